@@ -151,6 +151,11 @@ __device__ __forceinline__ dd operator*(dd a, dd b) { return as_dd(df_mul(as_df(
 __device__ __forceinline__ dd operator-(dd a) { return dd(-a.hi, -a.lo); }
 __device__ __forceinline__ double to_double(dd a) { return f64_of(a.hi) + f64_of(a.lo); }
 __device__ __forceinline__ double to_double(double a) { return a; }
+// a / 2 (exact) and a n, n a small whole number
+__device__ __forceinline__ dd halved(dd a) { return dd(0.5f * a.hi, 0.5f * a.lo); }
+__device__ __forceinline__ double halved(double a) { return 0.5 * a; }
+__device__ __forceinline__ dd scaled(dd a, int n) { return as_dd(df_mul(as_df(a), (float)n)); }
+__device__ __forceinline__ double scaled(double a, int n) { return n * a; }
 // nearest FP32 (the high part of a normalised pair)
 __device__ __forceinline__ float to_float(dd a) { return a.hi; }
 __device__ __forceinline__ float to_float(double a) { return (float)a; }

@@ -546,25 +546,20 @@ __global__ void __launch_bounds__(128) k_sums(Params P, const T2* __restrict__ f
 // in the FP64 form; first-order terms FP64 and slope-carrying terms FP32 in the FP32-f form.
 // -------------------------------------------------------------------------------------
 
-// Moments <x^n>, n = 0..6, of the normalised 1D Gaussian sqrt(lam/pi) exp(-lam (x-U)^2):
-// full range, x > 0 and x < 0.  Integration by parts gives
-// <x^{n+2}> = U <x^{n+1}> + (n+1)/(2 lam) <x^n> on every range.
-// h = 1/(2 lam); the starting values come from gauss_half_start (FP64): the half-range
-// masses mp0, mn0 and e = <x>_{x>0} - U mp0 = sqrt(lam/pi) exp(-lam U^2) / (2 lam).
+// Central half-range moments m_n = <x^n>, x = u - U, n = 0..6, of the normalised 1D Gaussian
+// sqrt(lam/pi) exp(-lam x^2) over u > 0 or u < 0: integration by parts gives
+// m_{n+2} = (n+1) h m_n + (-U)^{n+1} e with h = 1/(2 lam) and the range's starting values from
+// gauss_half_start (FP64): m0 its mass (mp0 or mn0) and e = m_1 = +-h sqrt(lam/pi) exp(-lam U^2).
 template <typename T>
-__device__ void gauss_moments7(T U, T h, T mp0, T mn0, T e, T* M, T* Mp, T* Mn) {
-  M[0] = T(1);
-  M[1] = U;
-  Mp[0] = mp0;
-  Mn[0] = mn0;
-  Mp[1] = U * Mp[0] + e;
-  Mn[1] = U * Mn[0] - e;
+__device__ __forceinline__ void gauss_central7(T U, T h, T m0, T e, T* m) {
+  m[0] = m0;
+  m[1] = e;
+  const T nU = -U;
+  T z = e;  // (-U)^n e
 #pragma unroll
   for (int n = 0; n < 5; n++) {
-    const T nh = T(n + 1) * h;
-    M[n + 2] = U * M[n + 1] + nh * M[n];
-    Mp[n + 2] = U * Mp[n + 1] + nh * Mp[n];
-    Mn[n + 2] = U * Mn[n + 1] + nh * Mn[n];
+    z = z * nU;
+    m[n + 2] = scaled(h, n + 1) * m[n] + z;
   }
 }
 // One erfc: the half-range mass on the far side of U is erfc(sqrt(lam)|U|)/2, the near side
@@ -588,61 +583,59 @@ __device__ void gauss_moments7_full(T U, T h, T* M) {
   for (int n = 0; n < 5; n++) M[n + 2] = U * M[n + 1] + T(n + 1) * h * M[n];
 }
 
-// <u^a v^b psi> for the normalised Maxwellian, u-moments Mu (one range), v-moments Mv,
-// <xi^2> = X2.
-template <typename T>
-__device__ __forceinline__ void psi_mom(const T* Mu, const T* Mv, T X2, int a, int b, T* o) {
-  o[0] = Mu[a] * Mv[b];
-  o[1] = Mu[a + 1] * Mv[b];
-  o[2] = Mu[a] * Mv[b + 1];
-  o[3] = T(0.5) * (Mu[a + 2] * Mv[b] + Mu[a] * Mv[b + 2] + Mu[a] * Mv[b] * X2);
-}
-// <u^a v^b psi (c . psi)>, c . psi = c1 + c2 u + c3 v + c4 (u^2 + v^2 + xi^2)/2, from the
-// factorised moments: with M(p, q) = Mu[p] Mv[q] and h = c4/2,
-//   T(p, q) = <u^p v^q (c . psi)> = Mu[p] A(q) + Mu[p+1] c2 Mv[q] + Mu[p+2] h Mv[q],
-//   A(q) = (c1 + h X2) Mv[q] + c3 Mv[q+1] + h Mv[q+2];
-// the components are T(a, b), T(a+1, b), T(a, b+1), and for the energy
-// (T(a+2, b) + T(a, b+2) + X2 T(a, b) + h (X4 - X2^2) M(a, b)) / 2, since
-// <xi^2 (c . psi)> = X2 (c . psi with xi^2 -> X2) + h (X4 - X2^2).
-// The tables A, B, C depend on (c, Mv, b) only and are shared by evaluations at several
-// (Mu, a); X4m = X4 - X2^2.
-template <typename T>
-struct APsi {
-  T A[3], B[3], C[3], h, mvb;
-};
-template <typename T>
-__device__ __forceinline__ void apsi_prep(const T* Mv, T X2, int b, const T* c, APsi<T>& t) {
-  t.h = T(0.5) * c[3];
-  const T c0x = c[0] + t.h * X2;
-#pragma unroll
-  for (int q = 0; q < 3; q++) {
-    t.A[q] = c0x * Mv[b + q] + c[2] * Mv[b + q + 1] + t.h * Mv[b + q + 2];
-    t.B[q] = c[1] * Mv[b + q];
-    t.C[q] = t.h * Mv[b + q];
-  }
-  t.mvb = Mv[b];
-}
-template <typename T>
-__device__ __forceinline__ void apsi_eval(const APsi<T>& t, const T* Mu, T X2, T X4m, int a, T* o) {
-  auto Tm = [&](int p, int q) { return Mu[a + p] * t.A[q] + Mu[a + p + 1] * t.B[q] + Mu[a + p + 2] * t.C[q]; };
-  const T t00 = Tm(0, 0);
-  o[0] = t00;
-  o[1] = Tm(1, 0);
-  o[2] = Tm(0, 1);
-  o[3] = T(0.5) * (Tm(2, 0) + Tm(0, 2) + X2 * t00 + t.h * X4m * (Mu[a] * t.mvb));
-}
+// S2-S5 in the frame that moves with the interface: x = un - U, y = ut - V and
+// psi' = (1, x, y, (x^2 + y^2 + xi^2)/2).  There the y and xi averages of the Maxwellian are
+// closed forms of h = 1/(2 lam) (<y^2> = h, <y^4> = 3 h^2, <xi^2> = K h,
+// <(y^2 + xi^2)^2> = (K+1)(K+3) h^2, odd powers 0), the moment matrix of the slope solve is
+// diagonal but for one entry, and every full-range moment of a slope is a moment of its own
+// solve (<psi' (a . psi')> = s').  About 310 operations against 530 with the moment tables of
+// the laboratory frame.
 
-// q = (K+2)/(4 lam) is the mean internal plus thermal energy per unit mass, c4 = lam/q.
+// s' = <psi' (a . psi)> of a slope target s = <psi (a . psi)>; ke = (U^2 + V^2)/2.
 template <typename T>
-__device__ void micro_slope(T U, T V, T lam, T q, T c4, const T* s, T* a) {
-  const T a4 = c4 * (T(2) * s[3] - T(2) * (U * s[1] + V * s[2]) + s[0] * (U * U + V * V - T(2) * q));
-  const T a3 = T(2) * lam * (s[2] - V * s[0]) - V * a4;
-  const T a2 = T(2) * lam * (s[1] - U * s[0]) - U * a4;
-  const T a1 = s[0] - U * a2 - V * a3 - a4 * (T(0.5) * (U * U + V * V) + q);
-  a[0] = a1;
-  a[1] = a2;
-  a[2] = a3;
-  a[3] = a4;
+__device__ __forceinline__ void to_moving(T U, T V, T ke, T* s) {
+  s[3] = s[3] - (U * s[1] + V * s[2]) + ke * s[0];
+  s[1] = s[1] - U * s[0];
+  s[2] = s[2] - V * s[0];
+}
+// Slope a (on psi') with <psi' (a . psi')> = s: q = (K+2) h / 2, il = 2 lam, c8 = 8 lam^2 / (K+2).
+template <typename T>
+__device__ __forceinline__ void micro_slope(T q, T il, T c8, const T* s, T* a) {
+  a[3] = c8 * (s[3] - q * s[0]);
+  a[1] = il * s[1];
+  a[2] = il * s[2];
+  a[0] = s[0] - q * a[3];
+}
+// The slope on psi = (1, un, ut, (un^2 + ut^2 + xi^2)/2) of a slope on psi'.
+template <typename T>
+__device__ __forceinline__ void to_lab(T U, T V, T ke, T* a) {
+  a[0] = a[0] - (U * a[1] + V * a[2]) + ke * a[3];
+  a[1] = a[1] - U * a[3];
+  a[2] = a[2] - V * a[3];
+}
+// Half-range moments of a normal slope: t = <un psi' (a . psi')>, n = <un^2 psi' (a . psi')>
+// over the range of the central moments m.  Averaged over y and xi, a . psi' is
+// p(x) = p0 + a1 x + (a3/2) x^2 with p0 = a0 + a3 (K+1) h / 2, its y moment is a2 h = s2', and
+// its moment with (y^2 + xi^2) is (K+1) h (p + a3 h).  With w_n = <un x^n> = U m_n + m_{n+1} and
+// d_n = <un x^n p>: t = (d0, d1, s2' w0, (d2 + (K+1) h (d0 + a3 h w0))/2), and since
+// un^2 = un (U + x), n = U t + (d1, d2, s2' w1, (d3 + (K+1) h (d1 + a3 h w1))/2).
+// k1h = (K+1) h; adds n to ns.
+template <typename T>
+__device__ __forceinline__ void half_moments(T U, T h, T k1h, const T* m, const T* a, T s2, T* t, T* ns) {
+  T w[6], d[4];
+#pragma unroll
+  for (int n = 0; n < 6; n++) w[n] = U * m[n] + m[n + 1];
+  const T p2 = halved(a[3]), p0 = a[0] + p2 * k1h, a3h = a[3] * h;
+#pragma unroll
+  for (int n = 0; n < 4; n++) d[n] = p0 * w[n] + a[1] * w[n + 1] + p2 * w[n + 2];
+  t[0] = d[0];
+  t[1] = d[1];
+  t[2] = s2 * w[0];
+  t[3] = halved(d[2] + k1h * (d[0] + a3h * w[0]));
+  ns[0] = ns[0] + (U * t[0] + d[1]);
+  ns[1] = ns[1] + (U * t[1] + d[2]);
+  ns[2] = ns[2] + (U * t[2] + s2 * w[1]);
+  ns[3] = ns[3] + (U * t[3] + halved(d[3] + k1h * (d[1] + a3h * w[1])));
 }
 
 // 1/n! as a constant expression (the loops that use it are unrolled).
@@ -752,7 +745,7 @@ __device__ __forceinline__ void wall_face_f32(const Params& P, bool isx, double 
 // Arithmetic: the primitive variables, exp and erfc of the half-range moments, tau and
 // Mt1..Mt5, the slope targets and the free-transport part of F in FP64; the moment
 // recurrences, the micro-slope solves, the compatibility moments and the equilibrium part of
-// F in T: double (FP64 form) or dd, double-FP32 on the FP32 pipe (FP32-f and DF64 forms,
+// F in T (in the frame that moves with the interface): double (FP64 form) or dd, double-FP32 on the FP32 pipe (FP32-f and DF64 forms,
 // about 2^-48 relative per operation, where FP64 would spend ~420 of its ~610 operations per
 // face on the 1/64-rate FP64 pipe).
 template <typename T>
@@ -816,66 +809,77 @@ __device__ __forceinline__ void face_core(const Params& P, const double* W0, con
   const double rl = rsqrt(lam);
   double mp0, mn0, e;
   gauss_half_start(U, lam, rl, mp0, mn0, e);
-  const T Ut = T(U), Vt = T(V), ht = T(h);
-  T Mu[7], Mup[7], Mun[7], Mv[7];
-  gauss_moments7<T>(Ut, ht, T(mp0), T(mn0), T(e), Mu, Mup, Mun);
-  gauss_moments7_full<T>(Vt, ht, Mv);
   const double X2 = 2.0 * K * ilam4, X4 = (K * K + 2.0 * K) * 4.0 * ilam4 * ilam4;
-  const T X2t = T(X2), X4m = T(X4 - X2 * X2);
   // S3: collision time tau = mu/p, mu = mu_ref T^omega, p = rho/(2 lam), and Mt1..Mt5 of
   // x = dt/tau (omega = 1/2: x = dt rho / (2 mu_ref sqrt(lam)))
   const double x = P.omega_half ? P.half_dt_mu * rho * rl : P.dt / collision_time(P, rho, lam);
   time_weights(P.dt, x, c.Mt);
   const double* Mt = c.Mt;
-  // S4: micro slopes
+  // S4: micro slopes a_L, a_R (normal), b (tangential), on psi' of the moving frame
   const double inv = irho * tdelta;
-  const T lamt = T(lam), q = T((K + 2) * ilam4), c4 = T(4.0 * lam * lam * P.inv_kp2);
-  T sL[4], sR[4], sT[4], sA[4];
+  const T Ut = T(U), Vt = T(V), ht = T(h), ke = halved(Ut * Ut + Vt * Vt);
+  const T q = scaled(halved(ht), K + 2), k1h = scaled(ht, K + 1), il = T(2.0 * lam);
+  const T c8 = T(8.0 * lam * lam * P.inv_kp2);
+  T t[4], sA[4] = {T(0.0), T(0.0), T(0.0), T(0.0)}, ns[4] = {T(0.0), T(0.0), T(0.0), T(0.0)};
+  // a_L on u > 0, then a_R on u < 0: one copy of the code for both (it is straight-line code
+  // run once per face, bound by instruction fetch on small meshes)
+#pragma unroll 1
+  for (int sd = 0; sd < 2; sd++) {
+    T s[4], m[7], a[4];
 #pragma unroll
-  for (int k = 0; k < 4; k++) {
-    sL[k] = T((W0[k] - WL[k]) * inv);
-    sR[k] = T((WR[k] - W0[k]) * inv);
-    sT[k] = T(St[k] * irho);
-  }
-  micro_slope<T>(Ut, Vt, lamt, q, c4, sL, c.aL);
-  micro_slope<T>(Ut, Vt, lamt, q, c4, sR, c.aR);
-  micro_slope<T>(Ut, Vt, lamt, q, c4, sT, c.b);
-  // moments of (u_n a_L, u_n a_R, u_t b) . psi g at the orders the compatibility condition
-  // (t) and the flux (n: one more u_n) need; each table is dropped once evaluated
-  T t1[4], t2[4], t3[4], n1[4], n2[4], n3[4], t4[4], p1[4];
-  {
-    APsi<T> tL;
-    apsi_prep<T>(Mv, X2t, 0, c.aL, tL);
-    apsi_eval<T>(tL, Mup, X2t, X4m, 1, t1);
-    apsi_eval<T>(tL, Mup, X2t, X4m, 2, n1);
-  }
-  {
-    APsi<T> tR;
-    apsi_prep<T>(Mv, X2t, 0, c.aR, tR);
-    apsi_eval<T>(tR, Mun, X2t, X4m, 1, t2);
-    apsi_eval<T>(tR, Mun, X2t, X4m, 2, n2);
-  }
-  {
-    APsi<T> tb;
-    apsi_prep<T>(Mv, X2t, 1, c.b, tb);
-    apsi_eval<T>(tb, Mu, X2t, X4m, 0, t3);
-    apsi_eval<T>(tb, Mu, X2t, X4m, 1, n3);
-  }
+    for (int k = 0; k < 4; k++) s[k] = T((sd == 0 ? W0[k] - WL[k] : WR[k] - W0[k]) * inv);
+    to_moving<T>(Ut, Vt, ke, s);
+    micro_slope<T>(q, il, c8, s, a);
+    gauss_central7<T>(Ut, ht, T(sd == 0 ? mp0 : mn0), T(sd == 0 ? e : -e), m);
+    half_moments<T>(Ut, ht, k1h, m, a, s[2], t, ns);
 #pragma unroll
-  for (int k = 0; k < 4; k++) sA[k] = -(t1[k] + t2[k] + t3[k]);
-  micro_slope<T>(Ut, Vt, lamt, q, c4, sA, c.A);
-  {
-    APsi<T> tA;
-    apsi_prep<T>(Mv, X2t, 0, c.A, tA);
-    apsi_eval<T>(tA, Mu, X2t, X4m, 1, t4);
+    for (int k = 0; k < 4; k++) sA[k] = sA[k] + t[k];
+    to_lab<T>(Ut, Vt, ke, a);
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      c.aR[k] = a[k];
+      if (sd == 0) c.aL[k] = a[k];
+    }
   }
-  // S5: equilibrium part of the macroscopic flux; S7 free transport part from the sums
-  psi_mom<T>(Mu, Mv, X2t, 1, 0, p1);
+  const T k4h = scaled(halved(ht), K + 4);  // <x^2 (x^2 + y^2 + xi^2)/2> = h k4h
+  {
+    // tangential: t = <ut psi' (b . psi')> and <un ut psi' (b . psi')> = U t + <x ut psi' (b . psi')>,
+    // ut = V + y, over the full range
+    T s[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) s[k] = T(St[k] * irho);
+    to_moving<T>(Ut, Vt, ke, s);
+    micro_slope<T>(q, il, c8, s, c.b);
+    const T y2 = ht * (s[0] + c.b[3] * ht);  // <y^2 (b . psi')> = <x^2 (b . psi')>
+    t[0] = Vt * s[0] + s[2];
+    t[1] = Vt * s[1];
+    t[2] = Vt * s[2] + y2;
+    t[3] = Vt * s[3] + k4h * s[2];
+    ns[0] = ns[0] + (Ut * t[0] + Vt * s[1]);
+    ns[1] = ns[1] + (Ut * t[1] + (Vt * y2 + ht * s[2]));
+    ns[2] = ns[2] + (Ut * t[2] + ht * s[1]);
+    ns[3] = ns[3] + (Ut * t[3] + Vt * (k4h * s[1]));
+#pragma unroll
+    for (int k = 0; k < 4; k++) sA[k] = -(sA[k] + t[k]);
+  }
+  // the compatibility condition gives the time slope A
+  micro_slope<T>(q, il, c8, sA, c.A);
+  // S5: equilibrium part of the macroscopic flux, on psi' and then on psi; S7 free transport
+  // part from the sums.  <un psi'> = (U, h, 0, U q);
+  // <un psi' (A . psi')> = U sA + (sA1, h (sA0 + A3 h), 0, k4h sA1)
   const T M1 = T(Mt[0]), M2 = T(Mt[1]), M3 = T(Mt[2]), rhot = T(rho);
+  T Fe[4];
+  Fe[0] = M1 * Ut + M2 * ns[0] + M3 * (Ut * sA[0] + sA[1]);
+  Fe[1] = M1 * ht + M2 * ns[1] + M3 * (Ut * sA[1] + ht * (sA[0] + c.A[3] * ht));
+  Fe[2] = M2 * ns[2] + M3 * (Ut * sA[2]);
+  Fe[3] = M1 * (Ut * q) + M2 * ns[3] + M3 * (Ut * sA[3] + k4h * sA[1]);
+  Fe[3] = Fe[3] + (Ut * Fe[1] + Vt * Fe[2]) + ke * Fe[0];
+  Fe[1] = Fe[1] + Ut * Fe[0];
+  Fe[2] = Fe[2] + Vt * Fe[0];
 #pragma unroll
-  for (int k = 0; k < 4; k++)
-    F[k] = to_double(rhot * (M1 * p1[k] + M2 * (n1[k] + n2[k] + n3[k]) + M3 * t4[k])) + Mt[3] * Sf[k] -
-           Mt[4] * Ss[k];
+  for (int k = 0; k < 4; k++) F[k] = to_double(rhot * Fe[k]) + Mt[3] * Sf[k] - Mt[4] * Ss[k];
+  to_lab<T>(Ut, Vt, ke, c.b);
+  to_lab<T>(Ut, Vt, ke, c.A);
   c.rho = rho;
   c.U = U;
   c.V = V;
