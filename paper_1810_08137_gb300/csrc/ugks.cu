@@ -49,13 +49,14 @@ struct ugks_ctx {
   float2* gdf = nullptr;
   int nchunk_neg = 0, nchunk_pos = 0;
   int sums_split = 1;        // FP32 form: warps per cell of the sums kernel (velocity-space split)
+  bool sums_tiled = false;   // FP32 form: sums with one thread per cell
   double* hs = nullptr;      // Shakhov model: heat-flux moment sums, kNHeat per cell
   CellShkF* cshk = nullptr;  // Shakhov model, FP32-f form: per-cell Shakhov factors
   // FP32 form: the step runs the batch kernels over a one-instance table, so an instance
   // stepped alone executes exactly the code it executes inside a batch
   SlotDev* d_slot = nullptr;
   BatchWork* d_work = nullptr;
-  int grid1[kPhases] = {0};
+  int grid1[16] = {0};       // per step kernel: blocks of its launch
   double* rpart = nullptr;
   int nrblocks = 0;
   int* err = nullptr;
@@ -195,7 +196,7 @@ size_t predict_bytes(const ugks_config* c) {
   if (f32) {
     const size_t row_d = nx * nq * 2 * sizeof(double);
     b += 2 * stage_half_bytes(row_d, ny) + sizeof(float4) * fs + sizeof(double2) * nq +
-         sizeof(float) * (12 * pr_all + 2 * (size_t)c->nu);
+         sizeof(float) * (12 * (pr_all + 1) + 14 * (size_t)c->nu);
     b += sizeof(SlotDev) + sizeof(BatchWork);
   }
   return b;
@@ -254,6 +255,7 @@ cudaError_t launch_step_f32(ugks_ctx* h, cudaStream_t st);
 cudaError_t setup_single_f32(ugks_ctx* h);
 cudaError_t upload_single_f32(ugks_ctx* h);
 int auto_sums_split(const Params& P, int sms);
+bool use_sums_tiles(const Params& P, int split, int sms);
 SlotDev slot_desc(const ugks_ctx* h, int walk_rows, int walk_vtile = 0);
 
 template <typename T>
@@ -888,6 +890,11 @@ ugks_status ugks_create(const ugks_config* cfg, void* cuda_stream, ugks_handle* 
   P.m_neg = 0;
   for (int m = 0; m < P.nv; m++)
     if (h->hv[m] < 0) P.m_neg = m + 1;
+  P.k_pos = P.nu;
+  for (int k = 0; k < P.nu; k++)
+    if (h->hu[k] > 0) { P.k_pos = k; break; }
+  for (int k = 0; k < P.nu; k++)
+    if (h->hu[k] < 0) P.k_neg = k + 1;
   {
     const std::pair<int, int> rp = f32_row_pairs(P.nv, cfg->vmin, cfg->vmax);
     P.pr_neg = rp.first;
@@ -1004,7 +1011,7 @@ ugks_status ugks_create(const ugks_config* cfg, void* cuda_stream, ugks_handle* 
     h->stage_bytes = 2 * stage_half_bytes(row_d, P.ny);
     ok = alloc((void**)&h->stage, h->stage_bytes) && alloc((void**)&h->gref4, sizeof(float4) * (size_t)P.fs) &&
          alloc((void**)&h->grefd, sizeof(double2) * (size_t)P.nq) &&
-         alloc((void**)&h->ftab, sizeof(float) * (12 * (size_t)P.pr_all + 2 * (size_t)P.nu));
+         alloc((void**)&h->ftab, sizeof(float) * (12 * ((size_t)P.pr_all + 1) + 14 * (size_t)P.nu));
     if (ok) {
       e = cudaStreamCreateWithFlags(&h->xstream, cudaStreamNonBlocking);
       for (int b = 0; b < 2 && e == cudaSuccess; b++) {
@@ -1055,8 +1062,9 @@ ugks_status ugks_create(const ugks_config* cfg, void* cuda_stream, ugks_handle* 
   }
   std::vector<float> ftab_host;
   if (h->ftab) {
-    // [pr_all][12]: (w0 w0' w1 w1') (w2 w2' w3 w3') (w4 w4' v v'), then u[nu], wu[nu]
-    ftab_host.assign(12 * (size_t)P.pr_all + 2 * (size_t)P.nu, 0.f);
+    // [pr_all][12]: (w0 w0' w1 w1') (w2 w2' w3 w3') (w4 w4' v v'), then [nu][12]: (w0 w0 w1 w1)
+    // (w2 w2 w3 w3) (w4 w4 u u) and a row of zeros, then u[nu], wu[nu]
+    ftab_host.assign(12 * ((size_t)P.pr_all + 1) + 14 * (size_t)P.nu, 0.f);
     const bool v0 = P.m_pos > P.m_neg;
     for (int pr = 0; pr < P.pr_all; pr++)
       for (int h2 = 0; h2 < 2; h2++) {
@@ -1070,11 +1078,17 @@ ugks_status ugks_create(const ugks_config* cfg, void* cuda_stream, ugks_handle* 
         t[10 + h2] = (float)vv;
       }
     for (int k = 0; k < P.nu; k++) {
-      ftab_host[12 * (size_t)P.pr_all + k] = (float)h->hu[k];
-      ftab_host[12 * (size_t)P.pr_all + P.nu + k] = (float)h->hwu[k];
+      float* t = &ftab_host[12 * ((size_t)P.pr_all + k)];
+      const double w = h->hu[k] == 0.0 ? 0.5 * h->hwu[k] : h->hwu[k];  // u = 0: half to each half
+      for (int n = 0; n < 5; n++) t[2 * n] = t[2 * n + 1] = (float)(w * std::pow(h->hu[k], n));
+      t[10] = t[11] = (float)h->hu[k];
+      float* uwf = &ftab_host[12 * ((size_t)P.pr_all + P.nu + 1)];
+      uwf[k] = (float)h->hu[k];
+      uwf[P.nu + k] = (float)h->hwu[k];
     }
     P.pwt = reinterpret_cast<const float4*>(h->ftab);
-    P.uwf = h->ftab + 12 * (size_t)P.pr_all;
+    P.uwt4 = P.pwt + 3 * (size_t)P.pr_all;
+    P.uwf = h->ftab + 12 * ((size_t)P.pr_all + P.nu + 1);
   }
   auto setup = [&]() -> cudaError_t {
     cudaError_t r;
@@ -1272,6 +1286,7 @@ ugks_status ugks_set_sums_split(ugks_handle h, int warps) {
   CK(cudaGetDevice(&dev));
   CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   h->sums_split = warps == 0 ? auto_sums_split(h->P, sms) : warps;
+  h->sums_tiled = use_sums_tiles(h->P, h->sums_split, sms);
   CK(upload_single_f32(h));
   for (int b = 0; b < 2; b++)  // the captured steps hold the old grid: capture them again
     if (h->graph[b]) {
@@ -1383,15 +1398,51 @@ struct ugks_batch_ctx {
   BatchWork* d_work = nullptr;
   BatchWork h_work;
   cudaGraphExec_t graph = nullptr;
-  int grid[kPhases + 1] = {0};
+  int grid[16] = {0};               // per step kernel: resident blocks
+  int kinds = 0;                    // kinds of the active instances (the captured launches)
   std::string last_error;
 };
 
 namespace {
 
-constexpr size_t kBatchSumsSmem = 0;  // the FP32-f sums kernel keeps its sums in registers
-// dynamic shared memory of the batch kernel of phase p
-constexpr size_t phase_smem(int p) { return p == 2 ? kBatchSumsSmem : (p == 5 ? kStripSmem : 0); }
+// Kernels of the FP32-f step: a phase has one kernel per kind of instance
+enum StepKernel { kGhostX, kGhostY, kSumsTile, kSumsSplit, kSumsShk, kFaces, kFacesShk, kCells, kStrip, kStripShk,
+                  kStepKernels };
+struct StepKernelInfo {
+  const void* fn;
+  size_t smem;   // dynamic shared memory
+  int phase;
+  int kinds;     // kinds of instances it serves (bits of instance_kind)
+};
+// 1: BGK, one thread per cell in the sums; 2: BGK, one or more warps per cell; 4: Shakhov
+int instance_kind(const ugks_ctx* h) { return h->P.shk ? 4 : (h->sums_tiled ? 1 : 2); }
+const StepKernelInfo kStepInfo[kStepKernels] = {
+    {(const void*)kb_ghost_x, 0, 0, 7},        {(const void*)kb_ghost_y, 0, 1, 7},
+    {(const void*)kb_sums_tile, kTileSmem, 2, 1}, {(const void*)kb_sums, 0, 2, 2},
+    {(const void*)kb_sums_shk, 0, 2, 4},       {(const void*)kb_faces, 0, 3, 3},
+    {(const void*)kb_faces_shk, 0, 3, 4},      {(const void*)kb_cells, 0, 4, 7},
+    {(const void*)kb_strip, kStripSmem, 5, 3}, {(const void*)kb_strip_shk, kStripSmem, 5, 4}};
+
+// Shared-memory limits of the step kernels, and their resident blocks on the whole device.
+cudaError_t step_grids(int* grid) {
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  for (int k = 0; k < kStepKernels && e == cudaSuccess; k++) {
+    int nb = 0;
+    if (kStepInfo[k].smem)
+      e = cudaFuncSetAttribute(kStepInfo[k].fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStepInfo[k].smem);
+    if (e == cudaSuccess)
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kStepInfo[k].fn, 128, kStepInfo[k].smem);
+    grid[k] = (nb > 0 ? nb : 1) * sms;
+  }
+  return e;
+}
+
+cudaError_t launch_kernel(int k, int grid, const SlotDev* slots, const BatchWork* work, cudaStream_t st) {
+  void* args[2] = {(void*)&slots, (void*)&work};
+  return cudaLaunchKernel(kStepInfo[k].fn, dim3(grid), dim3(128), args, kStepInfo[k].smem, st);
+}
 
 ugks_status bfail(ugks_batch_ctx* b, ugks_status s, const std::string& m) {
   if (b) b->last_error = m;
@@ -1428,6 +1479,7 @@ SlotDev slot_desc(const ugks_ctx* h, int walk_rows, int walk_vtile) {
   S.walk_rows = walk_rows;
   S.walk_vtile = walk_vtile;
   S.sums_split = h->sums_split;
+  S.sums_tiled = h->sums_tiled;
   S.cur = h->cur;
   return S;
 }
@@ -1436,9 +1488,11 @@ SlotDev slot_desc(const ugks_ctx* h, int walk_rows, int walk_vtile) {
 ugks_status upload_work(ugks_batch_ctx* b) {
   BatchWork& w = b->h_work;
   w.n = 0;
+  int kinds = 0;
   for (int p = 0; p < kPhases; p++) w.start[p][0] = 0;
   for (int s = 0; s < b->max_slots; s++) {
     if (!b->ctx[s]) continue;
+    kinds |= instance_kind(b->ctx[s]);
     const SlotDev S = slot_desc(b->ctx[s], b->walk_rows[s], b->walk_vtile[s]);
     const int a = w.n++;
     w.slot[a] = s;
@@ -1450,6 +1504,11 @@ ugks_status upload_work(ugks_batch_ctx* b) {
   }
   BCK(cudaMemcpyAsync(b->d_work, &w, sizeof(BatchWork), cudaMemcpyHostToDevice, b->stream));
   BCK(cudaStreamSynchronize(b->stream));  // w is host memory reused by the next update
+  if (kinds != b->kinds && b->graph && !b->persistent) {  // other kernels: capture again at the next step
+    BCK(cudaGraphExecDestroy(b->graph));
+    b->graph = nullptr;
+  }
+  b->kinds = kinds;
   return UGKS_OK;
 }
 
@@ -1478,15 +1537,11 @@ cudaError_t launch_batch(ugks_batch_ctx* b, cudaStream_t st) {
     lc.numAttrs = 1;
     return cudaLaunchKernelEx(&lc, kb_step, b->d_slots, (const BatchWork*)b->d_work, b->d_bar);
   }
-  kb_ghost_x<<<b->grid[0], 128, 0, st>>>(b->d_slots, b->d_work);
-  kb_ghost_y<<<b->grid[1], 128, 0, st>>>(b->d_slots, b->d_work);
-  kb_sums<<<b->grid[2], 128, kBatchSumsSmem, st>>>(b->d_slots, b->d_work);
-  kb_sums_shk<<<b->grid[2], 128, 0, st>>>(b->d_slots, b->d_work);  // Shakhov instances
-  kb_faces<<<b->grid[3], 128, 0, st>>>(b->d_slots, b->d_work);
-  kb_faces_shk<<<b->grid[3], 128, 0, st>>>(b->d_slots, b->d_work);
-  kb_cells<<<b->grid[4], 128, 0, st>>>(b->d_slots, b->d_work);
-  kb_strip<<<b->grid[5], 128, kStripSmem, st>>>(b->d_slots, b->d_work);
-  kb_strip_shk<<<b->grid[5], 128, kStripSmem, st>>>(b->d_slots, b->d_work);
+  for (int k = 0; k < kStepKernels; k++)
+    if (kStepInfo[k].kinds & b->kinds) {
+      const cudaError_t e = launch_kernel(k, b->grid[k], b->d_slots, b->d_work, st);
+      if (e != cudaSuccess) return e;
+    }
   kb_flip<<<1, 256, 0, st>>>(b->d_slots, b->d_work);
   return cudaGetLastError();
 }
@@ -1506,6 +1561,14 @@ int auto_sums_split(const Params& P, int sms) {
   return split;
 }
 
+// Sums with one thread per cell (sums_tile_body) where its tiles keep the device busy: from one
+// and a half blocks per SM.  Measured, warp per cell -> thread per cell, 28^2 velocities: 100x50
+// (169 tiles) 32.6 -> 38.3 us, 120x60 (256 tiles) 45.0 -> 38.9 us, 166x83 (462, just past a wave
+// of resident blocks) 76.6 -> 69.2 us, 800x400 1430 -> 842 us; 64^2: 120x60 175 -> 159 us.
+bool use_sums_tiles(const Params& P, int split, int sms) {
+  return !P.shk && split == 1 && 2L * tiles_x(P) * tiles_y(P) >= 3L * sms;
+}
+
 // Slot descriptor, one-instance work table and grid sizes of the FP32-f step (uploaded again
 // when a tile shape or the sums split changes).
 cudaError_t upload_single_f32(ugks_ctx* h) {
@@ -1515,18 +1578,12 @@ cudaError_t upload_single_f32(ugks_ctx* h) {
   memset(&w, 0, sizeof w);
   w.n = 1;
   w.slot[0] = 0;
-  int dev = 0, sms = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  const void* fns[kPhases] = {(const void*)kb_ghost_x, (const void*)kb_ghost_y, (const void*)kb_sums,
-                              (const void*)kb_faces, (const void*)kb_cells, (const void*)kb_strip};
-  for (int p = 0; p < kPhases; p++) {
-    w.start[p][1] = phase_blocks(S, p);
-    int nb = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fns[p], 128, phase_smem(p))) != cudaSuccess)
-      return e;
-    const int cap = (nb > 0 ? nb : 1) * sms;
-    h->grid1[p] = w.start[p][1] < cap ? (w.start[p][1] > 0 ? w.start[p][1] : 1) : cap;
+  for (int p = 0; p < kPhases; p++) w.start[p][1] = phase_blocks(S, p);
+  int cap[kStepKernels];
+  if ((e = step_grids(cap)) != cudaSuccess) return e;
+  for (int k = 0; k < kStepKernels; k++) {
+    const int want = w.start[kStepInfo[k].phase][1];
+    h->grid1[k] = want < 1 ? 1 : (want < cap[k] ? want : cap[k]);
   }
   if ((e = cudaMemcpy(h->d_slot, &S, sizeof(SlotDev), cudaMemcpyHostToDevice)) != cudaSuccess) return e;
   return cudaMemcpy(h->d_work, &w, sizeof(BatchWork), cudaMemcpyHostToDevice);
@@ -1542,41 +1599,20 @@ cudaError_t setup_single_f32(ugks_ctx* h) {
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   h->sums_split = auto_sums_split(h->P, sms);
-  if ((e = cudaFuncSetAttribute(kb_sums, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSumsSmem)) !=
-      cudaSuccess)
-    return e;
-  if ((e = cudaFuncSetAttribute(kb_strip, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStripSmem)) !=
-      cudaSuccess)
-    return e;
-  if ((e = cudaFuncSetAttribute(kb_strip_shk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStripSmem)) !=
-      cudaSuccess)
-    return e;
+  h->sums_tiled = use_sums_tiles(h->P, h->sums_split, sms);
   return upload_single_f32(h);
 }
 
 cudaError_t launch_step_f32(ugks_ctx* h, cudaStream_t st) {
   cudaError_t r;
-  if ((r = mark(h, 0)) != cudaSuccess) return r;
-  kb_ghost_x<<<h->grid1[0], 128, 0, st>>>(h->d_slot, h->d_work);
-  if ((r = mark(h, 1)) != cudaSuccess) return r;
-  kb_ghost_y<<<h->grid1[1], 128, 0, st>>>(h->d_slot, h->d_work);
-  if ((r = mark(h, 2)) != cudaSuccess) return r;
-  if (h->P.shk)  // the Shakhov model's sums, interface and walk
-    kb_sums_shk<<<h->grid1[2], 128, 0, st>>>(h->d_slot, h->d_work);
-  else
-    kb_sums<<<h->grid1[2], 128, kBatchSumsSmem, st>>>(h->d_slot, h->d_work);
-  if ((r = mark(h, 3)) != cudaSuccess) return r;
-  if (h->P.shk)
-    kb_faces_shk<<<h->grid1[3], 128, 0, st>>>(h->d_slot, h->d_work);
-  else
-    kb_faces<<<h->grid1[3], 128, 0, st>>>(h->d_slot, h->d_work);
-  if ((r = mark(h, 4)) != cudaSuccess) return r;
-  kb_cells<<<h->grid1[4], 128, 0, st>>>(h->d_slot, h->d_work);
-  if ((r = mark(h, 5)) != cudaSuccess) return r;
-  if (h->P.shk)
-    kb_strip_shk<<<h->grid1[5], 128, kStripSmem, st>>>(h->d_slot, h->d_work);
-  else
-    kb_strip<<<h->grid1[5], 128, kStripSmem, st>>>(h->d_slot, h->d_work);
+  const int kind = instance_kind(h);
+  int phase = -1;
+  for (int k = 0; k < kStepKernels; k++) {
+    if (!(kStepInfo[k].kinds & kind)) continue;
+    while (phase < kStepInfo[k].phase)
+      if ((r = mark(h, ++phase)) != cudaSuccess) return r;
+    if ((r = launch_kernel(k, h->grid1[k], h->d_slot, h->d_work, st)) != cudaSuccess) return r;
+  }
   kb_flip<<<1, 32, 0, st>>>(h->d_slot, h->d_work);
   if ((r = mark(h, 6)) != cudaSuccess) return r;
   if (h->profiling) h->events_used += UGKS_NKERNELS + 1;
@@ -1630,18 +1666,7 @@ ugks_status ugks_batch_create(int max_slots, size_t hbm_budget, void* cuda_strea
   int dev = 0, sms = 0;
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(kb_sums, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSumsSmem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(kb_strip, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStripSmem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(kb_strip_shk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStripSmem);
-  // persistent grids: resident blocks per SM x SMs
-  const void* fns[kPhases] = {(const void*)kb_ghost_x, (const void*)kb_ghost_y, (const void*)kb_sums,
-                              (const void*)kb_faces, (const void*)kb_cells, (const void*)kb_strip};
-  for (int p = 0; p < kPhases && e == cudaSuccess; p++) {
-    int nb = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fns[p], 128, phase_smem(p));
-    b->grid[p] = (nb > 0 ? nb : 1) * sms;
-  }
+  if (e == cudaSuccess) e = step_grids(b->grid);
   // persistent step: every block must be resident at once (cooperative launch)
   int coop = 0;
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);

@@ -31,6 +31,7 @@ struct SlotDev {
   int walk_rows;   // cell tile of the walk: rows per tile (autotuned per velocity-grid class)
   int walk_vtile;  // velocity tile of the walk: 32-slot chunks per tile, 0 = all (autotuned)
   int sums_split;  // warps per cell in the sums phase (1, 2 or 4): velocity-space split
+  int sums_tiled;  // sums with one thread per cell (sums_tile_body)
   int cur;         // ping-pong parity, flipped on the device after every step
 };
 
@@ -47,7 +48,9 @@ __host__ __device__ inline int phase_blocks(const SlotDev& S, int phase) {
   switch (phase) {
     case 0: return P.ny * 4;
     case 1: return (P.nx + 4) * 4;
-    case 2: return ((P.nx + 2) * (P.ny + 2) * S.sums_split + kWarpsPerBlock - 1) / kWarpsPerBlock;
+    case 2:
+      return S.sums_tiled ? tiles_x(P) * tiles_y(P)
+                           : ((P.nx + 2) * (P.ny + 2) * S.sums_split + kWarpsPerBlock - 1) / kWarpsPerBlock;
     case 3: return ((P.nx + 1) * P.ny + P.nx * (P.ny + 1) + 127) / 128;
     case 4: return S.nrblocks;
     default: {
@@ -101,11 +104,21 @@ __device__ __noinline__ void sums_phase(const SlotDev* __restrict__ slots, const
   for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
     const int a = find_instance(wk->start[2], wk->n, vb);
     const SlotDev& S = slots[wk->slot[a]];
-    if (S.P.shk) continue;  // Shakhov instances: sums_phase_shk
+    if (S.P.shk || S.sums_tiled) continue;  // sums_phase_shk, sums_tile_phase
     if (S.sums_split > 1)
       sums_body_split(S.P, S.f[S.cur], S.sums, vb - wk->start[2][a], S.sums_split, red);
     else
       sums_body_p<false>(S.P, S.f[S.cur], S.sums, vb - wk->start[2][a], 1, red);
+  }
+}
+
+__device__ __noinline__ void sums_tile_phase(const SlotDev* __restrict__ slots, const BatchWork* __restrict__ wk,
+                                             unsigned char* smem) {
+  const int total = wk->start[2][wk->n];
+  for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
+    const int a = find_instance(wk->start[2], wk->n, vb);
+    const SlotDev& S = slots[wk->slot[a]];
+    if (S.sums_tiled) sums_tile_body(S.P, S.f[S.cur], S.sums, vb - wk->start[2][a], smem);
   }
 }
 
@@ -275,6 +288,12 @@ __global__ void __launch_bounds__(128, 5) kb_sums(const SlotDev* __restrict__ sl
   sums_phase(slots, wk, red);
 }
 
+__global__ void __launch_bounds__(128, 3) kb_sums_tile(const SlotDev* __restrict__ slots,
+                                                    const BatchWork* __restrict__ wk) {
+  extern __shared__ __align__(16) unsigned char tile_sm[];  // kTileSmem bytes
+  sums_tile_phase(slots, wk, tile_sm);
+}
+
 // eight blocks per SM (64 registers, the rest on the stack): the interface is latency-bound
 // on its FP64 and double-FP32 chains, and 32 resident warps hide more of it than 12 (0.59 ->
 // 0.50 ms at 800x400x28^2; six blocks 0.52 ms)
@@ -366,7 +385,7 @@ __device__ __forceinline__ bool grid_sync(BarrierDev* g) {
 
 // dynamic shared memory of the persistent step: the largest phase's (the walk's rings; the
 // ghost tables and the cells reduction alias its start)
-constexpr size_t kStepSmem = kStripSmem;
+constexpr size_t kStepSmem = kStripSmem > kTileSmem ? kStripSmem : kTileSmem;
 static_assert(kStepSmem >= sizeof(double) * kGhostTab && kStepSmem >= sizeof(double) * 8 * 128 &&
                   kStepSmem >= sizeof(double) * kWarpsPerBlock * kNSum,
               "persistent step: shared memory of every phase");
@@ -382,6 +401,8 @@ __global__ void __launch_bounds__(128, 3) kb_step(SlotDev* __restrict__ slots,
   if (!grid_sync(bar)) return;
   sums_phase(slots, wk, reinterpret_cast<double(*)[kNSum]>(step_sm));
   sums_phase_shk(slots, wk);
+  __syncthreads();
+  sums_tile_phase(slots, wk, reinterpret_cast<unsigned char*>(step_sm));
   if (!grid_sync(bar)) return;
   faces_phase(slots, wk);
   faces_phase_shk(slots, wk);

@@ -470,6 +470,275 @@ __device__ __noinline__ void sums_body_split(const Params& P, const float4* __re
   sums_body_p<true>(P, f, sums, bx, split, red);
 }
 
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// 16-byte asynchronous copy to a shared-memory address, cached in L2 only
+__device__ __forceinline__ void cp_async16_cg_u(uint32_t sm, const void* gm) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sm), "l"(gm) : "memory");
+}
+
+// -------------------------------------------------------------------------------------
+// S1 + S7 with one thread per cell (meshes that fill the GPU with it, SlotDev::sums_tiled).  A block
+// owns a tile of 8 x 4 cells (lane = cell), its four warps the four quadrants of velocity space
+// (u >= 0 or u <= 0, v >= 0 or v <= 0), so a warp feeds one x side and one y side: 32 of the 64
+// face sums, in the registers of the thread that owns the cell.  No value crosses a lane: the
+// warp-per-cell kernel spends a third of its instructions on reducing its chunks across lanes,
+// and leaves lanes idle when nu is no multiple of 32.  A row pair of the quadrant is walked
+// along u; per row (packed pair) and with w_m = w_u u^m the thread sums
+//   A_m = sum w_m c_h (m < 4), X_m = sum w_m r_x,h (m < 5), Y_m = sum w_m r_y,h (m < 4),
+//   Ab_m (m < 2), Xb_m (m < 3), Yb_m (m < 2) of the b component,
+// from which the row's part of the 32 face sums follows with v and w_v.  The u = 0 column and
+// the v = 0 row enter both of their halves with half weight.
+// f is staged per warp, up to 8 slots of the 8 x 4 cells and their four-sided halo at a time,
+// with asynchronous copies one stage ahead; the 144-byte pitch of a cell puts the eight cells
+// of a row in different shared-memory banks.
+// What bounds it (400x200x28^2): latency at 12 warps per SM (168 registers, of them 72 sums):
+// issue 46 %, FMA pipe 38 %, shared-memory pipe 50 %, DRAM 2.6 TB/s; 64 instructions per
+// velocity-cell against 132 of the warp-per-cell kernel.  800x400x28^2: 1.431 -> 0.843 ms.
+// Stages of 8 slots 0.926 ms, 16 warps per SM (128 registers) 0.874 ms: more data in flight per
+// SM lowers the L2 hits of the halos.
+// Precision: FP32 sums over at most kTileSeg values of u in a row pair, these over at most
+// kTileTerms velocities of one cell; everything beyond in FP64 (as the warp-per-cell kernel, whose
+// chunks hold 8 rows x 32 lanes = 256 velocities).
+// -------------------------------------------------------------------------------------
+constexpr int kTileX = 8, kTileY = 4;            // cells of a tile
+constexpr int kTileSlots = 4;                    // slots per stage (at most)
+constexpr int kTileStages = 2;
+constexpr int kTileSeg = 16;                     // values of u per FP32 row sum
+constexpr int kTileTerms = 256;                  // velocities per FP32 chunk
+constexpr int kTilePitch = kTileSlots + 1;       // staged cell, in float4
+constexpr int kTileRow = kTileX + 2;             // staged cells per row
+constexpr int kTileStageF4 = (kTileY + 2) * kTileRow * kTilePitch;
+constexpr int kTileOut = 33;                     // doubles per face sum: 32 cells and a pad
+constexpr int kTileWarpBytes = kTileStages * kTileStageF4 * 16;
+static_assert(32 * kTileOut * 8 <= kTileWarpBytes, "the face sums reuse the staging buffers");
+constexpr size_t kTileSmem = (size_t)kWarpsPerBlock * kTileWarpBytes;
+
+__host__ __device__ __forceinline__ int tiles_x(const Params& P) { return (P.nx + 2 + kTileX - 1) / kTileX; }
+__host__ __device__ __forceinline__ int tiles_y(const Params& P) { return (P.ny + 2 + kTileY - 1) / kTileY; }
+
+__device__ __forceinline__ void sums_tile_body(const Params& P, const float4* __restrict__ f,
+                                               double* __restrict__ sums, int tile,
+                                               unsigned char* __restrict__ smem) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool un = warp & 1, vn = warp & 2;         // this warp's quadrant: u <= 0, v <= 0
+  const int nu = P.nu, fs = P.fs;
+  const int ntx = tiles_x(P);
+  const int x0 = (tile % ntx) * kTileX - 1, y0 = (tile / ntx) * kTileY - 1;  // first cell of the tile
+  const int tx = lane & 7, ty = lane >> 3;
+  const int i = x0 + tx, j = y0 + ty;
+  // a cell next to a pressure ghost (zero slopes) reads itself in place of its neighbours
+  const bool zs = (i < 0 && P.bc_kind[0] == 2) || (i >= P.nx && P.bc_kind[1] == 2) ||
+                  (j < 0 && P.bc_kind[2] == 2) || (j >= P.ny && P.bc_kind[3] == 2);
+  float4* st = reinterpret_cast<float4*>(smem + warp * kTileWarpBytes);
+  const int own = ((ty + 1) * kTileRow + tx + 1) * kTilePitch;
+  const int ox = zs ? 0 : kTilePitch, oy = zs ? 0 : kTileRow * kTilePitch;
+
+  // staging: lane (column lane / kTileSlots, slot lane % kTileSlots) copies every LC-th column of
+  // each of the 6 rows and its share of the left and right halo cells; rows and columns past the
+  // ghost ring repeat its last one
+  constexpr int LC = 32 / kTileSlots, NP = kTileX / LC;
+  const int sl = lane % kTileSlots, lc = lane / kTileSlots;
+  const size_t rs = (size_t)P.ex * fs;
+  const int xlast = P.nx + 1, yspan = P.ny + 2 - y0;  // last row the tile may read: y0 - 1 + yspan
+  const int hx = lc < LC / 2 ? x0 - 1 : min(x0 + kTileX, xlast), hr = lc % (LC / 2);
+  const float4* gcol = f + ((size_t)(y0 + 1) * P.ex + min(x0 + lc, xlast) + 2) * fs + sl;  // row y0 - 1
+  const float4* ghal = f + ((size_t)(min(y0 + hr, P.ny + 1) + 2) * P.ex + hx + 2) * fs + sl;
+  const int dcol2 = (min(x0 + lc + LC, xlast) - min(x0 + lc, xlast)) * fs;
+  const size_t dhal2 = (size_t)(min(y0 + hr + 2, P.ny + 1) - min(y0 + hr, P.ny + 1)) * rs;
+  const uint32_t dcol = smem_addr(st + (1 + lc) * kTilePitch + sl);
+  const uint32_t dhal = smem_addr(st + ((1 + hr) * kTileRow + (lc < LC / 2 ? 0 : kTileX + 1)) * kTilePitch + sl);
+
+  // u columns of the quadrant (u = 0 in both), in segments of kTileSeg; row pairs of the
+  // quadrant (for v <= 0 also the pair of the v = 0 row, with its other row at zero weight)
+  const int k0 = un ? 0 : P.k_neg, nk = (un ? P.k_pos : nu) - k0;
+  const int nseg = (nk + kTileSeg - 1) / kTileSeg;
+  const int pfirst = vn ? 0 : P.pr_neg, plast = vn ? P.pr_neg + (P.m_pos > P.m_neg ? 1 : 0) : P.pr_all;
+  const float4* uw = P.uwt4 + 3 * k0;
+  const float4* wt = P.pwt;
+  const float tdx = P.f_tdx, tdy = P.f_tdy;
+
+  // the next stage to be copied: segment, row pair, first column and end of the segment
+  int psg = 0, ppr = pfirst, pk = 0, pend = min(kTileSeg, nk);
+  uint32_t pslot = 0;
+  auto copy_stage = [&]() {
+    if (psg < nseg && ppr < plast) {
+      const int n = min(kTileSlots, pend - pk);
+      if (sl < n) {
+        const int s0 = ppr * nu + k0 + pk;
+        const float4* g = gcol + s0;
+        uint32_t d = dcol + pslot;
+#pragma unroll
+        for (int r = 0; r < kTileY + 2; r++) {
+          cp_async16_cg_u(d, g);
+          if (NP == 2) cp_async16_cg_u(d + LC * kTilePitch * 16, g + dcol2);
+          d += kTileRow * kTilePitch * 16;
+          if (r < yspan) g += rs;
+        }
+        cp_async16_cg_u(dhal + pslot, ghal + s0);
+        if (NP == 2) cp_async16_cg_u(dhal + pslot + 2 * kTileRow * kTilePitch * 16, ghal + s0 + dhal2);
+      }
+      pk += n;
+      if (pk >= pend) {
+        pk = pend - min(kTileSeg, nk - psg * kTileSeg);
+        if (++ppr == plast) {
+          ppr = pfirst;
+          pk = ++psg * kTileSeg;
+          pend = min(nk, pk + kTileSeg);
+        }
+      }
+      pslot ^= kTileStageF4 * 16;
+    }
+    cp_async_commit();
+  };
+
+  // FP64 face sums of the chunks done (local memory: touched once per chunk)
+  double accl[32];
+  double* acc = accl;
+  asm volatile("" : "+l"(acc));
+  float o[32];
+#pragma unroll
+  for (int e = 0; e < 32; e++) o[e] = 0.f;
+  int terms = 0;
+  bool first = true;
+  auto to_fp64 = [&]() {
+#pragma unroll
+    for (int e = 0; e < 32; e++) {
+      acc[e] = first ? (double)o[e] : acc[e] + (double)o[e];
+      o[e] = 0.f;
+    }
+    first = false;
+  };
+
+  copy_stage();
+  const float4* c = st + own;
+  int cflip = kTileStageF4;
+  for (int sg = 0; sg < nseg; sg++) {
+    const int ks = sg * kTileSeg, ke = min(nk, ks + kTileSeg);
+    for (int pr = pfirst; pr < plast; pr++) {
+      float2 A0, A1, A2, A3, X0, X1, X2, X3, X4, Y0, Y1, Y2, Y3, Ab0, Ab1, Xb0, Xb1, Xb2, Yb0, Yb1;
+      A0 = A1 = A2 = A3 = X0 = X1 = X2 = X3 = X4 = Y0 = Y1 = Y2 = Y3 = f2(0.f);
+      Ab0 = Ab1 = Xb0 = Xb1 = Xb2 = Yb0 = Yb1 = f2(0.f);
+      const float4* t = uw + 3 * ks;
+#pragma unroll 1
+      for (int k = ks; k < ke; k += kTileSlots) {
+        __syncwarp();  // every lane is done with the stage refilled next
+        copy_stage();
+        cp_async_wait<1>();
+        __syncwarp();
+        auto one = [&](const float4* cq, const float4* tq) {
+          const P4 C = ldp_s(cq), Wn = ldp_s(cq - ox), E = ldp_s(cq + ox);
+          const P4 S = ldp_s(cq - oy), N = ldp_s(cq + oy);
+          const float4 t0 = __ldg(tq), t1 = __ldg(tq + 1);
+          const float2 w4 = __ldg(reinterpret_cast<const float2*>(tq + 2));
+          const P4 rx = vl4(Wn, C, E), ry = vl4(S, C, N);
+          const float2 w0 = make_float2(t0.x, t0.y), w1 = make_float2(t0.z, t0.w);
+          const float2 w2 = make_float2(t1.x, t1.y), w3 = make_float2(t1.z, t1.w);
+          A0 = fma2(w0, C.h, A0); A1 = fma2(w1, C.h, A1); A2 = fma2(w2, C.h, A2); A3 = fma2(w3, C.h, A3);
+          X0 = fma2(w0, rx.h, X0); X1 = fma2(w1, rx.h, X1); X2 = fma2(w2, rx.h, X2);
+          X3 = fma2(w3, rx.h, X3); X4 = fma2(w4, rx.h, X4);
+          Y0 = fma2(w0, ry.h, Y0); Y1 = fma2(w1, ry.h, Y1); Y2 = fma2(w2, ry.h, Y2); Y3 = fma2(w3, ry.h, Y3);
+          Ab0 = fma2(w0, C.b, Ab0); Ab1 = fma2(w1, C.b, Ab1);
+          Xb0 = fma2(w0, rx.b, Xb0); Xb1 = fma2(w1, rx.b, Xb1); Xb2 = fma2(w2, rx.b, Xb2);
+          Yb0 = fma2(w0, ry.b, Yb0); Yb1 = fma2(w1, ry.b, Yb1);
+        };
+        // two slots at a time (their chains overlap), then an odd group's last one
+        const int n = min(kTileSlots, ke - k);
+        int q = 0;
+#pragma unroll 1
+        for (; q + 2 <= n; q += 2) {
+          one(c + q, t);
+          one(c + q + 1, t + 3);
+          t += 6;
+        }
+        if (q < n) {
+          one(c + q, t);
+          t += 3;
+        }
+        c += cflip;
+        cflip = -cflip;
+      }
+      // the row pair's part of the 32 face sums
+      const float4 wa = __ldg(wt + 3 * pr);
+      float2 w = make_float2(wa.x, wa.y);
+      const float4 wc = __ldg(wt + 3 * pr + 2);
+      float2 v = make_float2(wc.z, wc.w);
+      if (vn && pr == P.pr_neg) {  // the v = 0 row's half, nothing of its pair's other row
+        w.y = 0.f;
+      }
+      const float2 vv = mul2(v, v), wv = mul2(w, v), vt = mul2(v, f2(tdy));
+      const float2 sx = f2(un ? -1.f : 1.f), sy = f2(vn ? -1.f : 1.f);
+      // four face sums += g0 . x0, g1 . x1, g2 . x2, g3 . x3 (both rows)
+      auto add4s = [&](int e, float2 g0, float2 x0_, float2 g1, float2 x1_, float2 g2, float2 x2_, float2 g3,
+                       float2 x3_) {
+        o[e] = fmaf(g0.y, x0_.y, fmaf(g0.x, x0_.x, o[e]));
+        o[e + 1] = fmaf(g1.y, x1_.y, fmaf(g1.x, x1_.x, o[e + 1]));
+        o[e + 2] = fmaf(g2.y, x2_.y, fmaf(g2.x, x2_.x, o[e + 2]));
+        o[e + 3] = fmaf(g3.y, x3_.y, fmaf(g3.x, x3_.x, o[e + 3]));
+      };
+      auto en = [&](float2 q2, float2 q0, float2 b0) {  // energy component: (q2 + v^2 q0 + b0) / 2
+        return mul2(f2(0.5f), add2(fma2(vv, q0, q2), b0));
+      };
+      {  // x side: W0, tangential slope, Sf, Ss
+        const float2 F0 = fma2(sx, X0, A0), F1 = fma2(sx, X1, A1), F2 = fma2(sx, X2, A2), F3 = fma2(sx, X3, A3);
+        const float2 B0 = fma2(sx, Xb0, Ab0), B1 = fma2(sx, Xb1, Ab1);
+        add4s(kOffW0, w, F0, w, F1, wv, F0, w, en(F2, F0, B0));
+        const float2 wt_ = mul2(w, f2(tdy)), wvt = mul2(wv, f2(tdy));
+        add4s(kOffSt, wt_, Y0, wt_, Y1, wvt, Y0, wt_, en(Y2, Y0, Yb0));
+        add4s(kOffSf, w, F1, w, F2, wv, F1, w, en(F3, F1, B1));
+        const float2 Z1 = fma2(f2(tdx), X2, mul2(vt, Y1)), Z2 = fma2(f2(tdx), X3, mul2(vt, Y2));
+        const float2 Z3 = fma2(f2(tdx), X4, mul2(vt, Y3)), Zb = fma2(f2(tdx), Xb2, mul2(vt, Yb1));
+        add4s(kOffSs, w, Z1, w, Z2, wv, Z1, w, en(Z3, Z1, Zb));
+      }
+      {  // y side
+        const float2 F0 = fma2(sy, Y0, A0), F1 = fma2(sy, Y1, A1), F2 = fma2(sy, Y2, A2), B0 = fma2(sy, Yb0, Ab0);
+        const float2 ef = en(F2, F0, B0), wvv = mul2(w, vv);
+        add4s(16 + kOffW0, w, F0, w, F1, wv, F0, w, ef);
+        const float2 wt_ = mul2(w, f2(tdx)), wvt = mul2(wv, f2(tdx));
+        add4s(16 + kOffSt, wt_, X0, wt_, X1, wvt, X0, wt_, en(X2, X0, Xb0));
+        add4s(16 + kOffSf, wv, F0, wv, F1, wvv, F0, wv, ef);
+        const float2 D0 = fma2(f2(tdx), X1, mul2(vt, Y0)), D1 = fma2(f2(tdx), X2, mul2(vt, Y1));
+        const float2 D2 = fma2(f2(tdx), X3, mul2(vt, Y2)), Db = fma2(f2(tdx), Xb1, mul2(vt, Yb0));
+        add4s(16 + kOffSs, wv, D0, wv, D1, wvv, D0, wv, en(D2, D0, Db));
+      }
+      terms += 2 * (ke - ks);
+      if (terms + 2 * kTileSeg > kTileTerms) {
+        to_fp64();
+        terms = 0;
+      }
+    }
+  }
+  cp_async_wait<0>();
+  to_fp64();
+  __syncwarp();
+  {
+    double* out = reinterpret_cast<double*>(st) + lane;  // [32 face sums][cell]
+#pragma unroll
+    for (int e = 0; e < 32; e++) out[e * kTileOut] = acc[e];
+  }
+  __syncthreads();
+  // the quadrants' sums of each side, added in a fixed order: thread (entry, cell parity)
+  const bool xg = i < 0 || i >= P.nx, yg = j < 0 || j >= P.ny;
+  const unsigned need =  // cells whose sums are read: not corner ghosts, ghosts behind a wall, past the end
+      __ballot_sync(kFull, i <= P.nx && j <= P.ny && !(xg && yg) && !(i < 0 && P.bc_kind[0] == 1) &&
+                               !(i >= P.nx && P.bc_kind[1] == 1) && !(j < 0 && P.bc_kind[2] == 1) &&
+                               !(j >= P.ny && P.bc_kind[3] == 1));
+  {
+    const int e = threadIdx.x & (kNSum - 1), side = e >> 4, c0 = threadIdx.x >> 6;  // sides E W N S
+    const int el = (e & 15) + (side < 2 ? 0 : 16);
+    const int wa = side < 2 ? side : 2 * side - 4, wb = side < 2 ? side + 2 : 2 * side - 3;
+    const double* pa = reinterpret_cast<const double*>(smem + wa * kTileWarpBytes) + el * kTileOut + c0;
+    const double* pb = reinterpret_cast<const double*>(smem + wb * kTileWarpBytes) + el * kTileOut + c0;
+    double* row = sums + (size_t)wcell(P, x0 + c0, y0) * kNSum + e;
+#pragma unroll 1
+    for (int y = 0; y < kTileY; y++) {
+#pragma unroll
+      for (int x = 0; x < kTileX; x += 2)
+        if (need >> (8 * y + x + c0) & 1) row[x * kNSum] = pa[8 * y + x] + pb[8 * y + x];
+      row += (size_t)P.wx * kNSum;
+    }
+  }
+  __syncthreads();  // the block's next tile overwrites the partial sums
+}
 
 // -------------------------------------------------------------------------------------
 // S6 + S8 and Eq. 3 as an upwind strip walk.  For one velocity the micro flux through a face
@@ -500,7 +769,6 @@ constexpr size_t kStripSmem = (size_t)kWarpsPerBlock * kStripWarpF4 * sizeof(flo
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 
 // ---- bulk asynchronous copies (the tensor-memory-access unit) with mbarrier completion ----
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mbar_init(uint32_t bar, int count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }

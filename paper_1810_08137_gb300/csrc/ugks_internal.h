@@ -172,6 +172,9 @@ struct Params {
   // 2/dx, 2/dy, 1/dx, 1/dy
   double inv_kp2, half_dt_mu, quarter_dt_mu, d_tdx, d_tdy, d_idx, d_idy;
   const float* uwf;       // FP32 tables: [2][nu] u, wu
+  const float4* uwt4;     // FP32-f form: [nu + 1][3]: (w0 w0 w1 w1) (w2 w2 w3 w3) (w4 w4 u u),
+                          // w_m = wu u^m, half of wu at u = 0; the last row is zero
+  int k_neg, k_pos;       // number of u indices with u < 0; first u index with u > 0 (nu if none)
   const double* mvd;      // [5][nv] wv v^n, n = 0..4
   float f_tdx, f_tdy, f_idx, f_idy, f_dt;  // FP32 2/dx, 2/dy, 1/dx, 1/dy, dt
   int walk_wait_polls;    // FP32-f walk: bound of its wait for record copies (polls)
