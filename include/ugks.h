@@ -230,12 +230,12 @@ ugks_status ugks_fp64_rate(void* cuda_stream, double* gflops);
  * the step runs once per step for all active instances, as a persistent grid over a
  * device-resident table of (instance, tile) work items, and one step of the whole batch
  * is one CUDA graph replay.  By default the step is ONE cooperative launch of a persistent
- * kernel that runs the six phases (ghost x, ghost y, sums, interfaces, cells, walk) with a
- * grid-wide barrier between them; ugks_batch_set_persistent(b, 0) selects seven phase
- * launches instead (the same phase code and order of work).  Instances are admitted into free slots while the batch is in
- * use (admission checks an HBM budget) and retired when done; the table and each
- * instance's ping-pong parity live in device memory, so admission and retirement change
- * data, not the captured graph.  Each instance's results are bitwise those of the same
+ * kernel that runs the five phases (ghost ring, sums, interfaces, cells, walk) with a
+ * grid-wide barrier between them; ugks_batch_set_persistent(b, 0) selects one launch per
+ * phase instead (the same phase code and order of work).  Instances are admitted into free
+ * slots while the batch is in use (admission checks an HBM budget) and retired when done; the
+ * table and each instance's ping-pong parity live in device memory, so admission and retirement
+ * change data, not the captured graphs.  Each instance's results are bitwise those of the same
  * instance stepped alone with ugks_step (same kernels, same order of work). */
 typedef struct ugks_batch_ctx* ugks_batch;
 
@@ -270,7 +270,7 @@ ugks_status ugks_batch_step(ugks_batch b, int nsteps);
 ugks_status ugks_batch_sync(ugks_batch b);
 
 /* Step mode: enable != 0, one cooperative launch per step (the default where the device
- * supports cooperative launch); 0, seven phase launches.  Synchronises; UGKS_EINVAL if
+ * supports cooperative launch); 0, one launch per phase.  Synchronises; UGKS_EINVAL if
  * cooperative launch is unavailable. */
 ugks_status ugks_batch_set_persistent(ugks_batch b, int enable);
 int         ugks_batch_get_persistent(ugks_batch b);
@@ -280,8 +280,8 @@ int         ugks_batch_get_persistent(ugks_batch b);
  * up, ends the launch; ugks_batch_sync then reports UGKS_ETIMEOUT.  Synchronises. */
 ugks_status ugks_batch_set_wait_limit(ugks_batch b, unsigned long long polls);
 
-/* Tile shape of the f-update walk for one slot: the cell tile (rows per tile; a tile is
- * 4 columns wide) and the velocity tile (chunks of 32 velocity slots walked by consecutive
+/* Tile shape of the f-update walk for one slot: the cell tile (rows per tile, chosen by the
+ * library from the instances in flight until it is set or tuned; a tile is 4 columns wide) and the velocity tile (chunks of 32 velocity slots walked by consecutive
  * warps for the same cell tile; 0 = all chunks of the cell).  The autotuner: for each
  * velocity-grid class present (nu*nv <= 576, <= 1600, <= 4096, larger) it times
  * trial_steps batch steps for every cell tile of 16, 32, 64, 128 rows times velocity tile

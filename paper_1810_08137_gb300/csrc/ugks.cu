@@ -48,6 +48,7 @@ struct ugks_ctx {
   CellRecD* celld = nullptr;
   float2* gdf = nullptr;
   int nchunk_neg = 0, nchunk_pos = 0;
+  int walk_rows = kWalkRows; // FP32 form: rows per tile of the walk (stepped alone)
   int sums_split = 1;        // FP32 form: warps per cell of the sums kernel (velocity-space split)
   bool sums_tiled = false;   // FP32 form: sums with one thread per cell
   double* hs = nullptr;      // Shakhov model: heat-flux moment sums, kNHeat per cell
@@ -59,6 +60,8 @@ struct ugks_ctx {
   int grid1[16] = {0};       // per step kernel: blocks of its launch
   double* rpart = nullptr;
   int nrblocks = 0;
+  int face_block = 128;      // faces and cells per block of the interface and cell kernels
+  int cell_block = 128;
   int* err = nullptr;
   double* d_grid = nullptr;  // u[nu], v[nv], wu[nu], wv[nv], [5][nv] wv v^n
   double* stage = nullptr;   // FP64 staging for FP32 state conversion: two halves, stage_bytes
@@ -177,6 +180,11 @@ std::pair<int, int> f32_row_pairs(int nv, double vmin, double vmax) {
   return {pn, pn + (nv - mneg + 1) / 2};
 }
 
+// Threads per block of the interface and cell kernels (one thread per face or cell): one warp
+// where whole blocks would leave SMs idle (152 SMs), since their FP64 chains are bound by one SM's
+// FP64 pipe (2 operations per clock).  40x20: interface 36 -> 28 us, cells 15 -> 9 us.
+int small_block(long n) { return n < 152 * 128 ? 32 : 128; }
+
 // Device bytes ugks_create allocates for cfg (cudaMalloc sizes, without allocator rounding).
 size_t predict_bytes(const ugks_config* c) {
   const size_t nx = c->nx, ny = c->ny, nq = (size_t)c->nu * c->nv, nc = nx * ny;
@@ -184,7 +192,7 @@ size_t predict_bytes(const ugks_config* c) {
   const size_t pr_all = f32_row_pairs(c->nv, c->vmin, c->vmax).second, fs = pr_all * c->nu;
   const size_t fslot = f32 ? fs * sizeof(float4) : nq * sizeof(double2);  // f bytes per cell
   const size_t fcells = (nx + 4) * (ny + 4), nwe = (nx + 2) * (ny + 2);
-  const size_t nfx = (nx + 1) * ny, nfy = nx * (ny + 1), nrb = (nc + 127) / 128;
+  const size_t nfx = (nx + 1) * ny, nfy = nx * (ny + 1), cb = small_block(nc), nrb = (nc + cb - 1) / cb;
   size_t b = 2 * fcells * fslot + 2 * 4 * sizeof(double) * nwe + sizeof(double) * kNSum * nwe;
   if (shakhov_pr(c) != 1.0) b += sizeof(double) * kNHeat * nwe + (f32 ? sizeof(CellShkF) * nc : 0);
   b += f32 ? sizeof(FaceRecF) * (nfx + nfy) : (dfm ? sizeof(FaceRecD) : sizeof(FaceRec)) * (nfx + nfy);
@@ -256,7 +264,7 @@ cudaError_t setup_single_f32(ugks_ctx* h);
 cudaError_t upload_single_f32(ugks_ctx* h);
 int auto_sums_split(const Params& P, int sms);
 bool use_sums_tiles(const Params& P, int split, int sms);
-SlotDev slot_desc(const ugks_ctx* h, int walk_rows, int walk_vtile = 0);
+SlotDev slot_desc(const ugks_ctx* h, int par, int walk_rows, int walk_vtile = 0);
 
 template <typename T>
 cudaError_t launch_step(ugks_ctx* h, cudaStream_t st) {
@@ -271,9 +279,8 @@ cudaError_t launch_step(ugks_ctx* h, cudaStream_t st) {
   double* Wo = h->W[h->cur ^ 1];
   cudaError_t r;
   if ((r = mark(h, 0)) != cudaSuccess) return r;
-  k_ghost_x<T2><<<dim3(P.ny, 4), 128, 0, st>>>(P, fi, Wi, h->nwe);
+  k_ghost<T2><<<ghost_cells(P), 128, 0, st>>>(P, fi, Wi, h->nwe);
   if ((r = mark(h, 1)) != cudaSuccess) return r;
-  k_ghost_y<T2><<<dim3(P.nx + 4, 4), 128, 0, st>>>(P, fi, Wi, h->nwe);
   if ((r = mark(h, 2)) != cudaSuccess) return r;
   const int nce = (P.nx + 2) * (P.ny + 2);
   double* sums = h->sums;
@@ -281,11 +288,11 @@ cudaError_t launch_step(ugks_ctx* h, cudaStream_t st) {
       P, fi, sums, reinterpret_cast<T2*>(h->slopes));
   if ((r = mark(h, 3)) != cudaSuccess) return r;
   const int nf = (P.nx + 1) * P.ny + P.nx * (P.ny + 1);
-  k_faces<kRecF64><<<(nf + 127) / 128, 128, 0, st>>>(P, sums, Wi, h->nwe, h->fxr, h->fyr, h->Fx, h->Fy,
+  k_faces<kRecF64><<<(nf + h->face_block - 1) / h->face_block, h->face_block, 0, st>>>(P, sums, Wi, h->nwe, h->fxr, h->fyr, h->Fx, h->Fy,
                                                      h->mt4);
   if ((r = mark(h, 4)) != cudaSuccess) return r;
   const int nc = P.nx * P.ny;
-  k_cells<<<h->nrblocks, 128, 0, st>>>(P, Wi, Wo, h->nwe, h->Fx, h->Fy, h->cells, h->rpart, h->err,
+  k_cells<<<h->nrblocks, h->cell_block, 0, st>>>(P, Wi, Wo, h->nwe, h->Fx, h->Fy, h->cells, h->rpart, h->err,
                                        h->cellf, h->mt4);
   if ((r = mark(h, 5)) != cudaSuccess) return r;
   // the update in two passes: every face flux once, then Eq. 3 per velocity-cell
@@ -322,19 +329,18 @@ cudaError_t launch_step_df(ugks_ctx* h, cudaStream_t st) {
   DF4* sl = reinterpret_cast<DF4*>(h->slopes);
   cudaError_t r;
   if ((r = mark(h, 0)) != cudaSuccess) return r;
-  k_ghost_x<DF4><<<dim3(P.ny, 4), 128, 0, st>>>(P, fi, Wi, h->nwe);
+  k_ghost<DF4><<<ghost_cells(P), 128, 0, st>>>(P, fi, Wi, h->nwe);
   if ((r = mark(h, 1)) != cudaSuccess) return r;
-  k_ghost_y<DF4><<<dim3(P.nx + 4, 4), 128, 0, st>>>(P, fi, Wi, h->nwe);
   if ((r = mark(h, 2)) != cudaSuccess) return r;
   const int nce = (P.nx + 2) * (P.ny + 2);
   k_sums_df<<<(nce + kWarpsPerBlock - 1) / kWarpsPerBlock, 32 * kWarpsPerBlock, 0, st>>>(P, fi, h->sums, sl);
   if ((r = mark(h, 3)) != cudaSuccess) return r;
   const int nf = (P.nx + 1) * P.ny + P.nx * (P.ny + 1);
-  k_faces<kRecDF><<<(nf + 127) / 128, 128, 0, st>>>(P, h->sums, Wi, h->nwe, h->fxd, h->fyd, h->Fx, h->Fy,
+  k_faces<kRecDF><<<(nf + h->face_block - 1) / h->face_block, h->face_block, 0, st>>>(P, h->sums, Wi, h->nwe, h->fxd, h->fyd, h->Fx, h->Fy,
                                                     h->mt4);
   if ((r = mark(h, 4)) != cudaSuccess) return r;
   const int nc = P.nx * P.ny;
-  k_cells<<<h->nrblocks, 128, 0, st>>>(P, Wi, Wo, h->nwe, h->Fx, h->Fy, nullptr, h->rpart, h->err, nullptr,
+  k_cells<<<h->nrblocks, h->cell_block, 0, st>>>(P, Wi, Wo, h->nwe, h->Fx, h->Fy, nullptr, h->rpart, h->err, nullptr,
                                        h->mt4, h->celld);
   if ((r = mark(h, 5)) != cudaSuccess) return r;
   DF4* Xx = reinterpret_cast<DF4*>(h->xflux);
@@ -738,8 +744,7 @@ ugks_status ugks_step_noalloc(const ugks_config* cfg, const double* f_in, const 
                             W_in + (size_t)c * nc, nx * sizeof(double), nx * sizeof(double), ny,
                             cudaMemcpyDeviceToDevice, st));
   NA_CK(set_smem_limits_fp64(P.nv));
-  k_ghost_x<double2><<<dim3(ny, 4), 128, 0, st>>>(P, f0, W0, nwe);
-  k_ghost_y<double2><<<dim3(nx + 4, 4), 128, 0, st>>>(P, f0, W0, nwe);
+  k_ghost<double2><<<ghost_cells(P), 128, 0, st>>>(P, f0, W0, nwe);
   k_sums<double, double2><<<(nwe + kWarpsPerBlock - 1) / kWarpsPerBlock, 32 * kWarpsPerBlock,
                             smem_sums<double>(P.nv), st>>>(P, f0, sums, nullptr);
   k_faces<kRecF64><<<(nfx + nfy + 127) / 128, 128, 0, st>>>(P, sums, W0, nwe, fxr, fyr, Fx, Fy, mt4);
@@ -980,7 +985,9 @@ ugks_status ugks_create(const ugks_config* cfg, void* cuda_stream, ugks_handle* 
   h->nwe = (P.nx + 2) * (P.ny + 2);
   const size_t fbytes = h->fcells * (h->prec == UGKS_FP32F ? P.fs * sizeof(float4) : P.nq * sizeof(double2));
   const int nfx = (P.nx + 1) * P.ny, nfy = P.nx * (P.ny + 1), nc = P.nx * P.ny;
-  h->nrblocks = (nc + 127) / 128;
+  h->face_block = small_block(nfx + nfy);
+  h->cell_block = small_block(nc);
+  h->nrblocks = (nc + h->cell_block - 1) / h->cell_block;
   const bool f32 = h->prec == UGKS_FP32F, dfm = h->prec == UGKS_DF64;
   bool ok = alloc(&h->f[0], fbytes) && alloc(&h->f[1], fbytes) &&
             alloc((void**)&h->W[0], 4 * sizeof(double) * h->nwe) &&
@@ -1041,6 +1048,7 @@ ugks_status ugks_create(const ugks_config* cfg, void* cuda_stream, ugks_handle* 
   P.wu = h->d_grid + P.nu + P.nv;
   P.wv = h->d_grid + 2 * P.nu + P.nv;
   P.gref4 = h->gref4;
+  P.grefd = h->grefd;
   std::vector<float2> gdf_host;
   if (dfm) {
     // u[nu], wu[nu], v[nv], [5][nv] wv v^n and the mesh constants as double-FP32 pairs
@@ -1270,7 +1278,7 @@ ugks_status ugks_set_wait_limit(ugks_handle h, long long polls) {
   h->P.walk_wait_polls = polls > (1LL << 30) ? (1 << 30) : (int)polls;
   if (h->d_slot) {  // the FP32-f step reads its parameters from its slot descriptor
     CK(cudaStreamSynchronize(h->stream));
-    const SlotDev S = slot_desc(h, kWalkRows);
+    const SlotDev S = slot_desc(h, h->cur, h->walk_rows);
     CK(cudaMemcpy(h->d_slot, &S, sizeof(SlotDev), cudaMemcpyHostToDevice));
   }
   return UGKS_OK;
@@ -1389,7 +1397,8 @@ struct ugks_batch_ctx {
   int max_slots = 0;
   size_t budget = 0, used = 0;
   std::vector<ugks_ctx*> ctx;       // per slot, nullptr when free
-  std::vector<int> walk_rows;       // per slot: cell tile of the walk (rows)
+  std::vector<int> walk_rows;       // per slot: cell tile of the walk (rows), 0: automatic
+  std::vector<int> eff_rows;        // per slot: rows in use (0: descriptor not uploaded yet)
   std::vector<int> walk_vtile;      // per slot: velocity tile of the walk (chunks, 0 = all)
   bool persistent = false;          // one cooperative launch per step (else phase launches)
   int grid_step = 0;                // co-resident blocks of the persistent step kernel
@@ -1397,7 +1406,8 @@ struct ugks_batch_ctx {
   SlotDev* d_slots = nullptr;
   BatchWork* d_work = nullptr;
   BatchWork h_work;
-  cudaGraphExec_t graph = nullptr;
+  int par = 0;                      // parity of the next step
+  cudaGraphExec_t graph[2] = {nullptr, nullptr};  // captured step, per parity
   int grid[16] = {0};               // per step kernel: resident blocks
   int kinds = 0;                    // kinds of the active instances (the captured launches)
   std::string last_error;
@@ -1406,7 +1416,7 @@ struct ugks_batch_ctx {
 namespace {
 
 // Kernels of the FP32-f step: a phase has one kernel per kind of instance
-enum StepKernel { kGhostX, kGhostY, kSumsTile, kSumsSplit, kSumsShk, kFaces, kFacesShk, kCells, kStrip, kStripShk,
+enum StepKernel { kGhost, kSumsTile, kSumsWarp, kSumsShk, kFaces, kFacesShk, kCells, kStrip, kStripShk,
                   kStepKernels };
 struct StepKernelInfo {
   const void* fn;
@@ -1417,11 +1427,11 @@ struct StepKernelInfo {
 // 1: BGK, one thread per cell in the sums; 2: BGK, one or more warps per cell; 4: Shakhov
 int instance_kind(const ugks_ctx* h) { return h->P.shk ? 4 : (h->sums_tiled ? 1 : 2); }
 const StepKernelInfo kStepInfo[kStepKernels] = {
-    {(const void*)kb_ghost_x, 0, 0, 7},        {(const void*)kb_ghost_y, 0, 1, 7},
-    {(const void*)kb_sums_tile, kTileSmem, 2, 1}, {(const void*)kb_sums, 0, 2, 2},
-    {(const void*)kb_sums_shk, 0, 2, 4},       {(const void*)kb_faces, 0, 3, 3},
-    {(const void*)kb_faces_shk, 0, 3, 4},      {(const void*)kb_cells, 0, 4, 7},
-    {(const void*)kb_strip, kStripSmem, 5, 3}, {(const void*)kb_strip_shk, kStripSmem, 5, 4}};
+    {(const void*)kb_ghost, 0, 0, 7},          {(const void*)kb_sums_tile, kTileSmem, 1, 1},
+    {(const void*)kb_sums, 0, 1, 2},           {(const void*)kb_sums_shk, 0, 1, 4},
+    {(const void*)kb_faces, 0, 2, 3},          {(const void*)kb_faces_shk, 0, 2, 4},
+    {(const void*)kb_cells, 0, 3, 7},          {(const void*)kb_strip, kStripSmem, 4, 3},
+    {(const void*)kb_strip_shk, kStripSmem, 4, 4}};
 
 // Shared-memory limits of the step kernels, and their resident blocks on the whole device.
 cudaError_t step_grids(int* grid) {
@@ -1439,8 +1449,8 @@ cudaError_t step_grids(int* grid) {
   return e;
 }
 
-cudaError_t launch_kernel(int k, int grid, const SlotDev* slots, const BatchWork* work, cudaStream_t st) {
-  void* args[2] = {(void*)&slots, (void*)&work};
+cudaError_t launch_kernel(int k, int grid, const SlotDev* slots, const BatchWork* work, int par, cudaStream_t st) {
+  void* args[3] = {(void*)&slots, (void*)&work, (void*)&par};
   return cudaLaunchKernel(kStepInfo[k].fn, dim3(grid), dim3(128), args, kStepInfo[k].smem, st);
 }
 
@@ -1455,7 +1465,7 @@ ugks_status bfail(ugks_batch_ctx* b, ugks_status s, const std::string& m) {
     if (e_ != cudaSuccess) return bfail(b, UGKS_ECUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
   } while (0)
 
-SlotDev slot_desc(const ugks_ctx* h, int walk_rows, int walk_vtile) {
+SlotDev slot_desc(const ugks_ctx* h, int par, int walk_rows, int walk_vtile) {
   SlotDev S;
   memset(&S, 0, sizeof S);
   S.P = h->P;
@@ -1474,26 +1484,87 @@ SlotDev slot_desc(const ugks_ctx* h, int walk_rows, int walk_vtile) {
   S.err = h->err;
   S.nwe = h->nwe;
   S.nrblocks = h->nrblocks;
+  S.face_block = h->face_block;
+  S.cell_block = h->cell_block;
   S.nchunk_neg = h->nchunk_neg;
   S.nchunk_pos = h->nchunk_pos;
   S.walk_rows = walk_rows;
   S.walk_vtile = walk_vtile;
   S.sums_split = h->sums_split;
   S.sums_tiled = h->sums_tiled;
-  S.cur = h->cur;
+  S.cur = h->cur ^ par;
   return S;
 }
 
-// Rebuild the work table of the active slots and upload it (stream-ordered).
+// The captured steps are captured again at the next step.
+void drop_graphs(ugks_batch_ctx* b) {
+  for (int par = 0; par < 2; par++)
+    if (b->graph[par]) {
+      cudaGraphExecDestroy(b->graph[par]);
+      b->graph[par] = nullptr;
+    }
+}
+
+// Rows per tile of the walk for an instance that has `warps` resident warps to itself.  With
+// two waves or more of tiles of kWalkRows rows: equal tiles of at most that many (longer ones lose
+// the L2 hits of the strips' halos: 800x400x28^2 1.717 ms at 64 rows, 1.803 at 128; shorter ones
+// pay for their first face row and halo rows more often: 333x167x37^2 0.519 ms at 64, 0.549 at 14).
+// Below that the warps walk their tiles side by side and a step takes waves x (rows + 0.8) row
+// times: 40x20x20^2 one tile of 20 rows -> 1 row, 38.9 -> 14.1 us; 100x50x28^2 50 -> 10 rows,
+// 80 -> 39 us.
+int auto_walk_rows(const Params& P, int nchunk, long warps) {
+  const long per = (long)((P.nx + kStripW - 1) / kStripW) * nchunk;
+  const int tiles = (P.ny + kWalkRows - 1) / kWalkRows;
+  int best = (P.ny + tiles - 1) / tiles;
+  if (per * tiles >= 2 * warps) return best;
+  double best_t = 1e300;
+  for (int rows = 1; rows <= (P.ny < kWalkRows ? P.ny : kWalkRows); rows++) {
+    const long items = per * ((P.ny + rows - 1) / rows);
+    const double t = (double)((items + warps - 1) / warps) * (rows + 0.8);
+    if (t <= best_t) {
+      best_t = t;
+      best = rows;
+    }
+  }
+  return best;
+}
+
+ugks_status upload_slot(ugks_batch_ctx* b, int s) {
+  const SlotDev S = slot_desc(b->ctx[s], b->par, b->eff_rows[s], b->walk_vtile[s]);
+  BCK(cudaMemcpyAsync(b->d_slots + s, &S, sizeof(SlotDev), cudaMemcpyHostToDevice, b->stream));
+  BCK(cudaStreamSynchronize(b->stream));
+  return UGKS_OK;
+}
+
+// Choose the walk tiles, rebuild the work table of the active slots and upload both
+// (stream-ordered).  An instance without a set tile gets its share of the resident warps by
+// its velocity-cells.
 ugks_status upload_work(ugks_batch_ctx* b) {
   BatchWork& w = b->h_work;
+  double total = 0.0;
+  for (ugks_ctx* h : b->ctx)
+    if (h) total += (double)h->P.nx * h->P.ny * h->P.nq;
+  for (int s = 0; s < b->max_slots; s++) {
+    const ugks_ctx* h = b->ctx[s];
+    if (!h) continue;
+    int rows = b->walk_rows[s];
+    if (rows <= 0) {
+      const double share = (double)h->P.nx * h->P.ny * h->P.nq / total;
+      const long warps = (long)(share * b->grid[kStrip] * kWarpsPerBlock);
+      rows = auto_walk_rows(h->P, h->nchunk_neg + h->nchunk_pos, warps < 1 ? 1 : warps);
+    }
+    if (rows == b->eff_rows[s]) continue;
+    b->eff_rows[s] = rows;
+    const ugks_status r = upload_slot(b, s);
+    if (r) return r;
+  }
   w.n = 0;
   int kinds = 0;
   for (int p = 0; p < kPhases; p++) w.start[p][0] = 0;
   for (int s = 0; s < b->max_slots; s++) {
     if (!b->ctx[s]) continue;
     kinds |= instance_kind(b->ctx[s]);
-    const SlotDev S = slot_desc(b->ctx[s], b->walk_rows[s], b->walk_vtile[s]);
+    const SlotDev S = slot_desc(b->ctx[s], b->par, b->eff_rows[s], b->walk_vtile[s]);
     const int a = w.n++;
     w.slot[a] = s;
     for (int p = 0; p < kPhases; p++) {
@@ -1504,18 +1575,8 @@ ugks_status upload_work(ugks_batch_ctx* b) {
   }
   BCK(cudaMemcpyAsync(b->d_work, &w, sizeof(BatchWork), cudaMemcpyHostToDevice, b->stream));
   BCK(cudaStreamSynchronize(b->stream));  // w is host memory reused by the next update
-  if (kinds != b->kinds && b->graph && !b->persistent) {  // other kernels: capture again at the next step
-    BCK(cudaGraphExecDestroy(b->graph));
-    b->graph = nullptr;
-  }
+  if (kinds != b->kinds && !b->persistent) drop_graphs(b);  // other kernels
   b->kinds = kinds;
-  return UGKS_OK;
-}
-
-ugks_status upload_slot(ugks_batch_ctx* b, int s) {
-  const SlotDev S = slot_desc(b->ctx[s], b->walk_rows[s], b->walk_vtile[s]);
-  BCK(cudaMemcpyAsync(b->d_slots + s, &S, sizeof(SlotDev), cudaMemcpyHostToDevice, b->stream));
-  BCK(cudaStreamSynchronize(b->stream));
   return UGKS_OK;
 }
 
@@ -1535,14 +1596,13 @@ cudaError_t launch_batch(ugks_batch_ctx* b, cudaStream_t st) {
     lc.stream = st;
     lc.attrs = at;
     lc.numAttrs = 1;
-    return cudaLaunchKernelEx(&lc, kb_step, b->d_slots, (const BatchWork*)b->d_work, b->d_bar);
+    return cudaLaunchKernelEx(&lc, kb_step, (const SlotDev*)b->d_slots, (const BatchWork*)b->d_work, b->par, b->d_bar);
   }
   for (int k = 0; k < kStepKernels; k++)
     if (kStepInfo[k].kinds & b->kinds) {
-      const cudaError_t e = launch_kernel(k, b->grid[k], b->d_slots, b->d_work, st);
+      const cudaError_t e = launch_kernel(k, b->grid[k], b->d_slots, b->d_work, b->par, st);
       if (e != cudaSuccess) return e;
     }
-  kb_flip<<<1, 256, 0, st>>>(b->d_slots, b->d_work);
   return cudaGetLastError();
 }
 
@@ -1573,14 +1633,15 @@ bool use_sums_tiles(const Params& P, int split, int sms) {
 // when a tile shape or the sums split changes).
 cudaError_t upload_single_f32(ugks_ctx* h) {
   cudaError_t e;
-  const SlotDev S = slot_desc(h, kWalkRows);
+  int cap[kStepKernels];
+  if ((e = step_grids(cap)) != cudaSuccess) return e;
+  h->walk_rows = auto_walk_rows(h->P, h->nchunk_neg + h->nchunk_pos, (long)cap[kStrip] * kWarpsPerBlock);
+  const SlotDev S = slot_desc(h, h->cur, h->walk_rows);
   BatchWork w;
   memset(&w, 0, sizeof w);
   w.n = 1;
   w.slot[0] = 0;
   for (int p = 0; p < kPhases; p++) w.start[p][1] = phase_blocks(S, p);
-  int cap[kStepKernels];
-  if ((e = step_grids(cap)) != cudaSuccess) return e;
   for (int k = 0; k < kStepKernels; k++) {
     const int want = w.start[kStepInfo[k].phase][1];
     h->grid1[k] = want < 1 ? 1 : (want < cap[k] ? want : cap[k]);
@@ -1606,14 +1667,13 @@ cudaError_t setup_single_f32(ugks_ctx* h) {
 cudaError_t launch_step_f32(ugks_ctx* h, cudaStream_t st) {
   cudaError_t r;
   const int kind = instance_kind(h);
-  int phase = -1;
+  int next = 0;  // next event: the ring is the first of the step's six named parts, the second is empty
   for (int k = 0; k < kStepKernels; k++) {
     if (!(kStepInfo[k].kinds & kind)) continue;
-    while (phase < kStepInfo[k].phase)
-      if ((r = mark(h, ++phase)) != cudaSuccess) return r;
-    if ((r = launch_kernel(k, h->grid1[k], h->d_slot, h->d_work, st)) != cudaSuccess) return r;
+    while (next <= (kStepInfo[k].phase ? kStepInfo[k].phase + 1 : 0))
+      if ((r = mark(h, next++)) != cudaSuccess) return r;
+    if ((r = launch_kernel(k, h->grid1[k], h->d_slot, h->d_work, h->cur, st)) != cudaSuccess) return r;
   }
-  kb_flip<<<1, 32, 0, st>>>(h->d_slot, h->d_work);
   if ((r = mark(h, 6)) != cudaSuccess) return r;
   if (h->profiling) h->events_used += UGKS_NKERNELS + 1;
   return cudaGetLastError();
@@ -1628,7 +1688,7 @@ cudaError_t capture_batch(ugks_batch_ctx* b) {
   const cudaError_t el = launch_batch(b, b->cap_stream);
   e = cudaStreamEndCapture(b->cap_stream, &g);
   if (el != cudaSuccess) e = el;
-  if (e == cudaSuccess) e = cudaGraphInstantiate(&b->graph, g, 0);
+  if (e == cudaSuccess) e = cudaGraphInstantiate(&b->graph[b->par], g, 0);
   if (g) cudaGraphDestroy(g);
   return e;
 }
@@ -1657,7 +1717,8 @@ ugks_status ugks_batch_create(int max_slots, size_t hbm_budget, void* cuda_strea
   b->max_slots = max_slots;
   b->budget = hbm_budget;
   b->ctx.assign(max_slots, nullptr);
-  b->walk_rows.assign(max_slots, kWalkRows);
+  b->walk_rows.assign(max_slots, 0);
+  b->eff_rows.assign(max_slots, 0);
   b->walk_vtile.assign(max_slots, 0);
   memset(&b->h_work, 0, sizeof(BatchWork));
   cudaError_t e = cudaMalloc((void**)&b->d_slots, sizeof(SlotDev) * max_slots);
@@ -1699,7 +1760,7 @@ void ugks_batch_destroy(ugks_batch b) {
   if (b->stream) cudaStreamSynchronize(b->stream);
   for (ugks_ctx* h : b->ctx)
     if (h) ugks_destroy(h);
-  if (b->graph) cudaGraphExecDestroy(b->graph);
+  drop_graphs(b);
   if (b->cap_stream) {
     cudaStreamSynchronize(b->cap_stream);
     cudaStreamDestroy(b->cap_stream);
@@ -1730,7 +1791,7 @@ ugks_status ugks_batch_admit(ugks_batch b, const ugks_config* cfg, int* slot) {
   if (st) return bfail(b, st, "admit: instance allocation failed");
   b->ctx[s] = h;
   b->used += h->bytes;
-  int cls_rows = kWalkRows, cls_vt = 0;
+  int cls_rows = 0, cls_vt = 0;
   for (int k = 0; k < b->max_slots; k++)  // tuned tile of the same velocity class, if any
     if (k != s && b->ctx[k] && velocity_class(b->ctx[k]->cfg) == velocity_class(*cfg)) {
       cls_rows = b->walk_rows[k];
@@ -1738,8 +1799,8 @@ ugks_status ugks_batch_admit(ugks_batch b, const ugks_config* cfg, int* slot) {
     }
   b->walk_rows[s] = cls_rows;
   b->walk_vtile[s] = cls_vt;
-  ugks_status r = upload_slot(b, s);
-  if (!r) r = upload_work(b);
+  b->eff_rows[s] = 0;
+  ugks_status r = upload_work(b);
   if (r) {  // undo the admission: the caller gets no slot index to retire
     const std::string msg = b->last_error;
     cudaStreamSynchronize(b->stream);
@@ -1769,12 +1830,13 @@ ugks_handle ugks_batch_instance(ugks_batch b, int slot) {
 
 ugks_status ugks_batch_step(ugks_batch b, int nsteps) {
   if (!b || nsteps < 0) return bfail(b, UGKS_EINVAL, "batch step: bad argument");
-  if (!b->graph) {
-    const cudaError_t e = capture_batch(b);
-    if (e != cudaSuccess) return bfail(b, UGKS_ECUDA, std::string("batch capture: ") + cudaGetErrorString(e));
-  }
   for (int k = 0; k < nsteps; k++) {
-    BCK(cudaGraphLaunch(b->graph, b->stream));
+    if (!b->graph[b->par]) {
+      const cudaError_t e = capture_batch(b);
+      if (e != cudaSuccess) return bfail(b, UGKS_ECUDA, std::string("batch capture: ") + cudaGetErrorString(e));
+    }
+    BCK(cudaGraphLaunch(b->graph[b->par], b->stream));
+    b->par ^= 1;
     for (ugks_ctx* h : b->ctx)
       if (h) { h->cur ^= 1; h->steps_done++; }
   }
@@ -1788,14 +1850,6 @@ ugks_status ugks_batch_sync(ugks_batch b) {
   BCK(cudaMemcpy(&berr, &b->d_bar->err, sizeof(int), cudaMemcpyDeviceToHost));
   if (berr) {
     BCK(cudaMemset(&b->d_bar->err, 0, sizeof(int)));
-    // an interrupted launch did not flip the instances' buffers on the device: take each
-    // instance's parity back from the device so that state I/O addresses the right buffer
-    for (int s = 0; s < b->max_slots; s++)
-      if (b->ctx[s]) {
-        int cur = 0;
-        BCK(cudaMemcpy(&cur, &b->d_slots[s].cur, sizeof(int), cudaMemcpyDeviceToHost));
-        b->ctx[s]->cur = cur;
-      }
     return bfail(b, UGKS_ETIMEOUT,
                  "a grid barrier of the persistent step gave up waiting; the instances' states "
                  "are undefined (set them again)");
@@ -1811,12 +1865,11 @@ ugks_status ugks_batch_sync(ugks_batch b) {
 ugks_status ugks_batch_set_walk_rows(ugks_batch b, int slot, int rows) {
   if (!b || slot < 0 || slot >= b->max_slots || !b->ctx[slot] || rows < 1) return bfail(b, UGKS_EINVAL, "bad tile");
   b->walk_rows[slot] = rows;
-  ugks_status r = upload_slot(b, slot);
-  return r ? r : upload_work(b);
+  return upload_work(b);
 }
 
 int ugks_batch_get_walk_rows(ugks_batch b, int slot) {
-  return (b && slot >= 0 && slot < b->max_slots && b->ctx[slot]) ? b->walk_rows[slot] : 0;
+  return (b && slot >= 0 && slot < b->max_slots && b->ctx[slot]) ? b->eff_rows[slot] : 0;
 }
 
 ugks_status ugks_batch_set_walk_vtile(ugks_batch b, int slot, int chunks) {
@@ -1836,10 +1889,7 @@ ugks_status ugks_batch_set_persistent(ugks_batch b, int enable) {
   if (enable && !(b->grid_step > 0))
     return bfail(b, UGKS_EINVAL, "persistent step: cooperative launch unavailable on this device");
   BCK(cudaStreamSynchronize(b->stream));
-  if ((enable != 0) != b->persistent && b->graph) {
-    cudaGraphExecDestroy(b->graph);  // captured again at the next step
-    b->graph = nullptr;
-  }
+  if ((enable != 0) != b->persistent) drop_graphs(b);
   b->persistent = enable != 0;
   return UGKS_OK;
 }
@@ -1874,8 +1924,7 @@ ugks_status ugks_batch_tune(ugks_batch b, int trial_steps, double* best_ms) {
         if (b->ctx[s] && velocity_class(b->ctx[s]->cfg) == cls) {
           b->walk_rows[s] = rows;
           b->walk_vtile[s] = vt;
-          const ugks_status q = upload_slot(b, s);
-          if (q) return q;
+          b->eff_rows[s] = 0;
         }
       return upload_work(b);
     };

@@ -11,7 +11,7 @@
 namespace ugks {
 
 constexpr int kMaxSlots = 256;
-constexpr int kPhases = 6;  // ghost_x, ghost_y, sums, faces, cells, update (strip walk)
+constexpr int kPhases = 5;  // ghost ring, sums, faces, cells, update (strip walk)
 
 // What the phase kernels need about one instance.
 struct SlotDev {
@@ -32,7 +32,9 @@ struct SlotDev {
   int walk_vtile;  // velocity tile of the walk: 32-slot chunks per tile, 0 = all (autotuned)
   int sums_split;  // warps per cell in the sums phase (1, 2 or 4): velocity-space split
   int sums_tiled;  // sums with one thread per cell (sums_tile_body)
-  int cur;         // ping-pong parity, flipped on the device after every step
+  int face_block;  // faces per virtual block (32 spreads a small mesh over more SMs)
+  int cell_block;  // cells per virtual block
+  int cur;         // ping-pong parity in even steps: a step of parity par reads f[cur ^ par]
 };
 
 // Work table: virtual-block prefix sums per phase over the active instances.
@@ -46,13 +48,12 @@ struct BatchWork {
 __host__ __device__ inline int phase_blocks(const SlotDev& S, int phase) {
   const Params& P = S.P;
   switch (phase) {
-    case 0: return P.ny * 4;
-    case 1: return (P.nx + 4) * 4;
-    case 2:
+    case 0: return ghost_cells(P) * ghost_parts(P);
+    case 1:
       return S.sums_tiled ? tiles_x(P) * tiles_y(P)
                            : ((P.nx + 2) * (P.ny + 2) * S.sums_split + kWarpsPerBlock - 1) / kWarpsPerBlock;
-    case 3: return ((P.nx + 1) * P.ny + P.nx * (P.ny + 1) + 127) / 128;
-    case 4: return S.nrblocks;
+    case 2: return ((P.nx + 1) * P.ny + P.nx * (P.ny + 1) + S.face_block - 1) / S.face_block;
+    case 3: return S.nrblocks;
     default: {
       const long items = (long)((P.nx + kStripW - 1) / kStripW) *
                          ((P.ny + S.walk_rows - 1) / S.walk_rows) * (S.nchunk_neg + S.nchunk_pos);
@@ -76,98 +77,87 @@ __device__ __forceinline__ int find_instance(const int* start, int n, int vb) {
 // Not inlined: the persistent step and the phase kernels call the same compiled body, so an
 // instance's floating-point results do not depend on which of them runs it (inlined into
 // different kernels, the compiler may fuse a multiply and an add differently).
-__device__ __noinline__ void ghost_x_phase(const SlotDev* __restrict__ slots, const BatchWork* __restrict__ wk,
-                                              double* tab) {
+__device__ __noinline__ void ghost_phase(const SlotDev* __restrict__ slots, const BatchWork* __restrict__ wk, int par,
+                                         double* tab) {
   const int total = wk->start[0][wk->n];
   for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
     const int a = find_instance(wk->start[0], wk->n, vb);
     const SlotDev& S = slots[wk->slot[a]];
-    const int loc = vb - wk->start[0][a], c = S.cur;
-    ghost_x_body(S.P, S.f[c], S.W[c], S.nwe, loc % S.P.ny, loc / S.P.ny, tab);
+    const int c = S.cur ^ par;
+    ghost_body_f32(S.P, S.f[c], S.W[c], S.nwe, vb - wk->start[0][a], tab);
   }
 }
 
-__device__ __noinline__ void ghost_y_phase(const SlotDev* __restrict__ slots, const BatchWork* __restrict__ wk,
-                                              double* tab) {
+__device__ __noinline__ void sums_phase(const SlotDev* __restrict__ slots, const BatchWork* __restrict__ wk, int par,
+                                        double (*red)[kNSum]) {
   const int total = wk->start[1][wk->n];
   for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
     const int a = find_instance(wk->start[1], wk->n, vb);
     const SlotDev& S = slots[wk->slot[a]];
-    const int loc = vb - wk->start[1][a], c = S.cur, w = S.P.nx + 4;
-    ghost_y_body(S.P, S.f[c], S.W[c], S.nwe, loc % w, loc / w, tab);
-  }
-}
-
-__device__ __noinline__ void sums_phase(const SlotDev* __restrict__ slots, const BatchWork* __restrict__ wk,
-                                        double (*red)[kNSum]) {
-  const int total = wk->start[2][wk->n];
-  for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
-    const int a = find_instance(wk->start[2], wk->n, vb);
-    const SlotDev& S = slots[wk->slot[a]];
     if (S.P.shk || S.sums_tiled) continue;  // sums_phase_shk, sums_tile_phase
     if (S.sums_split > 1)
-      sums_body_split(S.P, S.f[S.cur], S.sums, vb - wk->start[2][a], S.sums_split, red);
+      sums_body_split(S.P, S.f[S.cur ^ par], S.sums, vb - wk->start[1][a], S.sums_split, red);
     else
-      sums_body_p<false>(S.P, S.f[S.cur], S.sums, vb - wk->start[2][a], 1, red);
+      sums_body_p<false>(S.P, S.f[S.cur ^ par], S.sums, vb - wk->start[1][a], 1, red);
   }
 }
 
-__device__ __noinline__ void sums_tile_phase(const SlotDev* __restrict__ slots, const BatchWork* __restrict__ wk,
+__device__ __noinline__ void sums_tile_phase(const SlotDev* __restrict__ slots, const BatchWork* __restrict__ wk, int par,
                                              unsigned char* smem) {
-  const int total = wk->start[2][wk->n];
+  const int total = wk->start[1][wk->n];
   for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
-    const int a = find_instance(wk->start[2], wk->n, vb);
+    const int a = find_instance(wk->start[1], wk->n, vb);
     const SlotDev& S = slots[wk->slot[a]];
-    if (S.sums_tiled) sums_tile_body(S.P, S.f[S.cur], S.sums, vb - wk->start[2][a], smem);
+    if (S.sums_tiled) sums_tile_body(S.P, S.f[S.cur ^ par], S.sums, vb - wk->start[1][a], smem);
   }
 }
 
 // The phases of the Shakhov model's instances (heat-flux sums, Shakhov interface, walk with
 // g+), over the same work table, skipping the BGK instances: functions and kernels of their
 // own, so that the BGK phases carry none of their code or registers.
-__device__ __noinline__ void sums_phase_shk(const SlotDev* __restrict__ slots, const BatchWork* __restrict__ wk) {
+__device__ __noinline__ void sums_phase_shk(const SlotDev* __restrict__ slots, const BatchWork* __restrict__ wk, int par) {
+  const int total = wk->start[1][wk->n];
+  for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
+    const int a = find_instance(wk->start[1], wk->n, vb);
+    const SlotDev& S = slots[wk->slot[a]];
+    if (S.P.shk) sums_body_p<false, true>(S.P, S.f[S.cur ^ par], S.sums, vb - wk->start[1][a], 1, nullptr);
+  }
+}
+
+__device__ __noinline__ void faces_phase(const SlotDev* __restrict__ slots, const BatchWork* __restrict__ wk, int par) {
   const int total = wk->start[2][wk->n];
   for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
     const int a = find_instance(wk->start[2], wk->n, vb);
     const SlotDev& S = slots[wk->slot[a]];
-    if (S.P.shk) sums_body_p<false, true>(S.P, S.f[S.cur], S.sums, vb - wk->start[2][a], 1, nullptr);
+    const int loc = vb - wk->start[2][a];
+    if (S.P.shk || (int)threadIdx.x >= S.face_block) continue;  // Shakhov instances: faces_phase_shk
+    faces_body<kRecF32>(S.P, S.sums, S.W[S.cur ^ par], S.nwe, S.fxf, S.fyf, S.Fx, S.Fy, S.mt4,
+                        loc * S.face_block + threadIdx.x);
   }
 }
 
-__device__ __noinline__ void faces_phase(const SlotDev* __restrict__ slots, const BatchWork* __restrict__ wk) {
-  const int total = wk->start[3][wk->n];
+__device__ __noinline__ void faces_phase_shk(const SlotDev* __restrict__ slots, const BatchWork* __restrict__ wk, int par) {
+  const int total = wk->start[2][wk->n];
   for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
-    const int a = find_instance(wk->start[3], wk->n, vb);
+    const int a = find_instance(wk->start[2], wk->n, vb);
     const SlotDev& S = slots[wk->slot[a]];
-    const int loc = vb - wk->start[3][a];
-    if (S.P.shk) continue;  // Shakhov instances: faces_phase_shk
-    faces_body<kRecF32>(S.P, S.sums, S.W[S.cur], S.nwe, S.fxf, S.fyf, S.Fx, S.Fy, S.mt4,
-                        loc * 128 + threadIdx.x);
+    if (!S.P.shk || (int)threadIdx.x >= S.face_block) continue;
+    const int loc = vb - wk->start[2][a];
+    faces_body<kRecF32, true>(S.P, S.sums, S.W[S.cur ^ par], S.nwe, S.fxf, S.fyf, S.Fx, S.Fy, S.mt4,
+                              loc * S.face_block + threadIdx.x);
   }
 }
 
-__device__ __noinline__ void faces_phase_shk(const SlotDev* __restrict__ slots, const BatchWork* __restrict__ wk) {
+__device__ __noinline__ void cells_phase(const SlotDev* __restrict__ slots, const BatchWork* __restrict__ wk, int par,
+                                            double (*red)[8]) {
   const int total = wk->start[3][wk->n];
-  for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
-    const int a = find_instance(wk->start[3], wk->n, vb);
-    const SlotDev& S = slots[wk->slot[a]];
-    if (!S.P.shk) continue;
-    const int loc = vb - wk->start[3][a];
-    faces_body<kRecF32, true>(S.P, S.sums, S.W[S.cur], S.nwe, S.fxf, S.fyf, S.Fx, S.Fy, S.mt4,
-                              loc * 128 + threadIdx.x);
-  }
-}
-
-__device__ __noinline__ void cells_phase(const SlotDev* __restrict__ slots, const BatchWork* __restrict__ wk,
-                                            double (*red)[128]) {
-  const int total = wk->start[4][wk->n];
   for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
     __syncthreads();  // red[] of the previous virtual block has been read
-    const int a = find_instance(wk->start[4], wk->n, vb);
+    const int a = find_instance(wk->start[3], wk->n, vb);
     const SlotDev& S = slots[wk->slot[a]];
-    const int c = S.cur;
+    const int c = S.cur ^ par;
     cells_body(S.P, S.W[c], S.W[c ^ 1], S.nwe, S.Fx, S.Fy, nullptr, S.rpart, S.err, S.cellf, S.mt4,
-               red, vb - wk->start[4][a]);
+               red, vb - wk->start[3][a], S.cell_block);
   }
 }
 
@@ -196,7 +186,7 @@ __device__ __forceinline__ void walk_item(const SlotDev& S, int ns, int nt, int 
 // Update sweep: one warp per work item (strip, row tile, velocity chunk).
 // Returns the record stages this warp has issued on its mbarriers (the Shakhov walk of the
 // persistent step continues on them).
-__device__ __noinline__ unsigned strip_phase(const SlotDev* __restrict__ slots, const BatchWork* __restrict__ wk,
+__device__ __noinline__ unsigned strip_phase(const SlotDev* __restrict__ slots, const BatchWork* __restrict__ wk, int par,
                                              float4* strip_sm) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // this warp's two mbarriers of the record ring (shared memory may have served another
@@ -211,15 +201,15 @@ __device__ __noinline__ unsigned strip_phase(const SlotDev* __restrict__ slots, 
   __syncwarp();
   unsigned nrec = 0;
   bool ok = true;
-  const int total = wk->start[5][wk->n];
+  const int total = wk->start[4][wk->n];
   for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
-    const int a = find_instance(wk->start[5], wk->n, vb);
+    const int a = find_instance(wk->start[4], wk->n, vb);
     const SlotDev& S = slots[wk->slot[a]];
     const int ns = (S.P.nx + kStripW - 1) / kStripW, nt = (S.P.ny + S.walk_rows - 1) / S.walk_rows;
-    const int it = (vb - wk->start[5][a]) * kWarpsPerBlock + warp;
+    const int it = (vb - wk->start[4][a]) * kWarpsPerBlock + warp;
     const int nch = S.nchunk_neg + S.nchunk_pos;
     if (it < ns * nt * nch) {
-      const int c = S.cur;
+      const int c = S.cur ^ par;
       int bx, by, ck;
       walk_item(S, ns, nt, it, bx, by, ck);
       // full strips (all but the last of a row when kStripW does not divide nx) with the
@@ -240,7 +230,7 @@ __device__ __noinline__ unsigned strip_phase(const SlotDev* __restrict__ slots, 
 // The walk of the Shakhov model's instances (g+ in the collision term; any strip width).
 // init: initialise this warp's mbarriers (a launch of its own); otherwise continue on the
 // ones strip_phase initialised in the same launch, after its nrec0 record stages.
-__device__ __noinline__ void strip_phase_shk(const SlotDev* __restrict__ slots, const BatchWork* __restrict__ wk,
+__device__ __noinline__ void strip_phase_shk(const SlotDev* __restrict__ slots, const BatchWork* __restrict__ wk, int par,
                                              float4* strip_sm, bool init, unsigned nrec0) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float4* wsm = strip_sm + warp * kStripWarpF4;
@@ -253,16 +243,16 @@ __device__ __noinline__ void strip_phase_shk(const SlotDev* __restrict__ slots, 
   __syncwarp();
   unsigned nrec = nrec0;
   bool ok = true;
-  const int total = wk->start[5][wk->n];
+  const int total = wk->start[4][wk->n];
   for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
-    const int a = find_instance(wk->start[5], wk->n, vb);
+    const int a = find_instance(wk->start[4], wk->n, vb);
     const SlotDev& S = slots[wk->slot[a]];
     if (!S.P.shk) continue;
     const int ns = (S.P.nx + kStripW - 1) / kStripW, nt = (S.P.ny + S.walk_rows - 1) / S.walk_rows;
-    const int it = (vb - wk->start[5][a]) * kWarpsPerBlock + warp;
+    const int it = (vb - wk->start[4][a]) * kWarpsPerBlock + warp;
     const int nch = S.nchunk_neg + S.nchunk_pos;
     if (it < ns * nt * nch && ok) {
-      const int c = S.cur;
+      const int c = S.cur ^ par;
       int bx, by, ck;
       walk_item(S, ns, nt, it, bx, by, ck);
       ok = strip_body_p<kStripW, false, true>(S.P, S.f[c], S.f[c ^ 1], S.fxf, S.fyf, S.cellf, S.nchunk_neg,
@@ -271,67 +261,58 @@ __device__ __noinline__ void strip_phase_shk(const SlotDev* __restrict__ slots, 
   }
 }
 
-// ---- one kernel per phase (the step as a graph of seven launches) ------------------------
-__global__ void kb_ghost_x(const SlotDev* __restrict__ slots, const BatchWork* __restrict__ wk) {
+// ---- one kernel per phase (the step as a graph of five launches) -------------------------
+// par: parity of the step (each instance's ping-pong parity is its SlotDev::cur ^ par)
+__global__ void kb_ghost(const SlotDev* __restrict__ slots, const BatchWork* __restrict__ wk, int par) {
   __shared__ double tab[kGhostTab];
-  ghost_x_phase(slots, wk, tab);
-}
-
-__global__ void kb_ghost_y(const SlotDev* __restrict__ slots, const BatchWork* __restrict__ wk) {
-  __shared__ double tab[kGhostTab];
-  ghost_y_phase(slots, wk, tab);
+  ghost_phase(slots, wk, par, tab);
 }
 
 __global__ void __launch_bounds__(128, 5) kb_sums(const SlotDev* __restrict__ slots,
-                                               const BatchWork* __restrict__ wk) {
+                                               const BatchWork* __restrict__ wk, int par) {
   __shared__ double red[kWarpsPerBlock][kNSum];  // face sums of split cells
-  sums_phase(slots, wk, red);
+  sums_phase(slots, wk, par, red);
 }
 
 __global__ void __launch_bounds__(128, 3) kb_sums_tile(const SlotDev* __restrict__ slots,
-                                                    const BatchWork* __restrict__ wk) {
+                                                    const BatchWork* __restrict__ wk, int par) {
   extern __shared__ __align__(16) unsigned char tile_sm[];  // kTileSmem bytes
-  sums_tile_phase(slots, wk, tile_sm);
+  sums_tile_phase(slots, wk, par, tile_sm);
 }
 
 // eight blocks per SM (64 registers, the rest on the stack): the interface is latency-bound
 // on its FP64 and double-FP32 chains, and 32 resident warps hide more of it than 12 (0.59 ->
 // 0.50 ms at 800x400x28^2; six blocks 0.52 ms)
 __global__ void __launch_bounds__(128, 8) kb_faces(const SlotDev* __restrict__ slots,
-                                                const BatchWork* __restrict__ wk) {
-  faces_phase(slots, wk);
+                                                const BatchWork* __restrict__ wk, int par) {
+  faces_phase(slots, wk, par);
 }
 
 __global__ void __launch_bounds__(128) kb_cells(const SlotDev* __restrict__ slots,
-                                                const BatchWork* __restrict__ wk) {
-  __shared__ double red[8][128];
-  cells_phase(slots, wk, red);
+                                                const BatchWork* __restrict__ wk, int par) {
+  __shared__ double red[4][8];
+  cells_phase(slots, wk, par, red);
 }
 
 __global__ void __launch_bounds__(128, 3) kb_strip(const SlotDev* __restrict__ slots,
-                                                const BatchWork* __restrict__ wk) {
+                                                const BatchWork* __restrict__ wk, int par) {
   extern __shared__ __align__(16) float4 strip_sm[];  // kStripSmem bytes
-  strip_phase(slots, wk, strip_sm);
+  strip_phase(slots, wk, par, strip_sm);
 }
 
 // The Shakhov model's phases (instances with pr != 1; the others are skipped).
 __global__ void __launch_bounds__(128, 4) kb_sums_shk(const SlotDev* __restrict__ slots,
-                                                   const BatchWork* __restrict__ wk) {
-  sums_phase_shk(slots, wk);
+                                                   const BatchWork* __restrict__ wk, int par) {
+  sums_phase_shk(slots, wk, par);
 }
 __global__ void __launch_bounds__(128, 4) kb_faces_shk(const SlotDev* __restrict__ slots,
-                                                    const BatchWork* __restrict__ wk) {
-  faces_phase_shk(slots, wk);
+                                                    const BatchWork* __restrict__ wk, int par) {
+  faces_phase_shk(slots, wk, par);
 }
 __global__ void __launch_bounds__(128, 3) kb_strip_shk(const SlotDev* __restrict__ slots,
-                                                    const BatchWork* __restrict__ wk) {
+                                                    const BatchWork* __restrict__ wk, int par) {
   extern __shared__ __align__(16) float4 strip_sm[];  // kStripSmem bytes
-  strip_phase_shk(slots, wk, strip_sm, true, 0u);
-}
-
-// After the step: every active instance swaps its buffers.
-__global__ void kb_flip(SlotDev* __restrict__ slots, const BatchWork* __restrict__ wk) {
-  for (int a = threadIdx.x; a < wk->n; a += blockDim.x) slots[wk->slot[a]].cur ^= 1;
+  strip_phase_shk(slots, wk, par, strip_sm, true, 0u);
 }
 
 // ---- the whole step as one persistent cooperative launch ---------------------------------
@@ -386,34 +367,27 @@ __device__ __forceinline__ bool grid_sync(BarrierDev* g) {
 // dynamic shared memory of the persistent step: the largest phase's (the walk's rings; the
 // ghost tables and the cells reduction alias its start)
 constexpr size_t kStepSmem = kStripSmem > kTileSmem ? kStripSmem : kTileSmem;
-static_assert(kStepSmem >= sizeof(double) * kGhostTab && kStepSmem >= sizeof(double) * 8 * 128 &&
-                  kStepSmem >= sizeof(double) * kWarpsPerBlock * kNSum,
+static_assert(kStepSmem >= sizeof(double) * kGhostTab && kStepSmem >= sizeof(double) * kWarpsPerBlock * kNSum,
               "persistent step: shared memory of every phase");
 
-__global__ void __launch_bounds__(128, 3) kb_step(SlotDev* __restrict__ slots,
-                                               const BatchWork* __restrict__ wk,
+__global__ void __launch_bounds__(128, 3) kb_step(const SlotDev* __restrict__ slots,
+                                               const BatchWork* __restrict__ wk, int par,
                                                BarrierDev* __restrict__ bar) {
   extern __shared__ __align__(16) float4 step_sm[];
-  double* tab = reinterpret_cast<double*>(step_sm);
-  ghost_x_phase(slots, wk, tab);
+  ghost_phase(slots, wk, par, reinterpret_cast<double*>(step_sm));
   if (!grid_sync(bar)) return;
-  ghost_y_phase(slots, wk, tab);
-  if (!grid_sync(bar)) return;
-  sums_phase(slots, wk, reinterpret_cast<double(*)[kNSum]>(step_sm));
-  sums_phase_shk(slots, wk);
+  sums_phase(slots, wk, par, reinterpret_cast<double(*)[kNSum]>(step_sm));
+  sums_phase_shk(slots, wk, par);
   __syncthreads();
-  sums_tile_phase(slots, wk, reinterpret_cast<unsigned char*>(step_sm));
+  sums_tile_phase(slots, wk, par, reinterpret_cast<unsigned char*>(step_sm));
   if (!grid_sync(bar)) return;
-  faces_phase(slots, wk);
-  faces_phase_shk(slots, wk);
+  faces_phase(slots, wk, par);
+  faces_phase_shk(slots, wk, par);
   if (!grid_sync(bar)) return;
-  cells_phase(slots, wk, reinterpret_cast<double(*)[128]>(step_sm));
+  cells_phase(slots, wk, par, reinterpret_cast<double(*)[8]>(step_sm));
   if (!grid_sync(bar)) return;
-  const unsigned nrec = strip_phase(slots, wk, step_sm);
-  strip_phase_shk(slots, wk, step_sm, false, nrec);
-  if (!grid_sync(bar)) return;
-  if (blockIdx.x == 0)
-    for (int a = threadIdx.x; a < wk->n; a += blockDim.x) slots[wk->slot[a]].cur ^= 1;
+  const unsigned nrec = strip_phase(slots, wk, par, step_sm);
+  strip_phase_shk(slots, wk, par, step_sm, false, nrec);
 }
 
 }  // namespace ugks

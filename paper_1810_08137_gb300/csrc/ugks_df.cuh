@@ -146,51 +146,8 @@ __device__ __forceinline__ df warp_reduce_scatter_df(df (&v)[N], int lane) {
   return r;
 }
 
-// Ghost ring: the FP64 form's rules (pressure Maxwellian in FP64, periodic image,
-// zero-gradient copy next to a wall), stored as double-FP32 pairs.
-__device__ void fill_ghost_cell(const Params& P, DF4* f, double* W, int nwe, int gi, int gj,
-                                int si, int sj, int side, bool write_W, int wi, int wj,
-                                double* tab) {
-  const int kind = P.bc_kind[side];
-  DF4* dst = f + fcell(P, gi, gj) * P.nq;
-  const DF4* src = f + fcell(P, si, sj) * P.nq;
-  const int sw = wcell(P, wi, wj);
-  if (kind == 2) {
-    double* fu = tab;
-    double* fv = tab + kMaxAxis;
-    const double rho_a = W[sw], U = W[nwe + sw] / rho_a, V = W[2 * nwe + sw] / rho_a;
-    const double lam = 1.0 / P.bc_T[side], rho = P.bc_rho[side];
-    const double G = rho * lam / kPi, bf = P.K / (2.0 * lam);
-    __syncthreads();  // the tables of the previous cell are no longer read
-    for (int k = threadIdx.x; k < P.nu; k += blockDim.x) {
-      const double du = P.u[k] - U;
-      fu[k] = G * exp(-lam * du * du);
-    }
-    for (int m = threadIdx.x; m < P.nv; m += blockDim.x) {
-      const double dv = P.v[m] - V;
-      fv[m] = exp(-lam * dv * dv);
-    }
-    __syncthreads();
-    for (int q = threadIdx.x; q < P.nq; q += blockDim.x) {
-      const int k = q % P.nu, m = q / P.nu;
-      const double gh = fu[k] * fv[m];
-      dst[q] = split4(gh, bf * gh);
-    }
-    if (write_W && threadIdx.x == 0) {
-      const int g = wcell(P, gi, gj);
-      W[g] = rho;
-      W[nwe + g] = rho * U;
-      W[2 * nwe + g] = rho * V;
-      W[3 * nwe + g] = rho * (0.5 * (U * U + V * V) + (P.K + 2) / (4.0 * lam));
-    }
-  } else {
-    for (int q = threadIdx.x; q < P.nq; q += blockDim.x) dst[q] = src[q];
-    if (write_W && threadIdx.x == 0) {
-      const int g = wcell(P, gi, gj), s = wcell(P, si, sj);
-      for (int c = 0; c < 4; c++) W[c * nwe + g] = W[c * nwe + s];
-    }
-  }
-}
+// Ghost ring: the FP64 form's, stored as double-FP32 pairs
+__device__ __forceinline__ DF4 ghost_value(DF4*, double h, double b) { return split4(h, b); }
 
 // State conversion (set-up and checkpoint paths): FP64 rows [cell][q][(h, b)] of rows
 // j0 .. j0+nrows-1 <-> double-FP32 f with its ghost ring; grid-stride over velocity-cells.

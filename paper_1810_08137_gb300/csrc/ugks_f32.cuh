@@ -66,56 +66,32 @@ __host__ __device__ __forceinline__ int padrow(const Params& P, int m) {
 }
 
 // -------------------------------------------------------------------------------------
-// Ghost ring (same rules as the FP64 form's fill_ghost_cell: pressure Maxwellian, periodic
-// image, zero-gradient copy next to a wall), over the slots of the paired layout.
+// Ghost ring over the slots of the paired layout (the FP64 form's rules): share `part` of
+// `parts` of ghost cell t.  A pressure Maxwellian is formed in FP64 and stored less g_ref: three
+// FP64 operations per velocity against g_ref's table (GB300 runs 2 of them per clock and SM),
+// rounded to FP32 on the integer pipe.
 // -------------------------------------------------------------------------------------
-__device__ void fill_ghost_cell(const Params& P, float4* f, double* W, int nwe, int gi, int gj,
-                                int si, int sj, int side, bool write_W, int wi, int wj,
-                                double* tab) {
-  const int kind = P.bc_kind[side];
-  float4* dst = f + fcell(P, gi, gj) * P.fs;
-  const float4* src = f + fcell(P, si, sj) * P.fs;
-  const int sw = wcell(P, wi, wj);
-  if (kind == 2) {
-    double* fu = tab;
-    double* fv = tab + kMaxAxis;
-    double* ru = tab + 2 * kMaxAxis;
-    double* rv = tab + 3 * kMaxAxis;
-    const double rho_a = W[sw], U = W[nwe + sw] / rho_a, V = W[2 * nwe + sw] / rho_a;
-    const double lam = 1.0 / P.bc_T[side], rho = P.bc_rho[side];
-    const double G = rho * lam / kPi, bf = P.K / (2.0 * lam);
-    __syncthreads();  // the tables of the previous cell are no longer read
-    for (int k = threadIdx.x; k < P.nu; k += blockDim.x) {
-      const double du = P.u[k] - U, dr = P.u[k] - P.ref_U;
-      fu[k] = G * exp(-lam * du * du);
-      ru[k] = P.ref_G * exp(-P.ref_lam * dr * dr);
-    }
-    for (int m = threadIdx.x; m < P.nv; m += blockDim.x) {
-      const double dv = P.v[m] - V, dr = P.v[m] - P.ref_V;
-      fv[m] = exp(-lam * dv * dv);
-      rv[m] = exp(-P.ref_lam * dr * dr);
-    }
-    __syncthreads();
-    for (int s = threadIdx.x; s < P.fs; s += blockDim.x) {
+constexpr int kGhostSlots = 2048;  // slots per share of a ghost cell, about
+__host__ __device__ __forceinline__ int ghost_parts(const Params& P) { return (P.fs + kGhostSlots - 1) / kGhostSlots; }
+__device__ __forceinline__ void ghost_body_f32(const Params& P, float4* f, double* W, int nwe, int t, double* tab) {
+  const int parts = ghost_parts(P), part = t % parts;
+  const int p0 = P.pr_all * part / parts, p1 = P.pr_all * (part + 1) / parts;  // row pairs of the share
+  GhostCell g = ghost_cell(P, t / parts);
+  if (part) g.write_W = false;
+  ghost_prepare(P, W, nwe, g, tab, prow(P, 2 * p0), prow(P, 2 * p1 - 1) + 1);
+  float4* dst = f + fcell(P, g.gi, g.gj) * P.fs;
+  if (g.side < 0) {
+    const float4* src = f + fcell(P, g.si, g.sj) * P.fs;
+    for (int s = p0 * P.nu + threadIdx.x; s < p1 * P.nu; s += blockDim.x) dst[s] = src[s];
+  } else {
+    const double bf = P.K * P.bc_T[g.side] * 0.5;
+    for (int s = p0 * P.nu + threadIdx.x; s < p1 * P.nu; s += blockDim.x) {
       const int pr = s / P.nu, k = s - pr * P.nu;
       const int m0 = prow(P, 2 * pr), m1 = prow(P, 2 * pr + 1);
-      const double g0 = fu[k] * fv[m0], r0 = ru[k] * rv[m0];
-      const double g1 = fu[k] * fv[m1], r1 = ru[k] * rv[m1];
-      dst[s] = make_float4((float)(g0 - r0), (float)(g1 - r1), (float)(bf * g0 - P.ref_bf * r0),
-                           (float)(bf * g1 - P.ref_bf * r1));
-    }
-    if (write_W && threadIdx.x == 0) {
-      const int g = wcell(P, gi, gj);
-      W[g] = rho;
-      W[nwe + g] = rho * U;
-      W[2 * nwe + g] = rho * V;
-      W[3 * nwe + g] = rho * (0.5 * (U * U + V * V) + (P.K + 2) / (4.0 * lam));
-    }
-  } else {
-    for (int s = threadIdx.x; s < P.fs; s += blockDim.x) dst[s] = src[s];
-    if (write_W && threadIdx.x == 0) {
-      const int g = wcell(P, gi, gj), s = wcell(P, si, sj);
-      for (int c = 0; c < 4; c++) W[c * nwe + g] = W[c * nwe + s];
+      const double2 r0 = P.grefd[m0 * P.nu + k], r1 = P.grefd[m1 * P.nu + k];
+      const double g0 = tab[k] * tab[kMaxAxis + m0], g1 = tab[k] * tab[kMaxAxis + m1];
+      dst[s] = make_float4(f32_rn(g0 - r0.x), f32_rn(g1 - r1.x), f32_rn(fma(bf, g0, -r0.y)),
+                           f32_rn(fma(bf, g1, -r1.y)));
     }
   }
 }

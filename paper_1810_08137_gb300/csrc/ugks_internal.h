@@ -164,6 +164,7 @@ struct Params {
   // row pairs in total, fs = pr_all * nu float4 slots per cell
   int pr_neg, pr_all, fs;
   const float4* gref4;    // [fs] g_ref of each slot (h, h', b, b')
+  const double2* grefd;   // [nq] g_ref (h, b) in FP64
   const float4* pwt;      // [pr_all][3]: (w0 w0' w1 w1') (w2 w2' w3 w3') (w4 w4' v v'),
                           // w_n = wv v^n of the pair's two rows; zero on padded rows, half
                           // of wv on the v = 0 row

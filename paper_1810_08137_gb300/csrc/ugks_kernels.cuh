@@ -1,7 +1,7 @@
 // Device kernels of one explicit 2D UGKS step (Liu, Hu & Li, arXiv:1810.08137, Sec. 2).
 //
 // Per step, on one stream:
-//   k_ghost_x, k_ghost_y  boundary ghost ring (periodic image, wall zero-gradient copy,
+//   k_ghost               boundary ghost ring (periodic image, wall zero-gradient copy,
 //                         pressure Maxwellian)
 //   k_sums                per cell and side, the velocity sums of steps S1 and S7 (W0,
 //                         tangential slope of W, free-transport sums) over one read of f
@@ -134,107 +134,113 @@ __host__ __device__ __forceinline__ void ref_maxwellian(const Params& P, double 
 }
 
 // -------------------------------------------------------------------------------------
-// Boundary ghost ring
+// Boundary ghost ring, one pass over its cells.  A ghost cell is a copy of an interior cell
+// (periodic image, zero gradient next to a wall) or a pressure Maxwellian with the velocity of
+// one; a corner's two rules compose to one of these (the y rule acts on what the x rule puts
+// there), so no ghost cell is read and the ring takes one launch.  The second layer is read
+// through periodic sides only: next to a wall the wall flux takes the place of the ghost's, and
+// a pressure ghost has zero slopes.
 // -------------------------------------------------------------------------------------
-// tab: shared memory of the block for 4 kMaxAxis doubles (per-axis Maxwellian factors)
-constexpr int kGhostTab = 4 * kMaxAxis;
+__host__ __device__ __forceinline__ int ghost_layers(const Params& P, int side) {
+  return P.bc_kind[side] == 0 ? 2 : 1;
+}
+// cells of the ring: rows 0..ny-1 of the x sides, then the y sides over every column
+__host__ __device__ __forceinline__ int ghost_cells(const Params& P) {
+  const int lx = ghost_layers(P, 0) + ghost_layers(P, 1), ly = ghost_layers(P, 2) + ghost_layers(P, 3);
+  return P.ny * lx + (P.nx + lx) * ly;
+}
+struct GhostCell {
+  int gi, gj;   // the ghost cell
+  int si, sj;   // interior cell it takes its values or its velocity from
+  int side;     // pressure side, or -1: a copy
+  bool write_W; // layer 1 (the W buffers hold one layer)
+};
+// interior index of ghost layer l beyond the low (side even) or high end of an axis of n cells
+__device__ __forceinline__ int ghost_source(int kind, bool low, int l, int n) {
+  if (kind == 0) return low ? n - l : l - 1;
+  return low ? 0 : n - 1;
+}
+__device__ __forceinline__ GhostCell ghost_cell(const Params& P, int t) {
+  const int l0 = ghost_layers(P, 0), lx = l0 + ghost_layers(P, 1);
+  const int l2 = ghost_layers(P, 2), ly = l2 + ghost_layers(P, 3);
+  GhostCell g;
+  int col, k;                // column of the ring (0 .. nx + lx), -1 for the interior
+  if (t < P.ny * lx) {
+    g.gj = t / lx;
+    k = t - g.gj * lx;
+    col = k < l0 ? k : P.nx + k;
+  } else {
+    t -= P.ny * lx;
+    col = t / ly;
+    k = t - col * ly;
+    g.gj = k < l2 ? -1 - k : P.ny + k - l2;
+  }
+  g.gi = col - l0;           // ghost columns -l0 .. -1 and nx ..
+  g.side = -1;
+  g.si = g.gi;
+  if (g.gi < 0 || g.gi >= P.nx) {
+    const int sd = g.gi < 0 ? 0 : 1, kind = P.bc_kind[sd];
+    g.si = ghost_source(kind, sd == 0, sd == 0 ? -g.gi : g.gi - P.nx + 1, P.nx);
+    if (kind == 2) g.side = sd;
+  }
+  g.sj = g.gj;
+  if (g.gj < 0 || g.gj >= P.ny) {
+    const int sd = g.gj < 0 ? 2 : 3, kind = P.bc_kind[sd];
+    g.sj = ghost_source(kind, sd == 2, sd == 2 ? -g.gj : g.gj - P.ny + 1, P.ny);
+    if (kind == 2) g.side = sd;
+  }
+  g.write_W = g.gi >= -1 && g.gi <= P.nx && g.gj >= -1 && g.gj <= P.ny;
+  return g;
+}
+// The ghost cell's W, and for a pressure side the per-axis factors of its Maxwellian
+// g_h = fu[k] fv[m] in the block's shared memory (tab: 2 kMaxAxis doubles), rows m0 .. m1-1.
+constexpr int kGhostTab = 2 * kMaxAxis;
+__device__ __forceinline__ void ghost_prepare(const Params& P, double* W, int nwe, const GhostCell& g, double* tab,
+                                              int m0, int m1) {
+  const int src = wcell(P, g.si, g.sj), dst = wcell(P, g.gi, g.gj);
+  if (g.side < 0) {
+    if (g.write_W && threadIdx.x < 4) W[threadIdx.x * nwe + dst] = W[threadIdx.x * nwe + src];
+    return;
+  }
+  const double rho_a = W[src], U = W[nwe + src] / rho_a, V = W[2 * nwe + src] / rho_a;
+  const double lam = 1.0 / P.bc_T[g.side], rho = P.bc_rho[g.side], G = rho * lam / kPi;
+  __syncthreads();  // the tables of the previous cell are no longer read
+  for (int t = threadIdx.x; t < P.nu + m1 - m0; t += blockDim.x) {
+    const double d = t < P.nu ? P.u[t] - U : P.v[m0 + t - P.nu] - V;
+    const double e = exp(-lam * d * d);
+    if (t < P.nu) tab[t] = G * e;
+    else tab[kMaxAxis + m0 + t - P.nu] = e;
+  }
+  if (g.write_W && threadIdx.x == 0) {
+    W[dst] = rho;
+    W[nwe + dst] = rho * U;
+    W[2 * nwe + dst] = rho * V;
+    W[3 * nwe + dst] = rho * (0.5 * (U * U + V * V) + (P.K + 2) / (4.0 * lam));
+  }
+  __syncthreads();
+}
+__device__ __forceinline__ double2 ghost_value(double2*, double h, double b) { return make_double2(h, b); }
 template <typename T2>
-__device__ void fill_ghost_cell(const Params& P, T2* f, double* W, int nwe, int gi, int gj,
-                                int si, int sj, int side, bool write_W, int wi, int wj,
-                                double* tab) {
-  const int kind = P.bc_kind[side];
-  T2* dst = f + fcell(P, gi, gj) * P.nq;
-  const T2* src = f + fcell(P, si, sj) * P.nq;
-  const int sw = wcell(P, wi, wj);
-  if (kind == 2) {  // pressure: Maxwellian(rho_bc, U and V of the adjacent cell, T_bc)
-    // both Maxwellians factor into a u part and a v part: per-axis tables in shared memory
-    double* fu = tab;
-    double* fv = tab + kMaxAxis;
-    double* ru = tab + 2 * kMaxAxis;
-    double* rv = tab + 3 * kMaxAxis;
-    const double rho_a = W[sw], U = W[nwe + sw] / rho_a, V = W[2 * nwe + sw] / rho_a;
-    const double lam = 1.0 / P.bc_T[side], rho = P.bc_rho[side];
-    const double G = rho * lam / kPi, bf = P.K / (2.0 * lam);
-    __syncthreads();  // the tables of the previous cell are no longer read
-    for (int k = threadIdx.x; k < P.nu; k += blockDim.x) {
-      const double du = P.u[k] - U, dr = P.u[k] - P.ref_U;
-      fu[k] = G * exp(-lam * du * du);
-      ru[k] = P.use_ref ? P.ref_G * exp(-P.ref_lam * dr * dr) : 0.0;
-    }
-    for (int m = threadIdx.x; m < P.nv; m += blockDim.x) {
-      const double dv = P.v[m] - V, dr = P.v[m] - P.ref_V;
-      fv[m] = exp(-lam * dv * dv);
-      rv[m] = exp(-P.ref_lam * dr * dr);
-    }
-    __syncthreads();
-    for (int q = threadIdx.x; q < P.nq; q += blockDim.x) {
-      const int k = q % P.nu, m = q / P.nu;
-      const double gh = fu[k] * fv[m], rh = ru[k] * rv[m];
-      T2 o;
-      o.x = gh - rh;
-      o.y = bf * gh - P.ref_bf * rh;
-      dst[q] = o;
-    }
-    if (write_W && threadIdx.x == 0) {
-      const int g = wcell(P, gi, gj);
-      W[g] = rho;
-      W[nwe + g] = rho * U;
-      W[2 * nwe + g] = rho * V;
-      W[3 * nwe + g] = rho * (0.5 * (U * U + V * V) + (P.K + 2) / (4.0 * lam));
-    }
-  } else {  // periodic image or zero-gradient copy next to a wall
+__device__ __forceinline__ void ghost_body(const Params& P, T2* f, double* W, int nwe, int t, double* tab) {
+  const GhostCell g = ghost_cell(P, t);
+  ghost_prepare(P, W, nwe, g, tab, 0, P.nv);
+  T2* dst = f + fcell(P, g.gi, g.gj) * P.nq;
+  if (g.side < 0) {
+    const T2* src = f + fcell(P, g.si, g.sj) * P.nq;
     for (int q = threadIdx.x; q < P.nq; q += blockDim.x) dst[q] = src[q];
-    if (write_W && threadIdx.x == 0) {
-      const int g = wcell(P, gi, gj), s = wcell(P, si, sj);
-      for (int c = 0; c < 4; c++) W[c * nwe + g] = W[c * nwe + s];
+  } else {
+    const double bf = P.K * P.bc_T[g.side] * 0.5;
+    for (int q = threadIdx.x; q < P.nq; q += blockDim.x) {
+      const int m = q / P.nu, k = q - m * P.nu;
+      const double gh = tab[k] * tab[kMaxAxis + m];
+      dst[q] = ghost_value(dst, gh, bf * gh);
     }
   }
 }
-
-// FP32 paired-row layout (ugks_f32.cuh)
-__device__ void fill_ghost_cell(const Params& P, float4* f, double* W, int nwe, int gi, int gj,
-                                int si, int sj, int side, bool write_W, int wi, int wj,
-                                double* tab);
-
-// x-sides, rows 0..ny-1; grid (ny, 4): blockIdx.y = side*2 + layer-1.
 template <typename T2>
-__device__ __forceinline__ void ghost_x_body(const Params& P, T2* f, double* W, int nwe, int bx, int by,
-                                             double* tab) {
-  const int j = bx, side = by >> 1, l = (by & 1) + 1;
-  const int kind = P.bc_kind[side];
-  const int gi = side == 0 ? -l : P.nx - 1 + l;
-  int si;
-  if (kind == 0) si = side == 0 ? P.nx - l : l - 1;
-  else si = side == 0 ? 0 : P.nx - 1;
-  const int ai = side == 0 ? 0 : P.nx - 1;  // adjacent interior cell (pressure velocity source)
-  fill_ghost_cell(P, f, W, nwe, gi, j, si, j, side, l == 1, kind == 2 ? ai : si, j, tab);
-}
-template <typename T2>
-__global__ void k_ghost_x(Params P, T2* f, double* W, int nwe) {
+__global__ void k_ghost(Params P, T2* f, double* W, int nwe) {
   __shared__ double tab[kGhostTab];
-  ghost_x_body(P, f, W, nwe, blockIdx.x, blockIdx.y, tab);
-}
-
-// y-sides over all columns -2..nx+1 (corners included, after the x-sides);
-// grid (nx+4, 4): blockIdx.y = side*2 + layer-1, side 0: S, 1: N.
-template <typename T2>
-__device__ __forceinline__ void ghost_y_body(const Params& P, T2* f, double* W, int nwe, int bx, int by,
-                                             double* tab) {
-  const int i = bx - 2, side = 2 + (by >> 1), l = (by & 1) + 1;
-  const int kind = P.bc_kind[side];
-  const int gj = side == 2 ? -l : P.ny - 1 + l;
-  int sj;
-  if (kind == 0) sj = side == 2 ? P.ny - l : l - 1;
-  else sj = side == 2 ? 0 : P.ny - 1;
-  const int aj = side == 2 ? 0 : P.ny - 1;
-  const bool wcol = i >= -1 && i <= P.nx;
-  const int wi = i < -1 ? -1 : (i > P.nx ? P.nx : i);
-  fill_ghost_cell(P, f, W, nwe, i, gj, i, sj, side, l == 1 && wcol, wi, kind == 2 ? aj : sj, tab);
-}
-template <typename T2>
-__global__ void k_ghost_y(Params P, T2* f, double* W, int nwe) {
-  __shared__ double tab[kGhostTab];
-  ghost_y_body(P, f, W, nwe, blockIdx.x, blockIdx.y, tab);
+  ghost_body(P, f, W, nwe, blockIdx.x, tab);
 }
 
 // -------------------------------------------------------------------------------------
@@ -1246,10 +1252,10 @@ __device__ __forceinline__ void cells_body(const Params& P, const double* __rest
                                            const double* __restrict__ Fy, CellRec* __restrict__ cr,
                                            double* __restrict__ rpart, int* __restrict__ err,
                                            CellRecF* __restrict__ crf,
-                                           const double* __restrict__ mt4, double (*red)[128],
-                                           int bx, CellRecD* __restrict__ crd = nullptr) {
-  const int c = bx * blockDim.x + threadIdx.x;
+                                           const double* __restrict__ mt4, double (*red)[8],
+                                           int bx, int cb, CellRecD* __restrict__ crd = nullptr) {
   const int nx = P.nx, nc = P.nx * P.ny;
+  const int c = threadIdx.x < cb ? bx * cb + threadIdx.x : nc;
   double d2[4] = {0, 0, 0, 0}, am[4] = {0, 0, 0, 0};
   if (c < nc) {
     const int i = c % nx, j = c / nx;
@@ -1371,20 +1377,37 @@ __device__ __forceinline__ void cells_body(const Params& P, const double* __rest
       cr[c] = R;
     }
   }
+  // the block's residual partials: sums of d2 on lanes 0..15, maxima of |W1| on lanes 16..31, by
+  // a transpose reduction within each warp, then over the warps
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool hi = lane & 16;
+  auto comb = [&](double x, double y) { return hi ? fmax(x, y) : x + y; };
+  double v[4];
+#pragma unroll
   for (int k = 0; k < 4; k++) {
-    red[k][threadIdx.x] = d2[k];
-    red[4 + k][threadIdx.x] = am[k];
+    const double got = __shfl_xor_sync(kFull, hi ? d2[k] : am[k], 16);
+    v[k] = comb(hi ? am[k] : d2[k], got);
   }
+#pragma unroll
+  for (int o = 8; o >= 4; o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int k = 0; k < o / 4; k++) {
+      const double got = __shfl_xor_sync(kFull, up ? v[k] : v[k + o / 4], o);
+      v[k] = comb(up ? v[k + o / 4] : v[k], got);
+    }
+  }
+  v[0] = comb(v[0], __shfl_xor_sync(kFull, v[0], 2));
+  v[0] = comb(v[0], __shfl_xor_sync(kFull, v[0], 1));
+  // lane bits 4, 3, 2: sum or maximum, then the component
+  if ((lane & 3) == 0) red[warp][lane >> 2] = v[0];
   __syncthreads();
-  for (int s = 64; s > 0; s >>= 1) {
-    if (threadIdx.x < s)
-      for (int k = 0; k < 4; k++) {
-        red[k][threadIdx.x] += red[k][threadIdx.x + s];
-        red[4 + k][threadIdx.x] = fmax(red[4 + k][threadIdx.x], red[4 + k][threadIdx.x + s]);
-      }
-    __syncthreads();
+  if (threadIdx.x < 8) {
+    double r = red[0][threadIdx.x];
+    for (int w = 1; w < (int)blockDim.x / 32; w++)
+      r = threadIdx.x < 4 ? r + red[w][threadIdx.x] : fmax(r, red[w][threadIdx.x]);
+    rpart[(size_t)bx * 8 + threadIdx.x] = r;
   }
-  if (threadIdx.x < 8) rpart[(size_t)bx * 8 + threadIdx.x] = red[threadIdx.x][0];
 }
 __global__ void __launch_bounds__(128) k_cells(Params P, const double* __restrict__ Win,
                                                double* __restrict__ Wout, int nwe,
@@ -1394,8 +1417,8 @@ __global__ void __launch_bounds__(128) k_cells(Params P, const double* __restric
                                                int* __restrict__ err, CellRecF* __restrict__ crf,
                                                const double* __restrict__ mt4,
                                                CellRecD* __restrict__ crd = nullptr) {
-  __shared__ double red[8][128];
-  cells_body(P, Win, Wout, nwe, Fx, Fy, cr, rpart, err, crf, mt4, red, blockIdx.x, crd);
+  __shared__ double red[4][8];
+  cells_body(P, Win, Wout, nwe, Fx, Fy, cr, rpart, err, crf, mt4, red, blockIdx.x, blockDim.x, crd);
 }
 
 // -------------------------------------------------------------------------------------
