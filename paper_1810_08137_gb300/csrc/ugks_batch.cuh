@@ -280,10 +280,11 @@ __global__ void __launch_bounds__(128, 3) kb_sums_tile(const SlotDev* __restrict
   sums_tile_phase(slots, wk, par, tile_sm);
 }
 
-// eight blocks per SM (64 registers, the rest on the stack): the interface is latency-bound
-// on its FP64 and double-FP32 chains, and 32 resident warps hide more of it than 12 (0.59 ->
-// 0.50 ms at 800x400x28^2; six blocks 0.52 ms)
-__global__ void __launch_bounds__(128, 8) kb_faces(const SlotDev* __restrict__ slots,
+// six blocks per SM (80 registers, the rest on the stack): bound by the FP64 pipe (about 200 FP64
+// instructions per face at 1/64 of the FP32 rate) and the latency of its FP64 and double-FP32
+// chains.  800x400x28^2 0.298 ms, 200x100 45 us (8 blocks 0.306 ms and 48 us, 4 blocks 0.334 ms and
+// 43 us).
+__global__ void __launch_bounds__(128, 6) kb_faces(const SlotDev* __restrict__ slots,
                                                 const BatchWork* __restrict__ wk, int par) {
   faces_phase(slots, wk, par);
 }

@@ -151,6 +151,9 @@ __device__ __forceinline__ dd operator*(dd a, dd b) { return as_dd(df_mul(as_df(
 __device__ __forceinline__ dd operator-(dd a) { return dd(-a.hi, -a.lo); }
 __device__ __forceinline__ double to_double(dd a) { return f64_of(a.hi) + f64_of(a.lo); }
 __device__ __forceinline__ double to_double(double a) { return a; }
+// a b + c with one renormalisation
+__device__ __forceinline__ dd mad(dd a, dd b, dd c) { return as_dd(df_fma(as_df(a), as_df(b), as_df(c))); }
+__device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
 // a / 2 (exact) and a n, n a small whole number
 __device__ __forceinline__ dd halved(dd a) { return dd(0.5f * a.hi, 0.5f * a.lo); }
 __device__ __forceinline__ double halved(double a) { return 0.5 * a; }

@@ -565,19 +565,35 @@ __device__ __forceinline__ void gauss_central7(T U, T h, T m0, T e, T* m) {
 #pragma unroll
   for (int n = 0; n < 5; n++) {
     z = z * nU;
-    m[n + 2] = scaled(h, n + 1) * m[n] + z;
+    m[n + 2] = mad(scaled(h, n + 1), m[n], z);
   }
 }
-// One erfc: the half-range mass on the far side of U is erfc(sqrt(lam)|U|)/2, the near side
-// 1 minus that; rl = 1/sqrt(lam).
+// The half-range masses are (1 +- erf(x))/2, x = sqrt(lam) U; rl = 1/sqrt(lam).  Subsonic
+// interfaces (|x| < 1/2) take erf from its Maclaurin series 2/sqrt(pi) sum (-1)^n x^(2n+1) /
+// (n! (2n+1)) (12 terms; the first one left out is below 1e-17 of the sum, and no term cancels
+// there), a third of the FP64 operations of erfc; beyond, erfc of the far side.
+__host__ __device__ constexpr double erf_coef(int n) {  // 2/sqrt(pi) (-1)^n / (n! (2n+1))
+  double f = 1.12837916709551257390 / (2 * n + 1);
+  for (int k = 1; k <= n; k++) f /= -k;
+  return f;
+}
 __device__ __forceinline__ void gauss_half_start(double U, double lam, double rl, double& mp0, double& mn0,
                                                  double& e) {
   constexpr double kHalfRsqrtPi = 0.28209479177387814347;  // 1 / (2 sqrt(pi))
-  const double sl = lam * rl;
-  e = exp(-lam * U * U) * (kHalfRsqrtPi * rl);
-  const double far = 0.5 * erfc(sl * fabs(U));
-  mp0 = U >= 0.0 ? 1.0 - far : far;
-  mn0 = U >= 0.0 ? far : 1.0 - far;
+  const double x = lam * rl * U, x2 = lam * U * U;
+  e = exp(-x2) * (kHalfRsqrtPi * rl);
+  if (x2 < 0.25) {
+    double p = erf_coef(11);
+#pragma unroll
+    for (int n = 10; n >= 0; n--) p = fma(p, x2, erf_coef(n));
+    const double d = 0.5 * x * p;
+    mp0 = 0.5 + d;
+    mn0 = 0.5 - d;
+  } else {
+    const double far = 0.5 * erfc(fabs(x));
+    mp0 = U >= 0.0 ? 1.0 - far : far;
+    mn0 = U >= 0.0 ? far : 1.0 - far;
+  }
 }
 
 // Full-range moments only (tangential axis).
@@ -600,24 +616,24 @@ __device__ void gauss_moments7_full(T U, T h, T* M) {
 // s' = <psi' (a . psi)> of a slope target s = <psi (a . psi)>; ke = (U^2 + V^2)/2.
 template <typename T>
 __device__ __forceinline__ void to_moving(T U, T V, T ke, T* s) {
-  s[3] = s[3] - (U * s[1] + V * s[2]) + ke * s[0];
-  s[1] = s[1] - U * s[0];
-  s[2] = s[2] - V * s[0];
+  s[3] = mad(ke, s[0], mad(-U, s[1], mad(-V, s[2], s[3])));
+  s[1] = mad(-U, s[0], s[1]);
+  s[2] = mad(-V, s[0], s[2]);
 }
 // Slope a (on psi') with <psi' (a . psi')> = s: q = (K+2) h / 2, il = 2 lam, c8 = 8 lam^2 / (K+2).
 template <typename T>
 __device__ __forceinline__ void micro_slope(T q, T il, T c8, const T* s, T* a) {
-  a[3] = c8 * (s[3] - q * s[0]);
+  a[3] = c8 * mad(-q, s[0], s[3]);
   a[1] = il * s[1];
   a[2] = il * s[2];
-  a[0] = s[0] - q * a[3];
+  a[0] = mad(-q, a[3], s[0]);
 }
 // The slope on psi = (1, un, ut, (un^2 + ut^2 + xi^2)/2) of a slope on psi'.
 template <typename T>
 __device__ __forceinline__ void to_lab(T U, T V, T ke, T* a) {
-  a[0] = a[0] - (U * a[1] + V * a[2]) + ke * a[3];
-  a[1] = a[1] - U * a[3];
-  a[2] = a[2] - V * a[3];
+  a[0] = mad(ke, a[3], mad(-U, a[1], mad(-V, a[2], a[0])));
+  a[1] = mad(-U, a[3], a[1]);
+  a[2] = mad(-V, a[3], a[2]);
 }
 // Half-range moments of a normal slope: t = <un psi' (a . psi')>, n = <un^2 psi' (a . psi')>
 // over the range of the central moments m.  Averaged over y and xi, a . psi' is
@@ -630,18 +646,18 @@ template <typename T>
 __device__ __forceinline__ void half_moments(T U, T h, T k1h, const T* m, const T* a, T s2, T* t, T* ns) {
   T w[6], d[4];
 #pragma unroll
-  for (int n = 0; n < 6; n++) w[n] = U * m[n] + m[n + 1];
-  const T p2 = halved(a[3]), p0 = a[0] + p2 * k1h, a3h = a[3] * h;
+  for (int n = 0; n < 6; n++) w[n] = mad(U, m[n], m[n + 1]);
+  const T p2 = halved(a[3]), p0 = mad(p2, k1h, a[0]), a3h = a[3] * h;
 #pragma unroll
-  for (int n = 0; n < 4; n++) d[n] = p0 * w[n] + a[1] * w[n + 1] + p2 * w[n + 2];
+  for (int n = 0; n < 4; n++) d[n] = mad(p2, w[n + 2], mad(a[1], w[n + 1], p0 * w[n]));
   t[0] = d[0];
   t[1] = d[1];
   t[2] = s2 * w[0];
-  t[3] = halved(d[2] + k1h * (d[0] + a3h * w[0]));
-  ns[0] = ns[0] + (U * t[0] + d[1]);
-  ns[1] = ns[1] + (U * t[1] + d[2]);
-  ns[2] = ns[2] + (U * t[2] + s2 * w[1]);
-  ns[3] = ns[3] + (U * t[3] + halved(d[3] + k1h * (d[1] + a3h * w[1])));
+  t[3] = halved(mad(k1h, mad(a3h, w[0], d[0]), d[2]));
+  ns[0] = ns[0] + mad(U, t[0], d[1]);
+  ns[1] = ns[1] + mad(U, t[1], d[2]);
+  ns[2] = mad(U, t[2], mad(s2, w[1], ns[2]));
+  ns[3] = ns[3] + mad(U, t[3], halved(mad(k1h, mad(a3h, w[1], d[1]), d[3])));
 }
 
 // 1/n! as a constant expression (the loops that use it are unrolled).
@@ -822,7 +838,7 @@ __device__ __forceinline__ void face_core(const Params& P, const double* W0, con
   time_weights(P.dt, x, c.Mt);
   const double* Mt = c.Mt;
   // S4: micro slopes a_L, a_R (normal), b (tangential), on psi' of the moving frame
-  const double inv = irho * tdelta;
+  const T irhot = T(irho), invt = irhot * T(tdelta);
   const T Ut = T(U), Vt = T(V), ht = T(h), ke = halved(Ut * Ut + Vt * Vt);
   const T q = scaled(halved(ht), K + 2), k1h = scaled(ht, K + 1), il = T(2.0 * lam);
   const T c8 = T(8.0 * lam * lam * P.inv_kp2);
@@ -833,7 +849,7 @@ __device__ __forceinline__ void face_core(const Params& P, const double* W0, con
   for (int sd = 0; sd < 2; sd++) {
     T s[4], m[7], a[4];
 #pragma unroll
-    for (int k = 0; k < 4; k++) s[k] = T((sd == 0 ? W0[k] - WL[k] : WR[k] - W0[k]) * inv);
+    for (int k = 0; k < 4; k++) s[k] = T(sd == 0 ? W0[k] - WL[k] : WR[k] - W0[k]) * invt;
     to_moving<T>(Ut, Vt, ke, s);
     micro_slope<T>(q, il, c8, s, a);
     gauss_central7<T>(Ut, ht, T(sd == 0 ? mp0 : mn0), T(sd == 0 ? e : -e), m);
@@ -853,18 +869,18 @@ __device__ __forceinline__ void face_core(const Params& P, const double* W0, con
     // ut = V + y, over the full range
     T s[4];
 #pragma unroll
-    for (int k = 0; k < 4; k++) s[k] = T(St[k] * irho);
+    for (int k = 0; k < 4; k++) s[k] = T(St[k]) * irhot;
     to_moving<T>(Ut, Vt, ke, s);
     micro_slope<T>(q, il, c8, s, c.b);
-    const T y2 = ht * (s[0] + c.b[3] * ht);  // <y^2 (b . psi')> = <x^2 (b . psi')>
-    t[0] = Vt * s[0] + s[2];
+    const T y2 = ht * mad(c.b[3], ht, s[0]);  // <y^2 (b . psi')> = <x^2 (b . psi')>
+    t[0] = mad(Vt, s[0], s[2]);
     t[1] = Vt * s[1];
-    t[2] = Vt * s[2] + y2;
-    t[3] = Vt * s[3] + k4h * s[2];
-    ns[0] = ns[0] + (Ut * t[0] + Vt * s[1]);
-    ns[1] = ns[1] + (Ut * t[1] + (Vt * y2 + ht * s[2]));
-    ns[2] = ns[2] + (Ut * t[2] + ht * s[1]);
-    ns[3] = ns[3] + (Ut * t[3] + Vt * (k4h * s[1]));
+    t[2] = mad(Vt, s[2], y2);
+    t[3] = mad(Vt, s[3], k4h * s[2]);
+    ns[0] = mad(Ut, t[0], mad(Vt, s[1], ns[0]));
+    ns[1] = mad(Ut, t[1], mad(Vt, y2, mad(ht, s[2], ns[1])));
+    ns[2] = mad(Ut, t[2], mad(ht, s[1], ns[2]));
+    ns[3] = mad(Ut, t[3], mad(Vt, k4h * s[1], ns[3]));
 #pragma unroll
     for (int k = 0; k < 4; k++) sA[k] = -(sA[k] + t[k]);
   }
@@ -875,13 +891,13 @@ __device__ __forceinline__ void face_core(const Params& P, const double* W0, con
   // <un psi' (A . psi')> = U sA + (sA1, h (sA0 + A3 h), 0, k4h sA1)
   const T M1 = T(Mt[0]), M2 = T(Mt[1]), M3 = T(Mt[2]), rhot = T(rho);
   T Fe[4];
-  Fe[0] = M1 * Ut + M2 * ns[0] + M3 * (Ut * sA[0] + sA[1]);
-  Fe[1] = M1 * ht + M2 * ns[1] + M3 * (Ut * sA[1] + ht * (sA[0] + c.A[3] * ht));
-  Fe[2] = M2 * ns[2] + M3 * (Ut * sA[2]);
-  Fe[3] = M1 * (Ut * q) + M2 * ns[3] + M3 * (Ut * sA[3] + k4h * sA[1]);
-  Fe[3] = Fe[3] + (Ut * Fe[1] + Vt * Fe[2]) + ke * Fe[0];
-  Fe[1] = Fe[1] + Ut * Fe[0];
-  Fe[2] = Fe[2] + Vt * Fe[0];
+  Fe[0] = mad(M3, mad(Ut, sA[0], sA[1]), mad(M2, ns[0], M1 * Ut));
+  Fe[1] = mad(M3, mad(Ut, sA[1], ht * mad(c.A[3], ht, sA[0])), mad(M2, ns[1], M1 * ht));
+  Fe[2] = mad(M3, Ut * sA[2], M2 * ns[2]);
+  Fe[3] = mad(M3, mad(Ut, sA[3], k4h * sA[1]), mad(M2, ns[3], M1 * (Ut * q)));
+  Fe[3] = mad(ke, Fe[0], mad(Ut, Fe[1], mad(Vt, Fe[2], Fe[3])));
+  Fe[1] = mad(Ut, Fe[0], Fe[1]);
+  Fe[2] = mad(Vt, Fe[0], Fe[2]);
 #pragma unroll
   for (int k = 0; k < 4; k++) F[k] = to_double(rhot * Fe[k]) + Mt[3] * Sf[k] - Mt[4] * Ss[k];
   to_lab<T>(Ut, Vt, ke, c.b);
