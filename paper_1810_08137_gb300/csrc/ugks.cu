@@ -16,6 +16,7 @@
 #include "ugks_kernels.cuh"
 #include "ugks_f32.cuh"
 #include "ugks_df.cuh"
+#include "ugks_tile.cuh"
 #include "ugks_batch.cuh"
 
 using namespace ugks;
@@ -185,6 +186,11 @@ std::pair<int, int> f32_row_pairs(int nv, double vmin, double vmax) {
 // FP64 pipe (2 operations per clock).  40x20 cells 14.9 -> 12.8 us.
 int small_block(long n) { return n < 152 * 128 ? 32 : 128; }
 
+// Velocity sums per cell: the FP64 and DF64 forms' BGK sums kernel keeps its four quadrants apart.
+int sums_per_cell(const ugks_config* c) {
+  return c->precision != UGKS_FP32F && shakhov_pr(c) == 1.0 ? kCellPart : kNSum;
+}
+
 // Device bytes ugks_create allocates for cfg (cudaMalloc sizes, without allocator rounding).
 size_t predict_bytes(const ugks_config* c) {
   const size_t nx = c->nx, ny = c->ny, nq = (size_t)c->nu * c->nv, nc = nx * ny;
@@ -193,13 +199,13 @@ size_t predict_bytes(const ugks_config* c) {
   const size_t fslot = f32 ? fs * sizeof(float4) : nq * sizeof(double2);  // f bytes per cell
   const size_t fcells = (nx + 4) * (ny + 4), nwe = (nx + 2) * (ny + 2);
   const size_t nfx = (nx + 1) * ny, nfy = nx * (ny + 1), cb = small_block(nc), nrb = (nc + cb - 1) / cb;
-  size_t b = 2 * fcells * fslot + 2 * 4 * sizeof(double) * nwe + sizeof(double) * kNSum * nwe;
+  size_t b = 2 * fcells * fslot + 2 * 4 * sizeof(double) * nwe + sizeof(double) * sums_per_cell(c) * nwe;
   if (shakhov_pr(c) != 1.0) b += sizeof(double) * kNHeat * nwe + (f32 ? sizeof(CellShkF) * nc : 0);
   b += f32 ? sizeof(FaceRecF) * (nfx + nfy) : (dfm ? sizeof(FaceRecD) : sizeof(FaceRec)) * (nfx + nfy);
   b += sizeof(double) * 4 * (nfx + nfy) + sizeof(double) * (nfx + nfy);
   b += f32 ? sizeof(CellRecF) * nc : (dfm ? sizeof(CellRecD) : sizeof(CellRec)) * nc;
-  if (dfm) b += sizeof(float2) * (2 * (size_t)c->nu + 6 * (size_t)c->nv);
-  b += sizeof(double) * 8 * nrb + sizeof(int) + sizeof(double) * (2 * (c->nu + c->nv) + 5 * c->nv);
+  if (dfm) b += sizeof(float2) * (8 * (size_t)c->nu + 8 * (size_t)c->nv);
+  b += sizeof(double) * 8 * nrb + sizeof(int) + sizeof(double) * (8 * (size_t)c->nu + 9 * (size_t)c->nv);
   if (!f32) b += nwe * nq * 2 * sizeof(double2) + (nfx + nfy) * nq * sizeof(double2);  // slopes, face fluxes
   if (f32) {
     const size_t row_d = nx * nq * 2 * sizeof(double);
@@ -232,6 +238,9 @@ size_t smem_cell_update(int nv) {
 cudaError_t set_smem_limits_fp64(int nv) {
   cudaError_t e = cudaFuncSetAttribute(k_sums<double, double2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem_sums<double>(nv));
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(k_sums_cell<NumF64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)(kWarpsPerBlock * kCellSumsWarp));
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_face_flux<double, double2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)smem_face_flux<double>(nv));
@@ -266,6 +275,12 @@ int auto_sums_split(const Params& P, int sms);
 bool use_sums_tiles(const Params& P, int split, int sms);
 SlotDev slot_desc(const ugks_ctx* h, int par, int walk_rows, int walk_vtile = 0);
 
+template <class N>
+void launch_sums_cell(const Params& P, const typename N::H* f, double* part, typename N::H* slopes, cudaStream_t st) {
+  k_sums_cell<N><<<4 * tiles_x(P) * tiles_y(P), 32 * kWarpsPerBlock, kWarpsPerBlock * kCellSumsWarp, st>>>(
+      P, f, part, slopes);
+}
+
 template <typename T>
 cudaError_t launch_step(ugks_ctx* h, cudaStream_t st) {
   if constexpr (sizeof(T) == 4) {
@@ -284,12 +299,17 @@ cudaError_t launch_step(ugks_ctx* h, cudaStream_t st) {
   if ((r = mark(h, 2)) != cudaSuccess) return r;
   const int nce = (P.nx + 2) * (P.ny + 2);
   double* sums = h->sums;
-  k_sums<T, T2><<<(nce + kWarpsPerBlock - 1) / kWarpsPerBlock, 32 * kWarpsPerBlock, smem_sums<T>(P.nv), st>>>(
-      P, fi, sums, reinterpret_cast<T2*>(h->slopes));
-  if ((r = mark(h, 3)) != cudaSuccess) return r;
-  const int nf = (P.nx + 1) * P.ny + P.nx * (P.ny + 1);
-  k_faces<kRecF64><<<(nf + h->face_block - 1) / h->face_block, h->face_block, 0, st>>>(P, sums, Wi, h->nwe, h->fxr, h->fyr, h->Fx, h->Fy,
-                                                     h->mt4);
+  const int nf = (P.nx + 1) * P.ny + P.nx * (P.ny + 1), fb = (nf + h->face_block - 1) / h->face_block;
+  if (P.shk) {  // the Shakhov model's heat-flux sums run one warp per cell
+    k_sums<T, T2><<<(nce + kWarpsPerBlock - 1) / kWarpsPerBlock, 32 * kWarpsPerBlock, smem_sums<T>(P.nv), st>>>(
+        P, fi, sums, reinterpret_cast<T2*>(h->slopes));
+    if ((r = mark(h, 3)) != cudaSuccess) return r;
+    k_faces<kRecF64, false><<<fb, h->face_block, 0, st>>>(P, sums, Wi, h->nwe, h->fxr, h->fyr, h->Fx, h->Fy, h->mt4);
+  } else {
+    launch_sums_cell<NumF64>(P, fi, sums, reinterpret_cast<T2*>(h->slopes), st);
+    if ((r = mark(h, 3)) != cudaSuccess) return r;
+    k_faces<kRecF64, true><<<fb, h->face_block, 0, st>>>(P, sums, Wi, h->nwe, h->fxr, h->fyr, h->Fx, h->Fy, h->mt4);
+  }
   if ((r = mark(h, 4)) != cudaSuccess) return r;
   const int nc = P.nx * P.ny;
   k_cells<<<h->nrblocks, h->cell_block, 0, st>>>(P, Wi, Wo, h->nwe, h->Fx, h->Fy, h->cells, h->rpart, h->err,
@@ -313,7 +333,10 @@ cudaError_t launch_step(ugks_ctx* h, cudaStream_t st) {
 size_t smem_face_flux_df(int nv) { return (size_t)4 * kWarpsPerBlock * nv * sizeof(df); }
 size_t smem_cell_update_df(int nv) { return (size_t)2 * kWarpsPerBlock * nv * sizeof(df); }
 cudaError_t set_smem_limits_df(int nv) {
-  cudaError_t e = cudaFuncSetAttribute(k_face_flux_df, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(k_sums_cell<NumDF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)(kWarpsPerBlock * kCellSumsWarp));
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(k_face_flux_df, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem_face_flux_df(nv));
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_cell_update_df, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -332,11 +355,10 @@ cudaError_t launch_step_df(ugks_ctx* h, cudaStream_t st) {
   k_ghost<DF4><<<ghost_cells(P), 128, 0, st>>>(P, fi, Wi, h->nwe);
   if ((r = mark(h, 1)) != cudaSuccess) return r;
   if ((r = mark(h, 2)) != cudaSuccess) return r;
-  const int nce = (P.nx + 2) * (P.ny + 2);
-  k_sums_df<<<(nce + kWarpsPerBlock - 1) / kWarpsPerBlock, 32 * kWarpsPerBlock, 0, st>>>(P, fi, h->sums, sl);
+  launch_sums_cell<NumDF>(P, fi, h->sums, sl, st);
   if ((r = mark(h, 3)) != cudaSuccess) return r;
   const int nf = (P.nx + 1) * P.ny + P.nx * (P.ny + 1);
-  k_faces<kRecDF><<<(nf + h->face_block - 1) / h->face_block, h->face_block, 0, st>>>(P, h->sums, Wi, h->nwe, h->fxd, h->fyd, h->Fx, h->Fy,
+  k_faces<kRecDF, true><<<(nf + h->face_block - 1) / h->face_block, h->face_block, 0, st>>>(P, h->sums, Wi, h->nwe, h->fxd, h->fyd, h->Fx, h->Fy,
                                                     h->mt4);
   if ((r = mark(h, 4)) != cudaSuccess) return r;
   const int nc = P.nx * P.ny;
@@ -747,7 +769,7 @@ ugks_status ugks_step_noalloc(const ugks_config* cfg, const double* f_in, const 
   k_ghost<double2><<<ghost_cells(P), 128, 0, st>>>(P, f0, W0, nwe);
   k_sums<double, double2><<<(nwe + kWarpsPerBlock - 1) / kWarpsPerBlock, 32 * kWarpsPerBlock,
                             smem_sums<double>(P.nv), st>>>(P, f0, sums, nullptr);
-  k_faces<kRecF64><<<(nfx + nfy + 127) / 128, 128, 0, st>>>(P, sums, W0, nwe, fxr, fyr, Fx, Fy, mt4);
+  k_faces<kRecF64, false><<<(nfx + nfy + 127) / 128, 128, 0, st>>>(P, sums, W0, nwe, fxr, fyr, Fx, Fy, mt4);
   k_cells<<<nrb, 128, 0, st>>>(P, W0, W1, nwe, Fx, Fy, cells, rpart, err, nullptr, mt4);
   // slopes are formed again in the update kernel: the scratch array holds no slope buffer
   k_update<double, double2><<<(nc + kWarpsPerBlock - 1) / kWarpsPerBlock, 32 * kWarpsPerBlock,
@@ -992,7 +1014,7 @@ ugks_status ugks_create(const ugks_config* cfg, void* cuda_stream, ugks_handle* 
   bool ok = alloc(&h->f[0], fbytes) && alloc(&h->f[1], fbytes) &&
             alloc((void**)&h->W[0], 4 * sizeof(double) * h->nwe) &&
             alloc((void**)&h->W[1], 4 * sizeof(double) * h->nwe) &&
-            alloc((void**)&h->sums, sizeof(double) * kNSum * (size_t)h->nwe) &&
+            alloc((void**)&h->sums, sizeof(double) * sums_per_cell(cfg) * (size_t)h->nwe) &&
             (!P.shk || alloc((void**)&h->hs, sizeof(double) * kNHeat * (size_t)h->nwe)) &&
             (f32 || alloc((void**)&h->slopes, sizeof(double2) * 2 * (size_t)h->nwe * P.nq)) &&
             (f32 || alloc((void**)&h->xflux, sizeof(double2) * (size_t)(nfx + nfy) * P.nq)) &&
@@ -1009,10 +1031,10 @@ ugks_status ugks_create(const ugks_config* cfg, void* cuda_stream, ugks_handle* 
             (f32 ? alloc((void**)&h->cellf, sizeof(CellRecF) * (size_t)nc)
                  : dfm ? alloc((void**)&h->celld, sizeof(CellRecD) * (size_t)nc)
                        : alloc((void**)&h->cells, sizeof(CellRec) * (size_t)nc)) &&
-            (!dfm || alloc((void**)&h->gdf, sizeof(float2) * (2 * (size_t)P.nu + 6 * (size_t)P.nv))) &&
+            (!dfm || alloc((void**)&h->gdf, sizeof(float2) * (8 * (size_t)P.nu + 8 * (size_t)P.nv))) &&
             alloc((void**)&h->rpart, sizeof(double) * 8 * (size_t)h->nrblocks) &&
             alloc((void**)&h->err, sizeof(int)) &&
-            alloc((void**)&h->d_grid, sizeof(double) * (2 * (P.nu + P.nv) + 5 * P.nv));
+            alloc((void**)&h->d_grid, sizeof(double) * (8 * (size_t)P.nu + 9 * (size_t)P.nv));
   if (ok && h->prec == UGKS_FP32F) {
     const size_t row_d = (size_t)P.nx * P.nq * 2 * sizeof(double);
     h->stage_bytes = 2 * stage_half_bytes(row_d, P.ny);
@@ -1040,6 +1062,19 @@ ugks_status ugks_create(const ugks_config* cfg, void* cuda_stream, ugks_handle* 
   grid.insert(grid.end(), h->hwv.begin(), h->hwv.end());
   for (int n = 0; n < 5; n++)
     for (int m = 0; m < P.nv; m++) grid.push_back(h->hwv[m] * std::pow(h->hv[m], n));
+  // tables of the thread-per-cell sums: [nu][6] w_u u^m (m = 0..4, half at u = 0) and u, [nv][2] v
+  // and w_v (half at v = 0)
+  std::vector<double> cell_tab;
+  for (int k = 0; k < P.nu; k++) {
+    for (int n = 0; n < 5; n++)
+      cell_tab.push_back((h->hu[k] == 0.0 ? 0.5 : 1.0) * h->hwu[k] * std::pow(h->hu[k], n));
+    cell_tab.push_back(h->hu[k]);
+  }
+  for (int m = 0; m < P.nv; m++) {
+    cell_tab.push_back(h->hv[m]);
+    cell_tab.push_back((h->hv[m] == 0.0 ? 0.5 : 1.0) * h->hwv[m]);
+  }
+  grid.insert(grid.end(), cell_tab.begin(), cell_tab.end());
   P.mvd = h->d_grid + 2 * (P.nu + P.nv);
   P.hs = h->hs;
   P.cshk = h->cshk;
@@ -1061,6 +1096,7 @@ ugks_status ugks_create(const ugks_config* cfg, void* cuda_stream, ugks_handle* 
     for (double x : h->hv) gdf_host.push_back(sp(x));
     for (int n = 0; n < 5; n++)
       for (int m = 0; m < P.nv; m++) gdf_host.push_back(sp(h->hwv[m] * std::pow(h->hv[m], n)));
+    for (double x : cell_tab) gdf_host.push_back(sp(x));
     P.gdf = h->gdf;
     P.df_tdx = sp(2.0 / P.dx);
     P.df_tdy = sp(2.0 / P.dy);

@@ -125,27 +125,6 @@ __device__ __forceinline__ df vl_df(df a, df c, df b) {
   return p.hi > 0.f ? r : df_zero();
 }
 
-// Warp sum of v[lane % N] returned to each lane (transpose reduce-scatter, as for FP64).
-template <int N>
-__device__ __forceinline__ df warp_reduce_scatter_df(df (&v)[N], int lane) {
-#pragma unroll
-  for (int o = N / 2; o >= 1; o >>= 1) {
-    const bool upper = (lane & o) != 0;
-#pragma unroll
-    for (int i = 0; i < o; i++) {
-      const df send = upper ? v[i] : v[i + o];
-      const df keep = upper ? v[i + o] : v[i];
-      const df got = {__shfl_xor_sync(kFull, send.hi, o), __shfl_xor_sync(kFull, send.lo, o)};
-      v[i] = df_add(keep, got);
-    }
-  }
-  df r = v[0];
-#pragma unroll
-  for (int o = N; o < 32; o <<= 1)
-    r = df_add(r, df{__shfl_xor_sync(kFull, r.hi, o), __shfl_xor_sync(kFull, r.lo, o)});
-  return r;
-}
-
 // Ghost ring: the FP64 form's, stored as double-FP32 pairs
 __device__ __forceinline__ DF4 ghost_value(DF4*, double h, double b) { return split4(h, b); }
 
@@ -195,212 +174,6 @@ __global__ void k_init_maxwellian_df(Params P, const double* __restrict__ prim, 
     W[nwe + w] = rho * U;
     W[2 * nwe + w] = rho * V;
     W[3 * nwe + w] = rho * (0.5 * (U * U + V * V) + (P.K + 2) / (4.0 * lam));
-  }
-}
-
-// -------------------------------------------------------------------------------------
-// S1 + S7 in double-FP32: the FP64 form's sums kernel (sums_body) with every velocity-cell
-// operation in double-FP32; the face sums each lane owns are accumulated in double-FP32
-// registers over velocity chunks and converted to FP64 once per cell.  The slopes of every
-// cell whose sums are formed go to the slope buffer (two DF4 per velocity-cell: r_x and r_y
-// of h and b) for the face-flux kernel.
-// -------------------------------------------------------------------------------------
-// The per-lane sums of one half of the v axis (a_n, ab_n, x_n, xb_n, y_n, yb_n as in sums_body).
-struct SumsHalfDF {
-  df a0, a1, a2, a3, ab0, ab1, x0, x1, x2, x3, xb0, xb1, y0, y1, y2, y3, y4, yb0, yb1, yb2;
-};
-// Close a half (north: the N side, else S): its 16 face sums reduced over the warp into
-// `side` (lanes < 16), and its sums added to the totals of the x sides.  Not inlined: one copy
-// of this long reduction serves both halves (the kernel's code otherwise misses the
-// instruction cache).
-__device__ __noinline__ void close_half_df(const SumsHalfDF& h, df u, df wu, df cu, df tdx, df tdy, bool north,
-                                           int lane, df& side, df* tot) {
-  auto pm = [&](df a, df y) { return north ? df_add(a, y) : df_sub(a, y); };
-  const df P0 = pm(h.a0, h.y0), P1 = pm(h.a1, h.y1), P2 = pm(h.a2, h.y2), P3 = pm(h.a3, h.y3);
-  const df Pb0 = pm(h.ab0, h.yb0), Pb1 = pm(h.ab1, h.yb1);
-  const df Z1 = df_fma(cu, h.x1, df_mul(tdy, h.y2)), Z2 = df_fma(cu, h.x2, df_mul(tdy, h.y3));
-  const df Z3 = df_fma(cu, h.x3, df_mul(tdy, h.y4)), Zb1 = df_fma(cu, h.xb1, df_mul(tdy, h.yb2));
-  const df uu = df_mul(u, u);
-  // (uu A + B)/2 + C/2
-  auto e4 = [&](df A, df B, df C) { return df_half(df_add(df_fma(uu, A, B), C)); };
-  df v[16];
-  v[0] = df_mul(wu, P0);
-  v[1] = df_mul(df_mul(wu, u), P0);
-  v[2] = df_mul(wu, P1);
-  v[3] = df_mul(wu, e4(P0, P2, Pb0));
-  const df ws = df_mul(wu, tdx);
-  v[4] = df_mul(ws, h.x0);
-  v[5] = df_mul(df_mul(ws, u), h.x0);
-  v[6] = df_mul(ws, h.x1);
-  v[7] = df_mul(ws, e4(h.x0, h.x2, h.xb0));
-  v[8] = df_mul(wu, P1);
-  v[9] = df_mul(df_mul(wu, u), P1);
-  v[10] = df_mul(wu, P2);
-  v[11] = df_mul(wu, e4(P1, P3, Pb1));
-  v[12] = df_mul(wu, Z1);
-  v[13] = df_mul(df_mul(wu, u), Z1);
-  v[14] = df_mul(wu, Z2);
-  v[15] = df_mul(wu, e4(Z1, Z3, Zb1));
-  const df r = warp_reduce_scatter_df<16>(v, lane);
-  if (lane < 16) side = df_add(side, r);
-  const df add[kSumsTotals] = {h.a0, h.a1, h.a2, h.ab0, h.x0, h.x1, h.x2, h.xb0, h.y0, h.y1, h.y2, h.y3, h.yb0, h.yb1};
-#pragma unroll
-  for (int t = 0; t < kSumsTotals; t++) tot[t] = df_add(tot[t], add[t]);
-}
-
-// The face sums of the x sides from the totals over both halves (E: u > 0 with f + r_x,
-// W: u < 0 with f - r_x, u = 0 half to each), reduced over the warp: entry `lane`.
-__device__ __noinline__ df x_sums_df(const df* tot, df u, df wu, df cu, df tdy, int lane) {
-  const df tA0 = tot[0], tA1 = tot[1], tA2 = tot[2], tAb = tot[3], tR0 = tot[4], tR1 = tot[5];
-  const df tR2 = tot[6], tRb = tot[7], tC0 = tot[8], tC1 = tot[9], tC2 = tot[10], tC3 = tot[11];
-  const df tCb0 = tot[12], tCb1 = tot[13];
-  const df D0 = df_fma(cu, tR0, df_mul(tdy, tC1)), D1 = df_fma(cu, tR1, df_mul(tdy, tC2));
-  const df D2 = df_fma(cu, tR2, df_mul(tdy, tC3)), Db = df_fma(cu, tRb, df_mul(tdy, tCb1));
-  const bool upos = u.hi > 0.f, uneg = u.hi < 0.f;
-  const df uu = df_mul(u, u);
-  auto e4 = [&](df A, df B, df C) { return df_half(df_add(df_fma(uu, A, B), C)); };
-  df xv[32];
-#pragma unroll
-  for (int sd = 0; sd < 2; sd++) {
-    // weight: wu on the upwind side, wu/2 on both sides for u = 0, 0 otherwise
-    const bool full = sd == 0 ? upos : uneg, none = sd == 0 ? uneg : upos;
-    const df wgt = none ? df_zero() : (full ? wu : df_half(wu));
-    auto pmx = [&](df a, df x) { return sd == 0 ? df_add(a, x) : df_sub(a, x); };
-    const df F0 = pmx(tA0, tR0), F1 = pmx(tA1, tR1), F2 = pmx(tA2, tR2), Fb = pmx(tAb, tRb);
-    df* o = xv + 16 * sd;
-    const df wgu = df_mul(wgt, u);
-    o[0] = df_mul(wgt, F0);
-    o[1] = df_mul(wgu, F0);
-    o[2] = df_mul(wgt, F1);
-    o[3] = df_mul(wgt, e4(F0, F2, Fb));
-    const df ws = df_mul(wgt, tdy);
-    o[4] = df_mul(ws, tC0);
-    o[5] = df_mul(df_mul(ws, u), tC0);
-    o[6] = df_mul(ws, tC1);
-    o[7] = df_mul(ws, e4(tC0, tC2, tCb0));
-    o[8] = df_mul(wgu, F0);
-    o[9] = df_mul(df_mul(wgu, u), F0);
-    o[10] = df_mul(wgu, F1);
-    o[11] = df_mul(wgu, e4(F0, F2, Fb));
-    o[12] = df_mul(wgu, D0);
-    o[13] = df_mul(df_mul(wgu, u), D0);
-    o[14] = df_mul(wgu, D1);
-    o[15] = df_mul(wgu, e4(D0, D2, Db));
-  }
-  return warp_reduce_scatter_df<32>(xv, lane);
-}
-
-__global__ void __launch_bounds__(128) k_sums_df(Params P, const DF4* __restrict__ f,
-                                                 double* __restrict__ sums, DF4* __restrict__ slopes) {
-  const int nv = P.nv, nu = P.nu, nq = P.nq;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int ncx = P.nx + 2;
-  const int cell = blockIdx.x * kWarpsPerBlock + warp;
-  if (cell >= ncx * (P.ny + 2)) return;
-  const int i = cell % ncx - 1, j = cell / ncx - 1;
-  const bool xg = i < 0 || i >= P.nx, yg = j < 0 || j >= P.ny;
-  if (xg && yg) return;
-  if ((i < 0 && P.bc_kind[0] == 1) || (i >= P.nx && P.bc_kind[1] == 1) ||
-      (j < 0 && P.bc_kind[2] == 1) || (j >= P.ny && P.bc_kind[3] == 1))
-    return;
-  const bool zs = (i < 0 && P.bc_kind[0] == 2) || (i >= P.nx && P.bc_kind[1] == 2) ||
-                  (j < 0 && P.bc_kind[2] == 2) || (j >= P.ny && P.bc_kind[3] == 2);
-  const DF4* fc = f + fcell(P, i, j) * nq;
-  const long rs = (long)P.ex * nq;
-  DF4* slc = slopes + (size_t)wcell(P, i, j) * nq * 2;
-  const df tdx = dfv(P.df_tdx), tdy = dfv(P.df_tdy);
-  const float2* tu = P.gdf;                 // u[nu]
-  const float2* twu = P.gdf + nu;           // wu[nu]
-  const float2* twn = P.gdf + 2 * nu + nv;  // [5][nv] wv v^n
-  const int mneg = P.m_neg, mpos = P.m_pos;
-  const bool v0 = mpos > mneg;
-  df ox = df_zero(), on = df_zero(), os = df_zero();  // owned face sums: E/W `lane`, N, S
-
-  for (int k0 = 0; k0 < nu; k0 += 32) {
-    const int k = k0 + lane;
-    const bool act = k < nu;
-    const int kk = act ? k : nu - 1;
-    const df u = dfv(tu[kk]);
-    const df wu = act ? dfv(twu[kk]) : df_zero();
-    const df cu = df_mul(u, tdx);
-    df a0, a1, a2, a3, ab0, ab1, x0, x1, x2, x3, xb0, xb1, y0, y1, y2, y3, y4, yb0, yb1, yb2;
-    // totals over both halves for the x sides: A0 A1 A2 Ab R0 R1 R2 Rb C0 C1 C2 C3 Cb0 Cb1
-    df tot[kSumsTotals];
-#pragma unroll
-    for (int t = 0; t < kSumsTotals; t++) tot[t] = df_zero();
-    auto zero = [&]() {
-      a0 = a1 = a2 = a3 = ab0 = ab1 = x0 = x1 = x2 = x3 = xb0 = xb1 = df_zero();
-      y0 = y1 = y2 = y3 = y4 = yb0 = yb1 = yb2 = df_zero();
-    };
-    // slopes of row m and the cell value
-    auto slopes_of = [&](int m, df& rxh, df& rxb, df& ryh, df& ryb, DF4& c) {
-      const DF4* src = fc + (size_t)m * nu + kk;
-      c = src[0];
-      if (zs) {
-        rxh = rxb = ryh = ryb = df_zero();
-      } else {
-        const DF4 w = src[-(long)nq], e = src[nq], s = src[-rs], n = src[rs];
-        rxh = vl_df(dh(w), dh(c), dh(e));
-        rxb = vl_df(db(w), db(c), db(e));
-        ryh = vl_df(dh(s), dh(c), dh(n));
-        ryb = vl_df(db(s), db(c), db(n));
-      }
-      if (act) {
-        DF4* q = slc + 2 * ((size_t)m * nu + k);
-        q[0] = mk4(rxh, rxb);
-        q[1] = mk4(ryh, ryb);
-      }
-    };
-    auto rows = [&](int m0, int m1) {
-#pragma unroll 1
-      for (int m = m0; m < m1; m++) {
-        df rxh, rxb, ryh, ryb;
-        DF4 c;
-        slopes_of(m, rxh, rxb, ryh, ryb, c);
-        const df w0 = dfv(twn[m]), w1 = dfv(twn[nv + m]), w2 = dfv(twn[2 * nv + m]);
-        const df w3 = dfv(twn[3 * nv + m]), w4 = dfv(twn[4 * nv + m]);
-        const df ch = dh(c), cb = db(c);
-        a0 = df_acc(a0, w0, ch); a1 = df_acc(a1, w1, ch); a2 = df_acc(a2, w2, ch); a3 = df_acc(a3, w3, ch);
-        ab0 = df_acc(ab0, w0, cb); ab1 = df_acc(ab1, w1, cb);
-        x0 = df_acc(x0, w0, rxh); x1 = df_acc(x1, w1, rxh); x2 = df_acc(x2, w2, rxh); x3 = df_acc(x3, w3, rxh);
-        xb0 = df_acc(xb0, w0, rxb); xb1 = df_acc(xb1, w1, rxb);
-        y0 = df_acc(y0, w0, ryh); y1 = df_acc(y1, w1, ryh); y2 = df_acc(y2, w2, ryh);
-        y3 = df_acc(y3, w3, ryh); y4 = df_acc(y4, w4, ryh);
-        yb0 = df_acc(yb0, w0, ryb); yb1 = df_acc(yb1, w1, ryb); yb2 = df_acc(yb2, w2, ryb);
-      }
-    };
-    auto row_v0 = [&](int m) {  // v = 0: only the w_0 sums, half weight
-      df rxh, rxb, ryh, ryb;
-      DF4 c;
-      slopes_of(m, rxh, rxb, ryh, ryb, c);
-      const df hw = df_half(dfv(twn[m]));
-      a0 = df_acc(a0, hw, dh(c)); ab0 = df_acc(ab0, hw, db(c));
-      x0 = df_acc(x0, hw, rxh); xb0 = df_acc(xb0, hw, rxb);
-      y0 = df_acc(y0, hw, ryh); yb0 = df_acc(yb0, hw, ryb);
-    };
-    // close a half: its face sums, then add it to the totals
-    auto close = [&](bool north, df& side) {
-      const SumsHalfDF h = {df_norm(a0), df_norm(a1), df_norm(a2), df_norm(a3), df_norm(ab0),
-                            df_norm(ab1), df_norm(x0), df_norm(x1), df_norm(x2), df_norm(x3),
-                            df_norm(xb0), df_norm(xb1), df_norm(y0), df_norm(y1), df_norm(y2),
-                            df_norm(y3), df_norm(y4), df_norm(yb0), df_norm(yb1), df_norm(yb2)};
-      close_half_df(h, u, wu, cu, tdx, tdy, north, lane, side, tot);
-    };
-    zero();
-    rows(0, mneg);
-    if (v0) row_v0(mneg);
-    close(false, os);
-    zero();
-    if (v0) row_v0(mneg);
-    rows(mpos, nv);
-    close(true, on);
-    ox = df_add(ox, x_sums_df(tot, u, wu, cu, tdy, lane));
-  }
-  double* out = sums + (size_t)cell * kNSum;
-  out[kSumE + lane] = to_double(ox);  // lanes 0..15: E side, 16..31: W side
-  if (lane < 16) {
-    out[kSumN + lane] = to_double(on);
-    out[kSumS + lane] = to_double(os);
   }
 }
 

@@ -60,10 +60,18 @@ __device__ __forceinline__ double rcp_nr(double s) {
 // van Leer limited slope of the stencil (a, c, b) times half the cell width:
 // r = sigma dx / 2 = d1 d2 / (d1 + d2) if d1 d2 > 0, else 0, with d1 = c - a, d2 = b - c.
 // (d1 d2 > 0 implies d1 + d2 != 0; a product small enough to make d1 + d2 subnormal
-// underflows to 0 and takes the zero branch.)
+// underflows to 0 and takes the zero branch.)  The quotient p / s from the reciprocal estimate r0
+// and one cubic step, q (1 + e + e^2) with q = p r0, e = 1 - s r0 (the estimate is good to about
+// 2^-20, so the cubic step leaves 2^-60): four FP64 operations instead of five, and the sign test
+// on the integer pipe (p > 0 read off its high word: neither zero, negative nor NaN; a subnormal p
+// whose high word is 0 counts as 0).
 __device__ __forceinline__ double vl_half(double a, double c, double b) {
-  double d1 = c - a, d2 = b - c, p = d1 * d2;
-  return p > 0.0 ? p * rcp_nr(d1 + d2) : 0.0;
+  const double d1 = c - a, d2 = b - c, p = d1 * d2, s = d1 + d2;
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(s));
+  const double e = fma(-s, r, 1.0), q = p * r;
+  const double t = fma(q, fma(e, e, e), q);
+  return (unsigned)(__double2hiint(p) - 1) <= 0x7fefffffu ? t : 0.0;
 }
 // 2^x and 1/x with subnormal results flushed to zero (PTX approximate forms).
 __device__ __forceinline__ float ex2_ftz(float x) {
@@ -1111,7 +1119,8 @@ __device__ __forceinline__ void face_rec_df(const FaceRec& R, FaceRecD& D) {
 // rx, ry: the x- and y-face records of kind REC (FaceRec, FaceRecF or FaceRecD).
 // SHK: the Shakhov model's interface heat flux and terms (a separate instance, so that the
 // BGK interface carries none of their code).
-template <int REC, bool SHK = false>
+// PART: the sums are the quadrants' partial sums of k_sums_cell, two of them per side.
+template <int REC, bool SHK = false, bool PART = false>
 __device__ __forceinline__ void faces_body(const Params& P, const double* __restrict__ sums,
                                            const double* __restrict__ W, int nwe,
                                            void* __restrict__ rx, void* __restrict__ ry,
@@ -1145,6 +1154,13 @@ __device__ __forceinline__ void faces_body(const Params& P, const double* __rest
     if (j == -1 && P.bc_kind[2] == 1) { wall = 1; side = 2; }
     if (j == ny - 1 && P.bc_kind[3] == 1) { wall = 2; side = 3; }
   }
+  // entry e of the sums of side o (kSumE ..) of a cell
+  auto side_sum = [&](int cell, int o, int e) {
+    if constexpr (!PART) return sums[(size_t)cell * kNSum + o + e];
+    // quadrants (E, N) (W, N) (E, S) (W, S): x side first, then y side
+    const double* p = sums + (size_t)cell * (4 * 32) + e;
+    return o == kSumE ? p[0] + p[64] : o == kSumW ? p[32] + p[96] : o == kSumN ? p[16] + p[48] : p[80] + p[112];
+  };
   FaceRec R;
   FaceRecF RF;
   constexpr bool f32 = REC == kRecF32;
@@ -1153,11 +1169,9 @@ __device__ __forceinline__ void faces_body(const Params& P, const double* __rest
     // diffuse wall: incoming half range from the gas cell's sums, outgoing wall Maxwellian
     // with the density that cancels the mass flux; first order in time
     const int oin = wall == 1 ? oR : oL;
-    const double* Se = wall == 1 ? sums + (size_t)cR * kNSum + oR + kOffSf
-                                 : sums + (size_t)cL * kNSum + oL + kOffSf;
     double Sin[4];
 #pragma unroll
-    for (int c = 0; c < 4; c++) Sin[c] = Se[c] + P.refsum[oin / 16][kOffSf + c];
+    for (int c = 0; c < 4; c++) Sin[c] = side_sum(wall == 1 ? cR : cL, oin, kOffSf + c) + P.refsum[oin / 16][kOffSf + c];
     const double rhow = -Sin[0] / P.wall_mom[side][0];
 #pragma unroll
     for (int c = 0; c < 4; c++) F[c] = P.dt * (Sin[c] + rhow * P.wall_mom[side][c]);
@@ -1176,17 +1190,15 @@ __device__ __forceinline__ void faces_body(const Params& P, const double* __rest
     if (f32) wall_face_f32(P, isx, R.bfac, lam, R.Ut, R.G, wall, RF);
   } else {
     const int pm[4] = {0, isx ? 1 : 2, isx ? 2 : 1, 3};  // natural -> face frame
-    const double* sL = sums + (size_t)cL * kNSum + oL;
-    const double* sR = sums + (size_t)cR * kNSum + oR;
     double W0[4], St[4], Sf[4], Ss[4], WL[4], WR[4], Fr[4];
     const double* rp = P.refpair[isx ? 0 : 1];  // g_ref sums of both sides (FP32-f form)
 #pragma unroll
     for (int c = 0; c < 4; c++) {
       const int s = pm[c];
-      W0[c] = (sL[kOffW0 + s] + sR[kOffW0 + s]) + rp[s];
-      Sf[c] = (sL[kOffSf + s] + sR[kOffSf + s]) + rp[4 + s];
-      St[c] = sL[kOffSt + s] + sR[kOffSt + s];
-      Ss[c] = sL[kOffSs + s] + sR[kOffSs + s];
+      W0[c] = (side_sum(cL, oL, kOffW0 + s) + side_sum(cR, oR, kOffW0 + s)) + rp[s];
+      Sf[c] = (side_sum(cL, oL, kOffSf + s) + side_sum(cR, oR, kOffSf + s)) + rp[4 + s];
+      St[c] = side_sum(cL, oL, kOffSt + s) + side_sum(cR, oR, kOffSt + s);
+      Ss[c] = side_sum(cL, oL, kOffSs + s) + side_sum(cR, oR, kOffSs + s);
       WL[c] = W[s * nwe + cL];
       WR[c] = W[s * nwe + cR];
     }
@@ -1246,14 +1258,14 @@ __device__ __forceinline__ void faces_body(const Params& P, const double* __rest
   }
 }
 // FP64 form (REC = kRecF64) and DF64 form (REC = kRecDF)
-template <int REC>
+template <int REC, bool PART>
 __global__ void __launch_bounds__(128, REC == kRecDF ? 4 : 3) k_faces(Params P, const double* __restrict__ sums, const double* __restrict__ W,
                         int nwe, void* __restrict__ rx, void* __restrict__ ry,
                         double* __restrict__ Fx, double* __restrict__ Fy, double* __restrict__ mt4) {
-  if (P.shk)
-    faces_body<REC, true>(P, sums, W, nwe, rx, ry, Fx, Fy, mt4, blockIdx.x * blockDim.x + threadIdx.x);
-  else
-    faces_body<REC, false>(P, sums, W, nwe, rx, ry, Fx, Fy, mt4, blockIdx.x * blockDim.x + threadIdx.x);
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if constexpr (PART) faces_body<REC, false, true>(P, sums, W, nwe, rx, ry, Fx, Fy, mt4, t);
+  else if (P.shk) faces_body<REC, true>(P, sums, W, nwe, rx, ry, Fx, Fy, mt4, t);
+  else faces_body<REC, false>(P, sums, W, nwe, rx, ry, Fx, Fy, mt4, t);
 }
 
 
