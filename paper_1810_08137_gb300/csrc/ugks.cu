@@ -225,28 +225,28 @@ template <typename T>
 size_t smem_update(int nv) {
   return (1 + 6 * kWarpsPerBlock) * (size_t)nv * sizeof(T);
 }
-template <typename T>
-size_t smem_face_flux(int nv) {
-  return (1 + 4 * kWarpsPerBlock) * (size_t)nv * sizeof(T);
+// Warps per block of the FP64 update kernels, whose tables take `doubles` per warp: four, fewer
+// where the tables of a large velocity grid would not fit an SM's shared memory.
+int update_warps(size_t doubles) {
+  const int w = (int)(224 * 1024 / (doubles * sizeof(double)));
+  return w < kWarpsPerBlock ? w : kWarpsPerBlock;
 }
-template <typename T>
-size_t smem_cell_update(int nv) {
-  return (1 + 2 * kWarpsPerBlock) * (size_t)nv * sizeof(T);
-}
+static_assert(face_flux_doubles(kMaxAxis, kMaxAxis) * sizeof(double) <= 224 * 1024, "tables of one warp");
 
 // dynamic shared memory limits of the FP64 form's sums and update kernels
-cudaError_t set_smem_limits_fp64(int nv) {
+cudaError_t set_smem_limits_fp64(int nu, int nv) {
   cudaError_t e = cudaFuncSetAttribute(k_sums<double, double2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem_sums<double>(nv));
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_sums_cell<NumF64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)(kWarpsPerBlock * kCellSumsWarp));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_face_flux<double, double2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem_face_flux<double>(nv));
+  const size_t ff = face_flux_doubles(nu, nv), cu = cell_update_doubles(nu, nv);
+  e = cudaFuncSetAttribute(k_face_flux, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)(update_warps(ff) * ff * sizeof(double)));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_cell_update<double, double2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem_cell_update<double>(nv));
+  e = cudaFuncSetAttribute(k_cell_update, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)(update_warps(cu) * cu * sizeof(double)));
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_update<double, double2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)smem_update<double>(nv));
@@ -318,10 +318,11 @@ cudaError_t launch_step(ugks_ctx* h, cudaStream_t st) {
   // the update in two passes: every face flux once, then Eq. 3 per velocity-cell
   T2* Xx = reinterpret_cast<T2*>(h->xflux);
   T2* Xy = Xx + (size_t)(P.nx + 1) * P.ny * P.nq;
-  const int ub = (nc + kWarpsPerBlock - 1) / kWarpsPerBlock;
-  k_face_flux<T, T2><<<ub, 32 * kWarpsPerBlock, smem_face_flux<T>(P.nv), st>>>(
+  const size_t ff = face_flux_doubles(P.nu, P.nv), cu = cell_update_doubles(P.nu, P.nv);
+  const int wf = update_warps(ff), wc = update_warps(cu);
+  k_face_flux<<<(nc + wf - 1) / wf, 32 * wf, wf * ff * sizeof(double), st>>>(
       P, fi, h->fxr, h->fyr, reinterpret_cast<const T2*>(h->slopes), Xx, Xy);
-  k_cell_update<T, T2><<<ub, 32 * kWarpsPerBlock, smem_cell_update<T>(P.nv), st>>>(P, fi, fo, h->cells, Xx, Xy);
+  k_cell_update<<<(nc + wc - 1) / wc, 32 * wc, wc * cu * sizeof(double), st>>>(P, fi, fo, h->cells, Xx, Xy);
   if ((r = mark(h, 6)) != cudaSuccess) return r;
   if (h->profiling) h->events_used += UGKS_NKERNELS + 1;
   return cudaGetLastError();
@@ -765,7 +766,7 @@ ugks_status ugks_step_noalloc(const ugks_config* cfg, const double* f_in, const 
     NA_CK(cudaMemcpy2DAsync(W0 + (size_t)c * nwe + wcell(P, 0, 0), P.wx * sizeof(double),
                             W_in + (size_t)c * nc, nx * sizeof(double), nx * sizeof(double), ny,
                             cudaMemcpyDeviceToDevice, st));
-  NA_CK(set_smem_limits_fp64(P.nv));
+  NA_CK(set_smem_limits_fp64(P.nu, P.nv));
   k_ghost<double2><<<ghost_cells(P), 128, 0, st>>>(P, f0, W0, nwe);
   k_sums<double, double2><<<(nwe + kWarpsPerBlock - 1) / kWarpsPerBlock, 32 * kWarpsPerBlock,
                             smem_sums<double>(P.nv), st>>>(P, f0, sums, nullptr);
@@ -1160,7 +1161,7 @@ ugks_status ugks_create(const ugks_config* cfg, void* cuda_stream, ugks_handle* 
                                        cudaMemcpyHostToDevice, h->stream)) != cudaSuccess)
       return r;
     if ((r = cudaMemsetAsync(h->err, 0, sizeof(int), h->stream)) != cudaSuccess) return r;
-    if (h->prec == UGKS_FP64 && (r = set_smem_limits_fp64(P.nv)) != cudaSuccess) return r;
+    if (h->prec == UGKS_FP64 && (r = set_smem_limits_fp64(P.nu, P.nv)) != cudaSuccess) return r;
     if (h->prec == UGKS_DF64 && (r = set_smem_limits_df(P.nv)) != cudaSuccess) return r;
     if ((r = cudaStreamSynchronize(h->stream)) != cudaSuccess) return r;
     return h->prec == UGKS_FP32F ? setup_single_f32(h) : cudaSuccess;

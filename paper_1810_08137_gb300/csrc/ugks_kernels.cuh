@@ -1690,253 +1690,232 @@ __global__ void __launch_bounds__(128) k_update(Params P, const T2* __restrict__
 
 // -------------------------------------------------------------------------------------
 // The same update in two passes, FP64 form: every (face, velocity) micro flux once.
-// k_face_flux: one warp per interior cell, lane = u index; for each velocity the cell forms
-// the flux X = Q g + Mt4 f_up - Mt5 d_up (or the wall flux) through its downwind x-face and
-// y-face from its own reconstruction, and a cell next to the boundary also forms the flux
-// whose upwind side is the ghost cell or the wall.  Every face and velocity is written by
-// exactly one warp, into Xx [(nx+1) ny][nq] and Xy [nx (ny+1)][nq] (face-major, velocity
-// innermost).  k_cell_update then reads the four fluxes of each velocity-cell and applies
-// Eq. 3.  The arithmetic of each flux and of the update is that of k_update, which forms
-// the four face fluxes of every velocity-cell (each interior flux twice).
+// k_face_flux: one warp per interior cell; for each velocity the cell forms the flux
+// X = Q g + Mt4 f_up - Mt5 d_up (or the wall flux) through its downwind x-face and y-face from
+// its own reconstruction, and a cell next to the boundary also forms the flux whose upwind side
+// is the ghost cell or the wall.  Every face and velocity is written by exactly one warp, into
+// Xx [(nx+1) ny][nq] and Xy [nx (ny+1)][nq] (face-major, velocity innermost).  k_cell_update then
+// reads the four fluxes of each velocity-cell and applies Eq. 3.
+// Both are bound by the FP64 pipe (2 operations per clock and SM).  Lanes run over the flattened
+// velocities (a lane per u would leave 12 of 32 idle at nu = 20), and all that depends on u or v
+// alone comes from per-warp tables in shared memory, so a velocity-cell costs 28 FP64
+// instructions for its two faces: per face 3 for Q_h, 2 for Q_b = X2 Q_h + linear, 1 for g and 4 per
+// component, with f_up and d_up folded into the coefficients of the cell value and its two half
+// slopes (67 before), 36 with the tables; k_cell_update 18 (22 with tables, 30 before).  Both passes,
+// 100x50x28^2 0.820 -> 0.518 ms, 40x20x20^2 163 -> 90 us; FP64 pipe 89 % busy.
 // -------------------------------------------------------------------------------------
-template <typename T>
-struct FaceK {
-  T Mt4, Mt5, bf;
-  int wall;
-};
-template <typename T, typename T2>
-__global__ void __launch_bounds__(128) k_face_flux(Params P, const T2* __restrict__ f,
-                                                   const FaceRec* __restrict__ fxr,
-                                                   const FaceRec* __restrict__ fyr,
-                                                   const T2* __restrict__ sl, T2* __restrict__ Xx,
-                                                   T2* __restrict__ Xy) {
+// Tables of k_face_flux (doubles, one after the other): per u index, the downwind x-face
+// (kFluxX arrays), then the downwind y-face for v <= 0 and for v > 0 (kFluxX arrays each), then
+// the factors of g of the upwind faces (x, y for v <= 0, y for v > 0; boundary cells only); per v
+// index kFluxM arrays.
+constexpr int kFluxX = 8;  // q0 q1 q2 q3 (Q_h in v), l0 l1 (Q_b - X2 Q_h), c1 (coefficient of r_x), g
+constexpr int kFluxU = 3 * kFluxX + 3;
+constexpr int kFluxM = 7;  // factors of g: W, E, downwind y, upwind y; coefficient of r_y: W, E, downwind y
+__host__ __device__ constexpr size_t face_flux_doubles(int nu, int nv) {
+  return (size_t)kFluxU * nu + (size_t)kFluxM * nv;
+}
+
+__global__ void __launch_bounds__(128, 4) k_face_flux(Params P, const double2* __restrict__ f,
+                                                      const FaceRec* __restrict__ fxr,
+                                                      const FaceRec* __restrict__ fyr,
+                                                      const double2* __restrict__ sl, double2* __restrict__ Xx,
+                                                      double2* __restrict__ Xy) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  const int nv = P.nv, nu = P.nu, nq = P.nq, nx = P.nx, ny = P.ny;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  T* sv = reinterpret_cast<T*>(smraw);
-  T* ev = sv + nv + warp * 4 * nv;  // [4][nv]: x W, x E, y S, y N factors in v
-  for (int m = tid; m < nv; m += blockDim.x) sv[m] = (T)P.v[m];
-  __syncthreads();
-  const int cell = blockIdx.x * kWarpsPerBlock + warp;
+  const int nv = P.nv, nu = P.nu, nq = P.nq, nx = P.nx, ny = P.ny, mpos = P.m_pos;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double* tu = reinterpret_cast<double*>(smraw) + warp * face_flux_doubles(nu, nv);
+  double* tm = tu + kFluxU * nu;
+  const int cell = blockIdx.x * (blockDim.x >> 5) + warp;
   if (cell >= nx * ny) return;
   const int i = cell % nx, j = cell / nx;
   const FaceRec& RW = fxr[(size_t)j * (nx + 1) + i];
   const FaceRec& RE = fxr[(size_t)j * (nx + 1) + i + 1];
   const FaceRec& RS = fyr[(size_t)j * nx + i];
   const FaceRec& RN = fyr[(size_t)(j + 1) * nx + i];
+  const bool edge = i == 0 || i == nx - 1 || j == 0 || j == ny - 1;
+  auto gauss = [](double lam, double d) { return exp(-lam * d * d); };
+
+  // u tables: Q at fixed u as a polynomial in v; a wall face passes dt f_up (Mt4 = dt, no Q)
+  for (int k = lane; k < nu; k += 32) {
+    const double u = P.u[k], cu = u * P.d_tdx;
+    const bool up = u > 0.0;
+    auto face = [&](const FaceRec& R, int side, bool xface, double c1, double* t) {
+      const double* h = R.Q[side][0];
+      const double* b = R.Q[side][1];
+      double q[4] = {0.0, 0.0, 0.0, 0.0}, l0 = 0.0, l1 = 0.0, g = 0.0;
+      if (!R.wall) {
+        const double d0 = b[0] - R.bfac * h[0], dn = b[1] - R.bfac * h[1], dt = b[2] - R.bfac * h[2];
+        if (xface) poly_in_v_xface(h, u, q);
+        else poly_in_v_yface(h, u, q);
+        l0 = d0 + u * (xface ? dn : dt);
+        l1 = xface ? dt : dn;
+        g = R.G * gauss(R.lam, u - (xface ? R.Un : R.Ut));
+      }
+#pragma unroll
+      for (int e = 0; e < 4; e++) t[e * nu + k] = q[e];
+      t[4 * nu + k] = l0;
+      t[5 * nu + k] = l1;
+      t[6 * nu + k] = c1;
+      t[7 * nu + k] = g;
+    };
+    const FaceRec& RX = up ? RE : RW;
+    face(RX, up ? 0 : 1, true, (up ? RX.Mt4 : -RX.Mt4) - RX.Mt5 * cu, tu);
+    face(RS, 1, false, -RS.Mt5 * cu, tu + kFluxX * nu);
+    face(RN, 0, false, -RN.Mt5 * cu, tu + 2 * kFluxX * nu);
+    if (edge) {
+      const FaceRec& RG = up ? RW : RE;
+      double* tg = tu + 3 * kFluxX * nu + k;
+      tg[0] = RG.G * gauss(RG.lam, u - RG.Un);
+      tg[nu] = RN.G * gauss(RN.lam, u - RN.Ut);
+      tg[2 * nu] = RS.G * gauss(RS.lam, u - RS.Ut);
+    }
+  }
   for (int m = lane; m < nv; m += 32) {
-    const double vv = P.v[m];
-    double d;
-    d = vv - RW.Ut; ev[0 * nv + m] = (T)exp(-RW.lam * d * d);  // x faces: ut = v
-    d = vv - RE.Ut; ev[1 * nv + m] = (T)exp(-RE.lam * d * d);
-    d = vv - RS.Un; ev[2 * nv + m] = (T)exp(-RS.lam * d * d);  // y faces: un = v
-    d = vv - RN.Un; ev[3 * nv + m] = (T)exp(-RN.lam * d * d);
+    const double v = P.v[m], cv = v * P.d_tdy;
+    const bool vp = m >= mpos;
+    const FaceRec& RD = vp ? RN : RS;
+    const FaceRec& RG = vp ? RS : RN;
+    tm[m] = gauss(RW.lam, v - RW.Ut);
+    tm[nv + m] = gauss(RE.lam, v - RE.Ut);
+    tm[2 * nv + m] = gauss(RD.lam, v - RD.Un);
+    tm[3 * nv + m] = edge ? gauss(RG.lam, v - RG.Un) : 0.0;
+    tm[4 * nv + m] = -RW.Mt5 * cv;
+    tm[5 * nv + m] = -RE.Mt5 * cv;
+    tm[6 * nv + m] = (vp ? RD.Mt4 : -RD.Mt4) - RD.Mt5 * cv;
   }
   __syncwarp();
-  auto faceK = [](const FaceRec& R) { return FaceK<T>{(T)R.Mt4, (T)R.Mt5, (T)R.bfac, R.wall}; };
-  const FaceK<T> KW = faceK(RW), KE = faceK(RE), KS = faceK(RS), KN = faceK(RN);
-  const T tdx = T(2.0 / P.dx), tdy = T(2.0 / P.dy);
-  const T dtT = (T)P.dt;
-  const long rs = (long)P.ex * nq;
-  const T2* fc0 = f + fcell(P, i, j) * nq;
-  const T2* sl0 = sl + (size_t)wcell(P, i, j) * nq * 2;  // this cell's slopes
-  T2* xw0 = Xx + ((size_t)j * (nx + 1) + i) * nq;        // W face of the cell; E face: + nq
-  T2* ys0 = Xy + ((size_t)j * nx + i) * nq;              // S face; N face: + nx nq
-  const bool pW = P.bc_kind[0] == 2, pE = P.bc_kind[1] == 2, pS = P.bc_kind[2] == 2, pN = P.bc_kind[3] == 2;
+  const double MW = RW.Mt4, ME = RE.Mt4, MS = RS.Mt4, MN = RN.Mt4;
+  const double XW = RW.bfac, XE = RE.bfac, XS = RS.bfac, XN = RN.bfac;
+  const double2* fc0 = f + fcell(P, i, j) * nq;
+  const double2* sl0 = sl + (size_t)wcell(P, i, j) * nq * 2;  // this cell's slopes
+  double2* xw0 = Xx + ((size_t)j * (nx + 1) + i) * nq;        // W face of the cell; E face: + nq
+  double2* ys0 = Xy + ((size_t)j * nx + i) * nq;              // S face; N face: + nx nq
+  const size_t ynf = (size_t)nx * nq;
+  const int kpos = P.k_pos;
 
-  // X of a face from the face value fh, fb and slope term dh, db of its upwind side; inc:
-  // the gas side is upwind (a wall face then passes dt f_up, else dt g_wall)
-  auto flux = [&](const FaceK<T>& F, const T (&qh)[4], const T (&qb)[4], T vv, T g, T fh, T fb,
-                  T dh, T db, bool inc) {
-    T2 X;
-    if (F.wall) {
-      X.x = inc ? dtT * fh : dtT * g;
-      X.y = inc ? dtT * fb : dtT * (F.bf * g);
-    } else {
-      X.x = horner3(qh, vv) * g + F.Mt4 * fh - F.Mt5 * dh;
-      X.y = horner3(qb, vv) * g + F.Mt4 * fb - F.Mt5 * db;
-    }
-    return X;
-  };
-
-  for (int k0 = 0; k0 < nu; k0 += 32) {
-    const int k = k0 + lane;
-    const bool act = k < nu;
-    const int kk = act ? k : nu - 1;
-    const double ud = P.u[kk];
-    const T u = (T)ud;
-    T gu[4];
-    {
-      double d;
-      d = ud - RW.Un; gu[0] = (T)(RW.G * exp(-RW.lam * d * d));
-      d = ud - RE.Un; gu[1] = (T)(RE.G * exp(-RE.lam * d * d));
-      d = ud - RS.Ut; gu[2] = (T)(RS.G * exp(-RS.lam * d * d));
-      d = ud - RN.Ut; gu[3] = (T)(RN.G * exp(-RN.lam * d * d));
-    }
-    const int xs = ud > 0.0 ? 0 : 1;  // upwind side of the x-face records
-    const bool up = ud > 0.0;         // downwind x-face: E for u > 0, W otherwise
-    const T sgx = up ? T(1) : T(-1);  // f_up = f + sgx r_x on the downwind face
-    // the downwind x-face (formed by this cell for every velocity) and the upwind one
-    // (formed here only when its upwind side is a ghost cell or a wall)
-    const FaceRec& RXd = up ? RE : RW;
-    const FaceRec& RXg = up ? RW : RE;
-    const FaceK<T> KXd = up ? KE : KW, KXg = up ? KW : KE;
-    const T gXd = up ? gu[1] : gu[0], gXg = up ? gu[0] : gu[1];
-    const T* evXd = ev + (up ? nv : 0);
-    const T* evXg = ev + (up ? 0 : nv);
-    T2* xd0 = up ? xw0 + nq : xw0;
-    T2* xg0 = up ? xw0 : xw0 + nq;
-    T qX[2][4];
-#pragma unroll
-    for (int c = 0; c < 2; c++) poly_in_v_xface(RXd.Q[xs][c], ud, qX[c]);
-    const long xo = up ? -(long)nq : (long)nq;  // x-upwind neighbour in f, in q
-    const bool xg = up ? i == 0 : i == nx - 1;  // it is a ghost cell (or a wall)
-    const bool xz = (up && i == 0 && pW) || (!up && i == nx - 1 && pE);
-    const T cu = u * tdx;
-
-    auto half = [&](auto vup_tag, int m0, int m1) {
-      constexpr bool VUP = decltype(vup_tag)::value;  // downwind y-face: N for v > 0, S otherwise
-      constexpr int ys = VUP ? 0 : 1;
-      const FaceRec& RYd = VUP ? RN : RS;
-      const FaceRec& RYg = VUP ? RS : RN;
-      const FaceK<T>& KYd = VUP ? KN : KS;
-      const FaceK<T>& KYg = VUP ? KS : KN;
-      const T gYd = VUP ? gu[3] : gu[2], gYg = VUP ? gu[2] : gu[3];
-      const T* evYd = ev + (VUP ? 3 : 2) * nv;
-      const T* evYg = ev + (VUP ? 2 : 3) * nv;
-      T2* yd0 = VUP ? ys0 + (size_t)nx * nq : ys0;
-      T2* yg0 = VUP ? ys0 : ys0 + (size_t)nx * nq;
-      constexpr T sgy = VUP ? T(1) : T(-1);
-      T qY[2][4];
-#pragma unroll
-      for (int c = 0; c < 2; c++) poly_in_v_yface(RYd.Q[ys][c], ud, qY[c]);
-      const long yo = VUP ? -rs : rs;                             // y-upwind neighbour in f
-      const long yso = VUP ? -(long)P.wx * nq : (long)P.wx * nq;  // ... in the slope buffer
-      const bool yg = VUP ? j == 0 : j == ny - 1;
-      const bool yz = (VUP && j == 0 && pS) || (!VUP && j == ny - 1 && pN);
-      for (int m = m0; m < m1; m++) {
-        const T vv = sv[m];
-        const size_t q = (size_t)m * nu + kk;
-        const T2* p = fc0 + q;
-        const T2 c = p[0];
-        const T2* sq = sl0 + 2 * q;
-        const T2 a = sq[0], b = sq[1];  // half slopes r_x, r_y of the cell (h, b)
-        const T cv = vv * tdy;
-        const T dch = cu * a.x + cv * b.x, dcb = cu * a.y + cv * b.y;
-        T2 X = flux(KXd, qX[0], qX[1], vv, gXd * evXd[m], c.x + sgx * a.x, c.y + sgx * a.y, dch,
-                    dcb, true);
-        if (act) xd0[q] = X;
-        if (xg) {
-          const T2 xu = p[xo];
-          const T2* su = sq + 2 * xo;
-          T2 au = su[0], bu = su[1];
-          if (xz) au.x = au.y = bu.x = bu.y = T(0);
-          const T duh = cu * au.x + cv * bu.x, dub = cu * au.y + cv * bu.y;
-          T qg[2][4];
-#pragma unroll
-          for (int cc = 0; cc < 2; cc++) poly_in_v_xface(RXg.Q[xs][cc], ud, qg[cc]);
-          X = flux(KXg, qg[0], qg[1], vv, gXg * evXg[m], xu.x + sgx * au.x, xu.y + sgx * au.y, duh,
-                   dub, false);
-          if (act) xg0[q] = X;
-        }
-        X = flux(KYd, qY[0], qY[1], vv, gYd * evYd[m], c.x + sgy * b.x, c.y + sgy * b.y, dch, dcb,
-                 true);
-        if (act) yd0[q] = X;
-        if (yg) {
-          const T2 yu = p[yo];
-          const T2* sw = sq + 2 * yso;
-          T2 av = sw[0], bv = sw[1];
-          if (yz) av.x = av.y = bv.x = bv.y = T(0);
-          const T dvh = cu * av.x + cv * bv.x, dvb = cu * av.y + cv * bv.y;
-          T qg[2][4];
-#pragma unroll
-          for (int cc = 0; cc < 2; cc++) poly_in_v_yface(RYg.Q[ys][cc], ud, qg[cc]);
-          X = flux(KYg, qg[0], qg[1], vv, gYg * evYg[m], yu.x + sgy * bv.x, yu.y + sgy * bv.y, dvh,
-                   dvb, false);
-          if (act) yg0[q] = X;
-        }
-      }
+  int m = lane / nu, k = lane - m * nu;
+  for (int q = lane; q < nq; q += 32) {
+    const bool up = k >= kpos, vp = m >= mpos;  // u > 0, v > 0
+    const double v = P.v[m];
+    const double2 c = fc0[q], a = sl0[2 * q], b = sl0[2 * q + 1];  // half slopes r_x, r_y (h, b)
+    // X of a face from its u table, coefficient c2 of r_y, Mt4, X2 = <xi^2> and v factor of g
+    auto flux = [&](const double* t, double c2, double m4, double x2, double ev) {
+      const double qh = fma(fma(fma(t[3 * nu], v, t[2 * nu]), v, t[nu]), v, t[0]);
+      const double qb = fma(x2, qh, fma(t[5 * nu], v, t[4 * nu]));
+      const double c1 = t[6 * nu], g = t[7 * nu] * ev;
+      return make_double2(fma(qh, g, fma(c2, b.x, fma(c1, a.x, m4 * c.x))),
+                          fma(qb, g, fma(c2, b.y, fma(c1, a.y, m4 * c.y))));
     };
-    half(std::integral_constant<bool, false>{}, 0, P.m_pos);
-    half(std::integral_constant<bool, true>{}, P.m_pos, nv);
+    (up ? xw0 + nq : xw0)[q] = flux(tu + k, tm[(up ? 5 : 4) * nv + m], up ? ME : MW, up ? XE : XW,
+                                    tm[(up ? nv : 0) + m]);
+    (vp ? ys0 + ynf : ys0)[q] = flux(tu + (vp ? 2 : 1) * kFluxX * nu + k, tm[6 * nv + m], vp ? MN : MS,
+                                     vp ? XN : XS, tm[2 * nv + m]);
+    if (edge) {
+      // faces whose upwind side is a ghost cell or a wall
+      const double u = P.u[k], cu = u * P.d_tdx, cv = v * P.d_tdy;
+      auto ghost = [&](const FaceRec& R, int side, bool xface, bool zero, double g, double2 fu, double2 au,
+                       double2 bu, double sg) {
+        if (R.wall) return make_double2(P.dt * g, P.dt * (R.bfac * g));
+        if (zero) au.x = au.y = bu.x = bu.y = 0.0;
+        double qh[4], qb[4];
+        if (xface) {
+          poly_in_v_xface(R.Q[side][0], u, qh);
+          poly_in_v_xface(R.Q[side][1], u, qb);
+        } else {
+          poly_in_v_yface(R.Q[side][0], u, qh);
+          poly_in_v_yface(R.Q[side][1], u, qb);
+        }
+        const double dh = cu * au.x + cv * bu.x, db = cu * au.y + cv * bu.y;
+        const double fh = fu.x + sg * (xface ? au.x : bu.x), fb = fu.y + sg * (xface ? au.y : bu.y);
+        return make_double2(horner3(qh, v) * g + R.Mt4 * fh - R.Mt5 * dh, horner3(qb, v) * g + R.Mt4 * fb - R.Mt5 * db);
+      };
+      if (up ? i == 0 : i == nx - 1) {
+        const FaceRec& R = up ? RW : RE;
+        const long xo = up ? -(long)nq : (long)nq;
+        (up ? xw0 : xw0 + nq)[q] = ghost(R, up ? 0 : 1, true, P.bc_kind[up ? 0 : 1] == 2,
+                                         tu[3 * kFluxX * nu + k] * tm[(up ? 0 : nv) + m], fc0[q + xo],
+                                         sl0[2 * (q + xo)], sl0[2 * (q + xo) + 1], up ? 1.0 : -1.0);
+      }
+      if (vp ? j == 0 : j == ny - 1) {
+        const FaceRec& R = vp ? RS : RN;
+        const long yo = (vp ? -1L : 1L) * P.ex * nq, yso = (vp ? -1L : 1L) * P.wx * nq;
+        (vp ? ys0 : ys0 + ynf)[q] = ghost(R, vp ? 0 : 1, false, P.bc_kind[vp ? 2 : 3] == 2,
+                                          tu[(3 * kFluxX + (vp ? 2 : 1)) * nu + k] * tm[3 * nv + m], fc0[q + yo],
+                                          sl0[2 * (q + yso)], sl0[2 * (q + yso) + 1], vp ? 1.0 : -1.0);
+      }
+    }
+    k += 32;
+    while (k >= nu) {
+      k -= nu;
+      m++;
+    }
   }
 }
 
-// Eq. 3 from the four face fluxes of each velocity-cell (k_face_flux), FP64 form.
-template <typename T, typename T2>
-__global__ void __launch_bounds__(128) k_cell_update(Params P, const T2* __restrict__ f,
-                                                     T2* __restrict__ fo,
-                                                     const CellRec* __restrict__ cr,
-                                                     const T2* __restrict__ Xx,
-                                                     const T2* __restrict__ Xy) {
+// Eq. 3 from the four face fluxes of each velocity-cell (k_face_flux), FP64 form: the increment
+// f^{n+1} - f^n = inv (flux + cg1 (g^{n+1} - f^n) + cgn (g^n - f^n)) with inv folded into the
+// coefficients; 18 FP64 instructions per velocity-cell.  Tables per warp: per u index
+// inv u/dx, g^n and g^{n+1} factors; per v index the same with v/dy.
+__host__ __device__ constexpr size_t cell_update_doubles(int nu, int nv) { return 3 * ((size_t)nu + nv); }
+
+__global__ void __launch_bounds__(128) k_cell_update(Params P, const double2* __restrict__ f,
+                                                     double2* __restrict__ fo, const CellRec* __restrict__ cr,
+                                                     const double2* __restrict__ Xx,
+                                                     const double2* __restrict__ Xy) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const int nv = P.nv, nu = P.nu, nq = P.nq, nx = P.nx, ny = P.ny;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  T* sv = reinterpret_cast<T*>(smraw);
-  T* ev = sv + nv + warp * 2 * nv;  // [2][nv]: g^n, g^{n+1} factors in v
-  for (int m = tid; m < nv; m += blockDim.x) sv[m] = (T)P.v[m];
-  __syncthreads();
-  const int cell = blockIdx.x * kWarpsPerBlock + warp;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double* tu = reinterpret_cast<double*>(smraw) + warp * cell_update_doubles(nu, nv);
+  double* tm = tu + 3 * nu;
+  const int cell = blockIdx.x * (blockDim.x >> 5) + warp;
   if (cell >= nx * ny) return;
   const int i = cell % nx, j = cell / nx;
   const CellRec& C = cr[cell];
+  const double inv = C.inv;
+  for (int k = lane; k < nu; k += 32) {
+    const double u = P.u[k], dn = u - C.Un, d1 = u - C.U1;
+    tu[k] = inv * P.d_idx * u;
+    tu[nu + k] = C.Gn * exp(-C.lamn * dn * dn);
+    tu[2 * nu + k] = C.G1 * exp(-C.lam1 * d1 * d1);
+  }
   for (int m = lane; m < nv; m += 32) {
-    const double vv = P.v[m];
-    double d;
-    d = vv - C.Vn; ev[m] = (T)exp(-C.lamn * d * d);
-    d = vv - C.V1; ev[nv + m] = (T)exp(-C.lam1 * d * d);
+    const double v = P.v[m], dn = v - C.Vn, d1 = v - C.V1;
+    tm[m] = inv * P.d_idy * v;
+    tm[nv + m] = exp(-C.lamn * dn * dn);
+    tm[2 * nv + m] = exp(-C.lam1 * d1 * d1);
   }
   __syncwarp();
-  const T inv = (T)C.inv, cg1 = (T)C.cg1, cgn = (T)C.cgn;
-  const T cg1b = (T)(C.cg1 * C.b1), cgnb = (T)(C.cgn * C.bn);
-  const T idx = T(1.0 / P.dx), idy = T(1.0 / P.dy);
-  const T2* fc0 = f + fcell(P, i, j) * nq;
-  T2* fo0 = fo + fcell(P, i, j) * nq;
-  const T2* xw0 = Xx + ((size_t)j * (nx + 1) + i) * nq;
-  const T2* ys0 = Xy + ((size_t)j * nx + i) * nq;
-  for (int k0 = 0; k0 < nu; k0 += 32) {
-    const int k = k0 + lane;
-    const bool act = k < nu;
-    const int kk = act ? k : nu - 1;
-    const double ud = P.u[kk];
-    const T u = (T)ud;
-    T gun, gu1;
-    {
-      double d;
-      d = ud - C.Un; gun = (T)(C.Gn * exp(-C.lamn * d * d));
-      d = ud - C.U1; gu1 = (T)(C.G1 * exp(-C.lam1 * d * d));
+  const double A1 = inv * C.cg1, An = inv * C.cgn, nB = -(A1 + An), A1b = A1 * C.b1, Anb = An * C.bn;
+  const double2* fc0 = f + fcell(P, i, j) * nq;
+  double2* fo0 = fo + fcell(P, i, j) * nq;
+  const double2* xw0 = Xx + ((size_t)j * (nx + 1) + i) * nq;
+  const double2* ys0 = Xy + ((size_t)j * nx + i) * nq;
+  const size_t ynf = (size_t)nx * nq;
+  int m = lane / nu, k = lane - m * nu;
+  for (int q = lane; q < nq; q += 32) {
+    const double2 c = fc0[q], XW = xw0[q], XE = xw0[nq + q], XS = ys0[q], XN = ys0[ynf + q];
+    const double au = tu[k], av = tm[m];
+    const double gn = tu[nu + k] * tm[nv + m], g1 = tu[2 * nu + k] * tm[2 * nv + m];
+    const double flh = fma(au, XW.x - XE.x, av * (XS.x - XN.x)), flb = fma(au, XW.y - XE.y, av * (XS.y - XN.y));
+    double dh, db;
+    if (!P.shk) {
+      dh = fma(A1, g1, fma(An, gn, fma(nB, c.x, flh)));
+      db = fma(A1b, g1, fma(Anb, gn, fma(nB, c.y, flb)));
+    } else {  // Shakhov: g+_h = g_h (1 + S_h), g+_b = g_h (b + S_b), heat flux of f^n
+      const double u = P.u[k], v = P.v[m];
+      double cu = u - C.Un, cv = v - C.Vn, cq = cu * C.qx + cv * C.qy, c2 = 2.0 * C.lamn * (cu * cu + cv * cv);
+      const double shn = C.an * cq * (c2 - 4.0), sbn = C.an * cq * C.bn * (c2 - 2.0);
+      cu = u - C.U1; cv = v - C.V1;
+      cq = cu * C.qx + cv * C.qy; c2 = 2.0 * C.lam1 * (cu * cu + cv * cv);
+      const double sh1 = C.a1 * cq * (c2 - 4.0), sb1 = C.a1 * cq * C.b1 * (c2 - 2.0);
+      dh = fma(A1, g1 + g1 * sh1, fma(An, gn + gn * shn, fma(nB, c.x, flh)));
+      db = fma(A1, g1 * (C.b1 + sb1), fma(An, gn * (C.bn + sbn), fma(nB, c.y, flb)));
     }
-    const T fxu = u * idx;
-    for (int m = 0; m < nv; m++) {
-      const T vv = sv[m];
-      const T fyv = vv * idy;
-      const size_t q = (size_t)m * nu + kk;
-      const T2 c = fc0[q];
-      const T2 XW = xw0[q], XE = xw0[nq + q], XS = ys0[q], XN = ys0[(size_t)nx * nq + q];
-      T flh = fxu * (XW.x - XE.x) + fyv * (XS.x - XN.x);
-      T flb = fxu * (XW.y - XE.y) + fyv * (XS.y - XN.y);
-      const T gnh = gun * ev[m], g1h = gu1 * ev[nv + m];
-      T dh, db;
-      if (!P.shk) {
-        dh = inv * (flh + cg1 * (g1h - c.x) + cgn * (gnh - c.x));
-        db = inv * (flb + (cg1b * g1h - cg1 * c.y) + (cgnb * gnh - cgn * c.y));
-      } else {  // Shakhov: g+_h = g_h (1 + S_h), g+_b = g_h (b + S_b), heat flux of f^n
-        const double vd = P.v[m];
-        double cu = ud - C.Un, cv = vd - C.Vn;
-        double cq = cu * C.qx + cv * C.qy, c2 = 2.0 * C.lamn * (cu * cu + cv * cv);
-        const T shn = (T)(C.an * cq * (c2 - 4.0)), sbn = (T)(C.an * cq * C.bn * (c2 - 2.0));
-        cu = ud - C.U1; cv = vd - C.V1;
-        cq = cu * C.qx + cv * C.qy; c2 = 2.0 * C.lam1 * (cu * cu + cv * cv);
-        const T sh1 = (T)(C.a1 * cq * (c2 - 4.0)), sb1 = (T)(C.a1 * cq * C.b1 * (c2 - 2.0));
-        const T gpnh = gnh + gnh * shn, gp1h = g1h + g1h * sh1;
-        const T gpnb = gnh * ((T)C.bn + sbn), gp1b = g1h * ((T)C.b1 + sb1);
-        dh = inv * (flh + cg1 * (gp1h - c.x) + cgn * (gpnh - c.x));
-        db = inv * (flb + cg1 * (gp1b - c.y) + cgn * (gpnb - c.y));
-      }
-      T2 o;
-      o.x = c.x + dh;
-      o.y = c.y + db;
-      if (act) fo0[q] = o;
+    fo0[q] = make_double2(c.x + dh, c.y + db);
+    k += 32;
+    while (k >= nu) {
+      k -= nu;
+      m++;
     }
   }
 }
