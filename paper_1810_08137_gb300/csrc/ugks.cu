@@ -231,7 +231,17 @@ int update_warps(size_t doubles) {
   const int w = (int)(224 * 1024 / (doubles * sizeof(double)));
   return w < kWarpsPerBlock ? w : kWarpsPerBlock;
 }
-static_assert(face_flux_doubles(kMaxAxis, kMaxAxis) * sizeof(double) <= 224 * 1024, "tables of one warp");
+static_assert(face_flux_doubles(kMaxAxis) * sizeof(double) <= 224 * 1024, "tables of one warp");
+
+template <class N>
+cudaError_t set_update_limits(int nu, int nv) {
+  const size_t ff = face_flux_doubles(nv), cu = cell_update_doubles(nu, nv);
+  const cudaError_t e = cudaFuncSetAttribute(k_face_flux<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)(update_warps(ff) * ff * sizeof(double)));
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_cell_update<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)(update_warps(cu) * cu * sizeof(double)));
+}
 
 // dynamic shared memory limits of the FP64 form's sums and update kernels
 cudaError_t set_smem_limits_fp64(int nu, int nv) {
@@ -241,13 +251,7 @@ cudaError_t set_smem_limits_fp64(int nu, int nv) {
   e = cudaFuncSetAttribute(k_sums_cell<NumF64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)(kWarpsPerBlock * kCellSumsWarp));
   if (e != cudaSuccess) return e;
-  const size_t ff = face_flux_doubles(nu, nv), cu = cell_update_doubles(nu, nv);
-  e = cudaFuncSetAttribute(k_face_flux, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)(update_warps(ff) * ff * sizeof(double)));
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_cell_update, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)(update_warps(cu) * cu * sizeof(double)));
-  if (e != cudaSuccess) return e;
+  if ((e = set_update_limits<NumF64>(nu, nv)) != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_update<double, double2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)smem_update<double>(nv));
 }
@@ -318,11 +322,11 @@ cudaError_t launch_step(ugks_ctx* h, cudaStream_t st) {
   // the update in two passes: every face flux once, then Eq. 3 per velocity-cell
   T2* Xx = reinterpret_cast<T2*>(h->xflux);
   T2* Xy = Xx + (size_t)(P.nx + 1) * P.ny * P.nq;
-  const size_t ff = face_flux_doubles(P.nu, P.nv), cu = cell_update_doubles(P.nu, P.nv);
+  const size_t ff = face_flux_doubles(P.nv), cu = cell_update_doubles(P.nu, P.nv);
   const int wf = update_warps(ff), wc = update_warps(cu);
-  k_face_flux<<<(nc + wf - 1) / wf, 32 * wf, wf * ff * sizeof(double), st>>>(
+  k_face_flux<NumF64><<<(nc + wf - 1) / wf, 32 * wf, wf * ff * sizeof(double), st>>>(
       P, fi, h->fxr, h->fyr, reinterpret_cast<const T2*>(h->slopes), Xx, Xy);
-  k_cell_update<<<(nc + wc - 1) / wc, 32 * wc, wc * cu * sizeof(double), st>>>(P, fi, fo, h->cells, Xx, Xy);
+  k_cell_update<NumF64><<<(nc + wc - 1) / wc, 32 * wc, wc * cu * sizeof(double), st>>>(P, fi, fo, h->cells, Xx, Xy);
   if ((r = mark(h, 6)) != cudaSuccess) return r;
   if (h->profiling) h->events_used += UGKS_NKERNELS + 1;
   return cudaGetLastError();
@@ -331,17 +335,11 @@ cudaError_t launch_step(ugks_ctx* h, cudaStream_t st) {
 
 // DF64 form: ghost ring, double-FP32 sums, FP64 interface and cell scalars (double-FP32
 // records), double-FP32 face fluxes and Eq. 3.
-size_t smem_face_flux_df(int nv) { return (size_t)4 * kWarpsPerBlock * nv * sizeof(df); }
-size_t smem_cell_update_df(int nv) { return (size_t)2 * kWarpsPerBlock * nv * sizeof(df); }
-cudaError_t set_smem_limits_df(int nv) {
-  cudaError_t e = cudaFuncSetAttribute(k_sums_cell<NumDF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(kWarpsPerBlock * kCellSumsWarp));
+cudaError_t set_smem_limits_df(int nu, int nv) {
+  const cudaError_t e = cudaFuncSetAttribute(k_sums_cell<NumDF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)(kWarpsPerBlock * kCellSumsWarp));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_face_flux_df, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem_face_flux_df(nv));
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_cell_update_df, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)smem_cell_update_df(nv));
+  return set_update_limits<NumDF>(nu, nv);
 }
 
 cudaError_t launch_step_df(ugks_ctx* h, cudaStream_t st) {
@@ -368,9 +366,10 @@ cudaError_t launch_step_df(ugks_ctx* h, cudaStream_t st) {
   if ((r = mark(h, 5)) != cudaSuccess) return r;
   DF4* Xx = reinterpret_cast<DF4*>(h->xflux);
   DF4* Xy = Xx + (size_t)(P.nx + 1) * P.ny * P.nq;
-  const int ub = (nc + kWarpsPerBlock - 1) / kWarpsPerBlock;
-  k_face_flux_df<<<ub, 32 * kWarpsPerBlock, smem_face_flux_df(P.nv), st>>>(P, fi, h->fxd, h->fyd, sl, Xx, Xy);
-  k_cell_update_df<<<ub, 32 * kWarpsPerBlock, smem_cell_update_df(P.nv), st>>>(P, fi, fo, h->celld, Xx, Xy);
+  const size_t ff = face_flux_doubles(P.nv), cu = cell_update_doubles(P.nu, P.nv);
+  const int wf = update_warps(ff), wc = update_warps(cu);
+  k_face_flux<NumDF><<<(nc + wf - 1) / wf, 32 * wf, wf * ff * sizeof(double), st>>>(P, fi, h->fxd, h->fyd, sl, Xx, Xy);
+  k_cell_update<NumDF><<<(nc + wc - 1) / wc, 32 * wc, wc * cu * sizeof(double), st>>>(P, fi, fo, h->celld, Xx, Xy);
   if ((r = mark(h, 6)) != cudaSuccess) return r;
   if (h->profiling) h->events_used += UGKS_NKERNELS + 1;
   return cudaGetLastError();
@@ -1162,7 +1161,7 @@ ugks_status ugks_create(const ugks_config* cfg, void* cuda_stream, ugks_handle* 
       return r;
     if ((r = cudaMemsetAsync(h->err, 0, sizeof(int), h->stream)) != cudaSuccess) return r;
     if (h->prec == UGKS_FP64 && (r = set_smem_limits_fp64(P.nu, P.nv)) != cudaSuccess) return r;
-    if (h->prec == UGKS_DF64 && (r = set_smem_limits_df(P.nv)) != cudaSuccess) return r;
+    if (h->prec == UGKS_DF64 && (r = set_smem_limits_df(P.nu, P.nv)) != cudaSuccess) return r;
     if ((r = cudaStreamSynchronize(h->stream)) != cudaSuccess) return r;
     return h->prec == UGKS_FP32F ? setup_single_f32(h) : cudaSuccess;
   };

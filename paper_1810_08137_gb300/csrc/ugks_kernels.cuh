@@ -1687,237 +1687,4 @@ __global__ void __launch_bounds__(128) k_update(Params P, const T2* __restrict__
   }
 }
 
-
-// -------------------------------------------------------------------------------------
-// The same update in two passes, FP64 form: every (face, velocity) micro flux once.
-// k_face_flux: one warp per interior cell; for each velocity the cell forms the flux
-// X = Q g + Mt4 f_up - Mt5 d_up (or the wall flux) through its downwind x-face and y-face from
-// its own reconstruction, and a cell next to the boundary also forms the flux whose upwind side
-// is the ghost cell or the wall.  Every face and velocity is written by exactly one warp, into
-// Xx [(nx+1) ny][nq] and Xy [nx (ny+1)][nq] (face-major, velocity innermost).  k_cell_update then
-// reads the four fluxes of each velocity-cell and applies Eq. 3.
-// Both are bound by the FP64 pipe (2 operations per clock and SM).  Lanes run over the flattened
-// velocities (a lane per u would leave 12 of 32 idle at nu = 20), and all that depends on u or v
-// alone comes from per-warp tables in shared memory, so a velocity-cell costs 28 FP64
-// instructions for its two faces: per face 3 for Q_h, 2 for Q_b = X2 Q_h + linear, 1 for g and 4 per
-// component, with f_up and d_up folded into the coefficients of the cell value and its two half
-// slopes (67 before), 36 with the tables; k_cell_update 18 (22 with tables, 30 before).  Both passes,
-// 100x50x28^2 0.820 -> 0.518 ms, 40x20x20^2 163 -> 90 us; FP64 pipe 89 % busy.
-// -------------------------------------------------------------------------------------
-// Tables of k_face_flux (doubles, one after the other): per u index, the downwind x-face
-// (kFluxX arrays), then the downwind y-face for v <= 0 and for v > 0 (kFluxX arrays each), then
-// the factors of g of the upwind faces (x, y for v <= 0, y for v > 0; boundary cells only); per v
-// index kFluxM arrays.
-constexpr int kFluxX = 8;  // q0 q1 q2 q3 (Q_h in v), l0 l1 (Q_b - X2 Q_h), c1 (coefficient of r_x), g
-constexpr int kFluxU = 3 * kFluxX + 3;
-constexpr int kFluxM = 7;  // factors of g: W, E, downwind y, upwind y; coefficient of r_y: W, E, downwind y
-__host__ __device__ constexpr size_t face_flux_doubles(int nu, int nv) {
-  return (size_t)kFluxU * nu + (size_t)kFluxM * nv;
-}
-
-__global__ void __launch_bounds__(128, 4) k_face_flux(Params P, const double2* __restrict__ f,
-                                                      const FaceRec* __restrict__ fxr,
-                                                      const FaceRec* __restrict__ fyr,
-                                                      const double2* __restrict__ sl, double2* __restrict__ Xx,
-                                                      double2* __restrict__ Xy) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  const int nv = P.nv, nu = P.nu, nq = P.nq, nx = P.nx, ny = P.ny, mpos = P.m_pos;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double* tu = reinterpret_cast<double*>(smraw) + warp * face_flux_doubles(nu, nv);
-  double* tm = tu + kFluxU * nu;
-  const int cell = blockIdx.x * (blockDim.x >> 5) + warp;
-  if (cell >= nx * ny) return;
-  const int i = cell % nx, j = cell / nx;
-  const FaceRec& RW = fxr[(size_t)j * (nx + 1) + i];
-  const FaceRec& RE = fxr[(size_t)j * (nx + 1) + i + 1];
-  const FaceRec& RS = fyr[(size_t)j * nx + i];
-  const FaceRec& RN = fyr[(size_t)(j + 1) * nx + i];
-  const bool edge = i == 0 || i == nx - 1 || j == 0 || j == ny - 1;
-  auto gauss = [](double lam, double d) { return exp(-lam * d * d); };
-
-  // u tables: Q at fixed u as a polynomial in v; a wall face passes dt f_up (Mt4 = dt, no Q)
-  for (int k = lane; k < nu; k += 32) {
-    const double u = P.u[k], cu = u * P.d_tdx;
-    const bool up = u > 0.0;
-    auto face = [&](const FaceRec& R, int side, bool xface, double c1, double* t) {
-      const double* h = R.Q[side][0];
-      const double* b = R.Q[side][1];
-      double q[4] = {0.0, 0.0, 0.0, 0.0}, l0 = 0.0, l1 = 0.0, g = 0.0;
-      if (!R.wall) {
-        const double d0 = b[0] - R.bfac * h[0], dn = b[1] - R.bfac * h[1], dt = b[2] - R.bfac * h[2];
-        if (xface) poly_in_v_xface(h, u, q);
-        else poly_in_v_yface(h, u, q);
-        l0 = d0 + u * (xface ? dn : dt);
-        l1 = xface ? dt : dn;
-        g = R.G * gauss(R.lam, u - (xface ? R.Un : R.Ut));
-      }
-#pragma unroll
-      for (int e = 0; e < 4; e++) t[e * nu + k] = q[e];
-      t[4 * nu + k] = l0;
-      t[5 * nu + k] = l1;
-      t[6 * nu + k] = c1;
-      t[7 * nu + k] = g;
-    };
-    const FaceRec& RX = up ? RE : RW;
-    face(RX, up ? 0 : 1, true, (up ? RX.Mt4 : -RX.Mt4) - RX.Mt5 * cu, tu);
-    face(RS, 1, false, -RS.Mt5 * cu, tu + kFluxX * nu);
-    face(RN, 0, false, -RN.Mt5 * cu, tu + 2 * kFluxX * nu);
-    if (edge) {
-      const FaceRec& RG = up ? RW : RE;
-      double* tg = tu + 3 * kFluxX * nu + k;
-      tg[0] = RG.G * gauss(RG.lam, u - RG.Un);
-      tg[nu] = RN.G * gauss(RN.lam, u - RN.Ut);
-      tg[2 * nu] = RS.G * gauss(RS.lam, u - RS.Ut);
-    }
-  }
-  for (int m = lane; m < nv; m += 32) {
-    const double v = P.v[m], cv = v * P.d_tdy;
-    const bool vp = m >= mpos;
-    const FaceRec& RD = vp ? RN : RS;
-    const FaceRec& RG = vp ? RS : RN;
-    tm[m] = gauss(RW.lam, v - RW.Ut);
-    tm[nv + m] = gauss(RE.lam, v - RE.Ut);
-    tm[2 * nv + m] = gauss(RD.lam, v - RD.Un);
-    tm[3 * nv + m] = edge ? gauss(RG.lam, v - RG.Un) : 0.0;
-    tm[4 * nv + m] = -RW.Mt5 * cv;
-    tm[5 * nv + m] = -RE.Mt5 * cv;
-    tm[6 * nv + m] = (vp ? RD.Mt4 : -RD.Mt4) - RD.Mt5 * cv;
-  }
-  __syncwarp();
-  const double MW = RW.Mt4, ME = RE.Mt4, MS = RS.Mt4, MN = RN.Mt4;
-  const double XW = RW.bfac, XE = RE.bfac, XS = RS.bfac, XN = RN.bfac;
-  const double2* fc0 = f + fcell(P, i, j) * nq;
-  const double2* sl0 = sl + (size_t)wcell(P, i, j) * nq * 2;  // this cell's slopes
-  double2* xw0 = Xx + ((size_t)j * (nx + 1) + i) * nq;        // W face of the cell; E face: + nq
-  double2* ys0 = Xy + ((size_t)j * nx + i) * nq;              // S face; N face: + nx nq
-  const size_t ynf = (size_t)nx * nq;
-  const int kpos = P.k_pos;
-
-  int m = lane / nu, k = lane - m * nu;
-  for (int q = lane; q < nq; q += 32) {
-    const bool up = k >= kpos, vp = m >= mpos;  // u > 0, v > 0
-    const double v = P.v[m];
-    const double2 c = fc0[q], a = sl0[2 * q], b = sl0[2 * q + 1];  // half slopes r_x, r_y (h, b)
-    // X of a face from its u table, coefficient c2 of r_y, Mt4, X2 = <xi^2> and v factor of g
-    auto flux = [&](const double* t, double c2, double m4, double x2, double ev) {
-      const double qh = fma(fma(fma(t[3 * nu], v, t[2 * nu]), v, t[nu]), v, t[0]);
-      const double qb = fma(x2, qh, fma(t[5 * nu], v, t[4 * nu]));
-      const double c1 = t[6 * nu], g = t[7 * nu] * ev;
-      return make_double2(fma(qh, g, fma(c2, b.x, fma(c1, a.x, m4 * c.x))),
-                          fma(qb, g, fma(c2, b.y, fma(c1, a.y, m4 * c.y))));
-    };
-    (up ? xw0 + nq : xw0)[q] = flux(tu + k, tm[(up ? 5 : 4) * nv + m], up ? ME : MW, up ? XE : XW,
-                                    tm[(up ? nv : 0) + m]);
-    (vp ? ys0 + ynf : ys0)[q] = flux(tu + (vp ? 2 : 1) * kFluxX * nu + k, tm[6 * nv + m], vp ? MN : MS,
-                                     vp ? XN : XS, tm[2 * nv + m]);
-    if (edge) {
-      // faces whose upwind side is a ghost cell or a wall
-      const double u = P.u[k], cu = u * P.d_tdx, cv = v * P.d_tdy;
-      auto ghost = [&](const FaceRec& R, int side, bool xface, bool zero, double g, double2 fu, double2 au,
-                       double2 bu, double sg) {
-        if (R.wall) return make_double2(P.dt * g, P.dt * (R.bfac * g));
-        if (zero) au.x = au.y = bu.x = bu.y = 0.0;
-        double qh[4], qb[4];
-        if (xface) {
-          poly_in_v_xface(R.Q[side][0], u, qh);
-          poly_in_v_xface(R.Q[side][1], u, qb);
-        } else {
-          poly_in_v_yface(R.Q[side][0], u, qh);
-          poly_in_v_yface(R.Q[side][1], u, qb);
-        }
-        const double dh = cu * au.x + cv * bu.x, db = cu * au.y + cv * bu.y;
-        const double fh = fu.x + sg * (xface ? au.x : bu.x), fb = fu.y + sg * (xface ? au.y : bu.y);
-        return make_double2(horner3(qh, v) * g + R.Mt4 * fh - R.Mt5 * dh, horner3(qb, v) * g + R.Mt4 * fb - R.Mt5 * db);
-      };
-      if (up ? i == 0 : i == nx - 1) {
-        const FaceRec& R = up ? RW : RE;
-        const long xo = up ? -(long)nq : (long)nq;
-        (up ? xw0 : xw0 + nq)[q] = ghost(R, up ? 0 : 1, true, P.bc_kind[up ? 0 : 1] == 2,
-                                         tu[3 * kFluxX * nu + k] * tm[(up ? 0 : nv) + m], fc0[q + xo],
-                                         sl0[2 * (q + xo)], sl0[2 * (q + xo) + 1], up ? 1.0 : -1.0);
-      }
-      if (vp ? j == 0 : j == ny - 1) {
-        const FaceRec& R = vp ? RS : RN;
-        const long yo = (vp ? -1L : 1L) * P.ex * nq, yso = (vp ? -1L : 1L) * P.wx * nq;
-        (vp ? ys0 : ys0 + ynf)[q] = ghost(R, vp ? 0 : 1, false, P.bc_kind[vp ? 2 : 3] == 2,
-                                          tu[(3 * kFluxX + (vp ? 2 : 1)) * nu + k] * tm[3 * nv + m], fc0[q + yo],
-                                          sl0[2 * (q + yso)], sl0[2 * (q + yso) + 1], vp ? 1.0 : -1.0);
-      }
-    }
-    k += 32;
-    while (k >= nu) {
-      k -= nu;
-      m++;
-    }
-  }
-}
-
-// Eq. 3 from the four face fluxes of each velocity-cell (k_face_flux), FP64 form: the increment
-// f^{n+1} - f^n = inv (flux + cg1 (g^{n+1} - f^n) + cgn (g^n - f^n)) with inv folded into the
-// coefficients; 18 FP64 instructions per velocity-cell.  Tables per warp: per u index
-// inv u/dx, g^n and g^{n+1} factors; per v index the same with v/dy.
-__host__ __device__ constexpr size_t cell_update_doubles(int nu, int nv) { return 3 * ((size_t)nu + nv); }
-
-__global__ void __launch_bounds__(128) k_cell_update(Params P, const double2* __restrict__ f,
-                                                     double2* __restrict__ fo, const CellRec* __restrict__ cr,
-                                                     const double2* __restrict__ Xx,
-                                                     const double2* __restrict__ Xy) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  const int nv = P.nv, nu = P.nu, nq = P.nq, nx = P.nx, ny = P.ny;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double* tu = reinterpret_cast<double*>(smraw) + warp * cell_update_doubles(nu, nv);
-  double* tm = tu + 3 * nu;
-  const int cell = blockIdx.x * (blockDim.x >> 5) + warp;
-  if (cell >= nx * ny) return;
-  const int i = cell % nx, j = cell / nx;
-  const CellRec& C = cr[cell];
-  const double inv = C.inv;
-  for (int k = lane; k < nu; k += 32) {
-    const double u = P.u[k], dn = u - C.Un, d1 = u - C.U1;
-    tu[k] = inv * P.d_idx * u;
-    tu[nu + k] = C.Gn * exp(-C.lamn * dn * dn);
-    tu[2 * nu + k] = C.G1 * exp(-C.lam1 * d1 * d1);
-  }
-  for (int m = lane; m < nv; m += 32) {
-    const double v = P.v[m], dn = v - C.Vn, d1 = v - C.V1;
-    tm[m] = inv * P.d_idy * v;
-    tm[nv + m] = exp(-C.lamn * dn * dn);
-    tm[2 * nv + m] = exp(-C.lam1 * d1 * d1);
-  }
-  __syncwarp();
-  const double A1 = inv * C.cg1, An = inv * C.cgn, nB = -(A1 + An), A1b = A1 * C.b1, Anb = An * C.bn;
-  const double2* fc0 = f + fcell(P, i, j) * nq;
-  double2* fo0 = fo + fcell(P, i, j) * nq;
-  const double2* xw0 = Xx + ((size_t)j * (nx + 1) + i) * nq;
-  const double2* ys0 = Xy + ((size_t)j * nx + i) * nq;
-  const size_t ynf = (size_t)nx * nq;
-  int m = lane / nu, k = lane - m * nu;
-  for (int q = lane; q < nq; q += 32) {
-    const double2 c = fc0[q], XW = xw0[q], XE = xw0[nq + q], XS = ys0[q], XN = ys0[ynf + q];
-    const double au = tu[k], av = tm[m];
-    const double gn = tu[nu + k] * tm[nv + m], g1 = tu[2 * nu + k] * tm[2 * nv + m];
-    const double flh = fma(au, XW.x - XE.x, av * (XS.x - XN.x)), flb = fma(au, XW.y - XE.y, av * (XS.y - XN.y));
-    double dh, db;
-    if (!P.shk) {
-      dh = fma(A1, g1, fma(An, gn, fma(nB, c.x, flh)));
-      db = fma(A1b, g1, fma(Anb, gn, fma(nB, c.y, flb)));
-    } else {  // Shakhov: g+_h = g_h (1 + S_h), g+_b = g_h (b + S_b), heat flux of f^n
-      const double u = P.u[k], v = P.v[m];
-      double cu = u - C.Un, cv = v - C.Vn, cq = cu * C.qx + cv * C.qy, c2 = 2.0 * C.lamn * (cu * cu + cv * cv);
-      const double shn = C.an * cq * (c2 - 4.0), sbn = C.an * cq * C.bn * (c2 - 2.0);
-      cu = u - C.U1; cv = v - C.V1;
-      cq = cu * C.qx + cv * C.qy; c2 = 2.0 * C.lam1 * (cu * cu + cv * cv);
-      const double sh1 = C.a1 * cq * (c2 - 4.0), sb1 = C.a1 * cq * C.b1 * (c2 - 2.0);
-      dh = fma(A1, g1 + g1 * sh1, fma(An, gn + gn * shn, fma(nB, c.x, flh)));
-      db = fma(A1, g1 * (C.b1 + sb1), fma(An, gn * (C.bn + sbn), fma(nB, c.y, flb)));
-    }
-    fo0[q] = make_double2(c.x + dh, c.y + db);
-    k += 32;
-    while (k >= nu) {
-      k -= nu;
-      m++;
-    }
-  }
-}
-
 }  // namespace ugks

@@ -1,6 +1,7 @@
-// S1 + S7 of the FP64 and DF64 forms with one thread per cell: the FP32-f form's sums_tile_body
-// (ugks_f32.cuh) in FP64 or double-FP32 arithmetic, plus the slope buffer these forms' face-flux
-// kernels read.  A block owns a tile of 8 x 4 cells (lane = cell) and one quadrant of velocity
+// Velocity sums and update of the FP64 and DF64 forms, one source for both arithmetics.
+//
+// S1 + S7 with one thread per cell: the FP32-f form's sums_tile_body (ugks_f32.cuh) in FP64 or
+// double-FP32 arithmetic, plus the slope buffer the face-flux kernel reads.  A block owns a tile of 8 x 4 cells (lane = cell) and one quadrant of velocity
 // space, so it feeds one x side and one y side; its four warps take a share of the quadrant's
 // rows each, and the interface kernel adds the two quadrants of a side.
 #pragma once
@@ -25,8 +26,18 @@ struct NumF64 {
   static __device__ __forceinline__ V neg(V a) { return -a; }
   static __device__ __forceinline__ V vl(V a, V c, V b) { return vl_half(a, c, b); }
   static __device__ __forceinline__ double f64(V a) { return a; }
+  using Face = FaceRec;
+  using Cell = CellRec;
+  static constexpr bool kShakhov = true;
+  static __device__ __forceinline__ V val(double a) { return a; }  // a record's field
+  static __device__ __forceinline__ V exp(V a) { return ::exp(a); }
+  static __device__ __forceinline__ V u(const Params& P, int k) { return P.u[k]; }
+  static __device__ __forceinline__ V v(const Params& P, int m) { return P.v[m]; }
   static __device__ __forceinline__ V tdx(const Params& P) { return P.d_tdx; }
   static __device__ __forceinline__ V tdy(const Params& P) { return P.d_tdy; }
+  static __device__ __forceinline__ V idx(const Params& P) { return P.d_idx; }
+  static __device__ __forceinline__ V idy(const Params& P) { return P.d_idy; }
+  static __device__ __forceinline__ V dt(const Params& P) { return P.dt; }
   // [nu][6]: w_u u^m (m = 0..4; half at u = 0) and u; [nv][2]: v and w_v (half at v = 0)
   static __device__ __forceinline__ const V* utab(const Params& P) { return P.mvd + 5 * P.nv; }
 };
@@ -47,8 +58,18 @@ struct NumDF {
   static __device__ __forceinline__ V neg(V a) { return df_neg(a); }
   static __device__ __forceinline__ V vl(V a, V c, V b) { return vl_df(a, c, b); }
   static __device__ __forceinline__ double f64(V a) { return to_double(a); }
+  using Face = FaceRecD;
+  using Cell = CellRecD;
+  static constexpr bool kShakhov = false;
+  static __device__ __forceinline__ V val(float2 a) { return dfv(a); }
+  static __device__ __forceinline__ V exp(V a) { return df_exp(a); }
+  static __device__ __forceinline__ V u(const Params& P, int k) { return dfv(__ldg(P.gdf + k)); }
+  static __device__ __forceinline__ V v(const Params& P, int m) { return dfv(__ldg(P.gdf + 2 * P.nu + m)); }
   static __device__ __forceinline__ V tdx(const Params& P) { return dfv(P.df_tdx); }
   static __device__ __forceinline__ V tdy(const Params& P) { return dfv(P.df_tdy); }
+  static __device__ __forceinline__ V idx(const Params& P) { return dfv(P.df_idx); }
+  static __device__ __forceinline__ V idy(const Params& P) { return dfv(P.df_idy); }
+  static __device__ __forceinline__ V dt(const Params& P) { return dfv(P.df_dt); }
   static __device__ __forceinline__ const V* utab(const Params& P) {
     return reinterpret_cast<const V*>(P.gdf + 2 * P.nu + 6 * P.nv);
   }
@@ -224,6 +245,287 @@ __global__ void __launch_bounds__(128, 3) k_sums_cell(Params P, const typename N
         r += N::f64(reinterpret_cast<const V*>(all + w * kCellSumsWarp)[t]);
       part[(size_t)wcell(P, x0 + (t & 7), y0 + (t >> 3)) * kCellPart + quad * 32 + lane] = r;
     }
+}
+
+// -------------------------------------------------------------------------------------
+// S6 + S8 and Eq. 3 of the FP64 and DF64 forms in two passes: every (face, velocity) micro flux
+// once.
+// k_face_flux: one warp per interior cell; for each velocity the cell forms the flux
+// X = Q g + Mt4 f_up - Mt5 d_up (or the wall flux) through its downwind x-face and y-face from
+// its own reconstruction, and a cell next to the boundary also forms the flux whose upwind side
+// is the ghost cell or the wall.  Every face and velocity is written by exactly one warp, into
+// Xx [(nx+1) ny][nq] and Xy [nx (ny+1)][nq] (face-major, velocity innermost).  k_cell_update then
+// reads the four fluxes of each velocity-cell and applies Eq. 3.
+// Both are bound by arithmetic: the FP64 form by the FP64 pipe (2 operations per clock and SM),
+// the DF64 form by the FP32 pipe.  Lanes run over the flattened
+// velocities (a lane per u would leave 12 of 32 idle at nu = 20), and all that depends on u or v
+// alone comes from per-warp tables in shared memory, so a velocity-cell costs 28 FP64
+// instructions for its two faces: per face 3 for Q_h, 2 for Q_b = X2 Q_h + linear, 1 for g and 4 per
+// component, with f_up and d_up folded into the coefficients of the cell value and its two half
+// slopes (67 before), 36 with the tables; k_cell_update 18 (22 with tables, 30 before).  Both passes,
+// 100x50x28^2 0.820 -> 0.518 ms, 40x20x20^2 163 -> 90 us; FP64 pipe 89 % busy.
+// -------------------------------------------------------------------------------------
+// Q at fixed u as a polynomial in v, from a record's eight coefficients: x face (un = u, ut = v) or
+// y face (un = v, ut = u).
+template <class N, typename C>
+__device__ __forceinline__ void poly_in_v(const C* c, typename N::V u, bool xface, typename N::V* q) {
+  auto k = [&](int i) { return N::val(c[i]); };
+  const int n1 = xface ? 1 : 2, n2 = xface ? 3 : 5, n3 = xface ? 6 : 7;  // powers of u
+  const int t1 = xface ? 2 : 1, t2 = xface ? 5 : 3, t3 = xface ? 7 : 6;  // powers of v
+  q[0] = N::mad(u, N::mad(u, N::mad(u, k(n3), k(n2)), k(n1)), k(0));
+  q[1] = N::mad(u, N::mad(u, k(t3), k(4)), k(t1));
+  q[2] = N::mad(u, k(n3), k(t2));
+  q[3] = k(t3);
+}
+
+// Tables of k_face_flux (doubles, one after the other): per u index, the downwind x-face
+// (kFluxX arrays), then the downwind y-face for v <= 0 and for v > 0 (kFluxX arrays each), then
+// the factors of g of the upwind faces (x, y for v <= 0, y for v > 0; boundary cells only); per v
+// index kFluxM values.
+// The u tables hold up to kFluxUB values of u at a time (a larger grid is walked in blocks of u), so
+// that their arrays lie at fixed distances and a wide velocity grid does not cost residency.
+constexpr int kFluxUB = 40;
+constexpr int kFluxX = 8;  // q0 q1 q2 q3 (Q_h in v), l0 l1 (Q_b - X2 Q_h), c1 (coefficient of r_x), g
+constexpr int kFluxU = 3 * kFluxX + 3;
+constexpr int kFluxM = 8;  // v; factors of g: W, E, downwind y, upwind y; coefficient of r_y: W, E, downwind y
+__host__ __device__ constexpr size_t face_flux_doubles(int nv) { return kFluxU * kFluxUB + (size_t)kFluxM * nv; }
+
+template <class N>
+__global__ void __launch_bounds__(128, 4) k_face_flux(Params P, const typename N::H* __restrict__ f,
+                                                      const typename N::Face* __restrict__ fxr,
+                                                      const typename N::Face* __restrict__ fyr,
+                                                      const typename N::H* __restrict__ sl,
+                                                      typename N::H* __restrict__ Xx,
+                                                      typename N::H* __restrict__ Xy) {
+  using V = typename N::V;
+  using H = typename N::H;
+  using Face = typename N::Face;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int nv = P.nv, nu = P.nu, nq = P.nq, nx = P.nx, ny = P.ny, mpos = P.m_pos;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  V* tu = reinterpret_cast<V*>(smraw) + warp * face_flux_doubles(nv);
+  V* tm = tu + kFluxU * kFluxUB;
+  const int cell = blockIdx.x * (blockDim.x >> 5) + warp;
+  if (cell >= nx * ny) return;
+  const int i = cell % nx, j = cell / nx;
+  const Face& RW = fxr[(size_t)j * (nx + 1) + i];
+  const Face& RE = fxr[(size_t)j * (nx + 1) + i + 1];
+  const Face& RS = fyr[(size_t)j * nx + i];
+  const Face& RN = fyr[(size_t)(j + 1) * nx + i];
+  const bool edge = i == 0 || i == nx - 1 || j == 0 || j == ny - 1;
+  auto val = [](const auto& x) { return N::val(x); };
+  auto gauss = [](V lam, V d) { return N::exp(N::neg(N::mul(lam, N::mul(d, d)))); };
+  const V tdx = N::tdx(P), tdy = N::tdy(P), dtv = N::dt(P);
+
+  for (int m = lane; m < nv; m += 32) {
+    const V v = N::v(P, m), cv = N::mul(v, tdy);
+    const bool vp = m >= mpos;
+    const Face& RD = vp ? RN : RS;
+    const Face& RG = vp ? RS : RN;
+    auto vg = [&](const Face& R, V U) { return gauss(val(R.lam), N::sub(v, U)); };
+    V* t = tm + kFluxM * m;
+    t[0] = v;
+    t[1] = vg(RW, val(RW.Ut));
+    t[2] = vg(RE, val(RE.Ut));
+    t[3] = vg(RD, val(RD.Un));
+    t[4] = edge ? vg(RG, val(RG.Un)) : N::zero();
+    t[5] = N::neg(N::mul(val(RW.Mt5), cv));
+    t[6] = N::neg(N::mul(val(RE.Mt5), cv));
+    t[7] = N::sub(vp ? val(RD.Mt4) : N::neg(val(RD.Mt4)), N::mul(val(RD.Mt5), cv));
+  }
+  const V MW = val(RW.Mt4), ME = val(RE.Mt4), MS = val(RS.Mt4), MN = val(RN.Mt4);
+  const V XW = val(RW.bfac), XE = val(RE.bfac), XS = val(RS.bfac), XN = val(RN.bfac);
+  const H* fc0 = f + fcell(P, i, j) * nq;
+  const H* sl0 = sl + (size_t)wcell(P, i, j) * nq * 2;  // this cell's slopes
+  H* xw0 = Xx + ((size_t)j * (nx + 1) + i) * nq;        // W face of the cell; E face: + nq
+  H* ys0 = Xy + ((size_t)j * nx + i) * nq;              // S face; N face: + nx nq
+  const size_t ynf = (size_t)nx * nq;
+  const int kpos = P.k_pos;
+
+  const int blocks = (nu + kFluxUB - 1) / kFluxUB;
+  for (int ub = 0; ub < blocks; ub++) {
+    const int kb = nu * ub / blocks, kw = nu * (ub + 1) / blocks - kb;  // this block's values of u
+    __syncwarp();  // the tables of the previous block are no longer read
+    // u tables: Q at fixed u as a polynomial in v; a wall face passes dt f_up (Mt4 = dt, no Q)
+    for (int kk = lane; kk < kw; kk += 32) {
+      const int k = kb + kk;
+      const V u = N::u(P, k), cu = N::mul(u, tdx);
+      const bool up = k >= P.k_pos;
+      // coefficient of a slope: +-Mt4 (the face value) - Mt5 c
+      auto coef = [&](const Face& R, int sg, V c) {
+        const V m5 = N::mul(val(R.Mt5), c);
+        return sg == 0 ? N::neg(m5) : N::sub(sg > 0 ? val(R.Mt4) : N::neg(val(R.Mt4)), m5);
+      };
+      auto face = [&](const Face& R, int side, bool xface, V c1, V* t) {
+        const auto* h = R.Q[side][0];
+        const auto* b = R.Q[side][1];
+        V q[4] = {N::zero(), N::zero(), N::zero(), N::zero()}, l0 = N::zero(), l1 = N::zero(), g = N::zero();
+        if (!R.wall) {
+          const V bf = val(R.bfac);
+          auto diff = [&](int c) { return N::sub(val(b[c]), N::mul(bf, val(h[c]))); };
+          const V dn = diff(1), dt = diff(2);
+          poly_in_v<N>(h, u, xface, q);
+          l0 = N::mad(u, xface ? dn : dt, diff(0));
+          l1 = xface ? dt : dn;
+          g = N::mul(val(R.G), gauss(val(R.lam), N::sub(u, val(xface ? R.Un : R.Ut))));
+        }
+#pragma unroll
+        for (int e = 0; e < 4; e++) t[e * kFluxUB + kk] = q[e];
+        t[4 * kFluxUB + kk] = l0;
+        t[5 * kFluxUB + kk] = l1;
+        t[6 * kFluxUB + kk] = c1;
+        t[7 * kFluxUB + kk] = g;
+      };
+      const Face& RX = up ? RE : RW;
+      face(RX, up ? 0 : 1, true, coef(RX, up ? 1 : -1, cu), tu);
+      face(RS, 1, false, coef(RS, 0, cu), tu + kFluxX * kFluxUB);
+      face(RN, 0, false, coef(RN, 0, cu), tu + 2 * kFluxX * kFluxUB);
+      if (edge) {
+        const Face& RG = up ? RW : RE;
+        V* tg = tu + 3 * kFluxX * kFluxUB + kk;
+        auto ug = [&](const Face& R, V U) { return N::mul(val(R.G), gauss(val(R.lam), N::sub(u, U))); };
+        tg[0] = ug(RG, val(RG.Un));
+        tg[kFluxUB] = ug(RN, val(RN.Ut));
+        tg[2 * kFluxUB] = ug(RS, val(RS.Ut));
+      }
+    }
+    __syncwarp();
+    int m = lane / kw, kk = lane - m * kw;
+    while (m < nv) {
+      const int k = kb + kk, q = m * nu + k;
+      const bool up = k >= kpos, vp = m >= mpos;  // u > 0, v > 0
+      const V* mt = tm + kFluxM * m;
+      const V v = mt[0];
+      const H c = fc0[q], a = sl0[2 * q], b = sl0[2 * q + 1];  // half slopes r_x, r_y (h, b)
+      // X of a face from its u table, coefficient c2 of r_y, Mt4, X2 = <xi^2> and v factor of g
+      auto flux = [&](const V* t, V c2, V m4, V x2, V ev) {
+        const V qh = N::mad(N::mad(N::mad(t[3 * kFluxUB], v, t[2 * kFluxUB]), v, t[kFluxUB]), v, t[0]);
+        const V qb = N::mad(x2, qh, N::mad(t[5 * kFluxUB], v, t[4 * kFluxUB]));
+        const V c1 = t[6 * kFluxUB], g = N::mul(t[7 * kFluxUB], ev);
+        return N::pack(N::mad(qh, g, N::mad(c2, N::h(b), N::mad(c1, N::h(a), N::mul(m4, N::h(c))))),
+                       N::mad(qb, g, N::mad(c2, N::b(b), N::mad(c1, N::b(a), N::mul(m4, N::b(c))))));
+      };
+      (up ? xw0 + nq : xw0)[q] = flux(tu + kk, mt[up ? 6 : 5], up ? ME : MW, up ? XE : XW, mt[up ? 2 : 1]);
+      (vp ? ys0 + ynf : ys0)[q] = flux(tu + (vp ? 2 : 1) * kFluxX * kFluxUB + kk, mt[7], vp ? MN : MS,
+                                       vp ? XN : XS, mt[3]);
+      if (edge) {
+        // faces whose upwind side is a ghost cell or a wall
+        const V u = N::u(P, k), cu = N::mul(u, tdx), cv = N::mul(v, tdy);
+        auto ghost = [&](const Face& R, int side, bool xface, bool zero, V g, H fu, H au, H bu, bool plus) {
+          if (R.wall) return N::pack(N::mul(dtv, g), N::mul(dtv, N::mul(val(R.bfac), g)));
+          if (zero) au = bu = N::pack(N::zero(), N::zero());
+          const V m4 = val(R.Mt4), m5 = val(R.Mt5);
+          auto comp = [&](const auto* Q, V f0, V ax, V by) {
+            V p[4];
+            poly_in_v<N>(Q, u, xface, p);
+            const V r = xface ? ax : by, fv = plus ? N::add(f0, r) : N::sub(f0, r);
+            const V d = N::mad(cu, ax, N::mul(cv, by));
+            const V qq = N::mad(N::mad(N::mad(p[3], v, p[2]), v, p[1]), v, p[0]);
+            return N::sub(N::mad(qq, g, N::mul(m4, fv)), N::mul(m5, d));
+          };
+          return N::pack(comp(R.Q[side][0], N::h(fu), N::h(au), N::h(bu)),
+                         comp(R.Q[side][1], N::b(fu), N::b(au), N::b(bu)));
+        };
+        if (up ? i == 0 : i == nx - 1) {
+          const Face& R = up ? RW : RE;
+          const long xo = up ? -(long)nq : (long)nq;
+          (up ? xw0 : xw0 + nq)[q] = ghost(R, up ? 0 : 1, true, P.bc_kind[up ? 0 : 1] == 2,
+                                           N::mul(tu[3 * kFluxX * kFluxUB + kk], mt[up ? 1 : 2]), fc0[q + xo],
+                                           sl0[2 * (q + xo)], sl0[2 * (q + xo) + 1], up);
+        }
+        if (vp ? j == 0 : j == ny - 1) {
+          const Face& R = vp ? RS : RN;
+          const long yo = (vp ? -1L : 1L) * P.ex * nq, yso = (vp ? -1L : 1L) * P.wx * nq;
+          (vp ? ys0 : ys0 + ynf)[q] = ghost(R, vp ? 0 : 1, false, P.bc_kind[vp ? 2 : 3] == 2,
+                                            N::mul(tu[(3 * kFluxX + (vp ? 2 : 1)) * kFluxUB + kk], mt[4]), fc0[q + yo],
+                                            sl0[2 * (q + yso)], sl0[2 * (q + yso) + 1], vp);
+        }
+      }
+      kk += 32;
+      while (kk >= kw) {
+        kk -= kw;
+        m++;
+      }
+    }
+  }
+}
+
+// Eq. 3 from the four face fluxes of each velocity-cell (k_face_flux): the increment
+// f^{n+1} - f^n = inv (flux + cg1 (g^{n+1} - f^n) + cgn (g^n - f^n)) with inv folded into the
+// coefficients; 18 FP64 instructions per velocity-cell.  Tables per warp: per u index
+// inv u/dx, g^n and g^{n+1} factors; per v index the same with v/dy.
+__host__ __device__ constexpr size_t cell_update_doubles(int nu, int nv) { return 3 * ((size_t)nu + nv); }
+
+template <class N>
+__global__ void __launch_bounds__(128) k_cell_update(Params P, const typename N::H* __restrict__ f,
+                                                     typename N::H* __restrict__ fo,
+                                                     const typename N::Cell* __restrict__ cr,
+                                                     const typename N::H* __restrict__ Xx,
+                                                     const typename N::H* __restrict__ Xy) {
+  using V = typename N::V;
+  using H = typename N::H;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int nv = P.nv, nu = P.nu, nq = P.nq, nx = P.nx, ny = P.ny;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  V* tu = reinterpret_cast<V*>(smraw) + warp * cell_update_doubles(nu, nv);
+  V* tm = tu + 3 * nu;
+  const int cell = blockIdx.x * (blockDim.x >> 5) + warp;
+  if (cell >= nx * ny) return;
+  const int i = cell % nx, j = cell / nx;
+  const typename N::Cell& C = cr[cell];
+  auto val = [](const auto& x) { return N::val(x); };
+  auto gauss = [](V lam, V d) { return N::exp(N::neg(N::mul(lam, N::mul(d, d)))); };
+  const V inv = val(C.inv), ix = N::mul(inv, N::idx(P)), iy = N::mul(inv, N::idy(P));
+  for (int k = lane; k < nu; k += 32) {
+    const V u = N::u(P, k);
+    tu[k] = N::mul(ix, u);
+    tu[nu + k] = N::mul(val(C.Gn), gauss(val(C.lamn), N::sub(u, val(C.Un))));
+    tu[2 * nu + k] = N::mul(val(C.G1), gauss(val(C.lam1), N::sub(u, val(C.U1))));
+  }
+  for (int m = lane; m < nv; m += 32) {
+    const V v = N::v(P, m);
+    tm[m] = N::mul(iy, v);
+    tm[nv + m] = gauss(val(C.lamn), N::sub(v, val(C.Vn)));
+    tm[2 * nv + m] = gauss(val(C.lam1), N::sub(v, val(C.V1)));
+  }
+  __syncwarp();
+  const V A1 = N::mul(inv, val(C.cg1)), An = N::mul(inv, val(C.cgn)), nB = N::neg(N::add(A1, An));
+  const V A1b = N::mul(A1, val(C.b1)), Anb = N::mul(An, val(C.bn));
+  const H* fc0 = f + fcell(P, i, j) * nq;
+  H* fo0 = fo + fcell(P, i, j) * nq;
+  const H* xw0 = Xx + ((size_t)j * (nx + 1) + i) * nq;
+  const H* ys0 = Xy + ((size_t)j * nx + i) * nq;
+  const size_t ynf = (size_t)nx * nq;
+  int m = lane / nu, k = lane - m * nu;
+  for (int q = lane; q < nq; q += 32) {
+    const H c = fc0[q], XW = xw0[q], XE = xw0[nq + q], XS = ys0[q], XN = ys0[ynf + q];
+    const V au = tu[k], av = tm[m];
+    const V gn = N::mul(tu[nu + k], tm[nv + m]), g1 = N::mul(tu[2 * nu + k], tm[2 * nv + m]);
+    const V flh = N::mad(au, N::sub(N::h(XW), N::h(XE)), N::mul(av, N::sub(N::h(XS), N::h(XN))));
+    const V flb = N::mad(au, N::sub(N::b(XW), N::b(XE)), N::mul(av, N::sub(N::b(XS), N::b(XN))));
+    V dh_ = N::mad(nB, N::h(c), flh), db_ = N::mad(nB, N::b(c), flb);
+    bool shk = false;
+    if constexpr (N::kShakhov) shk = P.shk;
+    if (!shk) {
+      dh_ = N::mad(A1, g1, N::mad(An, gn, dh_));
+      db_ = N::mad(A1b, g1, N::mad(Anb, gn, db_));
+    } else if constexpr (N::kShakhov) {  // g+_h = g_h (1 + S_h), g+_b = g_h (b + S_b), heat flux of f^n
+      const double u = P.u[k], v = P.v[m];
+      double cu = u - C.Un, cv = v - C.Vn, cq = cu * C.qx + cv * C.qy, c2 = 2.0 * C.lamn * (cu * cu + cv * cv);
+      const double shn = C.an * cq * (c2 - 4.0), sbn = C.an * cq * C.bn * (c2 - 2.0);
+      cu = u - C.U1; cv = v - C.V1;
+      cq = cu * C.qx + cv * C.qy; c2 = 2.0 * C.lam1 * (cu * cu + cv * cv);
+      const double sh1 = C.a1 * cq * (c2 - 4.0), sb1 = C.a1 * cq * C.b1 * (c2 - 2.0);
+      dh_ = fma(A1, g1 + g1 * sh1, fma(An, gn + gn * shn, dh_));
+      db_ = fma(A1, g1 * (C.b1 + sb1), fma(An, gn * (C.bn + sbn), db_));
+    }
+    fo0[q] = N::pack(N::add(N::h(c), dh_), N::add(N::b(c), db_));
+    k += 32;
+    while (k >= nu) {
+      k -= nu;
+      m++;
+    }
+  }
 }
 
 }  // namespace ugks
