@@ -225,33 +225,18 @@ template <typename T>
 size_t smem_update(int nv) {
   return (1 + 6 * kWarpsPerBlock) * (size_t)nv * sizeof(T);
 }
-// Warps per block of the FP64 update kernels, whose tables take `doubles` per warp: four, fewer
-// where the tables of a large velocity grid would not fit an SM's shared memory.
-int update_warps(size_t doubles) {
-  const int w = (int)(224 * 1024 / (doubles * sizeof(double)));
-  return w < kWarpsPerBlock ? w : kWarpsPerBlock;
-}
-static_assert(face_flux_doubles(kMaxAxis) * sizeof(double) <= 224 * 1024, "tables of one warp");
-
-template <class N>
-cudaError_t set_update_limits(int nu, int nv) {
-  const size_t ff = face_flux_doubles(nv), cu = cell_update_doubles(nu, nv);
-  const cudaError_t e = cudaFuncSetAttribute(k_face_flux<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)(update_warps(ff) * ff * sizeof(double)));
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_cell_update<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)(update_warps(cu) * cu * sizeof(double)));
-}
+static_assert(face_flux_doubles(kMaxAxis) * sizeof(double) <= 48 * 1024 &&
+                  cell_update_doubles(kMaxAxis, kMaxAxis) * sizeof(double) <= 48 * 1024,
+              "update tables: no raised shared-memory limit");
 
 // dynamic shared memory limits of the FP64 form's sums and update kernels
-cudaError_t set_smem_limits_fp64(int nu, int nv) {
+cudaError_t set_smem_limits_fp64(int nv) {
   cudaError_t e = cudaFuncSetAttribute(k_sums<double, double2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem_sums<double>(nv));
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_sums_cell<NumF64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)(kWarpsPerBlock * kCellSumsWarp));
   if (e != cudaSuccess) return e;
-  if ((e = set_update_limits<NumF64>(nu, nv)) != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_update<double, double2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)smem_update<double>(nv));
 }
@@ -285,6 +270,16 @@ void launch_sums_cell(const Params& P, const typename N::H* f, double* part, typ
       P, f, part, slopes);
 }
 
+// The update in two passes: every face flux once, then Eq. 3 per velocity-cell.
+template <class N>
+void launch_update(const Params& P, const typename N::H* fi, typename N::H* fo, const typename N::Face* fx,
+                   const typename N::Face* fy, const typename N::Cell* cells, const typename N::H* slopes,
+                   typename N::H* Xx, typename N::H* Xy, cudaStream_t st) {
+  const int nc = P.nx * P.ny;
+  k_face_flux<N><<<nc, 128, face_flux_doubles(P.nv) * sizeof(double), st>>>(P, fi, fx, fy, slopes, Xx, Xy);
+  k_cell_update<N><<<nc, 128, cell_update_doubles(P.nu, P.nv) * sizeof(double), st>>>(P, fi, fo, cells, Xx, Xy);
+}
+
 template <typename T>
 cudaError_t launch_step(ugks_ctx* h, cudaStream_t st) {
   if constexpr (sizeof(T) == 4) {
@@ -315,18 +310,12 @@ cudaError_t launch_step(ugks_ctx* h, cudaStream_t st) {
     k_faces<kRecF64, true><<<fb, h->face_block, 0, st>>>(P, sums, Wi, h->nwe, h->fxr, h->fyr, h->Fx, h->Fy, h->mt4);
   }
   if ((r = mark(h, 4)) != cudaSuccess) return r;
-  const int nc = P.nx * P.ny;
   k_cells<<<h->nrblocks, h->cell_block, 0, st>>>(P, Wi, Wo, h->nwe, h->Fx, h->Fy, h->cells, h->rpart, h->err,
                                        h->cellf, h->mt4);
   if ((r = mark(h, 5)) != cudaSuccess) return r;
-  // the update in two passes: every face flux once, then Eq. 3 per velocity-cell
   T2* Xx = reinterpret_cast<T2*>(h->xflux);
   T2* Xy = Xx + (size_t)(P.nx + 1) * P.ny * P.nq;
-  const size_t ff = face_flux_doubles(P.nv), cu = cell_update_doubles(P.nu, P.nv);
-  const int wf = update_warps(ff), wc = update_warps(cu);
-  k_face_flux<NumF64><<<(nc + wf - 1) / wf, 32 * wf, wf * ff * sizeof(double), st>>>(
-      P, fi, h->fxr, h->fyr, reinterpret_cast<const T2*>(h->slopes), Xx, Xy);
-  k_cell_update<NumF64><<<(nc + wc - 1) / wc, 32 * wc, wc * cu * sizeof(double), st>>>(P, fi, fo, h->cells, Xx, Xy);
+  launch_update<NumF64>(P, fi, fo, h->fxr, h->fyr, h->cells, reinterpret_cast<T2*>(h->slopes), Xx, Xy, st);
   if ((r = mark(h, 6)) != cudaSuccess) return r;
   if (h->profiling) h->events_used += UGKS_NKERNELS + 1;
   return cudaGetLastError();
@@ -335,11 +324,9 @@ cudaError_t launch_step(ugks_ctx* h, cudaStream_t st) {
 
 // DF64 form: ghost ring, double-FP32 sums, FP64 interface and cell scalars (double-FP32
 // records), double-FP32 face fluxes and Eq. 3.
-cudaError_t set_smem_limits_df(int nu, int nv) {
-  const cudaError_t e = cudaFuncSetAttribute(k_sums_cell<NumDF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)(kWarpsPerBlock * kCellSumsWarp));
-  if (e != cudaSuccess) return e;
-  return set_update_limits<NumDF>(nu, nv);
+cudaError_t set_smem_limits_df() {
+  return cudaFuncSetAttribute(k_sums_cell<NumDF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)(kWarpsPerBlock * kCellSumsWarp));
 }
 
 cudaError_t launch_step_df(ugks_ctx* h, cudaStream_t st) {
@@ -360,16 +347,12 @@ cudaError_t launch_step_df(ugks_ctx* h, cudaStream_t st) {
   k_faces<kRecDF, true><<<(nf + h->face_block - 1) / h->face_block, h->face_block, 0, st>>>(P, h->sums, Wi, h->nwe, h->fxd, h->fyd, h->Fx, h->Fy,
                                                     h->mt4);
   if ((r = mark(h, 4)) != cudaSuccess) return r;
-  const int nc = P.nx * P.ny;
   k_cells<<<h->nrblocks, h->cell_block, 0, st>>>(P, Wi, Wo, h->nwe, h->Fx, h->Fy, nullptr, h->rpart, h->err, nullptr,
                                        h->mt4, h->celld);
   if ((r = mark(h, 5)) != cudaSuccess) return r;
   DF4* Xx = reinterpret_cast<DF4*>(h->xflux);
   DF4* Xy = Xx + (size_t)(P.nx + 1) * P.ny * P.nq;
-  const size_t ff = face_flux_doubles(P.nv), cu = cell_update_doubles(P.nu, P.nv);
-  const int wf = update_warps(ff), wc = update_warps(cu);
-  k_face_flux<NumDF><<<(nc + wf - 1) / wf, 32 * wf, wf * ff * sizeof(double), st>>>(P, fi, h->fxd, h->fyd, sl, Xx, Xy);
-  k_cell_update<NumDF><<<(nc + wc - 1) / wc, 32 * wc, wc * cu * sizeof(double), st>>>(P, fi, fo, h->celld, Xx, Xy);
+  launch_update<NumDF>(P, fi, fo, h->fxd, h->fyd, h->celld, sl, Xx, Xy, st);
   if ((r = mark(h, 6)) != cudaSuccess) return r;
   if (h->profiling) h->events_used += UGKS_NKERNELS + 1;
   return cudaGetLastError();
@@ -765,7 +748,7 @@ ugks_status ugks_step_noalloc(const ugks_config* cfg, const double* f_in, const 
     NA_CK(cudaMemcpy2DAsync(W0 + (size_t)c * nwe + wcell(P, 0, 0), P.wx * sizeof(double),
                             W_in + (size_t)c * nc, nx * sizeof(double), nx * sizeof(double), ny,
                             cudaMemcpyDeviceToDevice, st));
-  NA_CK(set_smem_limits_fp64(P.nu, P.nv));
+  NA_CK(set_smem_limits_fp64(P.nv));
   k_ghost<double2><<<ghost_cells(P), 128, 0, st>>>(P, f0, W0, nwe);
   k_sums<double, double2><<<(nwe + kWarpsPerBlock - 1) / kWarpsPerBlock, 32 * kWarpsPerBlock,
                             smem_sums<double>(P.nv), st>>>(P, f0, sums, nullptr);
@@ -1160,8 +1143,8 @@ ugks_status ugks_create(const ugks_config* cfg, void* cuda_stream, ugks_handle* 
                                        cudaMemcpyHostToDevice, h->stream)) != cudaSuccess)
       return r;
     if ((r = cudaMemsetAsync(h->err, 0, sizeof(int), h->stream)) != cudaSuccess) return r;
-    if (h->prec == UGKS_FP64 && (r = set_smem_limits_fp64(P.nu, P.nv)) != cudaSuccess) return r;
-    if (h->prec == UGKS_DF64 && (r = set_smem_limits_df(P.nu, P.nv)) != cudaSuccess) return r;
+    if (h->prec == UGKS_FP64 && (r = set_smem_limits_fp64(P.nv)) != cudaSuccess) return r;
+    if (h->prec == UGKS_DF64 && (r = set_smem_limits_df()) != cudaSuccess) return r;
     if ((r = cudaStreamSynchronize(h->stream)) != cudaSuccess) return r;
     return h->prec == UGKS_FP32F ? setup_single_f32(h) : cudaSuccess;
   };

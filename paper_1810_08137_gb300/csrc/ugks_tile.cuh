@@ -250,20 +250,22 @@ __global__ void __launch_bounds__(128, 3) k_sums_cell(Params P, const typename N
 // -------------------------------------------------------------------------------------
 // S6 + S8 and Eq. 3 of the FP64 and DF64 forms in two passes: every (face, velocity) micro flux
 // once.
-// k_face_flux: one warp per interior cell; for each velocity the cell forms the flux
+// k_face_flux: one block per interior cell; for each velocity the cell forms the flux
 // X = Q g + Mt4 f_up - Mt5 d_up (or the wall flux) through its downwind x-face and y-face from
 // its own reconstruction, and a cell next to the boundary also forms the flux whose upwind side
-// is the ghost cell or the wall.  Every face and velocity is written by exactly one warp, into
+// is the ghost cell or the wall.  Every face and velocity is written by exactly one block, into
 // Xx [(nx+1) ny][nq] and Xy [nx (ny+1)][nq] (face-major, velocity innermost).  k_cell_update then
 // reads the four fluxes of each velocity-cell and applies Eq. 3.
 // Both are bound by arithmetic: the FP64 form by the FP64 pipe (2 operations per clock and SM),
 // the DF64 form by the FP32 pipe.  Lanes run over the flattened
 // velocities (a lane per u would leave 12 of 32 idle at nu = 20), and all that depends on u or v
-// alone comes from per-warp tables in shared memory, so a velocity-cell costs 28 FP64
+// alone comes from tables in shared memory (one kind per warp), so a velocity-cell costs 28 FP64
 // instructions for its two faces: per face 3 for Q_h, 2 for Q_b = X2 Q_h + linear, 1 for g and 4 per
 // component, with f_up and d_up folded into the coefficients of the cell value and its two half
-// slopes (67 before), 36 with the tables; k_cell_update 18 (22 with tables, 30 before).  Both passes,
-// 100x50x28^2 0.820 -> 0.518 ms, 40x20x20^2 163 -> 90 us; FP64 pipe 89 % busy.
+// slopes (67 before), 36 with the tables; k_cell_update 18 (22 with tables, 30 before).  A block per
+// cell shares the tables and spreads small meshes evenly.  Both passes, FP64: 100x50x28^2 0.820 ->
+// 0.433 ms (a warp per cell 0.518), 40x20x20^2 163 -> 70 us (90); FP64 pipe 89 % busy.  DF64:
+// 200x100x28^2 815 -> 569 us, 60x30x101^2 1478 -> 728 us (1125).
 // -------------------------------------------------------------------------------------
 // Q at fixed u as a polynomial in v, from a record's eight coefficients: x face (un = u, ut = v) or
 // y face (un = v, ut = u).
@@ -303,10 +305,9 @@ __global__ void __launch_bounds__(128, 4) k_face_flux(Params P, const typename N
   extern __shared__ __align__(16) unsigned char smraw[];
   const int nv = P.nv, nu = P.nu, nq = P.nq, nx = P.nx, ny = P.ny, mpos = P.m_pos;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  V* tu = reinterpret_cast<V*>(smraw) + warp * face_flux_doubles(nv);
+  V* tu = reinterpret_cast<V*>(smraw);
   V* tm = tu + kFluxU * kFluxUB;
-  const int cell = blockIdx.x * (blockDim.x >> 5) + warp;
-  if (cell >= nx * ny) return;
+  const int cell = blockIdx.x;
   const int i = cell % nx, j = cell / nx;
   const Face& RW = fxr[(size_t)j * (nx + 1) + i];
   const Face& RE = fxr[(size_t)j * (nx + 1) + i + 1];
@@ -317,7 +318,8 @@ __global__ void __launch_bounds__(128, 4) k_face_flux(Params P, const typename N
   auto gauss = [](V lam, V d) { return N::exp(N::neg(N::mul(lam, N::mul(d, d)))); };
   const V tdx = N::tdx(P), tdy = N::tdy(P), dtv = N::dt(P);
 
-  for (int m = lane; m < nv; m += 32) {
+  // the block's tables, one kind per warp: x-face, y-face for v <= 0, y-face for v > 0, v
+  for (int m = lane; m < (warp == 3 ? nv : 0); m += 32) {
     const V v = N::v(P, m), cv = N::mul(v, tdy);
     const bool vp = m >= mpos;
     const Face& RD = vp ? RN : RS;
@@ -345,9 +347,9 @@ __global__ void __launch_bounds__(128, 4) k_face_flux(Params P, const typename N
   const int blocks = (nu + kFluxUB - 1) / kFluxUB;
   for (int ub = 0; ub < blocks; ub++) {
     const int kb = nu * ub / blocks, kw = nu * (ub + 1) / blocks - kb;  // this block's values of u
-    __syncwarp();  // the tables of the previous block are no longer read
+    if (ub) __syncthreads();  // the tables of the previous block of u are no longer read
     // u tables: Q at fixed u as a polynomial in v; a wall face passes dt f_up (Mt4 = dt, no Q)
-    for (int kk = lane; kk < kw; kk += 32) {
+    for (int kk = lane; kk < (warp < 3 ? kw : 0); kk += 32) {
       const int k = kb + kk;
       const V u = N::u(P, k), cu = N::mul(u, tdx);
       const bool up = k >= P.k_pos;
@@ -376,21 +378,18 @@ __global__ void __launch_bounds__(128, 4) k_face_flux(Params P, const typename N
         t[6 * kFluxUB + kk] = c1;
         t[7 * kFluxUB + kk] = g;
       };
-      const Face& RX = up ? RE : RW;
-      face(RX, up ? 0 : 1, true, coef(RX, up ? 1 : -1, cu), tu);
-      face(RS, 1, false, coef(RS, 0, cu), tu + kFluxX * kFluxUB);
-      face(RN, 0, false, coef(RN, 0, cu), tu + 2 * kFluxX * kFluxUB);
-      if (edge) {
-        const Face& RG = up ? RW : RE;
-        V* tg = tu + 3 * kFluxX * kFluxUB + kk;
-        auto ug = [&](const Face& R, V U) { return N::mul(val(R.G), gauss(val(R.lam), N::sub(u, U))); };
-        tg[0] = ug(RG, val(RG.Un));
-        tg[kFluxUB] = ug(RN, val(RN.Ut));
-        tg[2 * kFluxUB] = ug(RS, val(RS.Ut));
+      const Face& RF = warp == 0 ? (up ? RE : RW) : warp == 1 ? RS : RN;
+      face(RF, warp == 0 ? (up ? 0 : 1) : warp == 1 ? 1 : 0, warp == 0, coef(RF, warp ? 0 : up ? 1 : -1, cu),
+           tu + warp * kFluxX * kFluxUB);
+      if (edge) {  // the upwind faces: x, y for v <= 0 (N), y for v > 0 (S)
+        const Face& RG = warp == 0 ? (up ? RW : RE) : warp == 1 ? RN : RS;
+        tu[(3 * kFluxX + warp) * kFluxUB + kk] =
+            N::mul(val(RG.G), gauss(val(RG.lam), N::sub(u, val(warp == 0 ? RG.Un : RG.Ut))));
       }
     }
-    __syncwarp();
-    int m = lane / kw, kk = lane - m * kw;
+    __syncthreads();
+    const int dm = 128 / kw, dk = 128 - dm * kw;  // 128 velocities on
+    int m = threadIdx.x / kw, kk = threadIdx.x - m * kw;
     while (m < nv) {
       const int k = kb + kk, q = m * nu + k;
       const bool up = k >= kpos, vp = m >= mpos;  // u > 0, v > 0
@@ -441,8 +440,9 @@ __global__ void __launch_bounds__(128, 4) k_face_flux(Params P, const typename N
                                             sl0[2 * (q + yso)], sl0[2 * (q + yso) + 1], vp);
         }
       }
-      kk += 32;
-      while (kk >= kw) {
+      m += dm;
+      kk += dk;
+      if (kk >= kw) {
         kk -= kw;
         m++;
       }
@@ -452,7 +452,7 @@ __global__ void __launch_bounds__(128, 4) k_face_flux(Params P, const typename N
 
 // Eq. 3 from the four face fluxes of each velocity-cell (k_face_flux): the increment
 // f^{n+1} - f^n = inv (flux + cg1 (g^{n+1} - f^n) + cgn (g^n - f^n)) with inv folded into the
-// coefficients; 18 FP64 instructions per velocity-cell.  Tables per warp: per u index
+// coefficients; 18 FP64 instructions per velocity-cell.  Tables of the block's cell: per u index
 // inv u/dx, g^n and g^{n+1} factors; per v index the same with v/dy.
 __host__ __device__ constexpr size_t cell_update_doubles(int nu, int nv) { return 3 * ((size_t)nu + nv); }
 
@@ -465,30 +465,28 @@ __global__ void __launch_bounds__(128) k_cell_update(Params P, const typename N:
   using V = typename N::V;
   using H = typename N::H;
   extern __shared__ __align__(16) unsigned char smraw[];
-  const int nv = P.nv, nu = P.nu, nq = P.nq, nx = P.nx, ny = P.ny;
+  const int nv = P.nv, nu = P.nu, nq = P.nq, nx = P.nx;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  V* tu = reinterpret_cast<V*>(smraw) + warp * cell_update_doubles(nu, nv);
+  V* tu = reinterpret_cast<V*>(smraw);
   V* tm = tu + 3 * nu;
-  const int cell = blockIdx.x * (blockDim.x >> 5) + warp;
-  if (cell >= nx * ny) return;
+  const int cell = blockIdx.x;
   const int i = cell % nx, j = cell / nx;
   const typename N::Cell& C = cr[cell];
   auto val = [](const auto& x) { return N::val(x); };
   auto gauss = [](V lam, V d) { return N::exp(N::neg(N::mul(lam, N::mul(d, d)))); };
   const V inv = val(C.inv), ix = N::mul(inv, N::idx(P)), iy = N::mul(inv, N::idy(P));
-  for (int k = lane; k < nu; k += 32) {
-    const V u = N::u(P, k);
-    tu[k] = N::mul(ix, u);
-    tu[nu + k] = N::mul(val(C.Gn), gauss(val(C.lamn), N::sub(u, val(C.Un))));
-    tu[2 * nu + k] = N::mul(val(C.G1), gauss(val(C.lam1), N::sub(u, val(C.U1))));
+  // one kind of table per warp: u with g^n, u with g^{n+1}, v with g^n, v with g^{n+1}
+  for (int t = lane; t < (warp < 2 ? nu : nv); t += 32) {
+    const V x = warp < 2 ? N::u(P, t) : N::v(P, t);
+    const V lam = val(warp & 1 ? C.lam1 : C.lamn);
+    const V c0 = val(warp == 0 ? C.Un : warp == 1 ? C.U1 : warp == 2 ? C.Vn : C.V1);
+    const V g = gauss(lam, N::sub(x, c0));
+    if (warp == 0) tu[t] = N::mul(ix, x);
+    if (warp == 2) tm[t] = N::mul(iy, x);
+    if (warp < 2) tu[(1 + warp) * nu + t] = N::mul(val(warp ? C.G1 : C.Gn), g);
+    else tm[(warp - 1) * nv + t] = g;
   }
-  for (int m = lane; m < nv; m += 32) {
-    const V v = N::v(P, m);
-    tm[m] = N::mul(iy, v);
-    tm[nv + m] = gauss(val(C.lamn), N::sub(v, val(C.Vn)));
-    tm[2 * nv + m] = gauss(val(C.lam1), N::sub(v, val(C.V1)));
-  }
-  __syncwarp();
+  __syncthreads();
   const V A1 = N::mul(inv, val(C.cg1)), An = N::mul(inv, val(C.cgn)), nB = N::neg(N::add(A1, An));
   const V A1b = N::mul(A1, val(C.b1)), Anb = N::mul(An, val(C.bn));
   const H* fc0 = f + fcell(P, i, j) * nq;
@@ -496,8 +494,9 @@ __global__ void __launch_bounds__(128) k_cell_update(Params P, const typename N:
   const H* xw0 = Xx + ((size_t)j * (nx + 1) + i) * nq;
   const H* ys0 = Xy + ((size_t)j * nx + i) * nq;
   const size_t ynf = (size_t)nx * nq;
-  int m = lane / nu, k = lane - m * nu;
-  for (int q = lane; q < nq; q += 32) {
+  const int dm = 128 / nu, dk = 128 - dm * nu;  // 128 velocities on
+  int m = threadIdx.x / nu, k = threadIdx.x - m * nu;
+  for (int q = threadIdx.x; q < nq; q += 128) {
     const H c = fc0[q], XW = xw0[q], XE = xw0[nq + q], XS = ys0[q], XN = ys0[ynf + q];
     const V au = tu[k], av = tm[m];
     const V gn = N::mul(tu[nu + k], tm[nv + m]), g1 = N::mul(tu[2 * nu + k], tm[2 * nv + m]);
@@ -520,8 +519,9 @@ __global__ void __launch_bounds__(128) k_cell_update(Params P, const typename N:
       db_ = fma(A1, g1 * (C.b1 + sb1), fma(An, gn * (C.bn + sbn), db_));
     }
     fo0[q] = N::pack(N::add(N::h(c), dh_), N::add(N::b(c), db_));
-    k += 32;
-    while (k >= nu) {
+    m += dm;
+    k += dk;
+    if (k >= nu) {
       k -= nu;
       m++;
     }
