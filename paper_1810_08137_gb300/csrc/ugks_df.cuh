@@ -8,14 +8,17 @@
 
 namespace ugks {
 
-// a / b: quotient of the high parts, one correction from the double-FP32 remainder
+// a / b: quotient q1 of the high parts, one correction from the remainder a - q1 b.  With r good to
+// about an ulp (one Newton step) q1 is within an ulp of a.hi / b.hi, so a.hi - q1 b.hi is exact in
+// one FMA; the rest of the remainder is added in FP32, 2^-24 of a correction of 2^-24: about 2^-48.
 __device__ __forceinline__ df df_div(df a, df b) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b.hi));
   r = __fmaf_rn(r, __fmaf_rn(-b.hi, r, 1.f), r);  // one Newton step: r to ~2^-24
   const float q1 = __fmul_rn(a.hi, r);
-  const df rem = df_sub(a, df_mul(b, q1));
-  return fast_two_sum(q1, __fmul_rn(rem.hi, r));
+  const float e = __fmaf_rn(-q1, b.hi, a.hi);
+  const float rem = __fmaf_rn(-q1, b.lo, __fadd_rn(e, a.lo));
+  return fast_two_sum(q1, __fmul_rn(rem, r));
 }
 // Running sum acc + a b without renormalising: the rounding error of the high-part sum and
 // the product's low parts go to acc.lo, which is left to grow (by at most an ulp of acc.hi
