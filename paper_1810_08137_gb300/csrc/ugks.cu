@@ -365,7 +365,7 @@ cudaError_t launch_any(ugks_ctx* h, cudaStream_t st) {
   return launch_step<float>(h, st);
 }
 
-constexpr int kConvBlocks = 1216;  // 8 per SM
+constexpr int kConvBlocks = 1216;  // blocks of the state conversion kernels: 8 per SM
 // 16-byte alignment of a caller's FP64 rows (the state conversion kernels then move each
 // (h, b) pair as one 16-byte access)
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
@@ -413,8 +413,36 @@ __global__ void k_prim(Params P, const double* __restrict__ W, int nwe, double* 
   out[3 * nc + c] = 1.0 / lam;
 }
 
+// W between its ghosted buffers and the caller's [4][nc] device rows, in one launch.
+__global__ void k_copy_W(Params P, double* __restrict__ Wg, int nwe, double* __restrict__ Wc, bool out) {
+  const int nc = P.nx * P.ny, t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= nc) return;
+  const int w = wcell(P, t % P.nx, t / P.nx);
+  for (int c = 0; c < 4; c++) {
+    if (out) Wc[(size_t)c * nc + t] = Wg[(size_t)c * nwe + w];
+    else Wg[(size_t)c * nwe + w] = Wc[(size_t)c * nc + t];
+  }
+}
+
+// FP64 form: the ghosted f buffer and the caller's device rows (8-byte aligned), a block per cell.
+__global__ void k_copy_f(Params P, double2* __restrict__ fg, double* __restrict__ fc, bool out) {
+  for (int c = blockIdx.x; c < P.nx * P.ny; c += gridDim.x) {
+    double* g = reinterpret_cast<double*>(fg + fcell(P, c % P.nx, c / P.nx) * P.nq);
+    double* u = fc + (size_t)c * P.nq * 2;
+    for (int q = threadIdx.x; q < 2 * P.nq; q += blockDim.x) {
+      if (out) u[q] = g[q];
+      else g[q] = u[q];
+    }
+  }
+}
+
 ugks_status copy_W_in(ugks_ctx* h, const double* W, cudaMemcpyKind kind) {
   const Params& P = h->P;
+  if (kind == cudaMemcpyDeviceToDevice) {
+    k_copy_W<<<(P.nx * P.ny + 127) / 128, 128, 0, h->stream>>>(P, h->W[h->cur], h->nwe, const_cast<double*>(W), false);
+    CK(cudaGetLastError());
+    return UGKS_OK;
+  }
   for (int c = 0; c < 4; c++) {
     double* dst = h->W[h->cur] + (size_t)c * h->nwe + wcell(P, 0, 0);
     CK(cudaMemcpy2DAsync(dst, P.wx * sizeof(double), W + (size_t)c * P.nx * P.ny, P.nx * sizeof(double),
@@ -425,6 +453,11 @@ ugks_status copy_W_in(ugks_ctx* h, const double* W, cudaMemcpyKind kind) {
 
 ugks_status copy_W_out(ugks_ctx* h, double* W, cudaMemcpyKind kind) {
   const Params& P = h->P;
+  if (kind == cudaMemcpyDeviceToDevice) {
+    k_copy_W<<<(P.nx * P.ny + 127) / 128, 128, 0, h->stream>>>(P, h->W[h->cur], h->nwe, W, true);
+    CK(cudaGetLastError());
+    return UGKS_OK;
+  }
   for (int c = 0; c < 4; c++) {
     const double* src = h->W[h->cur] + (size_t)c * h->nwe + wcell(P, 0, 0);
     CK(cudaMemcpy2DAsync(W + (size_t)c * P.nx * P.ny, P.nx * sizeof(double), src, P.wx * sizeof(double),
@@ -454,6 +487,11 @@ ugks_status copy_f_in(ugks_ctx* h, const double* f, bool from_host) {
   const Params& P = h->P;
   const size_t row_d = (size_t)P.nx * P.nq * 2 * sizeof(double);
   const cudaMemcpyKind kind = from_host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
+  if (h->prec == UGKS_FP64 && !from_host) {
+    k_copy_f<<<kConvBlocks, 256, 0, h->stream>>>(P, static_cast<double2*>(h->f[h->cur]), const_cast<double*>(f), false);
+    CK(cudaGetLastError());
+    return UGKS_OK;
+  }
   if (h->prec == UGKS_FP64) {
     char* dst = static_cast<char*>(h->f[h->cur]) + ((size_t)2 * P.ex + 2) * P.nq * h->t2;
     CK(cudaMemcpy2DAsync(dst, (size_t)P.ex * P.nq * h->t2, f, row_d, row_d, P.ny, kind, h->stream));
@@ -504,6 +542,11 @@ ugks_status copy_f_out(ugks_ctx* h, double* f, bool to_host) {
   const Params& P = h->P;
   const size_t row_d = (size_t)P.nx * P.nq * 2 * sizeof(double);
   const cudaMemcpyKind kind = to_host ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
+  if (h->prec == UGKS_FP64 && !to_host) {
+    k_copy_f<<<kConvBlocks, 256, 0, h->stream>>>(P, static_cast<double2*>(h->f[h->cur]), f, true);
+    CK(cudaGetLastError());
+    return UGKS_OK;
+  }
   if (h->prec == UGKS_FP64) {
     const char* src = static_cast<const char*>(h->f[h->cur]) + ((size_t)2 * P.ex + 2) * P.nq * h->t2;
     CK(cudaMemcpy2DAsync(f, row_d, src, (size_t)P.ex * P.nq * h->t2, row_d, P.ny, kind, h->stream));

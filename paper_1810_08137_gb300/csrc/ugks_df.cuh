@@ -92,27 +92,27 @@ __device__ __forceinline__ df vl_df(df a, df c, df b) {
 __device__ __forceinline__ DF4 ghost_value(DF4*, double h, double b) { return split4(h, b); }
 
 // State conversion (set-up and checkpoint paths): FP64 rows [cell][q][(h, b)] of rows
-// j0 .. j0+nrows-1 <-> double-FP32 f with its ghost ring; grid-stride over velocity-cells.
+// j0 .. j0+nrows-1 <-> double-FP32 f with its ghost ring; a block takes a cell at a time.
 __global__ void k_rows_to_df(const double* __restrict__ src, DF4* __restrict__ dst, Params P, int j0,
                              int nrows) {
-  const long n = (long)P.nx * nrows * P.nq;
-  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < n; t += (long)gridDim.x * blockDim.x) {
-    const long c = t / P.nq;
-    const int q = (int)(t - c * P.nq);
-    const int r = (int)(c / P.nx), i = (int)(c - (long)r * P.nx);
-    dst[((size_t)(j0 + r + 2) * P.ex + i + 2) * P.nq + q] = split4(src[2 * t], src[2 * t + 1]);
+  for (int c = blockIdx.x; c < P.nx * nrows; c += gridDim.x) {
+    const int r = c / P.nx, i = c - r * P.nx;
+    const double* s = src + (size_t)c * P.nq * 2;
+    DF4* d = dst + ((size_t)(j0 + r + 2) * P.ex + i + 2) * P.nq;
+    for (int q = threadIdx.x; q < P.nq; q += blockDim.x) d[q] = split4(s[2 * q], s[2 * q + 1]);
   }
 }
 __global__ void k_df_to_rows(const DF4* __restrict__ src, double* __restrict__ dst, Params P, int j0,
                              int nrows) {
-  const long n = (long)P.nx * nrows * P.nq;
-  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < n; t += (long)gridDim.x * blockDim.x) {
-    const long c = t / P.nq;
-    const int q = (int)(t - c * P.nq);
-    const int r = (int)(c / P.nx), i = (int)(c - (long)r * P.nx);
-    const DF4 v = src[((size_t)(j0 + r + 2) * P.ex + i + 2) * P.nq + q];
-    dst[2 * t] = (double)v.hh + (double)v.hl;
-    dst[2 * t + 1] = (double)v.bh + (double)v.bl;
+  for (int c = blockIdx.x; c < P.nx * nrows; c += gridDim.x) {
+    const int r = c / P.nx, i = c - r * P.nx;
+    const DF4* s = src + ((size_t)(j0 + r + 2) * P.ex + i + 2) * P.nq;
+    double* d = dst + (size_t)c * P.nq * 2;
+    for (int q = threadIdx.x; q < P.nq; q += blockDim.x) {
+      const DF4 v = s[q];
+      d[2 * q] = to_double(dh(v));
+      d[2 * q + 1] = to_double(db(v));
+    }
   }
 }
 // Pointwise Maxwellian of (rho, U, V, T) per cell (FP64, stored as double-FP32) and W.
