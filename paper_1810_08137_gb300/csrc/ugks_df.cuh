@@ -1,25 +1,13 @@
 // Double-FP32 arithmetic of the DF64 form beyond the scalar core of ugks_dfcore.cuh
-// (error-free transformations, sums, products): division, lazily normalised running sums,
-// e^x, and the same operations on packed FP32 pairs (two velocities per lane); then the DF64
-// form's kernels.
+// (error-free transformations, sums, products): lazily normalised running sums, e^x, and the sums
+// kernel's operations on packed FP32 pairs; then the DF64 form's ghost value, state conversion and
+// initial state (its step kernels are those of ugks_tile.cuh).
 #pragma once
 
 #include "ugks_dfcore.cuh"
 
 namespace ugks {
 
-// a / b: quotient q1 of the high parts, one correction from the remainder a - q1 b.  With r good to
-// about an ulp (one Newton step) q1 is within an ulp of a.hi / b.hi, so a.hi - q1 b.hi is exact in
-// one FMA; the rest of the remainder is added in FP32, 2^-24 of a correction of 2^-24: about 2^-48.
-__device__ __forceinline__ df df_div(df a, df b) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b.hi));
-  r = __fmaf_rn(r, __fmaf_rn(-b.hi, r, 1.f), r);  // one Newton step: r to ~2^-24
-  const float q1 = __fmul_rn(a.hi, r);
-  const float e = __fmaf_rn(-q1, b.hi, a.hi);
-  const float rem = __fmaf_rn(-q1, b.lo, __fadd_rn(e, a.lo));
-  return fast_two_sum(q1, __fmul_rn(rem, r));
-}
 // Running sum acc + a b without renormalising: the rounding error of the high-part sum and
 // the product's low parts go to acc.lo, which is left to grow (by at most an ulp of acc.hi
 // per term); df_norm restores |lo| <= ulp(hi)/2 once the sum is complete.
@@ -64,9 +52,9 @@ __device__ __forceinline__ df df_exp(df x) {
 // =====================================================================================
 // DF64 form of the step: f stored as double-FP32 pairs (DF4), the per-velocity arithmetic of
 // the sums (S1, S7), the micro flux (S6, S8) and the implicit update (Eq. 3) in double-FP32
-// on the FP32 pipe; the interface (S2-S5) and cell (Eq. 4) scalars in FP64 (the shared
-// kernels, which write double-FP32 copies of their records).  The kernels follow the FP64
-// form's kernels step for step: warp per cell, lane = u index, loop over the v rows.
+// on the FP32 pipe; the interface (S2-S5) in FP64 and double-FP32 and the cell scalars (Eq. 4) in
+// FP64 (the shared kernels, which write double-FP32 copies of their records).  The sums and the
+// update run on the FP64 form's kernels (ugks_tile.cuh, arithmetic NumDF).
 // =====================================================================================
 __device__ __forceinline__ df dfv(float2 a) { return {a.x, a.y}; }
 __device__ __forceinline__ df dh(const DF4& v) { return {v.hh, v.hl}; }
@@ -80,12 +68,59 @@ __device__ __forceinline__ DF4 split4(double h, double b) { return mk4(df_of(h),
 __device__ __forceinline__ df df_half(df a) { return {0.5f * a.hi, 0.5f * a.lo}; }  // exact
 __device__ __forceinline__ df df_zero() { return {0.f, 0.f}; }
 
-// van Leer half slope d1 d2 / (d1 + d2) if d1 d2 > 0 else 0, d1 = c - a, d2 = b - c
-__device__ __forceinline__ df vl_df(df a, df c, df b) {
-  const df d1 = df_sub(c, a), d2 = df_sub(b, c);
-  const df p = df_mul(d1, d2);
-  const df r = df_div(p, df_add(d1, d2));
-  return p.hi > 0.f ? r : df_zero();
+// ---- the same operations on two numbers at a time (packed FP32 pairs: one instruction for both),
+// lane by lane the scalar operation's results ----
+struct df2 {
+  float2 hi, lo;
+};
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ df2 two_sum2(float2 a, float2 b) {
+  const float2 s = add2(a, b), bb = sub2(s, a);
+  return {s, add2(sub2(a, sub2(s, bb)), sub2(b, bb))};
+}
+__device__ __forceinline__ df2 fast_two_sum2(float2 a, float2 b) {
+  const float2 s = add2(a, b);
+  return {s, sub2(b, sub2(s, a))};
+}
+__device__ __forceinline__ df2 df2_add(df2 a, df2 b) {
+  const df2 s = two_sum2(a.hi, b.hi);
+  return fast_two_sum2(s.hi, add2(s.lo, add2(a.lo, b.lo)));
+}
+__device__ __forceinline__ df2 df2_sub(df2 a, df2 b) {  // df_add(a, -b)
+  const float2 s = sub2(a.hi, b.hi), bb = sub2(s, a.hi);
+  const float2 e = sub2(sub2(a.hi, sub2(s, bb)), add2(b.hi, bb));
+  return fast_two_sum2(s, add2(e, sub2(a.lo, b.lo)));
+}
+// a b without renormalising: product of the high parts, and its rounding error plus the cross terms
+__device__ __forceinline__ df2 df2_prod(df2 a, df2 b) {
+  const float2 p = mul2(a.hi, b.hi);
+  return {p, fma2(a.lo, b.hi, fma2(a.hi, b.lo, fma2(a.hi, b.hi, neg2(p))))};
+}
+__device__ __forceinline__ df2 df2_mul(df2 a, df2 b) {
+  const df2 p = df2_prod(a, b);
+  return fast_two_sum2(p.hi, p.lo);
+}
+__device__ __forceinline__ df2 df2_acc(df2 acc, df2 a, df2 b) {
+  const df2 p = df2_prod(a, b), s = two_sum2(acc.hi, p.hi);
+  return {s.hi, add2(acc.lo, add2(s.lo, p.lo))};
+}
+// van Leer half slope d1 d2 / (d1 + d2) if d1 d2 > 0 else 0, d1 = c - a, d2 = b - c.  The quotient p / t:
+// q1 of the high parts, one correction from the remainder p - q1 t.  With r good to about an ulp (one
+// Newton step) q1 is within an ulp of p.hi / t.hi, so p.hi - q1 t.hi is exact in one FMA; the rest of
+// the remainder is added in FP32, 2^-24 of a correction of 2^-24: about 2^-48.
+__device__ __forceinline__ df2 vl2_df(df2 a, df2 c, df2 b) {
+  const df2 d1 = df2_sub(c, a), d2 = df2_sub(b, c), p = df2_mul(d1, d2), t = df2_add(d1, d2);
+  float2 r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(t.hi.x));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(t.hi.y));
+  const float2 nt = neg2(t.hi);
+  r = fma2(r, fma2(nt, r, f2(1.f)), r);
+  const float2 q1 = mul2(p.hi, r), nq = neg2(q1);
+  const float2 rem = fma2(nq, t.lo, add2(fma2(nq, t.hi, p.hi), p.lo));
+  df2 o = fast_two_sum2(q1, mul2(rem, r));
+  if (!(p.hi.x > 0.f)) o.hi.x = o.lo.x = 0.f;
+  if (!(p.hi.y > 0.f)) o.hi.y = o.lo.y = 0.f;
+  return o;
 }
 
 // Ghost ring: the FP64 form's, stored as double-FP32 pairs

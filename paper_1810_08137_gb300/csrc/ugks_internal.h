@@ -114,9 +114,10 @@ struct __align__(16) CellShkF {
   float ln[4], l1[4];
 };
 
-// DF64 form: f of one velocity, (h, b) as double-FP32 pairs (h = hh + hl, b = bh + bl)
+// DF64 form: f of one velocity, (h, b) as double-FP32 pairs (h = hh + hl, b = bh + bl); h beside
+// b, so that a loaded value is two packed FP32 pairs
 struct __align__(16) DF4 {
-  float hh, hl, bh, bl;
+  float hh, bh, hl, bl;
 };
 // DF64 form: the FP64 records (FaceRec, CellRec) as double-FP32 pairs, written by the FP64
 // interface and cell kernels for the DF64 update kernels (which do no FP64 arithmetic)

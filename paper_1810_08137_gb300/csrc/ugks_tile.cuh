@@ -1,9 +1,13 @@
 // Velocity sums and update of the FP64 and DF64 forms, one source for both arithmetics.
 //
 // S1 + S7 with one thread per cell: the FP32-f form's sums_tile_body (ugks_f32.cuh) in FP64 or
-// double-FP32 arithmetic, plus the slope buffer the face-flux kernel reads.  A block owns a tile of 8 x 4 cells (lane = cell) and one quadrant of velocity
-// space, so it feeds one x side and one y side; its four warps take a share of the quadrant's
-// rows each, and the interface kernel adds the two quadrants of a side.
+// double-FP32 arithmetic, plus the slope buffer the face-flux kernel reads.  A block owns a tile of
+// 8 x 4 cells (lane = cell) and one quadrant of velocity space, so it feeds one x side and one y
+// side; its four warps take a share of the quadrant's rows each, and the interface kernel adds the
+// two quadrants of a side.  Bound by arithmetic: FP64 64 pipe instructions per velocity-cell, the
+// pipe 89 % busy (100x50x28^2 624 -> 517 us against a warp per cell); DF64 by FP32 issue, so h and b,
+// or two powers of u, go through packed pairs (200x100x28^2 538 -> 409 -> 363 us, 60x30x101^2 712 ->
+// 559 -> 501 us: a warp per cell, a thread per cell, packed pairs).
 #pragma once
 
 namespace ugks {
@@ -26,6 +30,16 @@ struct NumF64 {
   static __device__ __forceinline__ V neg(V a) { return -a; }
   static __device__ __forceinline__ V vl(V a, V c, V b) { return vl_half(a, c, b); }
   static __device__ __forceinline__ double f64(V a) { return a; }
+  // two values at a time: (h, b) of a velocity, or two powers of u
+  using V2 = double2;
+  static __device__ __forceinline__ V2 pair(const H& a) { return a; }
+  static __device__ __forceinline__ V2 of(V x, V y) { return make_double2(x, y); }
+  static __device__ __forceinline__ V x(V2 a) { return a.x; }
+  static __device__ __forceinline__ V y(V2 a) { return a.y; }
+  static __device__ __forceinline__ H pack2(V2 a) { return a; }
+  static __device__ __forceinline__ V2 acc2(V2 c, V2 a, V2 b) { return of(fma(a.x, b.x, c.x), fma(a.y, b.y, c.y)); }
+  static __device__ __forceinline__ V2 vl2(V2 a, V2 c, V2 b) { return of(vl(a.x, c.x, b.x), vl(a.y, c.y, b.y)); }
+  static __device__ __forceinline__ V ld(const V* p) { return *p; }
   using Face = FaceRec;
   using Cell = CellRec;
   static constexpr bool kShakhov = true;
@@ -56,8 +70,18 @@ struct NumDF {
   static __device__ __forceinline__ V norm(V a) { return df_norm(a); }
   static __device__ __forceinline__ V half(V a) { return df_half(a); }
   static __device__ __forceinline__ V neg(V a) { return df_neg(a); }
-  static __device__ __forceinline__ V vl(V a, V c, V b) { return vl_df(a, c, b); }
   static __device__ __forceinline__ double f64(V a) { return to_double(a); }
+  using V2 = df2;
+  static __device__ __forceinline__ V2 pair(const H& a) {
+    return {make_float2(a.hh, a.bh), make_float2(a.hl, a.bl)};
+  }
+  static __device__ __forceinline__ V2 of(V x, V y) { return {make_float2(x.hi, y.hi), make_float2(x.lo, y.lo)}; }
+  static __device__ __forceinline__ V x(V2 a) { return {a.hi.x, a.lo.x}; }
+  static __device__ __forceinline__ V y(V2 a) { return {a.hi.y, a.lo.y}; }
+  static __device__ __forceinline__ H pack2(V2 a) { return {a.hi.x, a.hi.y, a.lo.x, a.lo.y}; }
+  static __device__ __forceinline__ V2 acc2(V2 c, V2 a, V2 b) { return df2_acc(c, a, b); }
+  static __device__ __forceinline__ V2 vl2(V2 a, V2 c, V2 b) { return vl2_df(a, c, b); }
+  static __device__ __forceinline__ V ld(const V* p) { return dfv(*reinterpret_cast<const float2*>(p)); }
   using Face = FaceRecD;
   using Cell = CellRecD;
   static constexpr bool kShakhov = false;
@@ -86,6 +110,7 @@ __global__ void __launch_bounds__(128, 3) k_sums_cell(Params P, const typename N
                                                       double* __restrict__ part,
                                                       typename N::H* __restrict__ slopes) {
   using V = typename N::V;
+  using V2 = typename N::V2;
   using H = typename N::H;
   extern __shared__ __align__(16) unsigned char cell_sm[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -160,9 +185,9 @@ __global__ void __launch_bounds__(128, 3) k_sums_cell(Params P, const typename N
   const H* c = st + own;
   int cflip = kTileStageF4;
   for (int m = m0; m < m1; m++) {
-    V A0, A1, A2, A3, X0, X1, X2, X3, X4, Y0, Y1, Y2, Y3, Ab0, Ab1, Xb0, Xb1, Xb2, Yb0, Yb1;
-    A0 = A1 = A2 = A3 = X0 = X1 = X2 = X3 = X4 = Y0 = Y1 = Y2 = Y3 = N::zero();
-    Ab0 = Ab1 = Xb0 = Xb1 = Xb2 = Yb0 = Yb1 = N::zero();
+    // sums over u^n of the value and its two half slopes: (h, b) for n < 2 or 3, then h of two powers
+    V2 a0, a1, a23, x0s, x1s, x2s, x34, y0s, y1s, y23;
+    a0 = a1 = a23 = x0s = x1s = x2s = x34 = y0s = y1s = y23 = N::of(N::zero(), N::zero());
     // slopes of a velocity of two quadrants (u = 0 or v = 0) are written by the upper one
     const bool wrow = need && !(vn && m >= P.m_neg);
 #pragma unroll 1
@@ -176,30 +201,30 @@ __global__ void __launch_bounds__(128, 3) k_sums_cell(Params P, const typename N
       for (int q = 0; q < n; q++) {
         const H C = c[q], Wn = c[q - ox], E = c[q + ox], S = c[q - oy], Nn = c[q + oy];
         const V* t = ut + 6 * (k + q);
-        const V w0 = t[0], w1 = t[1], w2 = t[2], w3 = t[3], w4 = t[4];
-        const V ch = N::h(C), cb = N::b(C);
-        const V rxh = N::vl(N::h(Wn), ch, N::h(E)), rxb = N::vl(N::b(Wn), cb, N::b(E));
-        const V ryh = N::vl(N::h(S), ch, N::h(Nn)), ryb = N::vl(N::b(S), cb, N::b(Nn));
+        const V w0 = N::ld(t), w1 = N::ld(t + 1), w2 = N::ld(t + 2), w3 = N::ld(t + 3), w4 = N::ld(t + 4);
+        const V2 cc = N::pair(C);
+        const V2 rx = N::vl2(N::pair(Wn), cc, N::pair(E)), ry = N::vl2(N::pair(S), cc, N::pair(Nn));
         if (wrow && !(un && k + q >= P.k_neg)) {
           H* q2 = slc + 2 * ((size_t)m * nu + k + q);
-          q2[0] = N::pack(rxh, rxb);
-          q2[1] = N::pack(ryh, ryb);
+          q2[0] = N::pack2(rx);
+          q2[1] = N::pack2(ry);
         }
-        A0 = N::acc(A0, w0, ch); A1 = N::acc(A1, w1, ch); A2 = N::acc(A2, w2, ch); A3 = N::acc(A3, w3, ch);
-        X0 = N::acc(X0, w0, rxh); X1 = N::acc(X1, w1, rxh); X2 = N::acc(X2, w2, rxh);
-        X3 = N::acc(X3, w3, rxh); X4 = N::acc(X4, w4, rxh);
-        Y0 = N::acc(Y0, w0, ryh); Y1 = N::acc(Y1, w1, ryh); Y2 = N::acc(Y2, w2, ryh); Y3 = N::acc(Y3, w3, ryh);
-        Ab0 = N::acc(Ab0, w0, cb); Ab1 = N::acc(Ab1, w1, cb);
-        Xb0 = N::acc(Xb0, w0, rxb); Xb1 = N::acc(Xb1, w1, rxb); Xb2 = N::acc(Xb2, w2, rxb);
-        Yb0 = N::acc(Yb0, w0, ryb); Yb1 = N::acc(Yb1, w1, ryb);
+        const V2 w00 = N::of(w0, w0), w11 = N::of(w1, w1), w22 = N::of(w2, w2), w23 = N::of(w2, w3);
+        a0 = N::acc2(a0, w00, cc); a1 = N::acc2(a1, w11, cc); a23 = N::acc2(a23, w23, N::of(N::x(cc), N::x(cc)));
+        x0s = N::acc2(x0s, w00, rx); x1s = N::acc2(x1s, w11, rx); x2s = N::acc2(x2s, w22, rx);
+        x34 = N::acc2(x34, N::of(w3, w4), N::of(N::x(rx), N::x(rx)));
+        y0s = N::acc2(y0s, w00, ry); y1s = N::acc2(y1s, w11, ry); y23 = N::acc2(y23, w23, N::of(N::x(ry), N::x(ry)));
       }
       c += cflip;
       cflip = -cflip;
     }
     // the row's part of the 32 face sums
-    auto nz = [](V& a) { a = N::norm(a); };
-    nz(A0); nz(A1); nz(A2); nz(A3); nz(X0); nz(X1); nz(X2); nz(X3); nz(X4); nz(Y0); nz(Y1); nz(Y2); nz(Y3);
-    nz(Ab0); nz(Ab1); nz(Xb0); nz(Xb1); nz(Xb2); nz(Yb0); nz(Yb1);
+    auto nx_ = [](V2 a) { return N::norm(N::x(a)); };
+    auto ny_ = [](V2 a) { return N::norm(N::y(a)); };
+    const V A0 = nx_(a0), A1 = nx_(a1), A2 = nx_(a23), A3 = ny_(a23), Ab0 = ny_(a0), Ab1 = ny_(a1);
+    const V X0 = nx_(x0s), X1 = nx_(x1s), X2 = nx_(x2s), X3 = nx_(x34), X4 = ny_(x34);
+    const V Xb0 = ny_(x0s), Xb1 = ny_(x1s), Xb2 = ny_(x2s);
+    const V Y0 = nx_(y0s), Y1 = nx_(y1s), Y2 = nx_(y23), Y3 = ny_(y23), Yb0 = ny_(y0s), Yb1 = ny_(y1s);
     const V v = vt[2 * m], w = vt[2 * m + 1];
     const V vv = N::mul(v, v), wv = N::mul(w, v), vty = N::mul(v, tdy);
     auto put = [&](int e, V g, V x) { out[e * kTileOut] = N::norm(N::acc(out[e * kTileOut], g, x)); };
