@@ -47,15 +47,15 @@ def peaks():
 # FP64 form: FP64 flops per velocity-cell as executed (FMA = 2 flops), from the ncu
 # instruction counts of its kernels (DFMA, DMUL, DADD per velocity-cell; the capture in
 # profiles/fp64_step_kernels_channel_200x100_v28.md): the update's two passes
-# 2 x 58.8 + 25.6 + 12.5, the sums kernel 2 x 43.4 + 13.3 + 18.4.  The peak is measured
+# 2 x 37.9 + 12.9 + 7.4, the sums kernel 2 x 38.1 + 10.3 + 15.7.  The peak is measured
 # in the run (ugks_fp64_rate: chains of FP64 FMAs on every SM).
-FP64_UPDATE_FLOPS_PER_VC = 2 * 58.8 + 25.6 + 12.5
-FP64_SUMS_FLOPS_PER_VC = 2 * 43.4 + 13.3 + 18.4
+FP64_UPDATE_FLOPS_PER_VC = 2 * 37.9 + 12.9 + 7.4
+FP64_SUMS_FLOPS_PER_VC = 2 * 38.1 + 10.3 + 15.7
 # DRAM traffic of the FP32-f update kernel per velocity-cell (read + write), from the ncu
 # capture of the current kernel summarised in profiles/fp32f_step_kernels_channel_400x200_v28.md
 # (dram__bytes_read.sum + dram__bytes_write.sum of one kb_strip launch at 400x200x28^2);
 # set to None when the kernel changes until it is captured again.
-UPDATE_TRAFFIC_PER_VC = (601.562112e6 + 465.784064e6) / 62.72e6
+UPDATE_TRAFFIC_PER_VC = (597.178624e6 + 464.608768e6) / 62.72e6
 # FP32 lane operations of the FP32-f update kernel per velocity-cell on the FMA pipe (a packed
 # pair instruction = 2), from the same capture's instruction mix: FFMA2 43.4, FMUL2 15.0,
 # FADD2 6.6, FFMA 5.0, FADD 3.4, FMUL 1.4 per velocity-cell; the peak is the FMA pipe's
@@ -335,7 +335,8 @@ def batch_bench(ugks, torch, stream, steps, warmup):
     B.sync()
     t_admit = time.perf_counter() - t0
     tuned_ms = B.tune(2)
-    # both step modes, same tiles: one persistent launch vs seven phase launches per step
+    # both step modes, same tiles: one persistent launch vs six phase launches per step (ghost ring,
+    # sums with a thread and with a warp per cell, faces, cells, update)
     mode_ms = {}
     tuned_mode = B.persistent
     for mode in (True, False):
@@ -368,7 +369,7 @@ def batch_bench(ugks, torch, stream, steps, warmup):
            "unit": UNIT, "ms_per_step": ms / steps, "steps": steps, "precision": "fp32f",
            "tuned_walk_rows": rows, "tuned_ms_per_step": tuned_ms,
            "admit_s": t_admit, "device_bytes": B.bytes_used,
-           "persistent": B.persistent, "launches_per_step": 1 if B.persistent else 7,
+           "persistent": B.persistent, "launches_per_step": 1 if B.persistent else 6,
            "ms_per_step_by_mode": mode_ms,
            "tuned_walk_vtile": sorted({B.walk_vtile(s) for s in slots})}
     B.close()
@@ -619,7 +620,8 @@ def main():
         "clocks": main["clocks"],
         "e2e": {"value": ws * cfg.vc * args.e2e_steps / t_e2e, "unit": UNIT,
                 "steps": args.e2e_steps, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
-        "gpu_launches": 7 * args.steps,  # 6 phase kernels + the buffer flip per step
+        # ghost ring, sums, faces, cells, update (FP64 form: the update is two kernels)
+        "gpu_launches": (5 if main_prec == ugks.FP32F else 6) * args.steps,
         "cpu_baseline": cpu,
         "batch": batch,
         "serving": serving,

@@ -3,20 +3,17 @@
 // Per step, on one stream:
 //   k_ghost               boundary ghost ring (periodic image, wall zero-gradient copy,
 //                         pressure Maxwellian)
-//   k_sums                per cell and side, the velocity sums of steps S1 and S7 (W0,
+//   sums                  per cell and side, the velocity sums of steps S1 and S7 (W0,
 //                         tangential slope of W, free-transport sums) over one read of f
 //   k_faces               per interface, steps S2-S5 (Maxwellian moments, Mt time weights,
-//                         micro slopes a_L a_R b A, equilibrium flux) in FP64, the total
-//                         macroscopic flux, and the coefficients of the micro flux (S6, S8);
-//                         the FP32-f form runs the terms that carry slopes in FP32
+//                         micro slopes a_L a_R b A, equilibrium flux), the total macroscopic
+//                         flux, and the coefficients of the micro flux (S6, S8): FP64, or with
+//                         the polynomial work in double-FP32 (FP32-f and DF64 forms)
 //   k_cells               conservative W update (Eq. 4), g^n, g^{n+1}, tau^n, tau^{n+1}
-//   k_face_flux           micro flux of every face and velocity (S6, S8), once, from its
-//                         upwind cell, into face-flux buffers (second read of f)
-//   k_cell_update         the implicit f update (Eq. 3) from the four fluxes of each
-//                         velocity-cell, one write of f^{n+1}
-//   (k_update, the same update in one pass that forms each interior flux twice, serves the
-//   allocation-free entry point)
-// These are the FP64 form's kernels; the FP32-f form (FP32 f in a paired-row layout) has
+//   update                micro flux (S6, S8) and the implicit f update (Eq. 3)
+// The sums and update of the FP64 and DF64 forms are in ugks_tile.cuh; here are the FP64 sums with a
+// warp per cell (k_sums: Shakhov model, allocation-free entry point) and the one-pass FP64 update of
+// the allocation-free entry point (k_update).  The FP32-f form (FP32 f in a paired-row layout) has
 // its own ghost fill, sums and update in ugks_f32.cuh and shares the interface and cell
 // bodies (faces_body, cells_body).
 //
@@ -85,11 +82,7 @@ __device__ __forceinline__ float rcp_ftz(float x) {
   return y;
 }
 // 16-byte asynchronous global -> shared copies (per thread), in commit groups.
-__device__ __forceinline__ void cp_async16(void* sm, const void* gm) {
-  const unsigned a = (unsigned)__cvta_generic_to_shared(sm);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(a), "l"(gm) : "memory");
-}
-// The same, cached in L2 only (data read once by this warp).
+// cached in L2 only (data read once by this warp)
 __device__ __forceinline__ void cp_async16_cg(void* sm, const void* gm) {
   const unsigned a = (unsigned)__cvta_generic_to_shared(sm);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(gm) : "memory");
@@ -97,14 +90,6 @@ __device__ __forceinline__ void cp_async16_cg(void* sm, const void* gm) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-__device__ __forceinline__ void cp_async8(void* sm, const void* gm) {
-  const unsigned a = (unsigned)__cvta_generic_to_shared(sm);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(a), "l"(gm) : "memory");
-}
-// one f value (float2: 8 bytes, double2: 16 bytes)
-__device__ __forceinline__ void cp_async_f(float2* sm, const float2* gm) { cp_async8(sm, gm); }
-__device__ __forceinline__ void cp_async_f(double2* sm, const double2* gm) { cp_async16(sm, gm); }
-
 
 // Collision time tau = mu / p with mu = mu_ref T^omega, T = 1/lam, p = rho / (2 lam).
 __device__ __forceinline__ double collision_time(const Params& P, double rho, double lam) {
