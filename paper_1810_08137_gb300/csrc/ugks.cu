@@ -186,10 +186,9 @@ std::pair<int, int> f32_row_pairs(int nv, double vmin, double vmax) {
 // FP64 pipe (2 operations per clock).  40x20 cells 14.9 -> 12.8 us.
 int small_block(long n) { return n < 152 * 128 ? 32 : 128; }
 
-// Velocity sums per cell: the FP64 and DF64 forms' BGK sums kernel keeps its four quadrants apart.
-int sums_per_cell(const ugks_config* c) {
-  return c->precision != UGKS_FP32F && shakhov_pr(c) == 1.0 ? kCellPart : kNSum;
-}
+// Velocity sums per cell: the FP64 and DF64 forms' BGK sums kernel keeps its four quadrants apart (the
+// Shakhov model's kernel, kNSum of them, gets the same room: the model adds only its own buffers).
+int sums_per_cell(const ugks_config* c) { return c->precision != UGKS_FP32F ? kCellPart : kNSum; }
 
 // Device bytes ugks_create allocates for cfg (cudaMalloc sizes, without allocator rounding).
 size_t predict_bytes(const ugks_config* c) {
