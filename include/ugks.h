@@ -182,8 +182,9 @@ ugks_status ugks_set_wait_limit(ugks_handle h, long long polls);
  * and their FP64 face sums are added in shared memory in a fixed order.  0 selects the
  * automatic choice that ugks_create also makes: more warps per cell while the cells alone
  * would leave the kernel's resident warps under-filled (small meshes, large velocity
- * grids) and every warp keeps at least 16 velocity rows.  The result depends on `warps` only
- * through the order of the FP64 additions.  UGKS_EINVAL for other values or another form.
+ * grids) and every warp keeps at least 16 velocity rows.  With 1, a mesh that fills the device
+ * with tiles of 8 x 4 cells is summed with a thread per cell.  The result depends on `warps` only
+ * through the order of the additions (FP64; FP32 within at most 256 terms).  UGKS_EINVAL for other values or another form.
  * Synchronises; the next ugks_step captures its graphs again. */
 ugks_status ugks_set_sums_split(ugks_handle h, int warps);
 /* Current warps per cell of the FP32-f sums (0 for another form or a NULL handle). */
