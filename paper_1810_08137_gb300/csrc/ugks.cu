@@ -2006,7 +2006,7 @@ ugks_status ugks_batch_tune(ugks_batch b, int trial_steps, double* best_ms) {
     if (!r) r = apply(best_r, best_v);
     best_total = best_t / trial_steps;
   }
-  // step mode: one persistent launch (six grid barriers per step) against seven phase
+  // step mode: one persistent launch (four grid barriers per step) against the phase
   // launches; the barriers cost more than the launches when the batch holds little work
   if (!r && b->grid_step > 0) {
     float t_mode[2] = {0.f, 0.f};

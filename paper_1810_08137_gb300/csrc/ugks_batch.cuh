@@ -1,7 +1,7 @@
 // Batched execution of many independent UGKS instances (FP32-f form): every phase of the
 // step runs once per step for all active instances, as a persistent grid that walks a
 // device-resident work table of virtual blocks.  The step is either one cooperative launch
-// of kb_step (all phases, grid barriers with bounded waits between them) or seven phase
+// of kb_step (all phases, grid barriers with bounded waits between them) or the phase
 // launches; either way one CUDA graph replay.  The table (and each instance's ping-pong
 // parity) lives in device memory, so admitting or retiring an instance changes data, not
 // the captured graph.

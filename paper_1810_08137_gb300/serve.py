@@ -157,8 +157,8 @@ def make_requests(cfgs, arrivals, prims):
 
 class ModeSwitchingBatch:
     """A batch engine whose step mode follows the work in flight: one persistent launch per
-    step (six grid barriers) when the active instances hold at least `persistent_min_vc`
-    velocity-cells, else seven phase launches, whose fixed cost is lower for small batches.
+    step (four grid barriers) when the active instances hold at least `persistent_min_vc`
+    velocity-cells, else a launch per phase, whose fixed cost is lower for small batches.
     The mode does not change results (the same phase code runs either way)."""
 
     def __init__(self, batch, persistent_min_vc: int):
