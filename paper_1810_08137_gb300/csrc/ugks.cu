@@ -1011,6 +1011,8 @@ ugks_status ugks_create(const ugks_config* cfg, void* cuda_stream, ugks_handle* 
       P.refpair[1][c] = P.refsum[kSumN / 16][kOffW0 + c] + P.refsum[kSumS / 16][kOffW0 + c];
       P.refpair[1][4 + c] = P.refsum[kSumN / 16][kOffSf + c] + P.refsum[kSumS / 16][kOffSf + c];
     }
+    for (int ax = 0; ax < 2; ax++)
+      for (int t = 0; t < 10; t++) P.refheatpair[ax][t] = P.refheat[2 * ax][t] + P.refheat[2 * ax + 1][t];
     // g_ref per slot of the paired-row layout (h, h', b, b')
     gref_host.resize((size_t)P.fs);
     for (int pr = 0; pr < P.pr_all; pr++)

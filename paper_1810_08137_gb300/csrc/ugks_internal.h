@@ -142,6 +142,7 @@ struct Params {
                           // (zero in the FP64 form): E, W, N, S (10 each), cell (first 10
                           // of its 13 in refheat[4], B-moments in refheatC)
   double refheatC[3];
+  double refheatpair[2][10];  // refheat of both sides of a face: x faces (E + W), y faces (N + S)
   int ex;                 // f row length in cells: nx + 4 (two-cell ghost ring)
   int wx;                 // W row length in cells: nx + 2 (one-cell ghost ring)
   double dx, dy, dt;
