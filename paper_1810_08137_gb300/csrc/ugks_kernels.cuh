@@ -797,7 +797,6 @@ __device__ __forceinline__ void shakhov_poly(double alpha, double U, double V, d
   p[3][0] = p[1][2] = a1 * l2;
   p[0][3] = p[2][1] = a2 * l2;
 }
-using FaceCore = FaceCoreT<double>;
 template <typename T>
 __device__ __forceinline__ void face_core(const Params& P, const double* W0, const double* St,
                                           const double* Sf, const double* Ss, const double* WL,
