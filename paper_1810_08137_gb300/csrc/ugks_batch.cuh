@@ -365,6 +365,8 @@ __device__ __forceinline__ bool grid_sync(BarrierDev* g) {
   return ok != 0;
 }
 
+__device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
+
 // dynamic shared memory of the persistent step: the largest phase's (the walk's rings; the
 // ghost tables and the cells reduction alias its start)
 constexpr size_t kStepSmem = kStripSmem > kTileSmem ? kStripSmem : kTileSmem;
@@ -386,7 +388,13 @@ __global__ void __launch_bounds__(128, 3) kb_step(const SlotDev* __restrict__ sl
   faces_phase_shk(slots, wk, par);
   if (!grid_sync(bar)) return;
   cells_phase(slots, wk, par, reinterpret_cast<double(*)[8]>(step_sm));
+  // The walk reads the face and cell records of this launch by bulk copies, through the async
+  // proxy: ordinary stores are ordered before such reads by a proxy fence only (grid_sync's fence is
+  // one of the generic proxy), on the writers before the barrier and on the readers after it.  The
+  // phase launches have the kernel boundary in its place.
+  fence_proxy_async_global();
   if (!grid_sync(bar)) return;
+  fence_proxy_async_global();
   const unsigned nrec = strip_phase(slots, wk, par, step_sm);
   strip_phase_shk(slots, wk, par, step_sm, false, nrec);
 }
