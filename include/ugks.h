@@ -172,7 +172,8 @@ ugks_status ugks_sync(ugks_handle h);
  * the mbarrier (each suspends the waiting lanes for a hardware-chosen time; the default
  * 2^22 is at least about a second).  When a wait runs out the walk records it and returns
  * after draining its copies in flight; the next synchronising call reports UGKS_ETIMEOUT
- * and the state is undefined until set again.  No effect on the other forms.
+ * and the state is undefined until set again.  No effect on the other forms; on an instance of a
+ * batch it takes effect in the batch's next step.
  * Synchronises. */
 ugks_status ugks_set_wait_limit(ugks_handle h, long long polls);
 
@@ -185,7 +186,8 @@ ugks_status ugks_set_wait_limit(ugks_handle h, long long polls);
  * grids) and every warp keeps at least 16 velocity rows.  With 1, a mesh that fills the device
  * with tiles of 8 x 4 cells is summed with a thread per cell.  The result depends on `warps` only
  * through the order of the additions (FP64; FP32 within at most 256 terms).  UGKS_EINVAL for other values or another form.
- * Synchronises; the next ugks_step captures its graphs again. */
+ * Synchronises; the next ugks_step captures its graphs again.  On an instance of a batch it takes
+ * effect in the batch's next step. */
 ugks_status ugks_set_sums_split(ugks_handle h, int warps);
 /* Current warps per cell of the FP32-f sums (0 for another form or a NULL handle). */
 int ugks_get_sums_split(ugks_handle h);
@@ -257,7 +259,7 @@ ugks_status ugks_batch_retire(ugks_batch b, int slot);
 
 /* The instance in a slot, for the single-instance calls that move state and read results
  * (ugks_init_maxwellian, ugks_set_state(_device), ugks_get_state(_device), ugks_moments,
- * ugks_residual, ugks_sync).  Do not call ugks_step or ugks_destroy on it.  NULL if the
+ * ugks_residual, ugks_sync) or set its sums (ugks_set_sums_split, ugks_set_wait_limit).  Do not call ugks_step or ugks_destroy on it.  NULL if the
  * slot is free. */
 ugks_handle ugks_batch_instance(ugks_batch b, int slot);
 

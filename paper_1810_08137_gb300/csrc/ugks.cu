@@ -21,6 +21,7 @@
 
 using namespace ugks;
 
+struct ugks_batch_ctx;
 struct ugks_ctx {
   ugks_config cfg;
   Params P;
@@ -59,6 +60,7 @@ struct ugks_ctx {
   SlotDev* d_slot = nullptr;
   BatchWork* d_work = nullptr;
   int grid1[16] = {0};       // per step kernel: blocks of its launch
+  ugks_batch_ctx* owner = nullptr;  // batch this instance is a slot of
   double* rpart = nullptr;
   int nrblocks = 0;
   int face_block = 128;      // faces and cells per block of the interface and cell kernels
@@ -262,6 +264,7 @@ cudaError_t upload_single_f32(ugks_ctx* h);
 int auto_sums_split(const Params& P, int sms);
 bool use_sums_tiles(const Params& P, int split, int sms);
 SlotDev slot_desc(const ugks_ctx* h, int par, int walk_rows, int walk_vtile = 0);
+ugks_status upload_owner(ugks_ctx* h);
 
 template <class N>
 void launch_sums_cell(const Params& P, const typename N::H* f, double* part, typename N::H* slopes, cudaStream_t st) {
@@ -1344,7 +1347,7 @@ ugks_status ugks_set_wait_limit(ugks_handle h, long long polls) {
     const SlotDev S = slot_desc(h, h->cur, h->walk_rows);
     CK(cudaMemcpy(h->d_slot, &S, sizeof(SlotDev), cudaMemcpyHostToDevice));
   }
-  return UGKS_OK;
+  return upload_owner(h);
 }
 
 ugks_status ugks_set_sums_split(ugks_handle h, int warps) {
@@ -1364,7 +1367,7 @@ ugks_status ugks_set_sums_split(ugks_handle h, int warps) {
       CK(cudaGraphExecDestroy(h->graph[b]));
       h->graph[b] = nullptr;
     }
-  return UGKS_OK;
+  return upload_owner(h);
 }
 
 int ugks_get_sums_split(ugks_handle h) { return (h && h->d_slot) ? h->sums_split : 0; }
@@ -1461,12 +1464,13 @@ struct ugks_batch_ctx {
   size_t budget = 0, used = 0;
   std::vector<ugks_ctx*> ctx;       // per slot, nullptr when free
   std::vector<int> walk_rows;       // per slot: cell tile of the walk (rows), 0: automatic
-  std::vector<int> eff_rows;        // per slot: rows in use (0: descriptor not uploaded yet)
+  std::vector<int> eff_rows;        // per slot: rows in use
   std::vector<int> walk_vtile;      // per slot: velocity tile of the walk (chunks, 0 = all)
   bool persistent = false;          // one cooperative launch per step (else phase launches)
   int grid_step = 0;                // co-resident blocks of the persistent step kernel
   BarrierDev* d_bar = nullptr;      // its grid barrier (count, gen, wait limit, timeout flag)
   SlotDev* d_slots = nullptr;
+  std::vector<SlotDev> h_slots;     // their host copies
   BatchWork* d_work = nullptr;
   BatchWork h_work;
   int par = 0;                      // parity of the next step
@@ -1592,21 +1596,20 @@ int auto_walk_rows(const Params& P, int nchunk, long warps) {
   return best;
 }
 
-ugks_status upload_slot(ugks_batch_ctx* b, int s) {
-  const SlotDev S = slot_desc(b->ctx[s], b->par, b->eff_rows[s], b->walk_vtile[s]);
-  BCK(cudaMemcpyAsync(b->d_slots + s, &S, sizeof(SlotDev), cudaMemcpyHostToDevice, b->stream));
-  BCK(cudaStreamSynchronize(b->stream));
-  return UGKS_OK;
-}
-
-// Choose the walk tiles, rebuild the work table of the active slots and upload both
-// (stream-ordered).  An instance without a set tile gets its share of the resident warps by
-// its velocity-cells.
+// Choose the walk tiles, rebuild the work table of the active slots and upload it together with
+// every slot's descriptor (stream-ordered, one wait): the table's block counts and the captured
+// kernels follow from the same descriptors that the device reads, whatever was set on an instance
+// since the last upload.  An instance without a set tile gets its share of the resident warps by
+// its velocity-cells.  An admission changes every share, so that single descriptors uploaded one
+// by one would cost a copy and a wait per slot.
 ugks_status upload_work(ugks_batch_ctx* b) {
   BatchWork& w = b->h_work;
   double total = 0.0;
   for (ugks_ctx* h : b->ctx)
     if (h) total += (double)h->P.nx * h->P.ny * h->P.nq;
+  w.n = 0;
+  int kinds = 0, last = 0;
+  for (int p = 0; p < kPhases; p++) w.start[p][0] = 0;
   for (int s = 0; s < b->max_slots; s++) {
     const ugks_ctx* h = b->ctx[s];
     if (!h) continue;
@@ -1616,31 +1619,32 @@ ugks_status upload_work(ugks_batch_ctx* b) {
       const long warps = (long)(share * b->grid[kStrip] * kWarpsPerBlock);
       rows = auto_walk_rows(h->P, h->nchunk_neg + h->nchunk_pos, warps < 1 ? 1 : warps);
     }
-    if (rows == b->eff_rows[s]) continue;
     b->eff_rows[s] = rows;
-    const ugks_status r = upload_slot(b, s);
-    if (r) return r;
-  }
-  w.n = 0;
-  int kinds = 0;
-  for (int p = 0; p < kPhases; p++) w.start[p][0] = 0;
-  for (int s = 0; s < b->max_slots; s++) {
-    if (!b->ctx[s]) continue;
-    kinds |= instance_kind(b->ctx[s]);
-    const SlotDev S = slot_desc(b->ctx[s], b->par, b->eff_rows[s], b->walk_vtile[s]);
+    b->h_slots[s] = slot_desc(h, b->par, rows, b->walk_vtile[s]);
+    kinds |= instance_kind(h);
+    last = s + 1;
     const int a = w.n++;
     w.slot[a] = s;
     for (int p = 0; p < kPhases; p++) {
-      const long next = (long)w.start[p][a] + phase_blocks(S, p);
+      const long next = (long)w.start[p][a] + phase_blocks(b->h_slots[s], p);
       if (next > 0x7fffffffL) return bfail(b, UGKS_EINVAL, "batch too large for the work table");
       w.start[p][a + 1] = (int)next;
     }
   }
+  if (last)
+    BCK(cudaMemcpyAsync(b->d_slots, b->h_slots.data(), sizeof(SlotDev) * last, cudaMemcpyHostToDevice, b->stream));
   BCK(cudaMemcpyAsync(b->d_work, &w, sizeof(BatchWork), cudaMemcpyHostToDevice, b->stream));
-  BCK(cudaStreamSynchronize(b->stream));  // w is host memory reused by the next update
+  BCK(cudaStreamSynchronize(b->stream));  // host memory reused by the next update
   if (kinds != b->kinds && !b->persistent) drop_graphs(b);  // other kernels
   b->kinds = kinds;
   return UGKS_OK;
+}
+
+// A setting of an instance in a batch takes effect in the batch's steps.
+ugks_status upload_owner(ugks_ctx* h) {
+  if (!h->owner) return UGKS_OK;
+  const ugks_status r = upload_work(h->owner);
+  return r ? fail(h, r, h->owner->last_error) : UGKS_OK;
 }
 
 cudaError_t launch_batch(ugks_batch_ctx* b, cudaStream_t st) {
@@ -1782,6 +1786,7 @@ ugks_status ugks_batch_create(int max_slots, size_t hbm_budget, void* cuda_strea
   b->ctx.assign(max_slots, nullptr);
   b->walk_rows.assign(max_slots, 0);
   b->eff_rows.assign(max_slots, 0);
+  b->h_slots.resize(max_slots);
   b->walk_vtile.assign(max_slots, 0);
   memset(&b->h_work, 0, sizeof(BatchWork));
   cudaError_t e = cudaMalloc((void**)&b->d_slots, sizeof(SlotDev) * max_slots);
@@ -1862,7 +1867,7 @@ ugks_status ugks_batch_admit(ugks_batch b, const ugks_config* cfg, int* slot) {
     }
   b->walk_rows[s] = cls_rows;
   b->walk_vtile[s] = cls_vt;
-  b->eff_rows[s] = 0;
+  h->owner = b;
   ugks_status r = upload_work(b);
   if (r) {  // undo the admission: the caller gets no slot index to retire
     const std::string msg = b->last_error;
@@ -1939,8 +1944,7 @@ ugks_status ugks_batch_set_walk_vtile(ugks_batch b, int slot, int chunks) {
   if (!b || slot < 0 || slot >= b->max_slots || !b->ctx[slot] || chunks < 0)
     return bfail(b, UGKS_EINVAL, "bad velocity tile");
   b->walk_vtile[slot] = chunks;
-  ugks_status r = upload_slot(b, slot);
-  return r ? r : upload_work(b);
+  return upload_work(b);
 }
 
 int ugks_batch_get_walk_vtile(ugks_batch b, int slot) {
@@ -1987,7 +1991,6 @@ ugks_status ugks_batch_tune(ugks_batch b, int trial_steps, double* best_ms) {
         if (b->ctx[s] && velocity_class(b->ctx[s]->cfg) == cls) {
           b->walk_rows[s] = rows;
           b->walk_vtile[s] = vt;
-          b->eff_rows[s] = 0;
         }
       return upload_work(b);
     };
