@@ -145,8 +145,8 @@ __global__ void k_df_to_rows(const DF4* __restrict__ src, double* __restrict__ d
     double* d = dst + (size_t)c * P.nq * 2;
     for (int q = threadIdx.x; q < P.nq; q += blockDim.x) {
       const DF4 v = s[q];
-      d[2 * q] = to_double(dh(v));
-      d[2 * q + 1] = to_double(db(v));
+      d[2 * q] = f64_of_any(v.hh) + f64_of_any(v.hl);
+      d[2 * q + 1] = f64_of_any(v.bh) + f64_of_any(v.bl);
     }
   }
 }

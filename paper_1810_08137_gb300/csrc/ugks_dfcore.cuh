@@ -60,6 +60,16 @@ __device__ __forceinline__ float f32_rn(double a) {
   const bool nan = m > 0x7ff00000u || (m == 0x7ff00000u && lw != 0u);
   return __uint_as_float(fin ? (normal ? sg | rb : sg) : (sg | (nan ? 0x7fc00000u : 0x7f800000u)));
 }
+// The same with FP32 subnormals kept (f itself: on a wide velocity grid its tails pass through that
+// range): the conversion instruction there, the integer pipe everywhere else.
+__device__ __forceinline__ double f64_of_any(float x) {
+  const unsigned m = __float_as_uint(x) & 0x7fffffffu;
+  return m - 1u < 0x007fffffu ? (double)x : f64_of(x);  // 0 < m < 2^23
+}
+__device__ __forceinline__ float f32_rn_any(double a) {
+  const unsigned m = (unsigned)__double2hiint(a) & 0x7fffffffu;
+  return m - 0x36900000u < 0x01800000u ? (float)a : f32_rn(a);  // 2^-150 <= |a| < 2^-126
+}
 // FP64 -> normalised pair: the cut high part, the remainder rounded to FP32, renormalised
 // (|lo| <= ulp(hi) / 2); |a - (hi + lo)| is a few 2^-48 |a|.  The remainder a - cut(a) is
 // +-(the 29 low significand bits) 2^(E - 1075) (E the biased exponent): its FP32 rounding is
