@@ -60,6 +60,7 @@ struct ugks_ctx {
   SlotDev* d_slot = nullptr;
   BatchWork* d_work = nullptr;
   int grid1[16] = {0};       // per step kernel: blocks of its launch
+  int device = -1;                  // device current at its creation
   ugks_batch_ctx* owner = nullptr;  // batch this instance is a slot of
   double* rpart = nullptr;
   int nrblocks = 0;
@@ -438,9 +439,26 @@ __global__ void k_copy_f(Params P, double2* __restrict__ fg, double* __restrict_
   }
 }
 
+// Whether a kernel of the handle may move the caller's device rows itself: memory of the handle's own
+// device from the first byte to the last, 8-byte aligned, with that device current.  Everything else
+// (another GPU's memory, managed or host memory, odd addresses) goes through the runtime's copies,
+// which reach it or refuse it without a fault.
+bool own_rows(const ugks_ctx* h, const void* p, size_t bytes) {
+  int dev = -1;
+  cudaPointerAttributes a0, a1;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev != h->device || (reinterpret_cast<uintptr_t>(p) & 7) != 0 ||
+      cudaPointerGetAttributes(&a0, p) != cudaSuccess ||
+      cudaPointerGetAttributes(&a1, static_cast<const char*>(p) + bytes - 1) != cudaSuccess) {
+    cudaGetLastError();  // clear the error of an unknown pointer
+    return false;
+  }
+  return a0.type == cudaMemoryTypeDevice && a1.type == cudaMemoryTypeDevice && a0.device == h->device &&
+         a1.device == h->device;
+}
+
 ugks_status copy_W_in(ugks_ctx* h, const double* W, cudaMemcpyKind kind) {
   const Params& P = h->P;
-  if (kind == cudaMemcpyDeviceToDevice) {
+  if (kind == cudaMemcpyDeviceToDevice && own_rows(h, W, 4 * sizeof(double) * P.nx * P.ny)) {
     k_copy_W<<<(P.nx * P.ny + 127) / 128, 128, 0, h->stream>>>(P, h->W[h->cur], h->nwe, const_cast<double*>(W), false);
     CK(cudaGetLastError());
     return UGKS_OK;
@@ -455,7 +473,7 @@ ugks_status copy_W_in(ugks_ctx* h, const double* W, cudaMemcpyKind kind) {
 
 ugks_status copy_W_out(ugks_ctx* h, double* W, cudaMemcpyKind kind) {
   const Params& P = h->P;
-  if (kind == cudaMemcpyDeviceToDevice) {
+  if (kind == cudaMemcpyDeviceToDevice && own_rows(h, W, 4 * sizeof(double) * P.nx * P.ny)) {
     k_copy_W<<<(P.nx * P.ny + 127) / 128, 128, 0, h->stream>>>(P, h->W[h->cur], h->nwe, W, true);
     CK(cudaGetLastError());
     return UGKS_OK;
@@ -489,7 +507,7 @@ ugks_status copy_f_in(ugks_ctx* h, const double* f, bool from_host) {
   const Params& P = h->P;
   const size_t row_d = (size_t)P.nx * P.nq * 2 * sizeof(double);
   const cudaMemcpyKind kind = from_host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
-  if (h->prec == UGKS_FP64 && !from_host) {
+  if (h->prec == UGKS_FP64 && !from_host && own_rows(h, f, row_d * P.ny)) {
     k_copy_f<<<kConvBlocks, 256, 0, h->stream>>>(P, static_cast<double2*>(h->f[h->cur]), const_cast<double*>(f), false);
     CK(cudaGetLastError());
     return UGKS_OK;
@@ -544,7 +562,7 @@ ugks_status copy_f_out(ugks_ctx* h, double* f, bool to_host) {
   const Params& P = h->P;
   const size_t row_d = (size_t)P.nx * P.nq * 2 * sizeof(double);
   const cudaMemcpyKind kind = to_host ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
-  if (h->prec == UGKS_FP64 && !to_host) {
+  if (h->prec == UGKS_FP64 && !to_host && own_rows(h, f, row_d * P.ny)) {
     k_copy_f<<<kConvBlocks, 256, 0, h->stream>>>(P, static_cast<double2*>(h->f[h->cur]), f, true);
     CK(cudaGetLastError());
     return UGKS_OK;
@@ -881,6 +899,7 @@ ugks_status ugks_create(const ugks_config* cfg, void* cuda_stream, ugks_handle* 
   h->cfg = *cfg;
   h->stream = static_cast<cudaStream_t>(cuda_stream);
   h->prec = cfg->precision;
+  cudaGetDevice(&h->device);
   h->t2 = sizeof(double2);  // FP64 form (the FP32-f form stores float4 slots of two velocities)
   Params& P = h->P;
   memset(&P, 0, sizeof P);
