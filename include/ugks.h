@@ -61,8 +61,9 @@ typedef enum {
   UGKS_FP64 = 0,   /* f stored and transported in FP64, all arithmetic FP64 */
   UGKS_FP32F = 1   /* f stored and transported in FP32 as f - g_ref.  FP64 for: the
                       velocity-space moment accumulation (FP32 products summed over chunks
-                      of at most 8 rows of one warp, every sum across chunks in FP64, then
-                      the exact FP64 sums of g_ref added), the interface scalars S2-S5 (W0,
+                      of at most 8 rows of one warp, or 64 velocities of one thread; sums across
+                      chunks in FP64, a thread's own in double-FP32, 48 bits; then the exact
+                      FP64 sums of g_ref added), the interface scalars S2-S5 (W0,
                       primitive variables, half-range moments, Mt1..Mt5 including the
                       exp(-dt/tau) series at small tau, the micro-slope solves a_L, a_R, b, A,
                       the macroscopic flux), the conservative W update (Eq. 4), the cell
@@ -185,7 +186,8 @@ ugks_status ugks_set_wait_limit(ugks_handle h, long long polls);
  * would leave the kernel's resident warps under-filled (small meshes, large velocity
  * grids) and every warp keeps at least 16 velocity rows.  With 1, a mesh that fills the device
  * with tiles of 8 x 4 cells is summed with a thread per cell.  The result depends on `warps` only
- * through the order of the additions (FP64; FP32 within at most 256 terms).  UGKS_EINVAL for other values or another form.
+ * through the order of the additions (FP64 and double-FP32; FP32 within a chunk of at most 256
+ * terms).  UGKS_EINVAL for other values or another form.
  * Synchronises; the next ugks_step captures its graphs again.  On an instance of a batch it takes
  * effect in the batch's next step. */
 ugks_status ugks_set_sums_split(ugks_handle h, int warps);

@@ -1133,13 +1133,15 @@ ugks_status ugks_create(const ugks_config* cfg, void* cuda_stream, ugks_handle* 
   P.wv = h->d_grid + 2 * P.nu + P.nv;
   P.gref4 = h->gref4;
   P.grefd = h->grefd;
+  auto sp = [](double x) {  // a double-FP32 pair
+    const float hi = (float)x;
+    return make_float2(hi, (float)(x - (double)hi));
+  };
+  P.df_tdx = sp(2.0 / P.dx);
+  P.df_tdy = sp(2.0 / P.dy);
   std::vector<float2> gdf_host;
   if (dfm) {
     // u[nu], wu[nu], v[nv], [5][nv] wv v^n and the mesh constants as double-FP32 pairs
-    auto sp = [](double x) {
-      const float hi = (float)x;
-      return make_float2(hi, (float)(x - (double)hi));
-    };
     for (double x : h->hu) gdf_host.push_back(sp(x));
     for (double x : h->hwu) gdf_host.push_back(sp(x));
     for (double x : h->hv) gdf_host.push_back(sp(x));
@@ -1147,8 +1149,6 @@ ugks_status ugks_create(const ugks_config* cfg, void* cuda_stream, ugks_handle* 
       for (int m = 0; m < P.nv; m++) gdf_host.push_back(sp(h->hwv[m] * std::pow(h->hv[m], n)));
     for (double x : cell_tab) gdf_host.push_back(sp(x));
     P.gdf = h->gdf;
-    P.df_tdx = sp(2.0 / P.dx);
-    P.df_tdy = sp(2.0 / P.dy);
     P.df_idx = sp(1.0 / P.dx);
     P.df_idy = sp(1.0 / P.dy);
     P.df_dt = sp(P.dt);
@@ -1708,9 +1708,10 @@ int auto_sums_split(const Params& P, int sms) {
 }
 
 // Sums with one thread per cell (sums_tile_body) where its tiles keep the device busy: from one
-// and a half blocks per SM.  Measured, warp per cell -> thread per cell, 28^2 velocities: 100x50
-// (169 tiles) 32.6 -> 38.3 us, 120x60 (256 tiles) 45.0 -> 38.9 us, 166x83 (462, just past a wave
-// of resident blocks) 76.6 -> 69.2 us, 800x400 1430 -> 842 us; 64^2: 120x60 175 -> 159 us.
+// and a half blocks per SM.  Measured, warp per cell -> thread per cell, 28^2 velocities: 120x60
+// (256 tiles) 43.0 -> 41.0 us, 140x70 61.3 -> 51.1 us, 166x83 (462, just past a wave of resident
+// blocks) 77.2 -> 72.2 us, 800x400 1448 -> 975 us; 120x60 at 16^2 26.8 -> 22.3 us, at 37^2 101.3 -> 71.7
+// us, at 64^2 176.3 -> 151.3 us.  Below, a block has an SM to itself and its four warps do not fill it.
 bool use_sums_tiles(const Params& P, int split, int sms) {
   return !P.shk && split == 1 && 2L * tiles_x(P) * tiles_y(P) >= 3L * sms;
 }

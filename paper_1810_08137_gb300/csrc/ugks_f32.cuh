@@ -467,24 +467,28 @@ __device__ __forceinline__ void cp_async16_cg_u(uint32_t sm, const void* gm) {
 // f is staged per warp, up to 8 slots of the 8 x 4 cells and their four-sided halo at a time,
 // with asynchronous copies one stage ahead; the 144-byte pitch of a cell puts the eight cells
 // of a row in different shared-memory banks.
-// What bounds it (400x200x28^2): latency at 12 warps per SM (168 registers, of them 72 sums):
-// issue 46 %, FMA pipe 38 %, shared-memory pipe 50 %, DRAM 2.6 TB/s; 64 instructions per
-// velocity-cell against 132 of the warp-per-cell kernel.  800x400x28^2: 1.431 -> 0.843 ms.
-// Stages of 8 slots 0.926 ms, 16 warps per SM (128 registers) 0.874 ms: more data in flight per
-// SM lowers the L2 hits of the halos.
-// Precision: FP32 sums over at most kTileSeg values of u in a row pair, these over at most
-// kTileTerms velocities of one cell; everything beyond in FP64 (as the warp-per-cell kernel, whose
-// chunks hold 8 rows x 32 lanes = 256 velocities).
+// What bounds it: latency at 12 warps per SM (168 registers, of them 72 sums).  Stages of 8 slots and
+// 16 warps per SM (128 registers) were slower: more data in flight per SM lowers the L2 hits of
+// the halos.  800x400x28^2: a warp per cell 1.431 ms, this kernel 0.977 ms.
+// Precision: FP32 sums over at most kTileSeg values of u in a row, both rows of a pair added
+// first, then at most kTileTerms velocities of one cell; the sums of these chunks in double-FP32 (48
+// bits, kept in local memory), the quadrants' and all that follows in FP64.  The weights w v^n come
+// rounded once from FP64, and the factor 2/dx or 2/dy of a tangential slope is applied to the sum.
+// A chain of additions rounds more than the warp-per-cell kernel's tree of the same length, hence
+// the shorter chunks: one step's error in W against FP64 from the same f (rms over 7200 cells, rho;
+// 28^2 / 64^2 velocities): a warp per cell 2.5e-10 / 1.9e-10, chunks of 256 in FP64 3.6e-10 /
+// 3.4e-10 (0.843 ms), of 96 2.3e-10 / 1.6e-10 (0.945 ms, but above the warp-per-cell kernel on
+// [-20, 20]^2), of 64 2.1e-10 / 1.5e-10.  The chunks' sums in FP64 took 1.114 ms.
 // -------------------------------------------------------------------------------------
 constexpr int kTileX = 8, kTileY = 4;            // cells of a tile
 constexpr int kTileSlots = 4;                    // slots per stage (at most)
 constexpr int kTileStages = 2;
 constexpr int kTileSeg = 16;                     // values of u per FP32 row sum
-constexpr int kTileTerms = 256;                  // velocities per FP32 chunk
+constexpr int kTileTerms = 64;                   // velocities per FP32 chunk
 constexpr int kTilePitch = kTileSlots + 1;       // staged cell, in float4
 constexpr int kTileRow = kTileX + 2;             // staged cells per row
 constexpr int kTileStageF4 = (kTileY + 2) * kTileRow * kTilePitch;
-constexpr int kTileOut = 33;                     // doubles per face sum: 32 cells and a pad
+constexpr int kTileOut = 33;                     // double-FP32 numbers per face sum: 32 cells and a pad
 constexpr int kTileWarpBytes = kTileStages * kTileStageF4 * 16;
 static_assert(32 * kTileOut * 8 <= kTileWarpBytes, "the face sums reuse the staging buffers");
 constexpr size_t kTileSmem = (size_t)kWarpsPerBlock * kTileWarpBytes;
@@ -567,22 +571,26 @@ __device__ __forceinline__ void sums_tile_body(const Params& P, const float4* __
     cp_async_commit();
   };
 
-  // FP64 face sums of the chunks done (local memory: touched once per chunk)
-  double accl[32];
-  double* acc = accl;
+  // face sums of the chunks done, as double-FP32 pairs, two of them per float4 (local memory)
+  float4 accl[16];
+  float4* acc = accl;
   asm volatile("" : "+l"(acc));
   float o[32];
 #pragma unroll
   for (int e = 0; e < 32; e++) o[e] = 0.f;
-  int terms = 0;
-  bool first = true;
-  auto to_fp64 = [&]() {
 #pragma unroll
-    for (int e = 0; e < 32; e++) {
-      acc[e] = first ? (double)o[e] : acc[e] + (double)o[e];
-      o[e] = 0.f;
+  for (int e = 0; e < 16; e++) acc[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+  int terms = 0;
+  auto close_chunk = [&]() {
+#pragma unroll
+    for (int e = 0; e < 16; e++) {
+      const float4 t = acc[e];
+      const float2 hi = make_float2(t.x, t.y), a = make_float2(o[2 * e], o[2 * e + 1]);
+      const float2 s = add2(hi, a), bb = sub2(s, hi);  // two_sum of both
+      const float2 lo = add2(make_float2(t.z, t.w), add2(sub2(hi, sub2(s, bb)), sub2(a, bb)));
+      acc[e] = make_float4(s.x, s.y, lo.x, lo.y);
+      o[2 * e] = o[2 * e + 1] = 0.f;
     }
-    first = false;
   };
 
   copy_stage();
@@ -633,63 +641,75 @@ __device__ __forceinline__ void sums_tile_body(const Params& P, const float4* __
         c += cflip;
         cflip = -cflip;
       }
-      // the row pair's part of the 32 face sums
-      const float4 wa = __ldg(wt + 3 * pr);
-      float2 w = make_float2(wa.x, wa.y);
-      const float4 wc = __ldg(wt + 3 * pr + 2);
-      float2 v = make_float2(wc.z, wc.w);
+      // the row pair's part of the 32 face sums; the tangential slopes without their factor 2/dy or
+      // 2/dx, the energy components as (w/2) (q2 + b0) + (w v^2/2) q0
+      const float4 wa = __ldg(wt + 3 * pr), wb = __ldg(wt + 3 * pr + 1), wc = __ldg(wt + 3 * pr + 2);
+      float2 w = make_float2(wa.x, wa.y), w1 = make_float2(wa.z, wa.w), w2 = make_float2(wb.x, wb.y);
+      float2 w3 = make_float2(wb.z, wb.w);
+      const float2 v = make_float2(wc.z, wc.w);
       if (vn && pr == P.pr_neg) {  // the v = 0 row's half, nothing of its pair's other row
-        w.y = 0.f;
+        w.y = w1.y = w2.y = w3.y = 0.f;
       }
-      const float2 vv = mul2(v, v), wv = mul2(w, v), vt = mul2(v, f2(tdy));
+      const float2 vt = mul2(v, f2(tdy)), hw = mul2(f2(0.5f), w), hw1 = mul2(f2(0.5f), w1), hw2 = mul2(f2(0.5f), w2);
       const float2 sx = f2(un ? -1.f : 1.f), sy = f2(vn ? -1.f : 1.f);
-      // four face sums += g0 . x0, g1 . x1, g2 . x2, g3 . x3 (both rows)
-      auto add4s = [&](int e, float2 g0, float2 x0_, float2 g1, float2 x1_, float2 g2, float2 x2_, float2 g3,
-                       float2 x3_) {
-        o[e] = fmaf(g0.y, x0_.y, fmaf(g0.x, x0_.x, o[e]));
-        o[e + 1] = fmaf(g1.y, x1_.y, fmaf(g1.x, x1_.x, o[e + 1]));
-        o[e + 2] = fmaf(g2.y, x2_.y, fmaf(g2.x, x2_.x, o[e + 2]));
-        o[e + 3] = fmaf(g3.y, x3_.y, fmaf(g3.x, x3_.x, o[e + 3]));
-      };
-      auto en = [&](float2 q2, float2 q0, float2 b0) {  // energy component: (q2 + v^2 q0 + b0) / 2
-        return mul2(f2(0.5f), add2(fma2(vv, q0, q2), b0));
+      // face sum += g . x, or g . x + g' . x' (both rows; their sum is formed first)
+      auto put = [&](int e, float2 g, float2 x) { o[e] += fmaf(g.y, x.y, g.x * x.x); };
+      auto put2 = [&](int e, float2 g, float2 x, float2 g_, float2 x_) {
+        o[e] += fmaf(g.y, x.y, fmaf(g_.y, x_.y, fmaf(g.x, x.x, g_.x * x_.x)));
       };
       {  // x side: W0, tangential slope, Sf, Ss
         const float2 F0 = fma2(sx, X0, A0), F1 = fma2(sx, X1, A1), F2 = fma2(sx, X2, A2), F3 = fma2(sx, X3, A3);
         const float2 B0 = fma2(sx, Xb0, Ab0), B1 = fma2(sx, Xb1, Ab1);
-        add4s(kOffW0, w, F0, w, F1, wv, F0, w, en(F2, F0, B0));
-        const float2 wt_ = mul2(w, f2(tdy)), wvt = mul2(wv, f2(tdy));
-        add4s(kOffSt, wt_, Y0, wt_, Y1, wvt, Y0, wt_, en(Y2, Y0, Yb0));
-        add4s(kOffSf, w, F1, w, F2, wv, F1, w, en(F3, F1, B1));
+        put(kOffW0, w, F0); put(kOffW0 + 1, w, F1); put(kOffW0 + 2, w1, F0);
+        put2(kOffW0 + 3, hw, add2(F2, B0), hw2, F0);
+        put(kOffSt, w, Y0); put(kOffSt + 1, w, Y1); put(kOffSt + 2, w1, Y0);
+        put2(kOffSt + 3, hw, add2(Y2, Yb0), hw2, Y0);
+        put(kOffSf, w, F1); put(kOffSf + 1, w, F2); put(kOffSf + 2, w1, F1);
+        put2(kOffSf + 3, hw, add2(F3, B1), hw2, F1);
         const float2 Z1 = fma2(f2(tdx), X2, mul2(vt, Y1)), Z2 = fma2(f2(tdx), X3, mul2(vt, Y2));
         const float2 Z3 = fma2(f2(tdx), X4, mul2(vt, Y3)), Zb = fma2(f2(tdx), Xb2, mul2(vt, Yb1));
-        add4s(kOffSs, w, Z1, w, Z2, wv, Z1, w, en(Z3, Z1, Zb));
+        put(kOffSs, w, Z1); put(kOffSs + 1, w, Z2); put(kOffSs + 2, w1, Z1);
+        put2(kOffSs + 3, hw, add2(Z3, Zb), hw2, Z1);
       }
       {  // y side
         const float2 F0 = fma2(sy, Y0, A0), F1 = fma2(sy, Y1, A1), F2 = fma2(sy, Y2, A2), B0 = fma2(sy, Yb0, Ab0);
-        const float2 ef = en(F2, F0, B0), wvv = mul2(w, vv);
-        add4s(16 + kOffW0, w, F0, w, F1, wv, F0, w, ef);
-        const float2 wt_ = mul2(w, f2(tdx)), wvt = mul2(wv, f2(tdx));
-        add4s(16 + kOffSt, wt_, X0, wt_, X1, wvt, X0, wt_, en(X2, X0, Xb0));
-        add4s(16 + kOffSf, wv, F0, wv, F1, wvv, F0, wv, ef);
+        const float2 FB = add2(F2, B0), hw3 = mul2(f2(0.5f), w3);
+        put(16 + kOffW0, w, F0); put(16 + kOffW0 + 1, w, F1); put(16 + kOffW0 + 2, w1, F0);
+        put2(16 + kOffW0 + 3, hw, FB, hw2, F0);
+        put(16 + kOffSt, w, X0); put(16 + kOffSt + 1, w, X1); put(16 + kOffSt + 2, w1, X0);
+        put2(16 + kOffSt + 3, hw, add2(X2, Xb0), hw2, X0);
+        put(16 + kOffSf, w1, F0); put(16 + kOffSf + 1, w1, F1); put(16 + kOffSf + 2, w2, F0);
+        put2(16 + kOffSf + 3, hw1, FB, hw3, F0);
         const float2 D0 = fma2(f2(tdx), X1, mul2(vt, Y0)), D1 = fma2(f2(tdx), X2, mul2(vt, Y1));
         const float2 D2 = fma2(f2(tdx), X3, mul2(vt, Y2)), Db = fma2(f2(tdx), Xb1, mul2(vt, Yb0));
-        add4s(16 + kOffSs, wv, D0, wv, D1, wvv, D0, wv, en(D2, D0, Db));
+        put(16 + kOffSs, w1, D0); put(16 + kOffSs + 1, w1, D1); put(16 + kOffSs + 2, w2, D0);
+        put2(16 + kOffSs + 3, hw1, add2(D2, Db), hw3, D0);
       }
       terms += 2 * (ke - ks);
       if (terms + 2 * kTileSeg > kTileTerms) {
-        to_fp64();
+        close_chunk();
         terms = 0;
       }
     }
   }
   cp_async_wait<0>();
-  to_fp64();
+  close_chunk();
   __syncwarp();
   {
-    double* out = reinterpret_cast<double*>(st) + lane;  // [32 face sums][cell]
+    df* out = reinterpret_cast<df*>(st) + lane;  // [32 face sums][cell]
 #pragma unroll
-    for (int e = 0; e < 32; e++) out[e * kTileOut] = acc[e];
+    for (int e = 0; e < 16; e++) {
+      const float4 t = acc[e];
+      df a = {t.x, t.z}, b = {t.y, t.w};
+      const int o4 = (2 * e) & 15;
+      if (o4 >= kOffSt && o4 < kOffSt + 4) {  // the factor of the tangential slope
+        const float2 q = e < 8 ? P.df_tdy : P.df_tdx;
+        a = df_mul(a, df{q.x, q.y});
+        b = df_mul(b, df{q.x, q.y});
+      }
+      out[2 * e * kTileOut] = a;
+      out[(2 * e + 1) * kTileOut] = b;
+    }
   }
   __syncthreads();
   // the quadrants' sums of each side, added in a fixed order: thread (entry, cell parity)
@@ -702,14 +722,14 @@ __device__ __forceinline__ void sums_tile_body(const Params& P, const float4* __
     const int e = threadIdx.x & (kNSum - 1), side = e >> 4, c0 = threadIdx.x >> 6;  // sides E W N S
     const int el = (e & 15) + (side < 2 ? 0 : 16);
     const int wa = side < 2 ? side : 2 * side - 4, wb = side < 2 ? side + 2 : 2 * side - 3;
-    const double* pa = reinterpret_cast<const double*>(smem + wa * kTileWarpBytes) + el * kTileOut + c0;
-    const double* pb = reinterpret_cast<const double*>(smem + wb * kTileWarpBytes) + el * kTileOut + c0;
+    const df* pa = reinterpret_cast<const df*>(smem + wa * kTileWarpBytes) + el * kTileOut + c0;
+    const df* pb = reinterpret_cast<const df*>(smem + wb * kTileWarpBytes) + el * kTileOut + c0;
     double* row = sums + (size_t)wcell(P, x0 + c0, y0) * kNSum + e;
 #pragma unroll 1
     for (int y = 0; y < kTileY; y++) {
 #pragma unroll
       for (int x = 0; x < kTileX; x += 2)
-        if (need >> (8 * y + x + c0) & 1) row[x * kNSum] = pa[8 * y + x] + pb[8 * y + x];
+        if (need >> (8 * y + x + c0) & 1) row[x * kNSum] = to_double(df_add(pa[8 * y + x], pb[8 * y + x]));
       row += (size_t)P.wx * kNSum;
     }
   }
