@@ -54,6 +54,8 @@ struct NumF64 {
   static __device__ __forceinline__ V dt(const Params& P) { return P.dt; }
   // [nu][6]: w_u u^m (m = 0..4; half at u = 0) and u; [nv][2]: v and w_v (half at v = 0)
   static __device__ __forceinline__ const V* utab(const Params& P) { return P.mvd + 5 * P.nv; }
+  // [5][nv]: w_v v^n, each rounded once
+  static __device__ __forceinline__ const V* vpow(const Params& P) { return P.mvd; }
 };
 struct NumDF {
   using V = df;
@@ -97,6 +99,9 @@ struct NumDF {
   static __device__ __forceinline__ const V* utab(const Params& P) {
     return reinterpret_cast<const V*>(P.gdf + 2 * P.nu + 6 * P.nv);
   }
+  static __device__ __forceinline__ const V* vpow(const Params& P) {
+    return reinterpret_cast<const V*>(P.gdf + 2 * P.nu + P.nv);
+  }
 };
 
 constexpr int kCellPart = 4 * 32;  // partial sums of a cell: [quadrant][x side 16, y side 16]
@@ -116,7 +121,7 @@ __global__ void __launch_bounds__(128, 3) k_sums_cell(Params P, const typename N
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int ntx = tiles_x(P), tile = blockIdx.x >> 2, quad = blockIdx.x & 3;
   const bool un = quad & 1, vn = quad & 2;
-  const int nu = P.nu, nq = P.nq;
+  const int nu = P.nu, nv = P.nv, nq = P.nq;
   const int x0 = (tile % ntx) * kTileX - 1, y0 = (tile / ntx) * kTileY - 1;
   const int tx = lane & 7, ty = lane >> 3, i = x0 + tx, j = y0 + ty;
   const bool xg = i < 0 || i >= P.nx, yg = j < 0 || j >= P.ny;
@@ -150,6 +155,7 @@ __global__ void __launch_bounds__(128, 3) k_sums_cell(Params P, const typename N
   const int m0 = ms + nm * warp / kWarpsPerBlock, m1 = ms + nm * (warp + 1) / kWarpsPerBlock;
   const V* ut = N::utab(P);
   const V* vt = ut + 6 * nu;
+  const V* vp = N::vpow(P);
   const V tdx = N::tdx(P), tdy = N::tdy(P);
   H* slc = slopes + (size_t)wcell(P, need ? i : 0, need ? j : 0) * nq * 2;
 
@@ -225,41 +231,48 @@ __global__ void __launch_bounds__(128, 3) k_sums_cell(Params P, const typename N
     const V X0 = nx_(x0s), X1 = nx_(x1s), X2 = nx_(x2s), X3 = nx_(x34), X4 = ny_(x34);
     const V Xb0 = ny_(x0s), Xb1 = ny_(x1s), Xb2 = ny_(x2s);
     const V Y0 = nx_(y0s), Y1 = nx_(y1s), Y2 = nx_(y23), Y3 = ny_(y23), Yb0 = ny_(y0s), Yb1 = ny_(y1s);
-    const V v = vt[2 * m], w = vt[2 * m + 1];
-    const V vv = N::mul(v, v), wv = N::mul(w, v), vty = N::mul(v, tdy);
+    // tangential slopes without their factor 2/dy or 2/dx, energy components as (w/2) (q2 + b0) +
+    // (w v^2/2) q0
+    const V w = vt[2 * m + 1], w1 = vp[nv + m], w2 = vp[2 * nv + m], vty = N::mul(vt[2 * m], tdy);
+    const V hw = N::half(w), hw1 = N::half(w1), hw2 = N::half(w2), hw3 = N::half(vp[3 * nv + m]);
     auto put = [&](int e, V g, V x) { out[e * kTileOut] = N::norm(N::acc(out[e * kTileOut], g, x)); };
-    auto en = [&](V q2, V q0, V b0) { return N::half(N::add(N::mad(vv, q0, q2), b0)); };
+    auto put2 = [&](int e, V g, V x, V g_, V x_) {
+      out[e * kTileOut] = N::norm(N::acc(N::acc(out[e * kTileOut], g_, x_), g, x));
+    };
     {  // x side: W0, tangential slope, Sf, Ss
       auto F = [&](V a, V x) { return un ? N::sub(a, x) : N::add(a, x); };
       const V F0 = F(A0, X0), F1 = F(A1, X1), F2 = F(A2, X2), F3 = F(A3, X3), B0 = F(Ab0, Xb0), B1 = F(Ab1, Xb1);
-      put(kOffW0, w, F0); put(kOffW0 + 1, w, F1); put(kOffW0 + 2, wv, F0); put(kOffW0 + 3, w, en(F2, F0, B0));
-      const V wt = N::mul(w, tdy), wvt = N::mul(wv, tdy);
-      put(kOffSt, wt, Y0); put(kOffSt + 1, wt, Y1); put(kOffSt + 2, wvt, Y0); put(kOffSt + 3, wt, en(Y2, Y0, Yb0));
-      put(kOffSf, w, F1); put(kOffSf + 1, w, F2); put(kOffSf + 2, wv, F1); put(kOffSf + 3, w, en(F3, F1, B1));
+      put(kOffW0, w, F0); put(kOffW0 + 1, w, F1); put(kOffW0 + 2, w1, F0);
+      put2(kOffW0 + 3, hw, N::add(F2, B0), hw2, F0);
+      put(kOffSt, w, Y0); put(kOffSt + 1, w, Y1); put(kOffSt + 2, w1, Y0);
+      put2(kOffSt + 3, hw, N::add(Y2, Yb0), hw2, Y0);
+      put(kOffSf, w, F1); put(kOffSf + 1, w, F2); put(kOffSf + 2, w1, F1);
+      put2(kOffSf + 3, hw, N::add(F3, B1), hw2, F1);
       const V Z1 = N::mad(tdx, X2, N::mul(vty, Y1)), Z2 = N::mad(tdx, X3, N::mul(vty, Y2));
       const V Z3 = N::mad(tdx, X4, N::mul(vty, Y3)), Zb = N::mad(tdx, Xb2, N::mul(vty, Yb1));
-      put(kOffSs, w, Z1); put(kOffSs + 1, w, Z2); put(kOffSs + 2, wv, Z1); put(kOffSs + 3, w, en(Z3, Z1, Zb));
+      put(kOffSs, w, Z1); put(kOffSs + 1, w, Z2); put(kOffSs + 2, w1, Z1);
+      put2(kOffSs + 3, hw, N::add(Z3, Zb), hw2, Z1);
     }
     {  // y side
       auto F = [&](V a, V y) { return vn ? N::sub(a, y) : N::add(a, y); };
-      const V F0 = F(A0, Y0), F1 = F(A1, Y1), F2 = F(A2, Y2), B0 = F(Ab0, Yb0);
-      const V ef = en(F2, F0, B0), wvv = N::mul(w, vv);
-      put(16 + kOffW0, w, F0); put(16 + kOffW0 + 1, w, F1); put(16 + kOffW0 + 2, wv, F0); put(16 + kOffW0 + 3, w, ef);
-      const V wt = N::mul(w, tdx), wvt = N::mul(wv, tdx);
-      put(16 + kOffSt, wt, X0); put(16 + kOffSt + 1, wt, X1); put(16 + kOffSt + 2, wvt, X0);
-      put(16 + kOffSt + 3, wt, en(X2, X0, Xb0));
-      put(16 + kOffSf, wv, F0); put(16 + kOffSf + 1, wv, F1); put(16 + kOffSf + 2, wvv, F0);
-      put(16 + kOffSf + 3, wv, ef);
+      const V F0 = F(A0, Y0), F1 = F(A1, Y1), FB = N::add(F(A2, Y2), F(Ab0, Yb0));
+      put(16 + kOffW0, w, F0); put(16 + kOffW0 + 1, w, F1); put(16 + kOffW0 + 2, w1, F0);
+      put2(16 + kOffW0 + 3, hw, FB, hw2, F0);
+      put(16 + kOffSt, w, X0); put(16 + kOffSt + 1, w, X1); put(16 + kOffSt + 2, w1, X0);
+      put2(16 + kOffSt + 3, hw, N::add(X2, Xb0), hw2, X0);
+      put(16 + kOffSf, w1, F0); put(16 + kOffSf + 1, w1, F1); put(16 + kOffSf + 2, w2, F0);
+      put2(16 + kOffSf + 3, hw1, FB, hw3, F0);
       const V D0 = N::mad(tdx, X1, N::mul(vty, Y0)), D1 = N::mad(tdx, X2, N::mul(vty, Y1));
       const V D2 = N::mad(tdx, X3, N::mul(vty, Y2)), Db = N::mad(tdx, Xb1, N::mul(vty, Yb0));
-      put(16 + kOffSs, wv, D0); put(16 + kOffSs + 1, wv, D1); put(16 + kOffSs + 2, wvv, D0);
-      put(16 + kOffSs + 3, wv, en(D2, D0, Db));
+      put(16 + kOffSs, w1, D0); put(16 + kOffSs + 1, w1, D1); put(16 + kOffSs + 2, w2, D0);
+      put2(16 + kOffSs + 3, hw1, N::add(D2, Db), hw3, D0);
     }
   }
   cp_async_wait<0>();
   const unsigned ok = __ballot_sync(kFull, need);
   __syncthreads();
   // the warps' sums, added in order: each warp writes eight cells, lane = entry
+  const double scale = (lane & 12) != kOffSt ? 1.0 : lane < 16 ? P.d_tdy : P.d_tdx;
   const unsigned char* all = cell_sm + kTileStages * kTileStageF4 * 16 + sizeof(V) * lane * kTileOut;
 #pragma unroll 1
   for (int t = 8 * warp; t < 8 * warp + 8; t++)
@@ -268,6 +281,7 @@ __global__ void __launch_bounds__(128, 3) k_sums_cell(Params P, const typename N
 #pragma unroll
       for (int w = 0; w < kWarpsPerBlock; w++)
         r += N::f64(reinterpret_cast<const V*>(all + w * kCellSumsWarp)[t]);
+      r *= scale;
       part[(size_t)wcell(P, x0 + (t & 7), y0 + (t >> 3)) * kCellPart + quad * 32 + lane] = r;
     }
 }
