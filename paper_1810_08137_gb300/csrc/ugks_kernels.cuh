@@ -541,8 +541,9 @@ __global__ void __launch_bounds__(128) k_sums(Params P, const T2* __restrict__ f
 }
 
 // -------------------------------------------------------------------------------------
-// Steps S2-S5 per interface, plus the coefficients of S6/S8 for the update kernel: all FP64
-// in the FP64 form; first-order terms FP64 and slope-carrying terms FP32 in the FP32-f form.
+// Steps S2-S5 per interface, plus the coefficients of S6/S8 for the update kernel: all FP64 in the
+// FP64 form; FP64 and double-FP32 in the others (face_core), whose records are rounded to FP32
+// (FP32-f form) or to double-FP32 (DF64 form).
 // -------------------------------------------------------------------------------------
 
 // Central half-range moments m_n = <x^n>, x = u - U, n = 0..6, of the normalised 1D Gaussian
@@ -751,9 +752,9 @@ __device__ __forceinline__ void wall_face_f32(const Params& P, bool isx, double 
 // Arithmetic: the primitive variables, exp and erfc of the half-range moments, tau and
 // Mt1..Mt5, the slope targets and the free-transport part of F in FP64; the moment
 // recurrences, the micro-slope solves, the compatibility moments and the equilibrium part of
-// F in T (in the frame that moves with the interface): double (FP64 form) or dd, double-FP32 on the FP32 pipe (FP32-f and DF64 forms,
-// about 2^-48 relative per operation, where FP64 would spend ~420 of its ~610 operations per
-// face on the 1/64-rate FP64 pipe).
+// F in T (in the frame that moves with the interface): double (FP64 form) or dd, double-FP32 on
+// the FP32 pipe (FP32-f and DF64 forms: about 310 operations per face, each good to about 2^-48, off
+// the 1/64-rate FP64 pipe).
 template <typename T>
 struct FaceCoreT {
   double rho, U, V, lam, X2, X4;
@@ -818,7 +819,7 @@ __device__ __forceinline__ void face_core(const Params& P, const double* W0, con
   time_weights(P.dt, x, c.Mt);
   const double* Mt = c.Mt;
   // S4: micro slopes a_L, a_R (normal), b (tangential), on psi' of the moving frame
-  const T irhot = T(irho), invt = irhot * T(tdelta);
+  const double inv = irho * tdelta;  // the slope targets are FP64 products, rounded to T once
   const T Ut = T(U), Vt = T(V), ht = T(h), ke = halved(Ut * Ut + Vt * Vt);
   const T q = scaled(halved(ht), K + 2), k1h = scaled(ht, K + 1), il = T(2.0 * lam);
   const T c8 = T(8.0 * lam * lam * P.inv_kp2);
@@ -829,7 +830,7 @@ __device__ __forceinline__ void face_core(const Params& P, const double* W0, con
   for (int sd = 0; sd < 2; sd++) {
     T s[4], m[7], a[4];
 #pragma unroll
-    for (int k = 0; k < 4; k++) s[k] = T(sd == 0 ? W0[k] - WL[k] : WR[k] - W0[k]) * invt;
+    for (int k = 0; k < 4; k++) s[k] = T((sd == 0 ? W0[k] - WL[k] : WR[k] - W0[k]) * inv);
     to_moving<T>(Ut, Vt, ke, s);
     micro_slope<T>(q, il, c8, s, a);
     gauss_central7<T>(Ut, ht, T(sd == 0 ? mp0 : mn0), T(sd == 0 ? e : -e), m);
@@ -849,7 +850,7 @@ __device__ __forceinline__ void face_core(const Params& P, const double* W0, con
     // ut = V + y, over the full range
     T s[4];
 #pragma unroll
-    for (int k = 0; k < 4; k++) s[k] = T(St[k]) * irhot;
+    for (int k = 0; k < 4; k++) s[k] = T(St[k] * irho);
     to_moving<T>(Ut, Vt, ke, s);
     micro_slope<T>(q, il, c8, s, c.b);
     const T y2 = ht * mad(c.b[3], ht, s[0]);  // <y^2 (b . psi')> = <x^2 (b . psi')>
