@@ -184,9 +184,11 @@ std::pair<int, int> f32_row_pairs(int nv, double vmin, double vmax) {
   return {pn, pn + (nv - mneg + 1) / 2};
 }
 
-// Threads per block of the interface and cell kernels (one thread per face or cell): one warp
-// where whole blocks would leave SMs idle (152 SMs), since their FP64 chains are bound by one SM's
-// FP64 pipe (2 operations per clock).  40x20 cells 14.9 -> 12.8 us.
+// Threads per block of the interface and cell kernels (one thread per face or cell) for n faces or
+// cells in a launch: one warp where whole blocks would leave SMs of a GB300 (152) idle, since their FP64
+// chains are bound by one SM's FP64 pipe (2 operations per clock).  40x20 cells 14.9 -> 12.8 us.  The
+// cell blocks fix the order in which a residual is added up and the device bytes of an instance, so
+// they depend on the instance alone, not on the device; a face's result does not depend on its block.
 int small_block(long n) { return n < 152 * 128 ? 32 : 128; }
 
 // Velocity sums per cell: the FP64 and DF64 forms' BGK sums kernel keeps its four quadrants apart (the
@@ -1624,8 +1626,16 @@ int auto_walk_rows(const Params& P, int nchunk, long warps) {
 ugks_status upload_work(ugks_batch_ctx* b) {
   BatchWork& w = b->h_work;
   double total = 0.0;
+  long faces = 0;
   for (ugks_ctx* h : b->ctx)
-    if (h) total += (double)h->P.nx * h->P.ny * h->P.nq;
+    if (h) {
+      total += (double)h->P.nx * h->P.ny * h->P.nq;
+      faces += (long)(h->P.nx + 1) * h->P.ny + (long)h->P.nx * (h->P.ny + 1);
+    }
+  // the faces per block follow from all instances' faces: a batch's blocks have four warps, and with
+  // one of them at work 64 serving requests took 625 us a step instead of 599, 16 uneven instances
+  // 4.18 ms instead of 4.13 (12 requests, below the line, 156 us instead of 162)
+  const int face_block = small_block(faces);
   w.n = 0;
   int kinds = 0, last = 0;
   for (int p = 0; p < kPhases; p++) w.start[p][0] = 0;
@@ -1640,6 +1650,7 @@ ugks_status upload_work(ugks_batch_ctx* b) {
     }
     b->eff_rows[s] = rows;
     b->h_slots[s] = slot_desc(h, b->par, rows, b->walk_vtile[s]);
+    b->h_slots[s].face_block = face_block;
     kinds |= instance_kind(h);
     last = s + 1;
     const int a = w.n++;

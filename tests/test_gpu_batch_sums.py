@@ -109,3 +109,22 @@ def test_sums_set_on_an_instance_of_a_batch(U, persistent):
         B.step(2)
         B.sync()
         check(B, sa, alone(U, a, pa, 2))
+
+
+@pytest.mark.parametrize("persistent", [True, False])
+def test_interface_blocks_follow_the_batch_not_the_result(U, persistent):
+    """Two instances of 15937 faces: blocks of 32 faces alone, of 128 together (past 152 x 128
+    faces), and back to 32 when one leaves."""
+    cfg = tiled()
+    prims = [prim_of(cfg, 30 + k) for k in range(2)]
+    with U.Batch(2) as B:
+        B.set_persistent(persistent)
+        slots = [B.admit(cfg), B.admit(cfg)]
+        for s, p in zip(slots, prims):
+            B.instance(s).init_maxwellian(*p)
+        B.step(3)
+        check(B, slots[1], alone(U, cfg, prims[1], 3))
+        B.retire(slots[1])
+        B.step(2)
+        B.sync()
+        check(B, slots[0], alone(U, cfg, prims[0], 5))
