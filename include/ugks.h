@@ -215,7 +215,8 @@ ugks_status ugks_residual(ugks_handle h, double res[4]);
  * stream around each of its kernels; enable == 0 stops recording and discards the
  * records.  ugks_kernel_times synchronises and returns, per kernel of the step (order:
  * ugks_kernel_name(0..UGKS_NKERNELS-1)), the launches recorded and their total device
- * time in ms.  ms and launches must hold UGKS_NKERNELS entries (either may be NULL). */
+ * time in ms.  ms and launches must hold UGKS_NKERNELS entries (either may be NULL).  The ghost
+ * ring is one launch and counts as "ghost_x"; "ghost_y" keeps its entry, with no launch and no time. */
 #define UGKS_NKERNELS 6
 ugks_status ugks_profile(ugks_handle h, int enable);
 ugks_status ugks_kernel_times(ugks_handle h, double* ms, long* launches);

@@ -513,20 +513,17 @@ __device__ __forceinline__ void sums_tile_body(const Params& P, const float4* __
   const int own = ((ty + 1) * kTileRow + tx + 1) * kTilePitch;
   const int ox = zs ? 0 : kTilePitch, oy = zs ? 0 : kTileRow * kTilePitch;
 
-  // staging: lane (column lane / kTileSlots, slot lane % kTileSlots) copies every LC-th column of
-  // each of the 6 rows and its share of the left and right halo cells; rows and columns past the
-  // ghost ring repeat its last one
-  constexpr int LC = 32 / kTileSlots, NP = kTileX / LC;
-  const int sl = lane % kTileSlots, lc = lane / kTileSlots;
+  // staging: lane (column lane / 4, slot lane % 4) copies its column of the 6 rows and one halo cell;
+  // rows and columns past the ghost ring repeat its last one
+  static_assert(kTileSlots == 4 && kTileX == 8, "one column of the tile per 4 lanes");
+  const int sl = lane & 3, lc = lane >> 2;
   const size_t rs = (size_t)P.ex * fs;
   const int xlast = P.nx + 1, yspan = P.ny + 2 - y0;  // last row the tile may read: y0 - 1 + yspan
-  const int hx = lc < LC / 2 ? x0 - 1 : min(x0 + kTileX, xlast), hr = lc % (LC / 2);
+  const int hx = lc < 4 ? x0 - 1 : min(x0 + kTileX, xlast), hr = lc & 3;
   const float4* gcol = f + ((size_t)(y0 + 1) * P.ex + min(x0 + lc, xlast) + 2) * fs + sl;  // row y0 - 1
   const float4* ghal = f + ((size_t)(min(y0 + hr, P.ny + 1) + 2) * P.ex + hx + 2) * fs + sl;
-  const int dcol2 = (min(x0 + lc + LC, xlast) - min(x0 + lc, xlast)) * fs;
-  const size_t dhal2 = (size_t)(min(y0 + hr + 2, P.ny + 1) - min(y0 + hr, P.ny + 1)) * rs;
   const uint32_t dcol = smem_addr(st + (1 + lc) * kTilePitch + sl);
-  const uint32_t dhal = smem_addr(st + ((1 + hr) * kTileRow + (lc < LC / 2 ? 0 : kTileX + 1)) * kTilePitch + sl);
+  const uint32_t dhal = smem_addr(st + ((1 + hr) * kTileRow + (lc < 4 ? 0 : kTileX + 1)) * kTilePitch + sl);
 
   // u columns of the quadrant (u = 0 in both), in segments of kTileSeg; row pairs of the
   // quadrant (for v <= 0 also the pair of the v = 0 row, with its other row at zero weight)
@@ -550,12 +547,10 @@ __device__ __forceinline__ void sums_tile_body(const Params& P, const float4* __
 #pragma unroll
         for (int r = 0; r < kTileY + 2; r++) {
           cp_async16_cg_u(d, g);
-          if (NP == 2) cp_async16_cg_u(d + LC * kTilePitch * 16, g + dcol2);
           d += kTileRow * kTilePitch * 16;
           if (r < yspan) g += rs;
         }
         cp_async16_cg_u(dhal + pslot, ghal + s0);
-        if (NP == 2) cp_async16_cg_u(dhal + pslot + 2 * kTileRow * kTilePitch * 16, ghal + s0 + dhal2);
       }
       pk += n;
       if (pk >= pend) {
