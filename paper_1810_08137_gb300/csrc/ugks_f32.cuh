@@ -90,8 +90,7 @@ __device__ __forceinline__ void ghost_body_f32(const Params& P, float4* f, doubl
       const int m0 = prow(P, 2 * pr), m1 = prow(P, 2 * pr + 1);
       const double2 r0 = P.grefd[m0 * P.nu + k], r1 = P.grefd[m1 * P.nu + k];
       const double g0 = tab[k] * tab[kMaxAxis + m0], g1 = tab[k] * tab[kMaxAxis + m1];
-      dst[s] = make_float4(f32_rn_any(g0 - r0.x), f32_rn_any(g1 - r1.x), f32_rn_any(fma(bf, g0, -r0.y)),
-                           f32_rn_any(fma(bf, g1, -r1.y)));
+      dst[s] = f32x4_rn_any(g0 - r0.x, g1 - r1.x, fma(bf, g0, -r0.y), fma(bf, g1, -r1.y));
     }
   }
 }
@@ -1161,8 +1160,7 @@ __global__ void k_rows_to_f32(const double* __restrict__ src, float4* __restrict
         b = make_double2(row[2 * q1], row[2 * q1 + 1]);
       }
       const double2 g0 = grefd[q0], g1 = grefd[q1];
-      d[s] = make_float4(f32_rn_any(a.x - g0.x), f32_rn_any(b.x - g1.x), f32_rn_any(a.y - g0.y),
-                         f32_rn_any(b.y - g1.y));
+      d[s] = f32x4_rn_any(a.x - g0.x, b.x - g1.x, a.y - g0.y, b.y - g1.y);
     }
   }
 }
