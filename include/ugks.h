@@ -61,7 +61,7 @@ typedef enum {
   UGKS_FP64 = 0,   /* f stored and transported in FP64, all arithmetic FP64 */
   UGKS_FP32F = 1   /* f stored and transported in FP32 as f - g_ref.  FP64 for: the
                       velocity-space moment accumulation (FP32 products summed over chunks
-                      of at most 8 rows of one warp, or 64 velocities of one thread; sums across
+                      of at most 8 rows of one warp, or 90 velocities of one thread; sums across
                       chunks in FP64, a thread's own in double-FP32, 48 bits; then the exact
                       FP64 sums of g_ref added), the interface scalars S2-S5 (W0,
                       primitive variables, half-range moments, Mt1..Mt5 including the

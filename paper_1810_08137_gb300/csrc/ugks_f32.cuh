@@ -466,24 +466,27 @@ __device__ __forceinline__ void cp_async16_cg_u(uint32_t sm, const void* gm) {
 // f is staged per warp, up to 8 slots of the 8 x 4 cells and their four-sided halo at a time,
 // with asynchronous copies one stage ahead; the 144-byte pitch of a cell puts the eight cells
 // of a row in different shared-memory banks.
-// What bounds it: latency at 12 warps per SM (168 registers, of them 72 sums).  Stages of 8 slots and
-// 16 warps per SM (128 registers) were slower: more data in flight per SM lowers the L2 hits of
-// the halos.  800x400x28^2: a warp per cell 1.431 ms, this kernel 0.977 ms.
+// What bounds it (400x200x28^2): latency at 12 warps per SM (168 registers, of them 72 sums): issue 47 %,
+// FMA pipe 37 %; 74 instructions per velocity-cell against 132 of the warp-per-cell kernel.  Stages
+// of 8 slots and 16 warps per SM (128 registers) were slower: more data in flight per SM lowers the
+// L2 hits of the halos.  800x400x28^2: a warp per cell 1.431 ms, this kernel 0.945 ms.
 // Precision: FP32 sums over at most kTileSeg values of u in a row, both rows of a pair added
-// first, then at most kTileTerms velocities of one cell; the sums of these chunks in double-FP32 (48
-// bits, kept in local memory), the quadrants' and all that follows in FP64.  The weights w v^n come
-// rounded once from FP64, and the factor 2/dx or 2/dy of a tangential slope is applied to the sum.
-// A chain of additions rounds more than the warp-per-cell kernel's tree of the same length, hence
-// the shorter chunks: one step's error in W against FP64 from the same f (rms over 7200 cells, rho;
-// 28^2 / 64^2 velocities): a warp per cell 2.5e-10 / 1.9e-10, chunks of 256 in FP64 3.6e-10 /
-// 3.4e-10 (0.843 ms), of 96 2.3e-10 / 1.6e-10 (0.945 ms, but above the warp-per-cell kernel on
-// [-20, 20]^2), of 64 2.1e-10 / 1.5e-10.  The chunks' sums in FP64 took 1.114 ms.
+// first, then over at most kTilePairs pairs and kTileTerms velocities of one cell; the sums of these
+// chunks in double-FP32 (48 bits, kept in local memory), the quadrants' and all that follows in
+// FP64.  The weights w v^n come rounded once from FP64, and the factor 2/dx or 2/dy of a tangential
+// slope is applied to the sum.  A chain of additions rounds more than the warp-per-cell kernel's
+// tree of the same length, hence the shorter chunks: one step's error in W against FP64 from the same
+// f (rms over 7200 cells, rho; 28^2, 64^2 velocities on [-4, 4]^2, 51^2 on [-20, 20]^2): a warp per
+// cell 2.5e-10, 1.9e-10, 1.27e-11; chunks of 256 in FP64 3.6e-10, 3.4e-10, 1.44e-11 (0.843 ms); of 96
+// 2.3e-10, 1.6e-10, 1.28e-11; as here 2.3e-10, 1.5e-10, 1.22e-11; of 64 2.1e-10, 1.5e-10, 1.18e-11
+// (0.975 ms).  Without the limit on pairs the narrow last segment of 40 values of u adds 11 pairs in a
+// row, 2 % above the warp-per-cell kernel.  The chunks' sums in FP64 took 1.11 ms at 64 terms.
 // -------------------------------------------------------------------------------------
 constexpr int kTileX = 8, kTileY = 4;            // cells of a tile
 constexpr int kTileSlots = 4;                    // slots per stage (at most)
 constexpr int kTileStages = 2;
 constexpr int kTileSeg = 16;                     // values of u per FP32 row sum
-constexpr int kTileTerms = 64;                   // velocities per FP32 chunk
+constexpr int kTileTerms = 90, kTilePairs = 4;   // velocities and row pairs per FP32 chunk (at most)
 constexpr int kTilePitch = kTileSlots + 1;       // staged cell, in float4
 constexpr int kTileRow = kTileX + 2;             // staged cells per row
 constexpr int kTileStageF4 = (kTileY + 2) * kTileRow * kTilePitch;
@@ -574,7 +577,7 @@ __device__ __forceinline__ void sums_tile_body(const Params& P, const float4* __
   for (int e = 0; e < 32; e++) o[e] = 0.f;
 #pragma unroll
   for (int e = 0; e < 16; e++) acc[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-  int terms = 0;
+  int terms = 0, pairs = 0;
   auto close_chunk = [&]() {
 #pragma unroll
     for (int e = 0; e < 16; e++) {
@@ -680,9 +683,9 @@ __device__ __forceinline__ void sums_tile_body(const Params& P, const float4* __
         put2(16 + kOffSs + 3, hw1, add2(D2, Db), hw3, D0);
       }
       terms += 2 * (ke - ks);
-      if (terms + 2 * kTileSeg > kTileTerms) {
+      if (++pairs == kTilePairs || terms + 2 * (ke - ks) > kTileTerms) {
         close_chunk();
-        terms = 0;
+        terms = pairs = 0;
       }
     }
   }
