@@ -44,18 +44,16 @@ def peaks():
         return 6800.0, "fallback"
 
 
-# FP64 form: FP64 flops per velocity-cell as executed (FMA = 2 flops), from the ncu
-# instruction counts of its kernels (DFMA, DMUL, DADD per velocity-cell; the capture in
-# profiles/fp64_step_kernels_channel_200x100_v28.md): the update's two passes
-# 2 x 37.9 + 12.9 + 7.4, the sums kernel 2 x 38.1 + 10.3 + 15.7.  The peak is measured
-# in the run (ugks_fp64_rate: chains of FP64 FMAs on every SM).
-FP64_UPDATE_FLOPS_PER_VC = 2 * 37.9 + 12.9 + 7.4
-FP64_SUMS_FLOPS_PER_VC = 2 * 38.1 + 10.3 + 15.7
-# DRAM traffic of the FP32-f update kernel per velocity-cell (read + write), from the ncu
-# capture of the current kernel summarised in profiles/fp32f_step_kernels_channel_400x200_v28.md
+# FP64 form: FP64 flops per velocity-cell as executed (FMA = 2 flops), from the instruction
+# counts that ncu reports for its kernels at 200x100x28^2 (DFMA, DMUL, DADD per velocity-cell): the
+# update's two passes 2 x 37.9 + 12.6 + 9.3, the sums kernel 2 x 38.2 + 9.7 + 15.7.  The peak is
+# measured in the run (ugks_fp64_rate: chains of FP64 FMAs on every SM).
+FP64_UPDATE_FLOPS_PER_VC = 2 * 37.9 + 12.6 + 9.3
+FP64_SUMS_FLOPS_PER_VC = 2 * 38.2 + 9.7 + 15.7
+# DRAM traffic of the FP32-f update kernel per velocity-cell (read + write), from an ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum of one kb_strip launch at 400x200x28^2);
 # set to None when the kernel changes until it is captured again.
-UPDATE_TRAFFIC_PER_VC = (597.178624e6 + 464.608768e6) / 62.72e6
+UPDATE_TRAFFIC_PER_VC = (596.786176e6 + 464.153856e6) / 62.72e6
 # FP32 lane operations of the FP32-f update kernel per velocity-cell on the FMA pipe (a packed
 # pair instruction = 2), from the same capture's instruction mix: FFMA2 43.4, FMUL2 15.0,
 # FADD2 6.6, FFMA 5.0, FADD 3.4, FMUL 1.4 per velocity-cell; the peak is the FMA pipe's
@@ -594,7 +592,7 @@ def main():
         "metric": METRIC, "value": main["value"], "unit": UNIT, "n_gpus": ws,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": main["ms_per_step"],
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-        "dtype": "f32 (f) + f64 (velocity sums across f32 chunks, W, cell scalars) + f64/double-f32 (interface scalars)" if main_prec == ugks.FP32F else "f64",
+        "dtype": "f32 (f) + f64 (W, cell scalars) + f64/double-f32 (velocity sums across f32 chunks, interface scalars)" if main_prec == ugks.FP32F else "f64",
         "data": "synthetic",
         "config": {"workload": cfg.name, "cells": cfg.nc, "velocities": cfg.nq,
                    "vc_per_step": cfg.vc, "kn": cfg.kn, "precision": args.prec,

@@ -240,9 +240,11 @@ ugks_status ugks_fp64_rate(void* cuda_stream, double* gflops);
  * grid-wide barrier between them; ugks_batch_set_persistent(b, 0) selects one launch per
  * phase instead (the same phase code and order of work).  Instances are admitted into free
  * slots while the batch is in use (admission checks an HBM budget) and retired when done; the
- * table and each instance's ping-pong parity live in device memory, so admission and retirement
- * change data, not the captured graphs.  Each instance's results are bitwise those of the same
- * instance stepped alone with ugks_step (same kernels, same order of work). */
+ * table and each instance's descriptor live in device memory, so admission and retirement change
+ * data and the captured graphs stay.  With one launch per phase the step is captured again when the
+ * kinds of instance present change (sums with a thread per cell, with a warp per cell, Shakhov): each
+ * kind has kernels of its own.  Each instance's results are bitwise those of the same instance
+ * stepped alone with ugks_step (same kernels, same order of work). */
 typedef struct ugks_batch_ctx* ugks_batch;
 
 /* max_slots <= 256 instances at a time; hbm_budget: total state bytes of the admitted
@@ -287,8 +289,9 @@ int         ugks_batch_get_persistent(ugks_batch b);
 ugks_status ugks_batch_set_wait_limit(ugks_batch b, unsigned long long polls);
 
 /* Tile shape of the f-update walk for one slot: the cell tile (rows per tile, chosen by the
- * library from the instances in flight until it is set or tuned; a tile is 4 columns wide) and the velocity tile (chunks of 32 velocity slots walked by consecutive
- * warps for the same cell tile; 0 = all chunks of the cell).  The autotuner: for each
+ * library from the instances in flight until it is set or tuned; a tile is 4 columns wide) and
+ * the velocity tile (chunks of 32 velocity slots walked by consecutive warps for the same cell
+ * tile; 0 = all chunks of the cell).  The autotuner: for each
  * velocity-grid class present (nu*nv <= 576, <= 1600, <= 4096, larger) it times
  * trial_steps batch steps for every cell tile of 16, 32, 64, 128 rows times velocity tile
  * of all, 2 and 1 chunks, and keeps the fastest for that class; then it times the step

@@ -1723,9 +1723,9 @@ int auto_sums_split(const Params& P, int sms) {
 
 // Sums with one thread per cell (sums_tile_body) where its tiles keep the device busy: from one
 // and a half blocks per SM.  Measured, warp per cell -> thread per cell, 28^2 velocities: 120x60
-// (256 tiles) 43.0 -> 41.0 us, 140x70 61.3 -> 51.1 us, 166x83 (462, just past a wave of resident
-// blocks) 77.2 -> 72.2 us, 800x400 1448 -> 975 us; 120x60 at 16^2 26.8 -> 22.3 us, at 37^2 101.3 -> 71.7
-// us, at 64^2 176.3 -> 151.3 us.  Below, a block has an SM to itself and its four warps do not fill it.
+// (256 tiles) 42.9 -> 40.8 us, 140x70 60.8 -> 49.5 us, 166x83 (462, just past a wave of resident
+// blocks) 77.3 -> 71.6 us, 800x400 1456 -> 947 us; 120x60 at 16^2 26.8 -> 22.2 us, at 37^2 100.8 -> 72.6
+// us, at 64^2 175.9 -> 151.4 us.  Below, a block has an SM to itself and its four warps do not fill it.
 bool use_sums_tiles(const Params& P, int split, int sms) {
   return !P.shk && split == 1 && 2L * tiles_x(P) * tiles_y(P) >= 3L * sms;
 }

@@ -2,9 +2,9 @@
 // step runs once per step for all active instances, as a persistent grid that walks a
 // device-resident work table of virtual blocks.  The step is either one cooperative launch
 // of kb_step (all phases, grid barriers with bounded waits between them) or the phase
-// launches; either way one CUDA graph replay.  The table (and each instance's ping-pong
-// parity) lives in device memory, so admitting or retiring an instance changes data, not
-// the captured graph.
+// launches; either way one CUDA graph replay.  The table and the descriptors live in device memory,
+// so admitting or retiring an instance changes data; only the phase launches are captured again, when
+// the kinds of instance present (and with them the kernels) change.
 // Included by ugks.cu (same translation unit as the single-instance kernels).
 #pragma once
 
@@ -32,7 +32,7 @@ struct SlotDev {
   int walk_vtile;  // velocity tile of the walk: 32-slot chunks per tile, 0 = all (autotuned)
   int sums_split;  // warps per cell in the sums phase (1, 2 or 4): velocity-space split
   int sums_tiled;  // sums with one thread per cell (sums_tile_body)
-  int face_block;  // faces per virtual block (32 spreads a small mesh over more SMs)
+  int face_block;  // faces per virtual block (32 spreads few faces over more SMs)
   int cell_block;  // cells per virtual block
   int cur;         // ping-pong parity in even steps: a step of parity par reads f[cur ^ par]
 };
@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(128, 3) kb_sums_tile(const SlotDev* __restrict
   sums_tile_phase(slots, wk, par, tile_sm);
 }
 
-// six blocks per SM (80 registers, the rest on the stack): bound by the FP64 pipe (about 200 FP64
+// six blocks per SM (80 registers, the rest on the stack): bound by the FP64 pipe (186 FP64
 // instructions per face at 1/64 of the FP32 rate) and the latency of its FP64 and double-FP32
 // chains.  800x400x28^2 0.298 ms, 200x100 45 us (8 blocks 0.306 ms and 48 us, 4 blocks 0.334 ms and
 // 43 us).

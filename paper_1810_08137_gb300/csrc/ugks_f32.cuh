@@ -466,8 +466,8 @@ __device__ __forceinline__ void cp_async16_cg_u(uint32_t sm, const void* gm) {
 // f is staged per warp, up to 8 slots of the 8 x 4 cells and their four-sided halo at a time,
 // with asynchronous copies one stage ahead; the 144-byte pitch of a cell puts the eight cells
 // of a row in different shared-memory banks.
-// What bounds it (400x200x28^2): latency at 12 warps per SM (168 registers, of them 72 sums): issue 47 %,
-// FMA pipe 37 %; 74 instructions per velocity-cell against 132 of the warp-per-cell kernel.  Stages
+// What bounds it (400x200x28^2): latency at 12 warps per SM (168 registers, of them 72 sums): issue 48 %,
+// FMA pipe 38 %; 73 instructions per velocity-cell against 132 of the warp-per-cell kernel.  Stages
 // of 8 slots and 16 warps per SM (128 registers) were slower: more data in flight per SM lowers the
 // L2 hits of the halos.  800x400x28^2: a warp per cell 1.431 ms, this kernel 0.945 ms.
 // Precision: FP32 sums over at most kTileSeg values of u in a row, both rows of a pair added

@@ -5,9 +5,11 @@
 // 8 x 4 cells (lane = cell) and one quadrant of velocity space, so it feeds one x side and one y
 // side; its four warps take a share of the quadrant's rows each, and the interface kernel adds the
 // two quadrants of a side.  Bound by arithmetic: FP64 64 pipe instructions per velocity-cell, the
-// pipe 89 % busy (100x50x28^2 624 -> 517 us against a warp per cell); DF64 by FP32 issue, so h and b,
-// or two powers of u, go through packed pairs (200x100x28^2 538 -> 409 -> 363 us, 60x30x101^2 712 ->
-// 559 -> 501 us: a warp per cell, a thread per cell, packed pairs).
+// pipe 90 % busy (100x50x28^2 624 -> 512 us against a warp per cell); DF64 by the FMA pipe (64 %) and
+// FP32 issue (55 %), so h and b, or two powers of u, go through packed pairs (200x100x28^2 538 -> 409 ->
+// 369 us, 60x30x101^2 712 -> 559 -> 508 us: a warp per cell, a thread per cell, packed pairs).  The
+// weights w v^n are those rounded once (formed from rounded v and w they put 13 % more error on rho V
+// than on rho U of the transposed flow).
 #pragma once
 
 namespace ugks {
@@ -301,10 +303,10 @@ __global__ void __launch_bounds__(128, 3) k_sums_cell(Params P, const typename N
 // alone comes from tables in shared memory (one kind per warp), so a velocity-cell costs 28 FP64
 // instructions for its two faces: per face 3 for Q_h, 2 for Q_b = X2 Q_h + linear, 1 for g and 4 per
 // component, with f_up and d_up folded into the coefficients of the cell value and its two half
-// slopes (67 before), 36 with the tables; k_cell_update 18 (22 with tables, 30 before).  A block per
+// slopes (67 before), 36 with the tables; k_cell_update 20 (24 with tables, 30 before).  A block per
 // cell shares the tables and spreads small meshes evenly.  Both passes, FP64: 100x50x28^2 0.820 ->
-// 0.433 ms (a warp per cell 0.518), 40x20x20^2 163 -> 70 us (90); FP64 pipe 89 % busy.  DF64:
-// 200x100x28^2 815 -> 569 us, 60x30x101^2 1478 -> 728 us (1125).
+// 0.447 ms (a warp per cell 0.518), 40x20x20^2 163 -> 70 us (90); FP64 pipe 94 % and 86 % busy.  DF64:
+// 200x100x28^2 815 -> 573 us, 60x30x101^2 1478 -> 728 us (1125).
 // -------------------------------------------------------------------------------------
 // Q at fixed u as a polynomial in v, from a record's eight coefficients: x face (un = u, ut = v) or
 // y face (un = v, ut = u).
