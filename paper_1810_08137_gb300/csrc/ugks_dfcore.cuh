@@ -62,23 +62,35 @@ __device__ __forceinline__ float f32_rn(double a) {
 }
 // The same with FP32 subnormals kept (f itself: on a wide velocity grid its tails pass through that
 // range).  To FP64: a subnormal is scaled by 2^64 on the FP32 pipe and the exponent taken back.  To
-// FP32: the conversion instruction for the few values that need it, in a function of its own, for a plain
-// cast under an `if` becomes a conversion of every value on the FP64 pipe and a select (800x400x28^2:
-// state out 2.1 ms against 1.16 ms, in 2.25 ms against 1.18 ms).
+// FP32: the 53-bit significand shifted to units of 2^-149 and rounded to nearest, ties to even, on the
+// integer pipe.  (A plain cast under an `if` becomes a conversion of every value on the FP64 pipe and a
+// select: 800x400x28^2 state out 2.1 ms against 1.16 ms, in 2.25 ms against 1.18 ms.)
 __device__ __forceinline__ double f64_of_any(float x) {
   const bool sub = (__float_as_uint(x) & 0x7f800000u) == 0u;
   const double d = f64_of(sub ? __fmul_rn(x, 0x1p64f) : x);
   return sub && x != 0.f ? __hiloint2double(__double2hiint(d) - (64 << 20), __double2loint(d)) : d;
 }
-__device__ __noinline__ float4 f32x4_cvt(double a, double b, double c, double d) {
-  return make_float4((float)a, (float)b, (float)c, (float)d);
+__device__ __forceinline__ bool to_f32_subnormal(double a) {  // 2^-150 <= |a| < 2^-126
+  return ((unsigned)__double2hiint(a) & 0x7fffffffu) - 0x36900000u < 0x01800000u;
+}
+__device__ __forceinline__ float f32_subnormal(double a) {  // of such an a
+  const unsigned long long b = (unsigned long long)__double_as_longlong(a);
+  const unsigned long long m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
+  const int s = 926 - (int)(b >> 52 & 0x7ffu);  // 30 .. 53: a = m 2^(E - 1075), in units of 2^-149 m 2^-s
+  const unsigned q = (unsigned)(m >> s);
+  const unsigned long long rest = m << (64 - s);
+  const bool up = rest > 1ull << 63 || (rest == 1ull << 63 && (q & 1u));
+  return __uint_as_float((unsigned)(b >> 32) & 0x80000000u | (q + up));
 }
 __device__ __forceinline__ float4 f32x4_rn_any(double a, double b, double c, double d) {
-  auto sub = [](double x) {  // 2^-150 <= |x| < 2^-126
-    return ((unsigned)__double2hiint(x) & 0x7fffffffu) - 0x36900000u < 0x01800000u;
-  };
-  if (sub(a) | sub(b) | sub(c) | sub(d)) return f32x4_cvt(a, b, c, d);
-  return make_float4(f32_rn(a), f32_rn(b), f32_rn(c), f32_rn(d));
+  float4 r = make_float4(f32_rn(a), f32_rn(b), f32_rn(c), f32_rn(d));
+  if (to_f32_subnormal(a) | to_f32_subnormal(b) | to_f32_subnormal(c) | to_f32_subnormal(d)) {
+    if (to_f32_subnormal(a)) r.x = f32_subnormal(a);
+    if (to_f32_subnormal(b)) r.y = f32_subnormal(b);
+    if (to_f32_subnormal(c)) r.z = f32_subnormal(c);
+    if (to_f32_subnormal(d)) r.w = f32_subnormal(d);
+  }
+  return r;
 }
 // FP64 -> normalised pair: the cut high part, the remainder rounded to FP32, renormalised
 // (|lo| <= ulp(hi) / 2); |a - (hi + lo)| is a few 2^-48 |a|.  The remainder a - cut(a) is

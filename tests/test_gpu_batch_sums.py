@@ -128,3 +128,18 @@ def test_interface_blocks_follow_the_batch_not_the_result(U, persistent):
         B.step(2)
         B.sync()
         check(B, slots[0], alone(U, cfg, prims[0], 5))
+
+
+@pytest.mark.parametrize("persistent", [True, False])
+def test_wide_grid_in_a_batch(U, persistent):
+    """On [-20, 20]^2 the pressure ghosts pass through FP32 subnormals."""
+    cfg = I.channel_config(nx=9, ny=4, n_vel=67, vrange=20.0, kn=0.02)
+    prim = prim_of(cfg, 40)
+    with U.Batch(2) as B:
+        B.set_persistent(persistent)
+        s, other = B.admit(cfg), B.admit(warps())
+        B.instance(s).init_maxwellian(*prim)
+        B.instance(other).init_maxwellian(*prim_of(warps(), 41))
+        B.step(4)
+        B.sync()
+        check(B, s, alone(U, cfg, prim, 4))
